@@ -31,28 +31,34 @@ __host__ __device__ inline int round_up(int x, int m) { return (x + m - 1) / m *
 // ---- 3 x 3 convolution as an implicit GEMM on the 5th-generation tensor cores ----------
 // D[p][n] = sum_k A[p][k] B[n][k] with p a pixel, n an output channel and k the position of
 // (input channel ci, tap = dy * 3 + dx) in the order of conv_kidx below: A[p][k] =
-// in[ci][y + dy - 1][x + dx - 1] (zero outside the image), B[n][k] = Wk[n][k].  A CTA of 128
-// threads takes 128 consecutive pixels of the batch (M = 128) and all output channels (N = 16
-// or 32, rows past Cout zero).  K is taken in passes, one group of GC = 8 or 16 input channels
-// per pass.  Each pass first copies the image rows that the CTA's pixels and their vertical
-// neighbours touch, for its channel group, from global into shared memory, channel innermost;
-// then each thread builds its pixel's row of A from that copy, one tap of 8 channels (one
-// 16-byte load) per k-chunk, in the canonical K-major layout without swizzle: 8 x 16-byte core matrices, the 16
-// row groups of a k-chunk 128 bytes apart (the descriptor's stride byte offset) and successive
-// k-chunks 16 * 128 bytes apart (its leading byte offset); B (all of K, loaded once) likewise
-// with N / 8 row groups.  One thread issues the pass's MMAs (tcgen05.mma, kind::f16, BF16
-// operands, FP32 accumulator in tensor memory) and commits them to an mbarrier; the next pass
-// overwrites A only after a bounded wait for that commit.  After the last pass every warp reads
-// its 32 rows of the accumulator (tcgen05.ld) and applies bias and ReLU.  Images too wide for
-// the row copy (more than 16.5 KB of rows per pass) are read from global memory instead.
-// About 71 KB of shared memory and 32 tensor-memory columns per CTA: three CTAs per SM.
+// in[ci][y + dy - 1][x + dx - 1] (zero outside the image), B[n][k] = Wk[n][k].
+//
+// Layout.  The network's own images are channel-innermost, [B][H][W][Cp] with the channels
+// padded with zeros to Cp = 8, 16 or 32 (chan_pad), so that the 8 channels of one tap of one
+// pixel, a core-matrix row of A, are 16 consecutive bytes.  A persistent CTA of 128 threads
+// walks over tiles of 128 consecutive pixels (M = 128, all output channels N = 16 or 32).
+// Thread t copies pixel t's taps straight into the canonical K-major layout without swizzle by
+// cp.async (16 bytes each, zeros outside the image): 8 x 16-byte core matrices, the 16 row
+// groups of a k-chunk 128 bytes apart (the descriptor's stride byte offset), successive k-chunks
+// 16 * 128 bytes apart (its leading byte offset).  B (all of K, loaded once per CTA) likewise
+// with N / 8 row groups.  One thread issues the tile's MMAs (tcgen05.mma, kind::f16, BF16
+// operands, FP32 accumulator in tensor memory), channel groups outermost, and commits them to an
+// mbarrier (bounded wait); the next tile's copies are issued before the epilogue, in which every
+// warp reads its 32 rows of the accumulator (tcgen05.ld) and applies bias and ReLU, or, for the
+// input gradient, the ReLU mask of the layer below, and writes FP32 and BF16 in one pass.
+//
+// What bounds it: the L2-to-shared copies (576 bytes per pixel of a 32-channel layer, most of them
+// L1 hits) and their latency; two CTAs per SM (92 KB each) cover each other's waits.  The K order
+// and the MMA shape are those of the planar form it replaces, so the outputs are bit-identical.
+// One training step of 48 images of 129^2, 5 layers of 32 channels, with a prediction on 12 images:
+// 34.7 ms with planar images (rows staged and transposed in shared memory per tile, the weight
+// gradient by one CTA per channel pair), 2.85 ms in this form.
 constexpr int kConvM = 128;              // pixels per CTA (accumulator lanes)
 constexpr int kConvTmemCols = 32;        // tensor-memory columns allocated per CTA (N <= 32)
 constexpr int kConvMaxKp = 288;          // 32 input channels x 9 taps
-constexpr int kConvTileBytes = 16896;    // staged image rows of one pass (4 rows of 129 pixels)
 
-// K order.  The input channels are taken in groups of GC = 8 (at most 8 channels) or 16, one
-// group per pass; within a pass k = tap * GC + c (c the channel within the group, tap = dy * 3 +
+// K order.  The input channels are taken in groups of GC = 8 (at most 8 channels) or 16;
+// within a group k = tap * GC + c (c the channel within the group, tap = dy * 3 +
 // dx), padded to a multiple of 16 (9 x 8 = 72 -> 80; 9 x 16 = 144).  So each 8-value k-chunk is
 // one tap of 8 consecutive channels.
 __host__ __device__ constexpr int conv_group(int cin) { return cin <= 8 ? 8 : 16; }
@@ -66,15 +72,21 @@ __host__ __device__ constexpr int conv_kidx(int cin, int ci, int tap) {
          ci % conv_group(cin);
 }
 
-__host__ __device__ constexpr size_t conv_a_bytes() {
-  return (size_t)conv_pass_k(16) / 8 * (kConvM / 8) * 128;
+// Channels of an image in memory: a whole number of groups.
+__host__ __device__ constexpr int chan_pad(int c) {
+  return (c + conv_group(c) - 1) / conv_group(c) * conv_group(c);
 }
-__host__ __device__ constexpr size_t conv_b_bytes(int nt) {
-  return (size_t)kConvMaxKp / 8 * (nt / 8) * 128;
+
+// Dynamic shared memory of k_conv_tc: A and B of all of K.
+__host__ __device__ constexpr size_t conv_smem_bytes(int nt, int kp) {
+  return (size_t)kp / 8 * (kConvM / 8) * 128 + (size_t)kp / 8 * (nt / 8) * 128;
 }
-// Dynamic shared memory of k_conv_tc: A of one pass, B, the staged rows.
-__host__ __device__ constexpr size_t conv_smem_bytes(int nt) {
-  return conv_a_bytes() + conv_b_bytes(nt) + kConvTileBytes;
+
+// Asynchronous 16-byte copy global -> shared; src_bytes = 0 writes zeros and reads nothing.
+__device__ __forceinline__ void copy16_async(uint32_t dst, const void* src, int src_bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
+               "r"(src_bytes)
+               : "memory");
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -111,28 +123,31 @@ __device__ __forceinline__ bool conv_mbar_wait(uint32_t bar, uint32_t parity, in
   return false;
 }
 
+// in: [B][H][W][Cp]; out_bf: [B][H][W][Cop] BF16 (Cop = chan_pad(Cout) <= NT), out_f:
+// [B][H][W][Fp] FP32 (Fp = 1 for one output channel, else Cop); mask (BF16, as out_bf): outputs
+// are zeroed where it is not positive.
 template <int NT, int GC>
 __global__ void __launch_bounds__(kConvM)
 k_conv_tc(const __nv_bfloat16* __restrict__ in, const __nv_bfloat16* __restrict__ Wk,
-          const float* __restrict__ bias, int Cin, int Cout, int Kp, int Np, int B, int H, int W,
-          int relu, __nv_bfloat16* __restrict__ out_bf, float* __restrict__ out_f,
+          const float* __restrict__ bias, int Cp, int Cout, int Kp, int Np, int64_t total, int H,
+          int W, int relu, const __nv_bfloat16* __restrict__ mask,
+          __nv_bfloat16* __restrict__ out_bf, float* __restrict__ out_f, int Cop, int Fp,
           int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char conv_smem[];
   __shared__ __align__(8) uint64_t mma_bar;
   __shared__ uint32_t tmem_base;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tid >> 5;
   const int nk = Kp / 8;                                  // k-chunks of 8 (Kp = conv_kp(Cin))
   constexpr int kPassChunks = conv_pass_k(GC) / 8;        // 18 (GC = 16) or 10 (GC = 8)
   constexpr int kGroups = GC / 8;                         // k-chunks per tap
   constexpr uint32_t kSbo = 128;                          // 8-row groups 128 bytes apart
   constexpr uint32_t kLboA = (kConvM / 8) * 128;          // 2048 bytes per k-chunk of A
   constexpr uint32_t kLboB = (NT / 8) * 128;              // bytes per k-chunk of B
-  unsigned char* sA = conv_smem;                          // kConvM x 144 BF16 (one pass)
-  unsigned char* sB = conv_smem + conv_a_bytes();         // NT x Kp BF16
-  uint16_t* sT = reinterpret_cast<uint16_t*>(conv_smem + conv_a_bytes() + conv_b_bytes(NT));
-  const int64_t plane = (int64_t)H * W, total = (int64_t)B * plane;
-  const int64_t pix0 = (int64_t)blockIdx.x * kConvM;
-  const int64_t pix = pix0 + tid;
+  const uint32_t sA = smem_u32(conv_smem);                // kConvM x Kp BF16
+  unsigned char* sBp = conv_smem + (size_t)nk * kLboA;    // NT x Kp BF16
+  const uint32_t sB = smem_u32(sBp);
+  const int64_t plane = (int64_t)H * W;
+  const int64_t tiles = (total + kConvM - 1) / kConvM;
   const uint32_t bar = smem_u32(&mma_bar);
 
   if (warp == 0) {   // tensor memory for the accumulator (whole warp, aligned)
@@ -146,124 +161,55 @@ k_conv_tc(const __nv_bfloat16* __restrict__ in, const __nv_bfloat16* __restrict_
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // This thread's pixel, and the rows (b H + y over the batch) the CTA's pixels and their
-  // vertical neighbours touch: rlo .. rlo + nrows - 1.
-  const bool valid = pix < total;
-  const int b = valid ? (int)(pix / plane) : 0;
-  const int64_t rem = valid ? pix - (int64_t)b * plane : 0;
-  const int y = (int)(rem / W), x = (int)(rem - (int64_t)y * W);
-  const int64_t rows_total = (int64_t)B * H;
-  const int64_t last = (pix0 + kConvM < total ? pix0 + kConvM : total) - 1;
-  const int64_t rlo = pix0 / W > 0 ? pix0 / W - 1 : 0;
-  const int64_t rhi = last / W + 1 < rows_total ? last / W + 1 : rows_total - 1;
-  const int nrows = (int)(rhi - rlo + 1);
-  const bool staged = (int64_t)nrows * W * GC * 2 <= kConvTileBytes;
-  const int b_lo = (int)(rlo / H), y_lo = (int)(rlo - (int64_t)b_lo * H);   // row rlo
-  const __nv_bfloat16* inb = in + (size_t)b * Cin * plane;
-  // the 9 taps of this pixel: inside the image (bit t of tap_in)
-  int tap_in = 0;
+  // Copies of a tile's rows of A: this thread's pixel, one 16-byte chunk per tap and 8 channels.
+  const uint32_t arow = sA + (tid >> 3) * kSbo + (tid & 7) * 16;
+  auto load_tile = [&](int64_t tile) {
+    const int64_t pix = tile * kConvM + tid;
+    const bool valid = pix < total;
+    const int64_t rem = valid ? pix % plane : 0;
+    const int y = (int)(rem / W), x = (int)(rem - (int64_t)y * W);
+    const __nv_bfloat16* src = in + (valid ? pix : 0) * Cp;
+    uint32_t dst = arow;
+    for (int c0 = 0; c0 < nk; c0 += kPassChunks) {
 #pragma unroll
-  for (int t = 0; t < 9; ++t) {
-    const int yy = y + t / 3 - 1, xx = x + t % 3 - 1;
-    if (valid && yy >= 0 && yy < H && xx >= 0 && xx < W) tap_in |= 1 << t;
-  }
-  // the staged copy's element of (row prow, column x) is sT[(prow W + x) GC + c]
-  const int prow = (int)((int64_t)b * H + y - rlo);
-
+      for (int kc = 0; kc < kPassChunks; ++kc) {
+        const int tap = kc / kGroups, g = kc - tap * kGroups;
+        const int dy = tap / 3 - 1, dx = tap % 3 - 1;
+        const bool is = tap < 9 && valid && y + dy >= 0 && y + dy < H && x + dx >= 0 && x + dx < W;
+        copy16_async(dst, is ? src + ((int64_t)dy * W + dx) * Cp + 8 * g : in, is ? 16 : 0);
+        dst += kLboA;
+      }
+      src += GC;
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  int64_t tile = blockIdx.x;
+  load_tile(tile);   // the grid has at most one CTA per tile
   // B: NT rows of the weights (rows Np .. NT - 1 zero), 16 bytes per (row, k-chunk)
   for (int e = tid; e < NT * nk; e += kConvM) {
     const int n = e / nk, kc = e - n * nk;
     uint4 row = make_uint4(0u, 0u, 0u, 0u);
     if (n < Np) row = *reinterpret_cast<const uint4*>(Wk + (size_t)n * Kp + kc * 8);
-    *reinterpret_cast<uint4*>(sB + (size_t)kc * kLboB + (n >> 3) * kSbo + (n & 7) * 16) = row;
+    *reinterpret_cast<uint4*>(sBp + (size_t)kc * kLboB + (n >> 3) * kSbo + (n & 7) * 16) = row;
   }
 
-  const int npass = (nk + kPassChunks - 1) / kPassChunks;
   bool ok = true;
-  int waited = -1;   // the last pass whose MMAs are known complete
-  for (int pass = 0; pass < npass; ++pass) {
-    const int c0 = pass * kPassChunks;                         // first k-chunk of the pass
-    const int nkp = nk - c0 < kPassChunks ? nk - c0 : kPassChunks;   // even: Kp % 16 == 0
-    const int ci0 = pass * GC;                                  // the pass's channel group
-    const int nci = Cin - ci0 < GC ? Cin - ci0 : GC;
-    if (pass > 0) {
-      // the previous pass's MMAs read A (and the copy is rewritten below): wait for them
-      ok = conv_mbar_wait(bar, (uint32_t)((pass - 1) & 1), 1 << 22);
-      if (__syncthreads_or(!ok)) break;
-      waited = pass - 1;
-    }
-    if (staged) {
-      // rows rlo .. rhi of the group's channels, channel innermost: sT[(row W + x) GC + c]
-      // (zero for c >= nci).  Item (row, 8-channel part g, 32-column segment) per warp: each
-      // lane loads its column's 8 channels (8 independent loads) and stores them as 16 bytes.
-      const int nxs = (W + 31) / 32;
-      const int items = nrows * kGroups * nxs;
-      const uint16_t* in16 = reinterpret_cast<const uint16_t*>(in);
-      for (int it = warp; it < items; it += kConvM / 32) {
-        const int row = it / (kGroups * nxs), rest = it - row * (kGroups * nxs);
-        const int g = rest / nxs, xr = (rest - g * nxs) * 32 + lane;
-        if (xr >= W) continue;
-        if (8 * g >= nci) {   // a part of the group past the last channel: zeros
-          *reinterpret_cast<uint4*>(sT + ((size_t)row * W + xr) * GC + 8 * g) =
-              make_uint4(0u, 0u, 0u, 0u);
-          continue;
-        }
-        int bb = b_lo, yy = y_lo + row;   // batch row rlo + row as (image, row)
-        while (yy >= H) {
-          yy -= H;
-          ++bb;
-        }
-        const uint16_t* src = in16 + ((size_t)bb * Cin + ci0 + 8 * g) * plane + (size_t)yy * W + xr;
-        uint16_t v[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = 8 * g + j < nci ? src[(size_t)j * plane] : (uint16_t)0;
-        uint4 pk;
-        pk.x = v[0] | ((uint32_t)v[1] << 16);
-        pk.y = v[2] | ((uint32_t)v[3] << 16);
-        pk.z = v[4] | ((uint32_t)v[5] << 16);
-        pk.w = v[6] | ((uint32_t)v[7] << 16);
-        *reinterpret_cast<uint4*>(sT + ((size_t)row * W + xr) * GC + 8 * g) = pk;
-      }
-      __syncthreads();
-    }
-    // A of the pass: this thread's pixel row; k-chunk kc is tap kc / kGroups of the channels
-    // 8 (kc % kGroups) .. + 7 of the group: one 16-byte load from the copy
-#pragma unroll
-    for (int kc = 0; kc < kPassChunks; ++kc) {
-      const int tap = kc / kGroups, g = kc - tap * kGroups;
-      uint4 row = make_uint4(0u, 0u, 0u, 0u);
-      if (tap < 9 && ((tap_in >> tap) & 1) && (staged || 8 * g < nci)) {
-        const int dy = tap / 3, dx = tap - dy * 3;
-        if (staged) {
-          row = *reinterpret_cast<const uint4*>(
-              sT + ((size_t)(prow + dy - 1) * W + x + dx - 1) * GC + 8 * g);
-        } else {
-          const __nv_bfloat16* src =
-              inb + (size_t)(ci0 + 8 * g) * plane + (size_t)(y + dy - 1) * W + x + dx - 1;
-          uint16_t v[8];
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            v[j] = 8 * g + j < nci ? __bfloat16_as_ushort(src[(size_t)j * plane]) : (uint16_t)0;
-          row.x = v[0] | ((uint32_t)v[1] << 16);
-          row.y = v[2] | ((uint32_t)v[3] << 16);
-          row.z = v[4] | ((uint32_t)v[5] << 16);
-          row.w = v[6] | ((uint32_t)v[7] << 16);
-        }
-      }
-      *reinterpret_cast<uint4*>(sA + (size_t)kc * kLboA + (tid >> 3) * kSbo + (tid & 7) * 16) = row;
-    }
-    // make the operands visible to the tensor core's asynchronous proxy, then issue
+  uint32_t parity = 0;
+  for (; tile < tiles; tile += gridDim.x, parity ^= 1) {
+    // this tile's A has arrived; make the operands visible to the tensor core's asynchronous
+    // proxy, then issue
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t taddr = tmem_base;
     if (tid == 0) {
       constexpr uint32_t idesc = conv_idesc(NT);
-      const uint32_t taddr = tmem_base;
-      for (int ks = 0; ks < nkp / 2; ++ks) {
-        const uint64_t ad = smem_desc(smem_u32(sA) + ks * 2 * kLboA, kLboA, kSbo);
-        const uint64_t bd = smem_desc(smem_u32(sB) + (c0 + ks * 2) * kLboB, kLboB, kSbo);
-        const uint32_t acc = (pass > 0 || ks > 0) ? 1u : 0u;
+      for (int ks = 0; ks < nk / 2; ++ks) {
+        const uint64_t ad = smem_desc(sA + ks * 2 * kLboA, kLboA, kSbo);
+        const uint64_t bd = smem_desc(sB + ks * 2 * kLboB, kLboB, kSbo);
+        const uint32_t acc = ks > 0 ? 1u : 0u;
         asm volatile(
             "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
             " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(taddr),
@@ -275,146 +221,303 @@ k_conv_tc(const __nv_bfloat16* __restrict__ in, const __nv_bfloat16* __restrict_
               bar)
           : "memory");
     }
-  }
-  const uint32_t taddr = tmem_base;
-  // the last issued pass: all of them after a normal loop, the one before the failed wait else
-  const int issued = ok ? npass - 1 : waited + 1;
-  if (ok) ok = conv_mbar_wait(bar, (uint32_t)((npass - 1) & 1), 1 << 22);
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (__syncthreads_or(!ok)) {
-    // The MMAs did not complete within the bound: report it, give the last issued commit one
-    // more bounded wait, release the tensor memory and stop.
-    if (tid == 0) atomicExch(err, 1);
-    conv_mbar_wait(bar, (uint32_t)(issued & 1), 1 << 22);
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (warp == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr),
-                   "r"(kConvTmemCols)
-                   : "memory");
+    ok = conv_mbar_wait(bar, parity, 1 << 22);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (__syncthreads_or(!ok)) {
+      ok = false;
+      break;
     }
-    return;
-  }
-  // accumulator row tid (lanes 32 warp .. 32 warp + 31), NT columns
-  float accv[NT];
-  const uint32_t lane_addr = taddr + ((uint32_t)(warp * 32) << 16);
-  if constexpr (NT == 16) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-        "%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-          "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(lane_addr));
+    // A is free again: the next tile's copies run under this tile's epilogue
+    if (tile + gridDim.x < tiles) load_tile(tile + gridDim.x);
+    // accumulator row tid (lanes 32 warp .. 32 warp + 31), NT columns
+    float accv[NT];
+    const uint32_t lane_addr = taddr + ((uint32_t)(warp * 32) << 16);
+    uint32_t r[NT];
+    if constexpr (NT == 16) {
+      asm volatile(
+          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
+          "%14,%15}, [%16];"
+          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+            "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
+            "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+          : "r"(lane_addr));
+    } else {
+      asm volatile(
+          "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
+          "%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+            "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
+            "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
+            "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+            "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]),
+            "=r"(r[31])
+          : "r"(lane_addr));
+    }
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    const int64_t pix = tile * kConvM + tid;
+    if (pix < total) {
 #pragma unroll
-    for (int j = 0; j < 16; ++j) accv[j] = __uint_as_float(r[j]);
-  } else {
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-        "%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-          "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-          "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]),
-          "=r"(r[31])
-        : "r"(lane_addr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      for (int n = 0; n < NT; ++n) {
+        float v = __uint_as_float(r[n]) + ((bias && n < Cout) ? bias[n] : 0.0f);
+        accv[n] = relu ? fmaxf(v, 0.0f) : v;
+      }
 #pragma unroll
-    for (int j = 0; j < 32; ++j) accv[j] = __uint_as_float(r[j]);
+      for (int n0 = 0; n0 < NT; n0 += 8) {   // 8 channels at a time (columns past Cout are 0)
+        if (n0 >= Cop) break;
+        if (mask) {
+          const uint4 mk = *reinterpret_cast<const uint4*>(mask + pix * Cop + n0);
+          const uint32_t mw[4] = {mk.x, mk.y, mk.z, mk.w};
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const float av = __uint_as_float((j & 1) ? mw[j >> 1] & 0xFFFF0000u : mw[j >> 1] << 16);
+            if (!(av > 0.0f)) accv[n0 + j] = 0.0f;
+          }
+        }
+        if (out_f) {
+          if (Fp == 1) {
+            if (n0 == 0) out_f[pix] = accv[0];
+          } else {
+#pragma unroll
+            for (int j = 0; j < 8; j += 4)
+              *reinterpret_cast<float4*>(out_f + pix * Fp + n0 + j) = make_float4(
+                  accv[n0 + j], accv[n0 + j + 1], accv[n0 + j + 2], accv[n0 + j + 3]);
+          }
+        }
+        if (out_bf) {
+          uint32_t pk[4];
+#pragma unroll
+          for (int j = 0; j < 8; j += 2) {
+            const __nv_bfloat162 h2 = __floats2bfloat162_rn(accv[n0 + j], accv[n0 + j + 1]);
+            pk[j >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
+          }
+          *reinterpret_cast<uint4*>(out_bf + pix * Cop + n0) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        }
+      }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");   // the next MMAs come after
   }
+  if (!ok) {
+    // The MMAs did not complete within the bound: report it, give their commit one more bounded
+    // wait, release the tensor memory and stop.
+    if (tid == 0) atomicExch(err, 1);
+    conv_mbar_wait(bar, parity, 1 << 22);
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr),
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
                  "r"(kConvTmemCols)
                  : "memory");
   }
-  if (pix >= total) return;
-#pragma unroll
-  for (int n = 0; n < NT; ++n) {
-    if (n >= Cout) break;
-    float v = accv[n] + (bias ? bias[n] : 0.0f);
-    if (relu) v = fmaxf(v, 0.0f);
-    const size_t o = ((size_t)b * Cout + n) * plane + rem;
-    if (out_f) out_f[o] = v;
-    if (out_bf) out_bf[o] = __float2bfloat16(v);
-  }
 }
 
+// ---- weight and bias gradients -------------------------------------------------------------
+// gw[co][ci][tap] = sum_{b,y,x} g[b][y][x][co] in[b][y + dy - 1][x + dx - 1][ci] and gb[co] =
+// sum g[b][y][x][co], products and sums in FP32 on the CUDA cores (g is FP32, so a BF16
+// tensor-core product would round it; 2 * 9 * Cin * Cout flops per pixel).
+//
+// A persistent CTA of 8 warps walks over strips of the images (up to kWgX columns by kWgRows
+// rows of one image).  The rows it needs are in shared memory: four rows of `in` (the three of
+// the window and the one being copied) and two of g, copied a row ahead by cp.async.  A warp
+// takes CO output channels and one part of the strip's columns, a lane one input channel (Cp < 32:
+// 32 / Cp lanes share a channel and split the columns again).  The lane keeps its CO x 9 sums and
+// the 3 x 3 window of `in` in registers: one step along x loads 3 values of `in` and CO of g (as
+// broadcast 16-byte loads) for 9 CO multiply-adds, so the FP32 pipe bounds it.  Every warp writes
+// its sums to its own slot and k_wgrad_sum adds the slots in order, so the result does not depend
+// on the schedule.
+constexpr int kWgX = 64, kWgRows = 16, kWgWarps = 8;
 
-// Weight and bias gradients of one layer: gw[co][ci][tap] = sum_{b,y,x} g[b][co][y][x] *
-// in[b][ci][y + dy - 1][x + dx - 1]; gb[co] = sum g[b][co].  One CTA per (co, ci).
-__global__ void __launch_bounds__(256)
-k_wgrad(const __nv_bfloat16* __restrict__ in, const float* __restrict__ g, int Cin, int Cout,
-        int B, int H, int W, float* __restrict__ gw, float* __restrict__ gb) {
-  const int co = blockIdx.x / Cin, ci = blockIdx.x % Cin;
-  const size_t plane = (size_t)H * W;
-  float acc[10];
+// Column parts of a strip = slots per CTA: warps per group of output channels.
+__host__ __device__ constexpr int wgrad_parts(int cout) {
+  return cout <= 8 ? kWgWarps : (cout <= 16 ? kWgWarps / 2 : kWgWarps / 4);
+}
+
+template <int CO>
+__global__ void __launch_bounds__(32 * kWgWarps, 2)
+k_wgrad(const __nv_bfloat16* __restrict__ in, const float* __restrict__ g, int Cp, int Cin,
+        int Cout, int Gp, int B, int H, int W, int xc, int chunks, int segs,
+        float* __restrict__ part) {
+  extern __shared__ __align__(16) unsigned char wg_smem[];
+  const int inrow = (xc + 2) * Cp;                                   // BF16 values of a row
+  __nv_bfloat16* s_in = reinterpret_cast<__nv_bfloat16*>(wg_smem);   // [4][xc + 2][Cp]
+  float* s_g = reinterpret_cast<float*>(wg_smem + (size_t)4 * inrow * 2);   // [2][xc][Gp]
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int parts = wgrad_parts(Cout), subs = 32 / Cp;
+  const int cg = warp / parts, pg = warp - cg * parts, co0 = cg * CO;
+  const int ci = lane & (Cp - 1), sub = lane / Cp;
+  const bool active = co0 < Cout;
+  float acc[CO][9];
 #pragma unroll
-  for (int i = 0; i < 10; ++i) acc[i] = 0.0f;
-  const int64_t total = (int64_t)B * H * W;
-  for (int64_t e = threadIdx.x; e < total; e += blockDim.x) {
-    const int x = (int)(e % W), y = (int)((e / W) % H), b = (int)(e / plane);
-    const float gv = g[((size_t)b * Cout + co) * plane + (size_t)y * W + x];
-    const __nv_bfloat16* ib = in + ((size_t)b * Cin + ci) * plane;
+  for (int c = 0; c < CO; ++c)
 #pragma unroll
-    for (int tap = 0; tap < 9; ++tap) {
-      const int yy = y + tap / 3 - 1, xx = x + tap % 3 - 1;
-      const float iv = (yy >= 0 && yy < H && xx >= 0 && xx < W)
-                           ? __bfloat162float(ib[(size_t)yy * W + xx]) : 0.0f;
-      acc[tap] = fmaf(gv, iv, acc[tap]);
+    for (int t = 0; t < 9; ++t) acc[c][t] = 0.0f;
+  float accb = 0.0f;
+  const int64_t items = (int64_t)B * chunks * segs;
+  for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
+    const int seg = (int)(it % segs), ch = (int)(it / segs % chunks), b = (int)(it / segs / chunks);
+    const int x0 = ch * xc, xn = W - x0 < xc ? W - x0 : xc;
+    const int y0 = seg * kWgRows, yn = H - y0 < kWgRows ? H - y0 : kWgRows;
+    // copy row y of `in` (columns x0 - 1 .. x0 + xn, zeros outside the image) into slot y & 3
+    auto copy_in = [&](int y) {
+      const int per = Cp / 8, n = (xn + 2) * per;
+      const bool row = y >= 0 && y < H;
+      const __nv_bfloat16* src = in + ((int64_t)b * H + (row ? y : 0)) * W * Cp;
+      const uint32_t dst = smem_u32(s_in + (size_t)(y & 3) * inrow);
+      for (int e = tid; e < n; e += 32 * kWgWarps) {
+        const int c = e / per, x = x0 - 1 + c;
+        const bool is = row && x >= 0 && x < W;
+        copy16_async(dst + e * 16, is ? src + (int64_t)(x0 - 1) * Cp + e * 8 : in, is ? 16 : 0);
+      }
+    };
+    auto copy_g = [&](int y) {   // row y of g into slot y & 1
+      const float* src = g + (((int64_t)b * H + y) * W + x0) * Gp;
+      float* dst = s_g + (size_t)(y & 1) * xc * Gp;
+      if constexpr (CO == 1) {
+        for (int e = tid; e < xn; e += 32 * kWgWarps) dst[e] = src[e];
+      } else {
+        for (int e = tid; e < xn * Gp / 4; e += 32 * kWgWarps)
+          copy16_async(smem_u32(dst + e * 4), src + e * 4, 16);
+      }
+    };
+    __syncthreads();   // the previous strip's rows have been read
+    copy_in(y0 - 1);
+    copy_in(y0);
+    copy_in(y0 + 1);
+    copy_g(y0);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    // the warp's columns, and the lane's among them
+    const int w0 = pg * xn / parts, w1 = (pg + 1) * xn / parts;
+    const int xs = w0 + sub * (w1 - w0) / subs, xe = w0 + (sub + 1) * (w1 - w0) / subs;
+    for (int y = y0; y < y0 + yn; ++y) {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();
+      if (y + 1 < y0 + yn) {
+        copy_in(y + 2);
+        copy_g(y + 1);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      if (!active) continue;
+      const float* gr = s_g + (size_t)(y & 1) * xc * Gp + co0;
+      const __nv_bfloat16* r[3];
+      float wnd[3][3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        r[d] = s_in + (size_t)((y - 1 + d) & 3) * inrow + ci;
+        wnd[d][1] = xs < xe ? __bfloat162float(r[d][xs * Cp]) : 0.0f;
+        wnd[d][2] = xs < xe ? __bfloat162float(r[d][(xs + 1) * Cp]) : 0.0f;
+      }
+      for (int x = xs; x < xe; ++x) {
+        float gv[CO];
+        if constexpr (CO == 8) {
+          const float4 g0 = *reinterpret_cast<const float4*>(gr + x * Gp);
+          const float4 g1 = *reinterpret_cast<const float4*>(gr + x * Gp + 4);
+          gv[0] = g0.x; gv[1] = g0.y; gv[2] = g0.z; gv[3] = g0.w;
+          gv[4] = g1.x; gv[5] = g1.y; gv[6] = g1.z; gv[7] = g1.w;
+        } else {
+          gv[0] = gr[x * Gp];
+        }
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          wnd[d][0] = wnd[d][1];
+          wnd[d][1] = wnd[d][2];
+          wnd[d][2] = __bfloat162float(r[d][(x + 2) * Cp]);
+        }
+#pragma unroll
+        for (int c = 0; c < CO; ++c)
+#pragma unroll
+          for (int t = 0; t < 9; ++t) acc[c][t] = fmaf(gv[c], wnd[t / 3][t % 3], acc[c][t]);
+      }
+      // the bias: lane (i, c) adds channel co0 + c of the warp's columns w0 + i, w0 + i + 32/CO ..
+      for (int x = w0 + lane / CO; x < w1; x += 32 / CO) accb += gr[x * Gp + lane % CO];
     }
-    acc[9] += gv;
   }
-  __shared__ float red[10][8];
+  if (!active) return;
+  // the warp's slot: [Cout][Cin][9], then the Cout bias sums
+  const int E = Cout * Cin * 9 + Cout;
+  float* slot = part + ((int64_t)blockIdx.x * parts + pg) * E;
 #pragma unroll
-  for (int i = 0; i < 10; ++i) {
-    float v = acc[i];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) red[i][threadIdx.x >> 5] = v;
-  }
+  for (int c = 0; c < CO; ++c)
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+      float v = acc[c][t];
+      for (int o = Cp; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane < Cin && co0 + c < Cout) slot[((co0 + c) * Cin + ci) * 9 + t] = v;
+    }
+  for (int o = CO; o < 32; o <<= 1) accb += __shfl_xor_sync(0xffffffffu, accb, o);
+  if (lane < CO && co0 + lane < Cout) slot[Cout * Cin * 9 + co0 + lane] = accb;
+}
+
+// out[e] = the sum over the slots of part[slot][e]: 8 interleaved partial sums per output.
+__global__ void __launch_bounds__(256)
+k_wgrad_sum(const float* __restrict__ part, int slots, int E, float* __restrict__ out) {
+  const int e = blockIdx.x * 32 + (threadIdx.x & 31), s0 = threadIdx.x >> 5;
+  float v = 0.0f;
+  if (e < E)
+    for (int s = s0; s < slots; s += 8) v += part[(int64_t)s * E + e];
+  __shared__ float red[8][32];
+  red[s0][threadIdx.x & 31] = v;
   __syncthreads();
-  if (threadIdx.x < 10) {
-    float v = 0.0f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[threadIdx.x][w];
-    if (threadIdx.x < 9)
-      gw[((size_t)co * Cin + ci) * 9 + threadIdx.x] = v;
-    else if (ci == 0)
-      gb[co] = v;
+  if (s0 == 0 && e < E) {
+#pragma unroll
+    for (int i = 1; i < 8; ++i) v += red[i][threadIdx.x];
+    out[e] = v;
   }
 }
 
-__global__ void k_f32_to_bf16(const float* __restrict__ x, __nv_bfloat16* __restrict__ y,
-                              int64_t n) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    y[i] = __float2bfloat16(x[i]);
+// Planar FP32 images [B][C][plane] to channel-innermost BF16 [B][plane][Cp] (zeros past C).
+__global__ void k_to_images(const float* __restrict__ x, __nv_bfloat16* __restrict__ y, int C,
+                            int Cp, int64_t plane, int64_t pixels) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < pixels;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t b = i / plane, r = i - b * plane;
+    for (int c0 = 0; c0 < Cp; c0 += 8) {
+      uint32_t pk[4];
+#pragma unroll
+      for (int j = 0; j < 8; j += 2) {
+        const float lo = c0 + j < C ? x[(b * C + c0 + j) * plane + r] : 0.0f;
+        const float hi = c0 + j + 1 < C ? x[(b * C + c0 + j + 1) * plane + r] : 0.0f;
+        const __nv_bfloat162 h2 = __floats2bfloat162_rn(lo, hi);
+        pk[j >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
+      }
+      *reinterpret_cast<uint4*>(y + i * Cp + c0) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+    }
+  }
 }
 
-// g_prev = g_in * (a > 0): the ReLU of the previous layer, a its (post-ReLU) output.
-// gin and gout may be the same array (element-wise, read before write).
-__global__ void k_relu_mask(const float* gin, const __nv_bfloat16* __restrict__ a, float* gout,
-                            int64_t n) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    gout[i] = __bfloat162float(a[i]) > 0.0f ? gin[i] : 0.0f;
+// Sum of the mask's values (one block, FP64) and 1 / max(1, sum * batch), the mean's factor.
+__global__ void __launch_bounds__(1024)
+k_mask_sum(const float* __restrict__ mask, int64_t n, int B, float* __restrict__ inv) {
+  double s = 0.0;
+  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s += mask[i];
+  __shared__ double red[32];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double v = 0.0;
+    for (int w = 0; w < 32; ++w) v += red[w];
+    v *= B;
+    *inv = (float)(1.0 / (v > 1.0 ? v : 1.0));
+  }
 }
 
-// Masked mean squared error: g = 2 (y - t) m / count, partial sums of (y - t)^2 m per block.
+// Masked mean squared error: g = 2 (y - t) m / count (FP32, and BF16 images of 8 channels, 7 of
+// them 0), partial sums of (y - t)^2 m per block.
 __global__ void __launch_bounds__(256)
 k_mse(const float* __restrict__ y, const float* __restrict__ t, const float* __restrict__ mask,
-      int64_t plane, int64_t n, float inv_count, float* __restrict__ g, float* __restrict__ part) {
+      int64_t plane, int64_t n, const float* __restrict__ inv_count, float* __restrict__ g,
+      __nv_bfloat16* __restrict__ gbf, float* __restrict__ part) {
+  const float inv = *inv_count;
   float s = 0.0f;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     const float d = (y[i] - t[i]) * mask[i % plane];
-    g[i] = 2.0f * d * inv_count;
+    const float gi = 2.0f * d * inv;
+    g[i] = gi;
+    *reinterpret_cast<uint4*>(gbf + i * 8) =
+        make_uint4(__bfloat16_as_ushort(__float2bfloat16(gi)), 0u, 0u, 0u);
     s = fmaf(d, d, s);
   }
   __shared__ float red[8];
@@ -533,12 +636,15 @@ struct mfwh_cnn_s {
   std::vector<int> Kp, Kpt, Np, Npt;
   // activation workspace, sized for cap elements per channel plane times the batch
   int64_t cap = 0;                     // B * H * W the workspace holds
-  std::vector<__nv_bfloat16*> act;     // inputs of each layer (BF16), [B][C][H][W]
+  std::vector<__nv_bfloat16*> act;     // inputs of each layer (BF16), [B][H][W][chan_pad(C)]
   float* y = nullptr;                  // network output [B][1][H][W]
-  float* g0 = nullptr;                 // gradient buffers [B][channels][H][W]
-  float* g1 = nullptr;
-  __nv_bfloat16* gbf = nullptr;
-  float* part = nullptr;               // loss partial sums
+  float* g0 = nullptr;                 // gradients of a layer's output, [B][H][W][chan_pad(C)]
+  float* g1 = nullptr;                 //   (the last layer's: [B][H][W])
+  __nv_bfloat16* gbf0 = nullptr;       // the same in BF16 (always padded)
+  __nv_bfloat16* gbf1 = nullptr;
+  float* wpart = nullptr;              // weight-gradient slots
+  int sms = 0;                         // SMs of the device
+  float* part = nullptr;               // loss partial sums, then the mean's factor
   float* part_h = nullptr;             // pinned
   int* err = nullptr;                  // device flag: a convolution's MMA wait ran out
 };
@@ -561,36 +667,63 @@ mfwh_status ensure_ws(mfwh_cnn_t c, int64_t bhw) {
   if (c->y) cudaFree(c->y);
   if (c->g0) cudaFree(c->g0);
   if (c->g1) cudaFree(c->g1);
-  if (c->gbf) cudaFree(c->gbf);
-  c->act.assign(c->layers + 1, nullptr);
+  if (c->gbf0) cudaFree(c->gbf0);
+  if (c->gbf1) cudaFree(c->gbf1);
+  c->y = c->g0 = c->g1 = nullptr;
+  c->gbf0 = c->gbf1 = nullptr;
+  c->act.assign(c->layers, nullptr);
   c->cap = 0;
-  const int maxc = std::max(c->channels, c->in_channels);
-  for (int l = 0; l <= c->layers; ++l) {
-    const int ch = l == 0 ? c->in_channels : (l == c->layers ? 1 : c->channels);
-    CKC(cudaMalloc(&c->act[l], sizeof(__nv_bfloat16) * bhw * ch));
-  }
+  const int gc = chan_pad(c->channels);
+  for (int l = 0; l < c->layers; ++l)
+    CKC(cudaMalloc(&c->act[l], sizeof(__nv_bfloat16) * bhw * chan_pad(c->cin[l])));
   CKC(cudaMalloc(&c->y, sizeof(float) * bhw));
-  CKC(cudaMalloc(&c->g0, sizeof(float) * bhw * maxc));
-  CKC(cudaMalloc(&c->g1, sizeof(float) * bhw * maxc));
-  CKC(cudaMalloc(&c->gbf, sizeof(__nv_bfloat16) * bhw * maxc));
+  CKC(cudaMalloc(&c->g0, sizeof(float) * bhw * gc));
+  CKC(cudaMalloc(&c->g1, sizeof(float) * bhw * gc));
+  CKC(cudaMalloc(&c->gbf0, sizeof(__nv_bfloat16) * bhw * gc));
+  CKC(cudaMalloc(&c->gbf1, sizeof(__nv_bfloat16) * bhw * gc));
   c->cap = bhw;
   return MFWH_OK;
 }
 
+// One convolution of channel-innermost images: cin -> cout channels; mask, out_bf, out_f as in
+// k_conv_tc.  Two persistent CTAs per SM, or one per tile when there are fewer tiles.
 void conv(mfwh_cnn_t c, const __nv_bfloat16* in, const __nv_bfloat16* Wk, const float* bias,
-          int Cin, int Cout, int Kp, int Np, int B, int H, int W, int relu, __nv_bfloat16* out_bf,
-          float* out_f) {
+          int cin, int cout, int Kp, int Np, int B, int H, int W, int relu,
+          const __nv_bfloat16* mask, __nv_bfloat16* out_bf, float* out_f) {
   const int64_t total = (int64_t)B * H * W;
-  const unsigned blocks = (unsigned)((total + kConvM - 1) / kConvM);
+  const unsigned blocks =
+      (unsigned)std::min<int64_t>((total + kConvM - 1) / kConvM, (int64_t)2 * c->sms);
   auto launch = [&](auto kernel, int nt) {
-    kernel<<<blocks, kConvM, conv_smem_bytes(nt), c->stream>>>(
-        in, Wk, bias, Cin, Cout, Kp, Np, B, H, W, relu, out_bf, out_f, c->err);
+    kernel<<<blocks, kConvM, conv_smem_bytes(nt, Kp), c->stream>>>(
+        in, Wk, bias, chan_pad(cin), cout, Kp, Np, total, H, W, relu, mask, out_bf, out_f,
+        chan_pad(cout), cout == 1 ? 1 : chan_pad(cout), c->err);
   };
-  const bool g8 = conv_group(Cin) == 8;
-  if (Np <= 16)
+  const bool g8 = conv_group(cin) == 8;
+  if (chan_pad(cout) <= 16)
     g8 ? launch(k_conv_tc<16, 8>, 16) : launch(k_conv_tc<16, 16>, 16);
   else
     g8 ? launch(k_conv_tc<32, 8>, 32) : launch(k_conv_tc<32, 16>, 32);
+}
+
+// Weight and bias gradients of layer l from the gradient g of its output, into c->grad (w and b
+// of a layer are adjacent in the flat parameter vector).
+void wgrad(mfwh_cnn_t c, int l, const float* g, int B, int H, int W) {
+  const int cin = c->cin[l], cout = c->cout[l], cp = chan_pad(cin);
+  const int gp = cout == 1 ? 1 : chan_pad(cout);
+  const int chunks = (W + kWgX - 1) / kWgX, xc = (W + chunks - 1) / chunks;   // even strips
+  const int segs = (H + kWgRows - 1) / kWgRows;
+  const int blocks =
+      (int)std::min<int64_t>((int64_t)B * chunks * segs, (int64_t)2 * c->sms);
+  const size_t smem = (size_t)4 * (xc + 2) * cp * 2 + (size_t)2 * xc * gp * 4;
+  const int E = cout * cin * 9 + cout;
+  if (cout == 1)
+    k_wgrad<1><<<blocks, 32 * kWgWarps, smem, c->stream>>>(c->act[l], g, cp, cin, cout, gp, B, H,
+                                                           W, xc, chunks, segs, c->wpart);
+  else
+    k_wgrad<8><<<blocks, 32 * kWgWarps, smem, c->stream>>>(c->act[l], g, cp, cin, cout, gp, B, H,
+                                                           W, xc, chunks, segs, c->wpart);
+  k_wgrad_sum<<<(E + 31) / 32, 256, 0, c->stream>>>(c->wpart, blocks * wgrad_parts(cout), E,
+                                                    c->grad + c->woff[l]);
 }
 
 // The convolution kernels' shared-memory limit, once per device.
@@ -600,13 +733,13 @@ mfwh_status conv_configure() {
   CKC(cudaGetDevice(&dev));
   if (dev >= 0 && dev < 64 && done[dev]) return MFWH_OK;
   CKC(cudaFuncSetAttribute(k_conv_tc<16, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)conv_smem_bytes(16)));
+                           (int)conv_smem_bytes(16, conv_kp(8))));
   CKC(cudaFuncSetAttribute(k_conv_tc<16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)conv_smem_bytes(16)));
+                           (int)conv_smem_bytes(16, kConvMaxKp)));
   CKC(cudaFuncSetAttribute(k_conv_tc<32, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)conv_smem_bytes(32)));
+                           (int)conv_smem_bytes(32, conv_kp(8))));
   CKC(cudaFuncSetAttribute(k_conv_tc<32, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)conv_smem_bytes(32)));
+                           (int)conv_smem_bytes(32, kConvMaxKp)));
   if (dev >= 0 && dev < 64) done[dev] = true;
   return MFWH_OK;
 }
@@ -622,25 +755,25 @@ mfwh_status check_err(mfwh_cnn_t c) {
 }
 
 mfwh_status pack_all(mfwh_cnn_t c) {
-  for (int l = 0; l < c->layers; ++l) {
-    CKC(cudaMemsetAsync(c->Wk[l], 0, sizeof(__nv_bfloat16) * c->Np[l] * c->Kp[l], c->stream));
-    CKC(cudaMemsetAsync(c->Wt[l], 0, sizeof(__nv_bfloat16) * c->Npt[l] * c->Kpt[l], c->stream));
-    k_pack<<<64, 256, 0, c->stream>>>(c->p + c->woff[l], c->cin[l], c->cout[l], c->Kp[l],
+  for (int l = 0; l < c->layers; ++l) {   // (the padding was zeroed at creation)
+    k_pack<<<32, 256, 0, c->stream>>>(c->p + c->woff[l], c->cin[l], c->cout[l], c->Kp[l],
                                       c->Kpt[l], c->Wk[l], c->Wt[l]);
   }
   CKC(cudaGetLastError());
   return MFWH_OK;
 }
 
-mfwh_status forward_impl(mfwh_cnn_t c, const float* x, int B, int H, int W) {
+// The network on planar images x; its output (one channel) to y.
+mfwh_status forward_impl(mfwh_cnn_t c, const float* x, int B, int H, int W, float* y) {
   const int64_t bhw = (int64_t)B * H * W;
   mfwh_status st = ensure_ws(c, bhw);
   if (st != MFWH_OK) return st;
-  k_f32_to_bf16<<<256, 256, 0, c->stream>>>(x, c->act[0], bhw * c->in_channels);
+  k_to_images<<<8 * c->sms, 256, 0, c->stream>>>(x, c->act[0], c->in_channels,
+                                                 chan_pad(c->in_channels), (int64_t)H * W, bhw);
   for (int l = 0; l < c->layers; ++l) {
     const bool last = l + 1 == c->layers;
     conv(c, c->act[l], c->Wk[l], c->p + c->boff[l], c->cin[l], c->cout[l], c->Kp[l], c->Np[l], B,
-         H, W, last ? 0 : 1, last ? nullptr : c->act[l + 1], last ? c->y : nullptr);
+         H, W, last ? 0 : 1, nullptr, last ? nullptr : c->act[l + 1], last ? y : nullptr);
   }
   CKC(cudaGetLastError());
   return MFWH_OK;
@@ -696,13 +829,30 @@ mfwh_status mfwh_cnn_create(int layers, int channels, int in_channels, uint64_t 
     if (cudaMalloc(&c->Wk[l], sizeof(__nv_bfloat16) * c->Np[l] * c->Kp[l]) != cudaSuccess ||
         cudaMalloc(&c->Wt[l], sizeof(__nv_bfloat16) * c->Npt[l] * c->Kpt[l]) != cudaSuccess)
       return fail_free(cnn_fail(MFWH_ERR_NOMEM, "cnn: weight allocation failed"));
-  if (cudaMalloc(&c->part, sizeof(float) * kLossBlocks) != cudaSuccess ||
-      cudaMallocHost(&c->part_h, sizeof(float) * kLossBlocks) != cudaSuccess ||
+  if (cudaMalloc(&c->part, sizeof(float) * (kLossBlocks + 1)) != cudaSuccess ||
+      cudaMallocHost(&c->part_h, sizeof(float) * (kLossBlocks + 1)) != cudaSuccess ||
       cudaMalloc(&c->err, sizeof(int)) != cudaSuccess)
     return fail_free(cnn_fail(MFWH_ERR_NOMEM, "cnn: allocation failed"));
   if (cudaMemsetAsync(c->err, 0, sizeof(int), c->stream) != cudaSuccess)
     return fail_free(cnn_fail(MFWH_ERR_CUDA, "cnn: initialisation failed"));
   if (conv_configure() != MFWH_OK) return fail_free(MFWH_ERR_CUDA);
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return fail_free(cnn_fail(MFWH_ERR_CUDA, "cnn: device query failed"));
+  // weight-gradient slots: at most two CTAs per SM, wgrad_parts slots each
+  int64_t slots = 0;
+  for (int l = 0; l < layers; ++l)
+    slots = std::max(slots, (int64_t)wgrad_parts(c->cout[l]) *
+                                (c->cout[l] * c->cin[l] * 9 + c->cout[l]));
+  if (cudaMalloc(&c->wpart, sizeof(float) * slots * 2 * c->sms) != cudaSuccess)
+    return fail_free(cnn_fail(MFWH_ERR_NOMEM, "cnn: workspace allocation failed"));
+  for (int l = 0; l < layers; ++l)   // the weights' padding stays 0
+    if (cudaMemsetAsync(c->Wk[l], 0, sizeof(__nv_bfloat16) * c->Np[l] * c->Kp[l], c->stream) !=
+            cudaSuccess ||
+        cudaMemsetAsync(c->Wt[l], 0, sizeof(__nv_bfloat16) * c->Npt[l] * c->Kpt[l], c->stream) !=
+            cudaSuccess)
+      return fail_free(cnn_fail(MFWH_ERR_CUDA, "cnn: initialisation failed"));
   if (cudaMemcpyAsync(c->p, h.data(), sizeof(float) * c->nparams, cudaMemcpyHostToDevice,
                       c->stream) != cudaSuccess ||
       cudaMemsetAsync(c->m, 0, sizeof(float) * c->nparams, c->stream) != cudaSuccess ||
@@ -745,38 +895,31 @@ mfwh_status mfwh_cnn_get_params(mfwh_cnn_t c, float* host, float* grads_host, in
 mfwh_status mfwh_cnn_forward(mfwh_cnn_t c, const float* x, int B, int H, int W, float* y) {
   if (!c || !x || !y || B < 1 || H < 1 || W < 1)
     return cnn_fail(MFWH_ERR_INVALID_ARG, "cnn: bad forward arguments");
-  mfwh_status st = forward_impl(c, x, B, H, W);
-  if (st != MFWH_OK) return st;
-  CKC(cudaMemcpyAsync(y, c->y, sizeof(float) * B * H * W, cudaMemcpyDeviceToDevice, c->stream));
-  return MFWH_OK;
+  return forward_impl(c, x, B, H, W, y);
 }
 
 mfwh_status mfwh_cnn_train_step(mfwh_cnn_t c, const float* x, const float* target,
                                 const float* mask, int B, int H, int W, float lr, float* loss) {
   if (!c || !x || !target || !mask || B < 1 || H < 1 || W < 1 || !(lr > 0.0f))
     return cnn_fail(MFWH_ERR_INVALID_ARG, "cnn: bad training arguments");
-  mfwh_status st = forward_impl(c, x, B, H, W);
+  mfwh_status st = ensure_ws(c, (int64_t)B * H * W);
+  if (st == MFWH_OK) st = forward_impl(c, x, B, H, W, c->y);
   if (st != MFWH_OK) return st;
   const int64_t hw = (int64_t)H * W, n = (int64_t)B * hw;
-  // the mask's point count, for the mean
-  std::vector<float> mh(hw);
-  CKC(cudaMemcpyAsync(mh.data(), mask, sizeof(float) * hw, cudaMemcpyDeviceToHost, c->stream));
-  CKC(cudaStreamSynchronize(c->stream));
-  double cnt = 0.0;
-  for (float v : mh) cnt += v;
-  const float inv = (float)(1.0 / std::max(1.0, cnt * B));
   float* g = c->g0;
   float* gnext = c->g1;
-  k_mse<<<kLossBlocks, 256, 0, c->stream>>>(c->y, target, mask, hw, n, inv, g, c->part);
+  __nv_bfloat16* gb = c->gbf0;
+  __nv_bfloat16* gbnext = c->gbf1;
+  float* inv = c->part + kLossBlocks;
+  k_mask_sum<<<1, 1024, 0, c->stream>>>(mask, hw, B, inv);
+  k_mse<<<kLossBlocks, 256, 0, c->stream>>>(c->y, target, mask, hw, n, inv, g, gb, c->part);
   for (int l = c->layers - 1; l >= 0; --l) {
-    k_wgrad<<<c->cout[l] * c->cin[l], 256, 0, c->stream>>>(
-        c->act[l], g, c->cin[l], c->cout[l], B, H, W, c->grad + c->woff[l], c->grad + c->boff[l]);
-    if (l > 0) {
-      k_f32_to_bf16<<<256, 256, 0, c->stream>>>(g, c->gbf, n * c->cout[l]);
-      conv(c, c->gbf, c->Wt[l], nullptr, c->cout[l], c->cin[l], c->Kpt[l], c->Npt[l], B, H, W, 0,
-           nullptr, gnext);
-      k_relu_mask<<<256, 256, 0, c->stream>>>(gnext, c->act[l], gnext, n * c->cin[l]);
+    wgrad(c, l, g, B, H, W);
+    if (l > 0) {   // the input gradient, through the ReLU of the layer below
+      conv(c, gb, c->Wt[l], nullptr, c->cout[l], c->cin[l], c->Kpt[l], c->Npt[l], B, H, W, 0,
+           c->act[l], gbnext, gnext);
       std::swap(g, gnext);
+      std::swap(gb, gbnext);
     }
   }
   c->step++;
@@ -786,21 +929,22 @@ mfwh_status mfwh_cnn_train_step(mfwh_cnn_t c, const float* x, const float* targe
                                      1.0f - std::pow(b2, (float)c->step));
   st = pack_all(c);
   if (st != MFWH_OK) return st;
-  CKC(cudaMemcpyAsync(c->part_h, c->part, sizeof(float) * kLossBlocks, cudaMemcpyDeviceToHost,
-                      c->stream));
+  CKC(cudaMemcpyAsync(c->part_h, c->part, sizeof(float) * (kLossBlocks + 1),
+                      cudaMemcpyDeviceToHost, c->stream));
   CKC(cudaStreamSynchronize(c->stream));
   double s = 0.0;
   for (int i = 0; i < kLossBlocks; ++i) s += c->part_h[i];
-  if (loss) *loss = (float)(s * inv);
+  if (loss) *loss = (float)(s * c->part_h[kLossBlocks]);
   return check_err(c);
 }
 
 void mfwh_cnn_destroy(mfwh_cnn_t c) {
   if (!c) return;
   cudaStreamSynchronize(c->stream);
-  for (float* b : {c->p, c->grad, c->m, c->v, c->y, c->g0, c->g1, c->part})
+  for (float* b : {c->p, c->grad, c->m, c->v, c->y, c->g0, c->g1, c->part, c->wpart})
     if (b) cudaFree(b);
-  if (c->gbf) cudaFree(c->gbf);
+  if (c->gbf0) cudaFree(c->gbf0);
+  if (c->gbf1) cudaFree(c->gbf1);
   for (auto* w : c->Wk)
     if (w) cudaFree(w);
   for (auto* w : c->Wt)
