@@ -49,9 +49,8 @@ typedef enum {
   MFWH_ERR_SPURIOUS = 6,      /* GMRES converged but the Helmholtz residual check failed */
   MFWH_ERR_NONFINITE = 7,     /* NaN or Inf in an iterate or residual */
   MFWH_ERR_TIMEOUT = 8        /* a bounded wait inside a kernel ran out: a grid-barrier wait of
-                                 the implicit step kernel (limit: mfwh_set_wait_limit) or a
-                                 tile's tensor copy of the FP32 blocked kernel; that wave solve's
-                                 results are invalid, the handle stays usable */
+                                 the implicit step kernel (limit: mfwh_set_wait_limit); that wave
+                                 solve's results are invalid, the handle stays usable */
 } mfwh_status;
 
 enum { MFWH_FILTER_OPTIMIZED = 0, MFWH_FILTER_TRADITIONAL = 1, MFWH_FILTER_USER = 2 };
@@ -117,9 +116,8 @@ typedef struct {
                                 filter of eq. vkUpdate; MFWH_UPDATE_EXPLICIT: B_mm V_m^{k+1} =
                                 q_m - sum_{j != m} B_mj V_j^k, the explicit filter of the
                                 footnote to eq. filterII (same fixed point) */
-  int tile_shape;            /* FP32 blocked kernel tile: 0 = 32x32, 512 threads (default);
-                                1 = 32x64, 512 threads; 2 = 64x64, 1024 threads (halved in
-                                y above 8 frequencies).  FP64 blocked kernel tile (points x by
+  int tile_shape;            /* FP32: 0, 1 or 2, no effect (the 2D blocked kernel has one tile:
+                                128x64 points with the halo).  FP64 blocked kernel tile (points x by
                                 y): 0 = 32x64, 512 threads; 1 = 32x32, 512 threads; 2 = 32x48,
                                 512 threads; 3 = 32x32, 256 threads, two CTAs per SM; 4 =
                                 32x16, 512 threads, two CTAs per SM; 5 = 32x16 tiles stepped by
@@ -342,7 +340,7 @@ mfwh_status mfwh_solve_batch_graph(const mfwh_handle_t* handles, int count, int 
 
 /* Autotuner for the blocked wave kernels.  Times the first steps (at most 96) of a
  * homogeneous wave solve of prob on the current device for each candidate temporal depth and
- * tile shape (FP32, 2D: depths 4, 8, 16 x tile shapes 0, 1, 2; FP64, 2D: depth 1, and depths
+ * tile shape (FP32, 2D: depths 4, 8, 16; FP64, 2D: depth 1, and depths
  * 4, 8 x tile shapes 1, 3; FP32, 3D: depths 1, 2, 4; FP64 3D, fourth order and c^2 fields:
  * depth 1), keeping the fastest:
  * *time_block and *tile_shape receive it, *ms_per_step

@@ -125,7 +125,7 @@ struct mfwh_handle_s {
   int nf = 0;
   int64_t P = 0, N = 0;            // points per grid function, nf * points
   int64_t PW = 0;                   // entries of one FP32 wave-level array (padded rows in 2D)
-  int* d_err = nullptr;             // device flag of the blocked FP32 kernel (tensor copy timeout)
+  int* d_err = nullptr;             // device flag of the implicit step kernel (barrier timeout)
   double inv_h2[3] = {0, 0, 0};
   double omega2[MFWH_MAX_NF] = {};
   double* f = nullptr;              // forcing [nf][P]
@@ -202,7 +202,7 @@ void reset_timing(mfwh_handle_t h) {
 }
 
 mfwh_status collect_timing(mfwh_handle_t h) {
-  if (h->d_err) {   // a bounded wait of a wave kernel ran out (1: FP32 tile copy; 2: barrier)
+  if (h->d_err) {   // a bounded barrier wait of the implicit step kernel ran out
     CK(cudaMemcpyAsync(h->pinned, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     int flag = 0;
@@ -211,9 +211,7 @@ mfwh_status collect_timing(mfwh_handle_t h) {
       CK(cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream));
       if (h->d_bar) CK(cudaMemsetAsync(h->d_bar, 0, 2 * sizeof(unsigned), h->stream));
       CK(cudaStreamSynchronize(h->stream));
-      return fail(MFWH_ERR_TIMEOUT,
-                  flag == 2 ? "implicit step kernel: a grid barrier wait timed out"
-                            : "FP32 wave kernel: a tile's tensor copy did not complete");
+      return fail(MFWH_ERR_TIMEOUT, "implicit step kernel: a grid barrier wait timed out");
     }
   }
   double ms = 0.0;
@@ -284,14 +282,14 @@ mfwh_status apply_pi32(mfwh_handle_t h, const double* vin, double* vout, int for
     a.first_hi = first_hi;
     a.wq = h->wq32;
     a.fc = h->fc32;
+    a.wq_host = h->wq32_h.data();
+    a.fc_host = h->fc32_h.data();
     a.binv = h->sh.binv;
     a.emat = h->sh.emat;
     a.has_e = h->sh.has_e;
     a.vprev = vin;
     a.depth = P.time_block;
-    a.shape = P.tile_shape;
     a.acc = P.precision == MFWH_PREC_FP32_BLOCKSUM ? 1 : 0;
-    a.err = h->d_err;
     a.forced = forced;
     int cur = 0;                 // pair holding the input: (W32[2 cur], W32[2 cur + 1])
     for (int n0 = 0; n0 < n_run;) {
@@ -906,11 +904,12 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
   g.layer_axis = P.layer_axis;
   g.layer_split = P.layer_split;
   g.order = P.order;
-  // FP32 2D wave levels: rows padded to 32 floats (16-byte aligned for tensor copies)
+  // FP32 2D wave levels and forcing: rows padded to 32 floats (16-byte aligned)
   const bool pad_w = P.precision != MFWH_PREC_FP64 && P.dim == 2;
   g.syw = pad_w ? (g.nx + 1 + 31) / 32 * 32 : g.sy;
   g.szw = pad_w ? g.syw * (g.ny + 1) : g.sz;
   h->PW = pad_w ? g.syw * (g.ny + 1) : h->P;
+  g.wpoints = h->PW;
 
   auto cleanup = [&](mfwh_status s) {
     mfwh_destroy(h);
@@ -955,7 +954,7 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
     struct {
       float** p;
       int64_t n;
-    } fb[] = {{&h->f32, h->N}, {&h->W32[0], h->PW}, {&h->W32[1], h->PW}, {&h->W32[2], h->PW},
+    } fb[] = {{&h->f32, h->PW * h->nf}, {&h->W32[0], h->PW}, {&h->W32[1], h->PW}, {&h->W32[2], h->PW},
               {&h->W32[3], h->PW}, {&h->qs, h->N}, {&h->qc, h->N},
               {&h->wq32, (int64_t)h->wq32_h.size()}, {&h->fc32, (int64_t)h->fc32_h.size()}};
     for (auto& b : fb) {
@@ -964,8 +963,6 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
     }
     for (int i = 0; i < 4 && e == cudaSuccess; ++i)
       e = cudaMemsetAsync(h->W32[i], 0, sizeof(float) * h->PW, h->stream);
-    if (e == cudaSuccess) e = cudaMalloc(&h->d_err, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(h->wq32, h->wq32_h.data(), sizeof(float) * h->wq32_h.size(),
                           cudaMemcpyHostToDevice, h->stream);
@@ -1104,7 +1101,7 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
   h->geom.fault = h->fault;
 #endif
   if (e == cudaSuccess && h->f32) {
-    launch_to_float(h->f, h->f32, h->N, h->stream);
+    launch_forcing32(h->nf, h->geom, h->f, h->f32, h->stream);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
@@ -1139,7 +1136,7 @@ mfwh_status mfwh_set_forcing(mfwh_handle_t h, const double* forcing) {
   if (!h || !forcing) return fail(MFWH_ERR_INVALID_ARG, "null argument");
   CK(cudaMemcpyAsync(h->f, forcing, sizeof(double) * h->N, cudaMemcpyDefault, h->stream));
   if (h->f32) {
-    launch_to_float(h->f, h->f32, h->N, h->stream);
+    launch_forcing32(h->nf, h->geom, h->f, h->f32, h->stream);
     h->total_launches++;
     CK(cudaGetLastError());
   }
@@ -2024,8 +2021,7 @@ mfwh_status mfwh_autotune(const mfwh_problem* prob, void* stream, int* time_bloc
   } else if (P.precision == MFWH_PREC_FP64) {
     cand = {{1, 0}, {2, 5}, {3, 5}, {4, 5}, {4, 4}, {4, 3}, {8, 3}};
   } else {
-    for (int T : {4, 8, 16})
-      for (int shape : {0, 1, 2}) cand.push_back({T, shape});
+    cand = {{4, 0}, {8, 0}, {16, 0}};
   }
   // Each candidate times the first tune_n steps of a homogeneous wave solve (whole launches
   // for every depth), after one untimed warm-up of the same length.

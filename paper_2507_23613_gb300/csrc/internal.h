@@ -23,7 +23,7 @@ struct Plan {
   int layer_axis = 0;
   int dim = 2;
   int time_block = 1;          // steps per wave-kernel launch (1, 4, 8 or 16)
-  int tile_shape = 0;          // FP32 blocked-kernel tile shape
+  int tile_shape = 0;          // tile of the FP64 blocked kernels (wave_tb.cu)
   int precision = MFWH_PREC_FP64;
   int order = 2;               // order of L_{ph}: 2 or 4
   int filter_update = MFWH_UPDATE_IMPLICIT;

@@ -20,8 +20,9 @@ struct Geom {
   int layer_axis;            // axis whose index selects the c^2 layer
   int64_t layer_split;       // indices >= layer_split use the upper-layer coefficients
   int order;                 // order of L_{ph}: 2 or 4 (0 reads as 2)
-  int64_t syw, szw;          // strides of j and k in the FP32 wave-level arrays W and D (2D
-                             // FP32 handles pad rows to 32 floats for tensor copies; else sy, sz)
+  int64_t syw, szw;          // strides of j and k in the FP32 arrays W, D and f (2D FP32 handles
+                             // pad rows to 32 floats for 16-byte accesses; else sy, sz)
+  int64_t wpoints;           // entries of one of them (stride between the frequencies of f)
   const double* c2f;         // c^2 per point [points] (MFWH_C_FIELD), else null; with a field
                              // the layer coefficients are those of c = 1 (lower layer only)
   BoundsFault* fault;        // device fault record of the index-checked build (check.cuh), or
@@ -101,13 +102,14 @@ struct TB32Host {
   Coef32 reg_lo, reg_hi, first_lo, first_hi;
   const float* wq;         // device [(N_t + 1) * nf]
   const float* fc;         // device [N_t * nf]
+  const float* wq_host;    // host copies of the two (the 2D kernel's travel as parameters)
+  const float* fc_host;
   const double* binv;      // host [MFWH_MAX_NF * MFWH_MAX_NF], row-major, leading dim 16 (C)
   const double* emat;      // host, same layout (E of the explicit filter)
   int has_e;
   const double* vprev;     // device V^k, or null
-  int n0, steps, depth, shape, forced, last;
+  int n0, steps, depth, forced, last;
   int acc;                 // 0: Kahan update every step; 1: per-launch partial sums folded
-  int* err;                // device flag set to 1 when a tile's tensor copy does not complete
 };
 // W^0 = fl32(sum_m v_m) (0 on the boundary), qs_m = w0_m W^0, qc_m = 0.
 void launch_init32(int nf, const Geom& g, const double* v, float* W0, float* qs, float* qc,
@@ -125,11 +127,12 @@ void launch_tb2d32(int nf, const Geom& g, const float* W_in, const float* D_in, 
                    float* D_out, const float* f, float* qs, float* qc, double* vout,
                    const double* vsub, const TB32Host& h, cudaStream_t st);
 // Up to h.depth (2 or 4) steps of a 3D grid per launch (second-order operator); outputs must
-// not alias inputs.  Same arguments as launch_tb2d32 (tile shape ignored).
+// not alias inputs.  Same arguments as launch_tb2d32.
 void launch_tb3d32(int nf, const Geom& g, const float* W_in, const float* D_in, float* W_out,
                    float* D_out, const float* f, float* qs, float* qc, double* vout,
                    const double* vsub, const TB32Host& h, cudaStream_t st);
-void launch_to_float(const double* x, float* y, int64_t n, cudaStream_t st);
+// The forcing [nf][points] rounded to FP32 in the layout of the FP32 wave levels.
+void launch_forcing32(int nf, const Geom& g, const double* x, float* y, cudaStream_t st);
 
 // In launch_init, launch_step, launch_last and launch_tb2d, q holds the N_f filter sums
 // [N_f][points], each as a float pair (hi, lo) in the 8 bytes of a double (fpair.cuh); only

@@ -8,10 +8,17 @@
 namespace mfwh {
 namespace {
 
-__global__ void k_to_float(const double* __restrict__ x, float* __restrict__ y, int64_t n) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    y[i] = (float)x[i];
+// A block takes rows (j, k) of one frequency; padding is written as 0.
+__global__ void __launch_bounds__(256)
+k_forcing32(const double* __restrict__ x, float* __restrict__ y, const Geom g, int64_t rows) {
+  const int64_t m = blockIdx.y;
+  for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
+    const int64_t k = r / (g.ny + 1), j = r - k * (g.ny + 1);
+    const double* src = x + m * g.points + k * g.sz + j * g.sy;
+    float* dst = y + m * g.wpoints + k * g.szw + j * g.syw;
+    for (int64_t i = threadIdx.x; i < g.syw; i += blockDim.x)
+      dst[i] = i <= g.nx ? (float)src[i] : 0.0f;
+  }
 }
 
 W32Ops ops_for(int nf) {
@@ -71,8 +78,10 @@ void launch_tb2d32(int nf, const Geom& g, const float* W_in, const float* D_in, 
   ops_for(nf).tb(g, W_in, D_in, W_out, D_out, f, qs, qc, vout, vsub, h, st);
 }
 
-void launch_to_float(const double* x, float* y, int64_t n, cudaStream_t st) {
-  k_to_float<<<4 * 152, 256, 0, st>>>(x, y, n);
+void launch_forcing32(int nf, const Geom& g, const double* x, float* y, cudaStream_t st) {
+  const int64_t rows = (g.ny + 1) * (g.dim == 3 ? g.nz + 1 : 1);
+  const dim3 grid((unsigned)(rows < 4096 ? rows : 4096), (unsigned)nf);
+  k_forcing32<<<grid, 256, 0, st>>>(x, y, g, rows);
 }
 
 }  // namespace mfwh

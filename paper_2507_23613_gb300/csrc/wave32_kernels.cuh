@@ -17,15 +17,13 @@
 // and everything after it are FP64.
 //
 // Two kernels advance the scheme:
-//  * k_tb2d32: 2D, T steps per launch on a 32 x (TY K) tile with a T-point halo in
-//    shared memory (the tile plus a ring of radius T-1-s updated at step s), the
-//    Kahan pairs of the tile's points in registers for all T steps;
+//  * k_tb2d32: 2D, T steps per launch on overlapped tiles whose points, halo included, live
+//    in the registers of one CTA for all T steps;
 //  * k_step32 / k_last32: one step per launch, 2D or 3D, second- or fourth-order L_h.
 // Both perform the same FP32 operations per point in the same order, so their
 // results are bit-identical.
 #pragma once
 
-#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -82,18 +80,19 @@ __device__ __forceinline__ void kahan_add(float& s, float& c, float w, float x) 
   s = t;
 }
 
-// kappa c^2 Delta_h W at a point whose value is w and whose neighbour sums of
-// differences are dxx, dyy, dzz, minus the forcing; same order in every kernel.
+// kappa c^2 Delta_h W at a point whose neighbour sums of differences are dxx, dyy, dzz, minus
+// the forcing (f is laid out like the wave levels, q the point's index there); same order in
+// every kernel.
 template <int NF, int DIM>
 __device__ __forceinline__ float increment(const Coef32& L, float dxx, float dyy, float dzz,
                                            const float* fc, const float* __restrict__ f,
-                                           int64_t p, int64_t points, int forced) {
+                                           int64_t q, int64_t wpoints, int forced) {
   float inc = L.Ay * dyy;
   if (DIM == 3) inc = fmaf(L.Az, dzz, inc);
   inc = fmaf(L.Ax, dxx, inc);
   if (forced) {
 #pragma unroll
-    for (int m = 0; m < NF; ++m) inc = fmaf(-fc[m], f[m * points + p], inc);
+    for (int m = 0; m < NF; ++m) inc = fmaf(-fc[m], f[m * wpoints + q], inc);
   }
   return inc;
 }
@@ -134,7 +133,7 @@ template <int NF, int DIM, int ORDER>
 __device__ __forceinline__ void step_point(const float* __restrict__ W, const float* D,
                                            const float* __restrict__ f, const Step32Args<NF>& a,
                                            const Geom& g, int64_t i, int64_t j, int64_t k,
-                                           int64_t p, float& wn, float& dn) {
+                                           float& wn, float& dn) {
   const int64_t li = g.layer_axis == 0 ? i : (g.layer_axis == 1 ? j : k);
   const Coef32& L = li >= g.layer_split ? a.hi : a.lo;
   const int64_t q = wpos(g, i, j, k);
@@ -147,7 +146,7 @@ __device__ __forceinline__ void step_point(const float* __restrict__ W, const fl
     dyy = comb4(W, q, g.syw, j, g.ny, w, dyy);
     if (DIM == 3) dzz = comb4(W, q, g.szw, k, g.nz, w, dzz);
   }
-  const float inc = increment<NF, DIM>(L, dxx, dyy, dzz, a.fc, f, p, g.points, a.forced);
+  const float inc = increment<NF, DIM>(L, dxx, dyy, dzz, a.fc, f, q, g.wpoints, a.forced);
   dn = (D ? D[q] : 0.0f) + inc;
   wn = w + dn;
 }
@@ -164,7 +163,7 @@ k_step32(const float* __restrict__ W, const float* D_in, float* __restrict__ W_o
   index_of<DIM>(g, i, j, k, p, interior);
   if (!interior) return;
   float wn, dn;
-  step_point<NF, DIM, ORDER>(W, D_in, f, a, g, i, j, k, p, wn, dn);
+  step_point<NF, DIM, ORDER>(W, D_in, f, a, g, i, j, k, wn, dn);
   W_out[wpos(g, i, j, k)] = wn;
   D_out[wpos(g, i, j, k)] = dn;
 #pragma unroll
@@ -216,7 +215,7 @@ k_last32(const float* __restrict__ W, const float* __restrict__ D, const float* 
   for (int m = 0; m < NF; ++m) s[m] = c[m] = 0.0f;
   if (interior) {
     float wn, dn;
-    step_point<NF, DIM, ORDER>(W, D, f, a, g, i, j, k, p, wn, dn);
+    step_point<NF, DIM, ORDER>(W, D, f, a, g, i, j, k, wn, dn);
 #pragma unroll
     for (int m = 0; m < NF; ++m) {
       s[m] = qs[m * g.points + p];
@@ -228,51 +227,55 @@ k_last32(const float* __restrict__ W, const float* __restrict__ D, const float* 
 }
 
 // ---- temporally blocked 2D kernel ----------------------------------------------
+//
+// One CTA per SM (16 warps) holds an extended tile of 128 x 64 points in registers, W and D of
+// 4 x 4 points per thread: lane l has columns 4l .. 4l + 3, warp w rows 4w .. 4w + 3.  Every step
+// updates all of them (the outermost ring of valid values shrinks by one point a step, so after
+// T steps the (128 - 2T) x (64 - 2T) points in the middle are exact), except that a warp rests
+// once no later step reads its rows.  Left and right neighbours come from the thread itself or by
+// one shuffle per row and side, vertical neighbours from the thread itself or, above and below
+// its four rows, from the edge rows that the warps exchange through shared memory (double
+// buffered: one barrier per step).  A step of a point is 8 FP32 operations (each neighbour
+// difference is formed once and serves both of its points: W_w - W at a point is exactly minus
+// W_e - W at its left neighbour) plus about 1.5 instructions of exchange, with no index
+// arithmetic and no per-point tests away from the boundary.  (The form it replaces, 32 x 32 tiles
+// with the halo ring in shared memory and a flat index over it, issued 169 instructions per
+// point-step at N_f = 5, this one 58: 30.1 against 19.2 ms for a map on 2049^2, N_f = 5, depth 16,
+// 1717 steps.)
+//
+// The filter sums are not touched while stepping.  Each step stores the owned points' new values
+// in shared memory (T x 4 bytes per owned point: 192 KB of the 227 KB, which sets the tile);
+// after the last step every thread takes owned points one by one, reads their T values back and
+// updates all N_f sums in registers, in step order, with the weights as constant operands.
+//   ACC = 0: Kahan update of (s_m, c_m) at every step.
+//   ACC = 1: plain FP32 partial sums over the steps of one launch, folded into the Kahan
+//            pair once per launch (compensated across launches; the partial of at most T
+//            terms carries a rounding error far below that of the FP32 wave levels).
+constexpr int kRtWarps = 16, kRtThreads = 32 * kRtWarps;
+constexpr int kRtEX = 128, kRtEY = 64;    // extended tile
 
+template <int NF, int T>
+struct RT32Args {
+  Coef32 reg_lo, reg_hi, first_lo, first_hi;
+  int n0, steps, forced, last, subtract;
+  float wq[T * NF];   // w_{n+1,m} of step s: [s * NF + m]
+  float fc[T * NF];   // kappa_n cos(omega~_m t^n)
+};
+
+template <int T>
+constexpr size_t rt32_smem_bytes() {
+  return sizeof(float) * ((size_t)T * (kRtEX - 2 * T) * (kRtEY - 2 * T) +
+                          (size_t)2 * kRtWarps * 2 * kRtEX);
+}
+
+// One parameter block for the kernel and the 3D kernel's table-driven coefficients.
 template <int NF>
 struct TB32Args {
   Coef32 reg_lo, reg_hi, first_lo, first_hi;
   const float* wq;   // [(N_t + 1) * NF]
   const float* fc;   // [N_t * NF]
-  int* err;          // set to 1 when a tile's tensor copy does not complete
   int n0, steps, forced, last, subtract;
 };
-
-// A global offset clamped into [lo, hi] as a 32-bit local coordinate.
-__device__ __forceinline__ int clamp_local(int64_t v, int lo, int hi) {
-  return v < lo ? lo : (v > hi ? hi : (int)v);
-}
-
-// One leapfrog update at local point l of the extended tile (increment form).
-template <int NF, int EX>
-__device__ __forceinline__ float tb_update(const float* Wc, float* Wn, float* Dv, int l,
-                                           const Coef32& L, const float* fc,
-                                           const float* __restrict__ f, int64_t p,
-                                           int64_t points, int forced) {
-  const float w = Wc[l];
-  const float dxx = (Wc[l - 1] - w) + (Wc[l + 1] - w);
-  const float dyy = (Wc[l - EX] - w) + (Wc[l + EX] - w);
-  const float inc = increment<NF, 2>(L, dxx, dyy, 0.0f, fc, f, p, points, forced);
-  const float dn = Dv[l] + inc;
-  const float wn = w + dn;
-  Dv[l] = dn;
-  Wn[l] = wn;
-  return wn;
-}
-
-// ceil(2^32 / d) for 2 <= d < 128, a table in constant memory filled at compile time: the
-// multiplier of the exact division floor(e / d) = (e * m) >> 32 for the small ring indices e
-// of the blocked kernels (e < 2^16; checked exhaustively on the host).
-struct DivMagic {
-  unsigned m[128];
-};
-constexpr DivMagic make_div_magic() {
-  DivMagic t{};
-  for (int d = 2; d < 128; ++d) t.m[d] = 0xFFFFFFFFu / (unsigned)d + 1u;
-  return t;
-}
-__constant__ DivMagic c_div_magic = make_div_magic();
-__device__ __forceinline__ unsigned div_magic(int d) { return c_div_magic.m[d]; }
 
 // Fold a partial sum x into the Kahan pair (s, c).
 __device__ __forceinline__ void kahan_fold(float& s, float& c, float x) {
@@ -282,305 +285,216 @@ __device__ __forceinline__ void kahan_fold(float& s, float& c, float x) {
   s = t;
 }
 
-// The halo ring of radius r around a BX x BY tile at one step, enumerated evenly over all
-// threads: first the 2r rows of BX + 2r points above and below the tile, then the BY rows of
-// 2r points to its left and right.  Quotients by the row lengths are exact integer divisions by
-// a multiplier: floor(e / d) = (e * ceil(2^32 / d)) >> 32 for the ring indices used here
-// (e < 2^16, d < 2^7; checked exhaustively on the host).
-// SIMPLE: every ring point is interior and has the same c^2 (no bounds or layer tests).
-template <int NF, int T, int BX, int BY, bool SIMPLE>
-__device__ __forceinline__ void ring_pass(const float* Wc, float* Wn, float* Dv, int r, int tid,
-                                          int nthreads, int ilx, int ihx, int ily, int ihy,
-                                          bool lay_x, int lay_thr, const Coef32& lo,
-                                          const Coef32& hi, const float* fc,
-                                          const float* __restrict__ f, int64_t y0, int64_t x0,
-                                          const Geom& g, int forced) {
-  constexpr int EX = BX + 2 * T;
-  const int RW = BX + 2 * r;
-  const int top = 2 * r * RW;
-  const int ring = top + 2 * r * BY;
-  const unsigned m_rw = div_magic(RW), m_2r = div_magic(2 * r);
-  for (int e = tid; e < ring; e += nthreads) {
-    int lx, ly;
-    if (e < top) {
-      const int row = (int)__umulhi((unsigned)e, m_rw);
-      lx = T - r + (e - row * RW);
-      ly = row < r ? T - r + row : T + BY + row - r;
-    } else {
-      const int e2 = e - top;
-      const int row = (int)__umulhi((unsigned)e2, m_2r);
-      const int col = e2 - row * 2 * r;
-      ly = T + row;
-      lx = col < r ? T - r + col : T + BX + col - r;
-    }
-    if (!SIMPLE && (lx < ilx || lx > ihx || ly < ily || ly > ihy)) continue;
-    const Coef32& L = SIMPLE ? lo : (((lay_x ? lx : ly) >= lay_thr) ? hi : lo);
-    tb_update<NF, EX>(Wc, Wn, Dv, ly * EX + lx, L, fc, f, (y0 + ly) * g.sy + x0 + lx, g.points,
-                      forced);
-  }
-}
 
-// ACC = 0: Kahan update of (s_m, c_m) at every step.
-// ACC = 1: plain FP32 partial sums over the steps of one launch, folded into the Kahan
-//          pair once per launch (compensated across launches; the partial of at most T
-//          terms carries a rounding error far below that of the FP32 wave levels).
-//
-// The CTA has BX x TY threads (BX = 32 or 64) and a BX x (TY K) tile.  Thread (tx, ty) owns
-// the K consecutive tile rows ty K .. ty K + K - 1 of column tx.  The wave values W and
-// increments D of its own points stay in registers for all T steps; only the left and right
-// neighbours and the rows just above and below the strip come from shared memory.  The halo
-// ring is updated from shared memory by all threads.
-// Tensor-memory-accelerator (TMA) copies of the extended tile: one 2D tiled copy of EX x EY
-// floats per array, completing on an mbarrier with a transaction count.  Points outside the
-// grid (negative or past the extents) arrive as zeros.
-__device__ __forceinline__ unsigned smem_addr(const void* p) {
-  return (unsigned)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ void tma_tile_2d(float* dst, const CUtensorMap* map, int x, int y,
-                                            unsigned bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%2, %3}], [%4];" ::"r"(smem_addr(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
-      : "memory");
-}
-
-// Bounded wait for phase `parity` of an mbarrier; false when the bound ran out.
-__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, int limit) {
-  for (int it = 0; it < limit; ++it) {
-    unsigned done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (done) return true;
-  }
-  return false;
-}
-
-template <int NF, int T, int BX, int TY, int K, int MB, int ACC>
-__global__ void __launch_bounds__(BX * TY, MB)
+template <int NF, int T, int ACC>
+__global__ void __launch_bounds__(kRtThreads, 1)
 k_tb2d32(const float* __restrict__ W_in, const float* __restrict__ D_in,
          float* __restrict__ W_out, float* __restrict__ D_out, const float* __restrict__ f,
          float* __restrict__ qs, float* __restrict__ qc, double* vout, const double* vsub,
-         const TB32Args<NF> a, const Last32Binv<NF> b, const Geom g,
-         const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmD,
-         int use_tma) {
-  constexpr int BY = TY * K, NT = BX * TY;
-  constexpr int EX = BX + 2 * T, EY = BY + 2 * T, E = EX * EY;
-  static_assert((E * sizeof(float)) % 128 == 0, "tile arrays must stay 128-byte aligned");
-  extern __shared__ __align__(128) float sm32[];
-  __shared__ __align__(8) uint64_t tile_bar;
-  float* Wc = sm32;             // W^n on the extended tile
-  float* Wn = sm32 + E;         // W^{n+1}
-  float* Dv = sm32 + 2 * E;     // D on the halo (the tile's own D lives in registers)
-  float* s_wq = sm32 + 3 * E;   // [T][NF]
-  float* s_fc = s_wq + T * NF;  // [T][NF]
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * BX + tx;
-  const int64_t x0 = (int64_t)blockIdx.x * BX - T, y0 = (int64_t)blockIdx.y * BY - T;
-  // Local-coordinate bounds (32-bit): grid points gl*, interior points il*.
-  const int glx = clamp_local(-x0, 0, EX), ghx = clamp_local(g.nx - x0, -1, EX - 1);
-  const int gly = clamp_local(-y0, 0, EY), ghy = clamp_local(g.ny - y0, -1, EY - 1);
-  const int ilx = clamp_local(1 - x0, 0, EX), ihx = clamp_local(g.nx - 1 - x0, -1, EX - 1);
-  const int ily = clamp_local(1 - y0, 0, EY), ihy = clamp_local(g.ny - 1 - y0, -1, EY - 1);
-  // c^2 layer: points whose local coordinate along the layer axis is >= lay_thr use hi.
+         const __grid_constant__ RT32Args<NF, T> a, const __grid_constant__ Last32Binv<NF> b,
+         const Geom g) {
+  constexpr int VX = kRtEX - 2 * T, VY = kRtEY - 2 * T;   // owned points
+  static_assert(T % 4 == 0 && VX > 0 && VY > 0, "owned points are whole 4 x 4 blocks");
+  extern __shared__ __align__(16) float sm32[];
+  float* hist = sm32;                       // [T][VY][VX] owned values step by step
+  float* edge = sm32 + T * VX * VY;         // [2][warp][top, bottom][128] edge rows
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t x0 = (int64_t)blockIdx.x * VX - T, y0 = (int64_t)blockIdx.y * VY - T;
+  const int lx = 4 * lane, ly = 4 * warp;
+  const int64_t gx = x0 + lx, gy = y0 + ly;   // this thread's first point
+  const bool owner = lx >= T && lx < T + VX && ly >= T && ly < T + VY;
   const bool lay_x = g.layer_axis == 0;
-  const int lay_thr = clamp_local(g.layer_split - (lay_x ? x0 : y0), -1, EX + EY);
-  // Every point of the largest ring interior, all with one c^2: the ring needs no tests.
-  const bool simple = ilx <= 1 && ihx >= EX - 2 && ily <= 1 && ihy >= EY - 2 &&
-                      (lay_thr <= 0 || lay_thr >= (lay_x ? EX : EY));
-  const bool all_hi = lay_thr <= 0;
-
-  if (use_tma) {
-    // W twice (current level and the buffer of the next one, whose boundary values must be
-    // in place) and D once, by tensor copies issued from one thread.
-    const unsigned bar = smem_addr(&tile_bar);
-    if (tid == 0) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-    if (tid == 0) {
-      const unsigned bytes = (D_in != nullptr ? 3u : 2u) * (unsigned)(E * sizeof(float));
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-                   : "memory");
-      tma_tile_2d(Wc, &tmW, (int)x0, (int)y0, bar);
-      tma_tile_2d(Wn, &tmW, (int)x0, (int)y0, bar);
-      if (D_in != nullptr) tma_tile_2d(Dv, &tmD, (int)x0, (int)y0, bar);
-    }
-    if (D_in == nullptr)
-      for (int e = tid; e < E; e += NT) Dv[e] = 0.0f;
-    const bool ok = mbar_wait(bar, 0, 1 << 22);
-    if (__syncthreads_or(!ok)) {
-      // The copies did not complete within the bound: report it (the host fails the call with
-      // MFWH_ERR_TIMEOUT), give them one more bounded wait to land while the CTA still owns its
-      // shared memory, and stop.  If that wait runs out too the CTA stops all the same: every
-      // wait in this kernel must end.
-      if (tid == 0) atomicExch(a.err, 1);
-      mbar_wait(bar, 0, 1 << 22);
-      return;
-    }
-  } else {
-    for (int ly = ty; ly < EY; ly += TY) {
-      const bool row = ly >= gly && ly <= ghy;
-      const int64_t rbase = (y0 + ly) * g.syw + x0;
-      for (int lx = tx; lx < EX; lx += BX) {
-        const bool in = row && lx >= glx && lx <= ghx;
-        const int l = ly * EX + lx;
-        const float w = in ? W_in[rbase + lx] : 0.0f;
-        Wc[l] = w;
-        Wn[l] = w;
-        Dv[l] = (in && D_in != nullptr) ? D_in[rbase + lx] : 0.0f;
+  // the thread's points: interior (bit 4k + c of in_mask), upper layer (of hi_mask)
+  unsigned in_mask = 0, hi_mask = 0;
+  float w[4][4], d[4][4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int64_t y = gy + k;
+    const bool row = y >= 0 && y <= g.ny;
+    const int64_t base = y * g.syw + gx;
+    if (row && gx >= 0 && gx + 3 <= g.nx) {
+      const float4 v = *reinterpret_cast<const float4*>(W_in + base);
+      w[k][0] = v.x; w[k][1] = v.y; w[k][2] = v.z; w[k][3] = v.w;
+      float4 u = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (D_in != nullptr) u = *reinterpret_cast<const float4*>(D_in + base);
+      d[k][0] = u.x; d[k][1] = u.y; d[k][2] = u.z; d[k][3] = u.w;
+    } else {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const bool in = row && gx + c >= 0 && gx + c <= g.nx;
+        w[k][c] = in ? W_in[base + c] : 0.0f;
+        d[k][c] = (in && D_in != nullptr) ? D_in[base + c] : 0.0f;
       }
     }
-  }
-  for (int e = tid; e < a.steps * NF; e += NT) {
-    const int st = e / NF, m = e - st * NF;
-    const int n = a.n0 + st;
-    s_wq[e] = a.wq[(n + 1) * NF + m];
-    s_fc[e] = a.forced ? a.fc[n * NF + m] : 0.0f;
-  }
-  // The strip: local column lxo, rows lyo .. lyo + K - 1.
-  const int lxo = T + tx, lyo = T + ty * K;
-  const int64_t p0 = (y0 + lyo) * g.sy + x0 + lxo;
-  if (ACC == 1) {
-    // Ask L2 for the Kahan pairs folded at the end of the launch.  A warp's 32 columns of
-    // one row span at most two 128-byte lines; each lane prefetches some of the warp's
-    // (row, frequency, array) lines.
-    const int lane = tid & 31;
-    const int64_t wbase = p0 - (tx & 31);
-    for (int c = lane; c < 4 * K * NF; c += 32) {
-      const int half = c & 1, k = (c >> 1) % K, m = ((c >> 1) / K) % NF, arr = c / (2 * K * NF);
-      const int64_t pl = wbase + k * g.sy + half * 31;
-      if (lxo - (tx & 31) + half * 31 <= ihx && lyo + k <= ihy) {
-        const float* ptr = (arr ? qc : qs) + m * g.points + pl;
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr));
-      }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int64_t x = gx + c;
+      if (x > 0 && x < g.nx && y > 0 && y < g.ny) in_mask |= 1u << (4 * k + c);
+      if ((lay_x ? x : y) >= g.layer_split) hi_mask |= 1u << (4 * k + c);
     }
   }
-  const bool col_int = lxo >= ilx && lxo <= ihx;
-  bool own_int[K], own_up[K];
-  float wr[K], dr[K], ks[K][NF], kc[K][NF], part[K][NF];
-  __syncthreads();
+  // Ask L2 for the sums that the end of the launch updates (an owner's rows of 4 points).
+  if (owner) {
+    for (int e = 0; e < 2 * NF; ++e) {
+      const float* base = (e & 1 ? qc : qs) + (int64_t)(e >> 1) * g.points;
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const int ly = lyo + k;
-    own_int[k] = col_int && ly >= ily && ly <= ihy;
-    own_up[k] = (lay_x ? lxo : ly) >= lay_thr;
-    wr[k] = Wc[ly * EX + lxo];
-    dr[k] = Dv[ly * EX + lxo];
-#pragma unroll
-    for (int m = 0; m < NF; ++m) {
-      part[k][m] = 0.0f;
-      if (ACC == 0) {
-        ks[k][m] = own_int[k] ? qs[m * g.points + p0 + k * g.sy] : 0.0f;
-        kc[k][m] = own_int[k] ? qc[m * g.points + p0 + k * g.sy] : 0.0f;
-      }
+      for (int k = 0; k < 4; ++k)
+        if ((in_mask >> (4 * k) & 1u) && (lane & 3) == 0)   // one request per 64 bytes
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(base + (gy + k) * g.sy + gx));
     }
   }
-
-  // The T steps in two compiled copies with the same arithmetic per point: ALLINT, for
-  // homogeneous launches of CTAs whose updated points are all interior with one c^2, without
-  // the forcing terms and the per-point interior and layer tests; and the general one.
-  auto run_steps = [&](auto allint_c) {
-    constexpr bool ALLINT = decltype(allint_c)::value;
-    const int forcing = ALLINT ? 0 : a.forced;
-    for (int s = 0; s < a.steps; ++s) {
-      const int r = a.steps - 1 - s;
-      const bool first = a.n0 + s == 0;
-      const Coef32 lo = first ? a.first_lo : a.reg_lo;
-      const Coef32 hi = first ? a.first_hi : a.reg_hi;
-      const float* fc = s_fc + s * NF;
-      float wq[NF];
+  auto edge_row = [&](int buf, int wp, int which) {
+    return reinterpret_cast<float4*>(edge + ((buf * kRtWarps + wp) * 2 + which) * kRtEX) + lane;
+  };
+  auto put_edges = [&](int buf) {
+    *edge_row(buf, warp, 0) = make_float4(w[0][0], w[0][1], w[0][2], w[0][3]);
+    *edge_row(buf, warp, 1) = make_float4(w[3][0], w[3][1], w[3][2], w[3][3]);
+  };
+  // One step of the thread's points from the edge rows of buffer buf.  PLAIN: every point is
+  // interior with one c^2 (a whole warp's); the values are the same.
+  auto step_points = [&](int s, int buf, auto plain_c, auto forced_c) {
+    constexpr bool PLAIN = decltype(plain_c)::value, FORCED = decltype(forced_c)::value;
+    const bool first = a.n0 + s == 0;
+    const Coef32 lo = first ? a.first_lo : a.reg_lo;
+    const Coef32 hi = first ? a.first_hi : a.reg_hi;
+    const Coef32 one = (hi_mask & 1) ? hi : lo;
+    // the outermost rows have no neighbour warp: their values are never read
+    const float4 u4 = *edge_row(buf, warp > 0 ? warp - 1 : 0, 1);
+    const float4 b4 = *edge_row(buf, warp < kRtWarps - 1 ? warp + 1 : warp, 0);
+    const float up[4] = {u4.x, u4.y, u4.z, u4.w}, below[4] = {b4.x, b4.y, b4.z, b4.w};
+    // W - W_above of the current row; row k + 1's is taken before row k is overwritten
+    float dv[4];
 #pragma unroll
-      for (int m = 0; m < NF; ++m) wq[m] = s_wq[s * NF + m];
-      // the strip: centre values from registers, neighbours from shared memory
-      {
-        const float above = Wc[(lyo - 1) * EX + lxo];
-        const float below = Wc[(lyo + K) * EX + lxo];
-        float wnew[K];
+    for (int c = 0; c < 4; ++c) dv[c] = w[0][c] - up[c];
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-          const float w = wr[k];
-          wnew[k] = w;
-          if (!ALLINT && !own_int[k]) continue;   // boundary and outside points keep W = 0
-          const int l = (lyo + k) * EX + lxo;
-          const float up = k == 0 ? above : wr[k - 1];
-          const float dn = k == K - 1 ? below : wr[k + 1];
-          const float dxx = (Wc[l - 1] - w) + (Wc[l + 1] - w);
-          const float dyy = (up - w) + (dn - w);
-          const Coef32 L = ALLINT ? (all_hi ? hi : lo) : (own_up[k] ? hi : lo);
-          const float inc = increment<NF, 2>(L, dxx, dyy, 0.0f, fc, f, p0 + k * g.sy, g.points,
-                                             forcing);
-          dr[k] = dr[k] + inc;
-          wnew[k] = w + dr[k];
-        }
+    for (int k = 0; k < 4; ++k) {
+      const float left = __shfl_up_sync(0xffffffffu, w[k][3], 1);
+      const float right = __shfl_down_sync(0xffffffffu, w[k][0], 1);
+      float dx[5];   // W - W_left of columns 0 .. 4
+      dx[0] = w[k][0] - left;
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-          wr[k] = wnew[k];
-          Wn[(lyo + k) * EX + lxo] = wnew[k];
-          if (ALLINT || own_int[k]) {
+      for (int c = 1; c < 4; ++c) dx[c] = w[k][c] - w[k][c - 1];
+      dx[4] = right - w[k][3];
+      float inc[4];
 #pragma unroll
-            for (int m = 0; m < NF; ++m) {
-              if (ACC == 0)
-                kahan_add(ks[k][m], kc[k][m], wq[m], wnew[k]);
-              else
-                part[k][m] = fmaf(wq[m], wnew[k], part[k][m]);
-            }
+      for (int c = 0; c < 4; ++c) {
+        const float wc = w[k][c];
+        const float dn = (k < 3 ? w[k < 3 ? k + 1 : 3][c] : below[c]) - wc;
+        const float dxx = dx[c + 1] - dx[c];   // (W_w - W) + (W_e - W)
+        const float dyy = dn - dv[c];
+        dv[c] = dn;
+        const bool upper = hi_mask >> (4 * k + c) & 1u;
+        const float Ax = PLAIN ? one.Ax : (upper ? hi.Ax : lo.Ax);
+        const float Ay = PLAIN ? one.Ay : (upper ? hi.Ay : lo.Ay);
+        inc[c] = Ay * dyy;
+        inc[c] = fmaf(Ax, dxx, inc[c]);
+      }
+      if constexpr (FORCED) {
+        if (in_mask >> (4 * k) & 15u) {   // rows of f are padded like those of W
+          const float* fp = f + (gy + k) * g.syw + gx;
+#pragma unroll 4
+          for (int m = 0; m < NF; ++m) {
+            const float4 v = *reinterpret_cast<const float4*>(fp + m * g.wpoints);
+            const float fc = a.fc[s * NF + m];
+            inc[0] = fmaf(-fc, v.x, inc[0]);
+            inc[1] = fmaf(-fc, v.y, inc[1]);
+            inc[2] = fmaf(-fc, v.z, inc[2]);
+            inc[3] = fmaf(-fc, v.w, inc[3]);
           }
         }
       }
-      if (r > 0) {
-        if (ALLINT || simple)
-          ring_pass<NF, T, BX, BY, true>(Wc, Wn, Dv, r, tid, NT, ilx, ihx, ily, ihy, lay_x,
-                                         lay_thr, all_hi ? hi : lo, hi, fc, f, y0, x0, g,
-                                         forcing);
-        else
-          ring_pass<NF, T, BX, BY, false>(Wc, Wn, Dv, r, tid, NT, ilx, ihx, ily, ihy, lay_x,
-                                          lay_thr, lo, hi, fc, f, y0, x0, g, forcing);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float dnew = d[k][c] + inc[c];
+        const float wnew = w[k][c] + dnew;
+        const bool in = PLAIN || (in_mask >> (4 * k + c) & 1u);
+        d[k][c] = in ? dnew : 0.0f;   // boundary and outside points keep W = 0
+        w[k][c] = in ? wnew : 0.0f;
       }
-      __syncthreads();
-      float* t = Wc;
-      Wc = Wn;
-      Wn = t;
     }
   };
-  if (simple && !a.forced)
-    run_steps(std::true_type{});
-  else
-    run_steps(std::false_type{});
-  // wr = W^{n0+steps}, dr = D^{n0+steps-1/2} on the strip
-  const bool col_in = lxo <= ghx;
+  const bool plain = __all_sync(0xffffffffu, in_mask == 0xFFFFu) &&
+                     (__all_sync(0xffffffffu, hi_mask == 0u) ||
+                      __all_sync(0xffffffffu, hi_mask == 0xFFFFu));
+  put_edges(0);
+  __syncthreads();
+  for (int s = 0; s < a.steps; ++s) {
+    const int r = a.steps - 1 - s;   // later steps read the owned points grown by r
+    if (ly + 3 >= T - r && ly < T + VY + r) {
+      if (a.forced)
+        step_points(s, s & 1, std::false_type{}, std::true_type{});
+      else if (plain)
+        step_points(s, s & 1, std::true_type{}, std::false_type{});
+      else
+        step_points(s, s & 1, std::false_type{}, std::false_type{});
+      put_edges((s + 1) & 1);
+      if (owner) {
+        float* h = hist + (size_t)s * VX * VY + (ly - T) * VX + lx - T;
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const int64_t p = p0 + k * g.sy;
-    if (ACC == 1 && own_int[k]) {
+        for (int k = 0; k < 4; ++k)
+          *reinterpret_cast<float4*>(h + k * VX) =
+              make_float4(w[k][0], w[k][1], w[k][2], w[k][3]);
+      }
+    }
+    __syncthreads();
+  }
+  if (owner && !a.last) {
 #pragma unroll
-      for (int m = 0; m < NF; ++m) {
-        ks[k][m] = qs[m * g.points + p];
-        kc[k][m] = qc[m * g.points + p];
-        kahan_fold(ks[k][m], kc[k][m], part[k][m]);
+    for (int k = 0; k < 4; ++k) {
+      if (gy + k > g.ny || gx >= g.syw) continue;
+      const int64_t base = (gy + k) * g.syw + gx;
+      *reinterpret_cast<float4*>(W_out + base) = make_float4(w[k][0], w[k][1], w[k][2], w[k][3]);
+      *reinterpret_cast<float4*>(D_out + base) = make_float4(d[k][0], d[k][1], d[k][2], d[k][3]);
+    }
+  }
+  // The filter sums of the owned points.
+  for (int i = tid; i < VX * VY; i += kRtThreads) {
+    const int ry = i / VX, rx = i - ry * VX;
+    const int64_t x = x0 + T + rx, y = y0 + T + ry;
+    const bool in = x > 0 && x < g.nx && y > 0 && y < g.ny;
+    if (!in && !(a.last && x <= g.nx && y <= g.ny)) continue;
+    const int64_t p = y * g.sy + x;
+    float ks[NF], kc[NF];
+#pragma unroll
+    for (int m = 0; m < NF; ++m) {
+      ks[m] = in ? qs[m * g.points + p] : 0.0f;
+      kc[m] = in ? qc[m * g.points + p] : 0.0f;
+    }
+    if (in) {
+      float part[ACC == 1 ? NF : 1];
+      if constexpr (ACC == 1) {
+#pragma unroll
+        for (int m = 0; m < NF; ++m) part[m] = 0.0f;
+      }
+      auto add = [&](int s, float v) {
+#pragma unroll
+        for (int m = 0; m < NF; ++m) {
+          if constexpr (ACC == 1)
+            part[m] = fmaf(a.wq[s * NF + m], v, part[m]);
+          else
+            kahan_add(ks[m], kc[m], a.wq[s * NF + m], v);
+        }
+      };
+      if (a.steps == T) {
+#pragma unroll
+        for (int s = 0; s < T; ++s) add(s, hist[s * VX * VY + i]);
+      } else {
+#pragma unroll 1
+        for (int s = 0; s < a.steps; ++s) add(s, hist[s * VX * VY + i]);
+      }
+      if constexpr (ACC == 1) {
+#pragma unroll
+        for (int m = 0; m < NF; ++m) kahan_fold(ks[m], kc[m], part[m]);
       }
     }
     if (!a.last) {
-      if (!own_int[k]) continue;
-      W_out[(y0 + lyo + k) * g.syw + x0 + lxo] = wr[k];
-      D_out[(y0 + lyo + k) * g.syw + x0 + lxo] = dr[k];
 #pragma unroll
       for (int m = 0; m < NF; ++m) {
-        qs[m * g.points + p] = ks[k][m];
-        qc[m * g.points + p] = kc[k][m];
+        qs[m * g.points + p] = ks[m];
+        qc[m * g.points + p] = kc[m];
       }
     } else {
-      if (!col_in || lyo + k > ghy) continue;
-      if (!own_int[k]) {
-#pragma unroll
-        for (int m = 0; m < NF; ++m) ks[k][m] = kc[k][m] = 0.0f;
-      }
-      filter_solve_out<NF>(ks[k], kc[k], b, a.subtract, vsub, vout, p, g.points, own_int[k]);
+      filter_solve_out<NF>(ks, kc, b, a.subtract, vsub, vout, p, g.points, in);
     }
   }
 }
@@ -702,8 +616,8 @@ k_tb3d32(const float* __restrict__ W_in, const float* __restrict__ D_in,
       const float dxx = (Wc[l - 1] - w) + (Wc[l + 1] - w);
       const float dyy = (Wc[l - EX] - w) + (Wc[l + EX] - w);
       const float dzz = (Wc[l - SXY] - w) + (Wc[l + SXY] - w);
-      const int64_t p = pz * g.sz + py * g.sy + px;
-      const float inc = increment<NF, 3>(L, dxx, dyy, dzz, fc, f, p, g.points, a.forced);
+      const int64_t q = pz * g.szw + py * g.syw + px;
+      const float inc = increment<NF, 3>(L, dxx, dyy, dzz, fc, f, q, g.wpoints, a.forced);
       const float dn = Dv[l] + inc;
       Dv[l] = dn;
       Wn[l] = w + dn;
@@ -843,107 +757,39 @@ void init32_nf(const Geom& g, const double* v, float* W0, float* qs, float* qc, 
     k_init32<NF, 2><<<grid_of(g), dim3(kBX, kBY), 0, st>>>(v, W0, qs, qc, a, g);
 }
 
-using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
-                                   const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// The driver's tensor-map encoder, looked up once through the runtime (no driver library link).
-inline EncodeTiledFn encode_tiled() {
-  static EncodeTiledFn fn = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                         &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess) {
-      cudaGetLastError();
-      p = nullptr;
-    }
-    return reinterpret_cast<EncodeTiledFn>(p);
-  }();
-  return fn;
-}
-
-// Tensor map of one 2D wave-level array for EX x EY boxes; false if unavailable, in which
-// case the kernel loads its tile with ordinary loads.
-inline bool wave_tensor_map(CUtensorMap* m, const float* base, const Geom& g, int ex, int ey) {
-  EncodeTiledFn fn = encode_tiled();
-  if (!fn || !base || g.dim != 2 || (g.syw * sizeof(float)) % 16 != 0 ||
-      (reinterpret_cast<uintptr_t>(base) & 15) != 0)
-    return false;
-  const cuuint64_t dims[2] = {(cuuint64_t)(g.nx + 1), (cuuint64_t)(g.ny + 1)};
-  const cuuint64_t strides[1] = {(cuuint64_t)(g.syw * sizeof(float))};
-  const cuuint32_t box[2] = {(cuuint32_t)ex, (cuuint32_t)ey};
-  const cuuint32_t estr[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box,
-            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-template <int NF, int T, int BX, int TY, int K, int MB, int ACC>
+template <int NF, int T, int ACC>
 void tb32_launch(const Geom& g, const float* W_in, const float* D_in, float* W_out, float* D_out,
                  const float* f, float* qs, float* qc, double* vout, const double* vsub,
                  const TB32Host& h, cudaStream_t st) {
-  constexpr int BY = TY * K;
-  constexpr int EX = BX + 2 * T, EY = BY + 2 * T;
-  constexpr size_t smem = sizeof(float) * (3 * EX * EY + 2 * T * NF);
+  constexpr size_t smem = rt32_smem_bytes<T>();
   static bool configured[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64 || !configured[dev]) {
-    cudaFuncSetAttribute(k_tb2d32<NF, T, BX, TY, K, MB, ACC>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(k_tb2d32<NF, T, ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
-  TB32Args<NF> a;
+  RT32Args<NF, T> a;
   a.reg_lo = h.reg_lo;
   a.reg_hi = h.reg_hi;
   a.first_lo = h.first_lo;
   a.first_hi = h.first_hi;
-  a.wq = h.wq;
-  a.fc = h.fc;
   a.n0 = h.n0;
   a.steps = h.steps;
   a.forced = h.forced;
   a.last = h.last;
   a.subtract = vsub != nullptr;
-  a.err = h.err;
+  for (int s = 0; s < T; ++s)
+    for (int m = 0; m < NF; ++m) {
+      a.wq[s * NF + m] = s < h.steps ? h.wq_host[(size_t)(h.n0 + s + 1) * NF + m] : 0.0f;
+      a.fc[s * NF + m] = s < h.steps && h.forced ? h.fc_host[(size_t)(h.n0 + s) * NF + m] : 0.0f;
+    }
   const Last32Binv<NF> b = binv_args<NF>(h.binv, h.emat, h.has_e, h.vprev);
-  dim3 grid((unsigned)((g.nx + BX) / BX), (unsigned)((g.ny + BY) / BY));
-  CUtensorMap tmW{}, tmD{};
-  int use_tma = h.err != nullptr && wave_tensor_map(&tmW, W_in, g, EX, EY) &&
-                (D_in == nullptr || wave_tensor_map(&tmD, D_in, g, EX, EY));
-  if (D_in == nullptr) tmD = tmW;
-  k_tb2d32<NF, T, BX, TY, K, MB, ACC><<<grid, dim3(BX, TY), smem, st>>>(
-      W_in, D_in, W_out, D_out, f, qs, qc, vout, vsub, a, b, g, tmW, tmD, use_tma);
-}
-
-template <int NF, int T, int ACC>
-void tb32_shape(const Geom& g, const float* W_in, const float* D_in, float* W_out, float* D_out,
-                const float* f, float* qs, float* qc, double* vout, const double* vsub,
-                const TB32Host& h, cudaStream_t st) {
-  // Tile shapes, K consecutive rows per thread (K halves above 8 frequencies to bound
-  // registers):
-  //  0: 512 threads, tile 32 x 32 (K = 2; 32 x 16), two CTAs per SM (one with ACC = 0);
-  //  1: 512 threads, tile 32 x 64 (K = 4; 32 x 32), one CTA per SM;
-  //  2: 1024 threads, tile 64 x 64 (K = 4; 64 x 32), one CTA per SM.
-  constexpr int KS = NF <= 8 ? 2 : 1;
-  constexpr int M2 = ACC == 0 ? 1 : 2;
-  switch (h.shape) {
-    case 1:
-      tb32_launch<NF, T, 32, 16, 2 * KS, 1, ACC>(g, W_in, D_in, W_out, D_out, f, qs, qc, vout,
-                                                 vsub, h, st);
-      break;
-    case 2:
-      tb32_launch<NF, T, 64, 16, 2 * KS, 1, ACC>(g, W_in, D_in, W_out, D_out, f, qs, qc, vout,
-                                                 vsub, h, st);
-      break;
-    default:
-      tb32_launch<NF, T, 32, 16, KS, M2, ACC>(g, W_in, D_in, W_out, D_out, f, qs, qc, vout, vsub,
-                                              h, st);
-      break;
-  }
+  constexpr int VX = kRtEX - 2 * T, VY = kRtEY - 2 * T;
+  const dim3 grid((unsigned)((g.nx + VX) / VX), (unsigned)((g.ny + VY) / VY));
+  k_tb2d32<NF, T, ACC><<<grid, kRtThreads, smem, st>>>(W_in, D_in, W_out, D_out, f, qs, qc, vout,
+                                                       vsub, a, b, g);
 }
 
 template <int NF, int T>
@@ -951,9 +797,9 @@ void tb32_acc(const Geom& g, const float* W_in, const float* D_in, float* W_out,
               const float* f, float* qs, float* qc, double* vout, const double* vsub,
               const TB32Host& h, cudaStream_t st) {
   if (h.acc == 1)
-    tb32_shape<NF, T, 1>(g, W_in, D_in, W_out, D_out, f, qs, qc, vout, vsub, h, st);
+    tb32_launch<NF, T, 1>(g, W_in, D_in, W_out, D_out, f, qs, qc, vout, vsub, h, st);
   else
-    tb32_shape<NF, T, 0>(g, W_in, D_in, W_out, D_out, f, qs, qc, vout, vsub, h, st);
+    tb32_launch<NF, T, 0>(g, W_in, D_in, W_out, D_out, f, qs, qc, vout, vsub, h, st);
 }
 
 template <int NF>
@@ -995,7 +841,6 @@ void tb3d32_launch(const Geom& g, const float* W_in, const float* D_in, float* W
   a.forced = h.forced;
   a.last = h.last;
   a.subtract = vsub != nullptr;
-  a.err = h.err;
   const Last32Binv<NF> b = binv_args<NF>(h.binv, h.emat, h.has_e, h.vprev);
   const dim3 grid((unsigned)((g.nx + BX) / BX), (unsigned)((g.ny + kT3Y) / kT3Y),
                   (unsigned)((g.nz + kT3Z) / kT3Z));
