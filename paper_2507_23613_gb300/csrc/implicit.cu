@@ -344,12 +344,23 @@ __device__ void prolong_pass(const MgLevel& C, const R* uc, const MgLevel& F, R*
 // them.  A point update, residual or restriction computes what rb_half, residual_at and
 // restrict_pass compute on the whole grid (same operations in the same order).
 
+// Quotients t / d by a multiplication for 0 <= t < 2^16 and 2 <= d < 2^16 (exact: the multiplier
+// exceeds 2^32 / d by less than 1, so the product's error stays below t < 2^32 / d).  The point
+// loops of the phases divide once per point; a run-time integer division is some 20
+// instructions.
+struct FastDiv {
+  unsigned d, m;
+  __device__ explicit FastDiv(int n) : d((unsigned)n), m(0xFFFFFFFFu / (unsigned)n + 1u) {}
+  __device__ __forceinline__ int quot(int t) const { return (int)__umulhi((unsigned)t, m); }
+};
+
 // Half-sweep of colour `color` over the square [ri, ri + S) x [rj, rj + S).
 __device__ void tile_half(const MgLevel& F, float* su, const float* sf, int Wd, int is, int js,
                           int ri, int rj, int S, int color, int axis) {
   const int hw = (S + 1) / 2;
+  const FastDiv dh(hw);
   for (int t = threadIdx.x; t < hw * S; t += blockDim.x) {
-    const int r = t / hw, it = t - r * hw;
+    const int r = dh.quot(t), it = t - r * hw;
     const int j = rj + r;
     const int i = ri + (((ri + j + color) & 1) ? 1 : 0) + 2 * it;
     if (i >= ri + S || i < 1 || i > F.nx - 1 || j < 1 || j > F.ny - 1) continue;
@@ -378,14 +389,15 @@ __device__ void tile_down_rest(const MgLevel& F, const MgLevel& C, float* su, co
     tile_half(F, su, sf, Wd, is, js, i0 - d, j0 - d, T + 2 * d, h & 1, axis);
     __syncthreads();
   }
+  const FastDiv dT(T), dTc(T / 2);
   for (int t = threadIdx.x; t < T * T; t += blockDim.x) {
-    const int i = i0 + t % T, j = j0 + t / T;
+    const int r = dT.quot(t), i = i0 + t - r * T, j = j0 + r;
     if (i > F.nx - 1 || j > F.ny - 1) continue;
     F.v32[(int64_t)j * F.sy + i] = su[(j - js) * Wd + (i - is)];
   }
   const int Tc = T / 2, I0 = (i0 + 1) / 2, J0 = (j0 + 1) / 2;
   for (int t = threadIdx.x; t < Tc * Tc; t += blockDim.x) {
-    const int I = I0 + t % Tc, J = J0 + t / Tc;
+    const int r = dTc.quot(t), I = I0 + t - r * Tc, J = J0 + r;
     if (I > C.nx - 1 || J > C.ny - 1) continue;
     float acc = 0.0f;
     for (int b = -1; b <= 1; ++b) {
@@ -421,14 +433,17 @@ __device__ double down0_tiles(const MgLevel& F, const MgLevel& C, int axis, unsi
   float* su = reinterpret_cast<float*>(zs + Wz * Wz);
   float* sf = su + Wd * Wd;
   double m = 0.0;
+  const FastDiv dz(Wz), dw(Wd);
   for (int tile = blockIdx.x; tile < ntx * nty; tile += gridDim.x) {
     const int i0 = 1 + (tile % ntx) * T, j0 = 1 + (tile / ntx) * T;
     const int is = i0 - H, js = j0 - H;
-    for (int t = threadIdx.x; t < Wz * Wz; t += blockDim.x)
-      zs[t] = z_ghost(F, is - 2 + t % Wz, js - 2 + t / Wz);
+    for (int t = threadIdx.x; t < Wz * Wz; t += blockDim.x) {
+      const int row = dz.quot(t);
+      zs[t] = z_ghost(F, is - 2 + t - row * Wz, js - 2 + row);
+    }
     __syncthreads();
     for (int t = threadIdx.x; t < Wd * Wd; t += blockDim.x) {
-      const int i = is + t % Wd, j = js + t / Wd;
+      const int row = dw.quot(t), i = is + t - row * Wd, j = js + row;
       double r = 0.0;
       if (i >= 1 && i <= F.nx - 1 && j >= 1 && j <= F.ny - 1) {
         const int64_t p = (int64_t)j * F.sy + i;
@@ -466,11 +481,12 @@ __device__ void down_tiles(const MgLevel& F, const MgLevel& C, int axis, unsigne
   const int ntx = (F.nx - 1 + T - 1) / T, nty = (F.ny - 1 + T - 1) / T;
   float* su = reinterpret_cast<float*>(smraw);
   float* sf = su + Wd * Wd;
+  const FastDiv dw(Wd);
   for (int tile = blockIdx.x; tile < ntx * nty; tile += gridDim.x) {
     const int i0 = 1 + (tile % ntx) * T, j0 = 1 + (tile / ntx) * T;
     const int is = i0 - H, js = j0 - H;
     for (int t = threadIdx.x; t < Wd * Wd; t += blockDim.x) {
-      const int i = is + t % Wd, j = js + t / Wd;
+      const int row = dw.quot(t), i = is + t - row * Wd, j = js + row;
       const bool in = i >= 1 && i <= F.nx - 1 && j >= 1 && j <= F.ny - 1;
       sf[t] = in ? F.f32[(int64_t)j * F.sy + i] : 0.0f;
       su[t] = 0.0f;
@@ -489,11 +505,12 @@ __device__ void up_tiles(const MgLevel& F, const MgLevel& C, const float* ec, bo
   const int ntx = (F.nx - 1 + T - 1) / T, nty = (F.ny - 1 + T - 1) / T;
   float* su = reinterpret_cast<float*>(smraw);
   float* sf = su + Wd * Wd;
+  const FastDiv dw(Wd);
   for (int tile = blockIdx.x; tile < ntx * nty; tile += gridDim.x) {
     const int i0 = 1 + (tile % ntx) * T, j0 = 1 + (tile / ntx) * T;
     const int is = i0 - H, js = j0 - H;
     for (int t = threadIdx.x; t < Wd * Wd; t += blockDim.x) {
-      const int i = is + t % Wd, j = js + t / Wd;
+      const int row = dw.quot(t), i = is + t - row * Wd, j = js + row;
       float uu = 0.0f, ff = 0.0f;
       if (i >= 1 && i <= F.nx - 1 && j >= 1 && j <= F.ny - 1) {
         const int64_t p = (int64_t)j * F.sy + i;
@@ -509,8 +526,9 @@ __device__ void up_tiles(const MgLevel& F, const MgLevel& C, const float* ec, bo
       tile_half(F, su, sf, Wd, is, js, i0 - d, j0 - d, T + 2 * d, h & 1, axis);
       __syncthreads();
     }
+    const FastDiv dT(T);
     for (int t = threadIdx.x; t < T * T; t += blockDim.x) {
-      const int i = i0 + t % T, j = j0 + t / T;
+      const int row = dT.quot(t), i = i0 + t - row * T, j = j0 + row;
       if (i > F.nx - 1 || j > F.ny - 1) continue;
       const int64_t p = (int64_t)j * F.sy + i;
       const float e = su[(j - js) * Wd + (i - is)];
@@ -525,14 +543,82 @@ __device__ void up_tiles(const MgLevel& F, const MgLevel& C, const float* ec, bo
 
 // ---- the coarse CTA: levels lc..nlev-1 in shared memory -----------------------------
 
+// 2D point loops of the coarse CTA: f(it, j) for j = 1 .. rows and column index it = 0 .. cols - 1,
+// a power-of-two group of lanes per row (no division per point).  The coarse V-cycle is a chain of
+// short phases between block barriers while all other CTAs wait: the index arithmetic and the
+// repeated residuals were most of a phase.  Map on 513^2, N_f = 6, N_t = 71: 45.0 -> 41.8 ms
+// (with the multiplications in place of the tiled phases' divisions).
+template <class F>
+__device__ __forceinline__ void cta_rows(int rows, int cols, F&& f) {
+  const int lg = cols > 16 ? 5 : (cols > 8 ? 4 : (cols > 4 ? 3 : (cols > 2 ? 2 : 1)));
+  const int lane = threadIdx.x & ((1 << lg) - 1), step = blockDim.x >> lg;
+  for (int j = 1 + (threadIdx.x >> lg); j <= rows; j += step)
+    for (int it = lane; it < cols; it += 1 << lg) f(it, j);
+}
+
 template <int DIM, typename R>
 __device__ void cta_smooth(const MgLevel& L, R* u, const R* f, int sweeps, int axis) {
-  for (int s = 0; s < sweeps; ++s) {
-    rb_half<DIM, R>(L, u, f, 0, axis, threadIdx.x, blockDim.x);
-    __syncthreads();
-    rb_half<DIM, R>(L, u, f, 1, axis, threadIdx.x, blockDim.x);
-    __syncthreads();
+  if constexpr (DIM == 2) {
+    // one interior point: its neighbours are boundary zeros, so every sweep gives the same value
+    if (L.nx == 2 && L.ny == 2) sweeps = 1;
+    const int sy = (int)L.sy;
+    for (int h = 0; h < 2 * sweeps; ++h) {   // the operations of rb_half
+      cta_rows(L.ny - 1, L.nx / 2, [&](int it, int j) {
+        const int i = (((j + h) & 1) ? 1 : 2) + 2 * it;
+        if (i > L.nx - 1) return;
+        const int p = j * sy + i;
+        const bool hi = upper(L, axis, i, j, 0);
+        const R s = neighbours<2, R>(u, p, sy, 0, Co<R>::a(L, hi));
+        u[p] = (f[p] + s) * Co<R>::dinv(L, hi);
+      });
+      __syncthreads();
+    }
+  } else {
+    for (int s = 0; s < sweeps; ++s) {
+      rb_half<DIM, R>(L, u, f, 0, axis, threadIdx.x, blockDim.x);
+      __syncthreads();
+      rb_half<DIM, R>(L, u, f, 1, axis, threadIdx.x, blockDim.x);
+      __syncthreads();
+    }
   }
+}
+
+// The residual of a level restricted onto the next one (restrict_pass); in 2D FP32 hierarchies it
+// is evaluated once per fine point into the scratch behind the levels instead of up to four times.
+template <int DIM, typename R>
+__device__ void cta_restrict(const ImpArgs& a, const MgLevel& L, const MgLevel& C, R* sm) {
+  const int axis = a.layer_axis;
+  R* u = sm + L.smem;
+  R* uc = sm + C.smem;
+  if constexpr (DIM == 2 && sizeof(R) == 4) {
+    const MgLevel& last = a.lev[a.nlev - 1];
+    R* r = sm + last.smem + 2 * last.points;
+    const int sy = (int)L.sy;
+    cta_rows(L.ny - 1, L.nx - 1, [&](int it, int j) {
+      r[j * sy + it + 1] = residual_at<2, R>(L, u, u + L.points, axis, it + 1, j, 0);
+    });
+    __syncthreads();
+    cta_rows(C.ny - 1, C.nx - 1, [&](int it, int J) {
+      const int I = it + 1;
+      R acc = 0;
+#pragma unroll
+      for (int b = -1; b <= 1; ++b) {
+        const R wb = b == 0 ? R(0.5) : R(0.25);
+#pragma unroll
+        for (int aa = -1; aa <= 1; ++aa) {
+          const R wa = aa == 0 ? R(0.5) : R(0.25);
+          acc += R(1) * wb * wa * r[(2 * J + b) * sy + 2 * I + aa];
+        }
+      }
+      const int P = J * (int)C.sy + I;
+      uc[C.points + P] = acc;
+      uc[P] = 0;
+    });
+  } else {
+    restrict_pass<DIM, R>(L, nullptr, u, u + L.points, C, uc + C.points, uc, axis, threadIdx.x,
+                          blockDim.x);
+  }
+  __syncthreads();
 }
 
 // One V-cycle on levels l0..nlev-1 (l0's pre-smoothing skipped when presmoothed).
@@ -541,13 +627,9 @@ __device__ void cta_vcycle(const ImpArgs& a, R* sm, int l0, bool presmoothed) {
   const int axis = a.layer_axis;
   for (int l = l0; l < a.nlev - 1; ++l) {
     const MgLevel& L = a.lev[l];
-    const MgLevel& C = a.lev[l + 1];
     R* u = sm + L.smem;
     if (!(presmoothed && l == l0)) cta_smooth<DIM, R>(L, u, u + L.points, a.nu1, axis);
-    R* uc = sm + C.smem;
-    restrict_pass<DIM, R>(L, nullptr, u, u + L.points, C, uc + C.points, uc, axis, threadIdx.x,
-                          blockDim.x);
-    __syncthreads();
+    cta_restrict<DIM, R>(a, L, a.lev[l + 1], sm);
   }
   {
     const MgLevel& L = a.lev[a.nlev - 1];
@@ -558,7 +640,14 @@ __device__ void cta_vcycle(const ImpArgs& a, R* sm, int l0, bool presmoothed) {
     const MgLevel& L = a.lev[l];
     const MgLevel& C = a.lev[l + 1];
     R* u = sm + L.smem;
-    prolong_pass<DIM, R>(C, sm + C.smem, L, u, threadIdx.x, blockDim.x);
+    if constexpr (DIM == 2) {
+      const R* uc = sm + C.smem;
+      cta_rows(L.ny - 1, L.nx - 1, [&](int it, int j) {
+        u[j * (int)L.sy + it + 1] += prolong_at<2, R>(C, uc, it + 1, j, 0);
+      });
+    } else {
+      prolong_pass<DIM, R>(C, sm + C.smem, L, u, threadIdx.x, blockDim.x);
+    }
     __syncthreads();
     cta_smooth<DIM, R>(L, u, u + L.points, a.nu2, axis);
   }
@@ -887,7 +976,10 @@ cudaError_t mg_launch_config(int dim, int lc, int64_t smem_elems, MgLevel* lev, 
   constexpr int kSmemBound = 120 * 1024;
   const bool mixed = mg_mixed(dim, lc);
   int64_t need = smem_elems * (mixed ? 4 : 8);
-  if (mixed && dim == 2) need = std::max(need, mg_tile_smem_bytes(kMgTileMax));
+  if (mixed && dim == 2) {   // the coarse levels with the restriction's scratch; the tiled phases
+    need += lev[lc].points * 4;
+    need = std::max(need, mg_tile_smem_bytes(kMgTileMax));
+  }
   *smem = (size_t)need;
   if (*smem > (size_t)kSmemBound) return cudaErrorInvalidValue;
   const void* fn = dim == 3 ? (const void*)k_imp_step<3> : (const void*)k_imp_step<2>;
