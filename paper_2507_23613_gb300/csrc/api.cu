@@ -174,9 +174,7 @@ struct mfwh_handle_s {
   float* W32[4] = {};               // (W, D) pairs: W32[0], W32[1] and W32[2], W32[3]
   float* qs = nullptr;              // Kahan sums [nf][P]
   float* qc = nullptr;              // Kahan compensations [nf][P]
-  float* wq32 = nullptr;            // device [(N_t + 1) * nf] w_{n,m}
-  float* fc32 = nullptr;            // device [N_t * nf] kappa_n cos(omega~_m t^n)
-  std::vector<float> wq32_h, fc32_h;
+  std::vector<float> wq32_h, fc32_h;   // [(N_t + 1) * nf] w_{n,m}, [N_t * nf] kappa_n cos(omega~_m t^n)
   // implicit time stepping (MFWH_TIME_IMPLICIT)
   bool implicit = false;
   ImpArgs* imp = nullptr;           // step-kernel arguments (levels filled at create)
@@ -274,27 +272,29 @@ mfwh_status apply_pi32(mfwh_handle_t h, const double* vin, double* vout, int for
   layer_coef32(h, P.c2_lo, 0.5 * dt * dt, &first_lo);
   layer_coef32(h, P.c2_hi, 0.5 * dt * dt, &first_hi);
   int launches = 0;
-  if (P.time_block > 1) {
+  // One step per launch (time_block 1, the 3D default) makes a Kahan update at every step, and
+  // the blocked kernels with such updates give the same bits: 3D runs 4 steps per launch then.
+  const bool kahan3 = P.dim == 3 && P.order == 2 && P.time_block <= 1;
+  const int depth = kahan3 ? 4 : P.time_block;
+  if (depth > 1) {
     TB32Host a;
     a.reg_lo = reg_lo;
     a.reg_hi = reg_hi;
     a.first_lo = first_lo;
     a.first_hi = first_hi;
-    a.wq = h->wq32;
-    a.fc = h->fc32;
     a.wq_host = h->wq32_h.data();
     a.fc_host = h->fc32_h.data();
     a.binv = h->sh.binv;
     a.emat = h->sh.emat;
     a.has_e = h->sh.has_e;
     a.vprev = vin;
-    a.depth = P.time_block;
-    a.acc = P.precision == MFWH_PREC_FP32_BLOCKSUM ? 1 : 0;
+    a.depth = depth;
+    a.acc = P.precision == MFWH_PREC_FP32_BLOCKSUM && !kahan3 ? 1 : 0;
     a.forced = forced;
     int cur = 0;                 // pair holding the input: (W32[2 cur], W32[2 cur + 1])
     for (int n0 = 0; n0 < n_run;) {
       a.n0 = n0;
-      a.steps = std::min(P.time_block, n_run - n0);
+      a.steps = std::min(depth, n_run - n0);
       a.last = n0 + a.steps == n_t;
       const float* D_in = n0 == 0 ? nullptr : h->W32[2 * cur + 1];
       if (P.dim == 3)
@@ -904,11 +904,11 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
   g.layer_axis = P.layer_axis;
   g.layer_split = P.layer_split;
   g.order = P.order;
-  // FP32 2D wave levels and forcing: rows padded to 32 floats (16-byte aligned)
-  const bool pad_w = P.precision != MFWH_PREC_FP64 && P.dim == 2;
+  // FP32 wave levels and forcing: rows padded to 32 floats (16-byte aligned)
+  const bool pad_w = P.precision != MFWH_PREC_FP64;
   g.syw = pad_w ? (g.nx + 1 + 31) / 32 * 32 : g.sy;
   g.szw = pad_w ? g.syw * (g.ny + 1) : g.sz;
-  h->PW = pad_w ? g.syw * (g.ny + 1) : h->P;
+  h->PW = pad_w ? g.szw * (g.dim == 3 ? g.nz + 1 : 1) : h->P;
   g.wpoints = h->PW;
 
   auto cleanup = [&](mfwh_status s) {
@@ -955,20 +955,13 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
       float** p;
       int64_t n;
     } fb[] = {{&h->f32, h->PW * h->nf}, {&h->W32[0], h->PW}, {&h->W32[1], h->PW}, {&h->W32[2], h->PW},
-              {&h->W32[3], h->PW}, {&h->qs, h->N}, {&h->qc, h->N},
-              {&h->wq32, (int64_t)h->wq32_h.size()}, {&h->fc32, (int64_t)h->fc32_h.size()}};
+              {&h->W32[3], h->PW}, {&h->qs, h->N}, {&h->qc, h->N}};
     for (auto& b : fb) {
       e = cudaMalloc(b.p, sizeof(float) * std::max<int64_t>(b.n, 1));
       if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaMalloc (FP32 workspace)"));
     }
     for (int i = 0; i < 4 && e == cudaSuccess; ++i)
       e = cudaMemsetAsync(h->W32[i], 0, sizeof(float) * h->PW, h->stream);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(h->wq32, h->wq32_h.data(), sizeof(float) * h->wq32_h.size(),
-                          cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess && !h->fc32_h.empty())
-      e = cudaMemcpyAsync(h->fc32, h->fc32_h.data(), sizeof(float) * h->fc32_h.size(),
-                          cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cleanup(cuda_fail(e, "initialising FP32 workspace"));
   }
@@ -1418,8 +1411,7 @@ void mfwh_destroy(mfwh_handle_t h) {
   if (h->d_bar) cudaFree(h->d_bar);
   if (h->d_mgc) cudaFree(h->d_mgc);
   delete h->imp;
-  float* fbufs[] = {h->f32, h->W32[0], h->W32[1], h->W32[2], h->W32[3], h->qs, h->qc,
-                    h->wq32, h->fc32};
+  float* fbufs[] = {h->f32, h->W32[0], h->W32[1], h->W32[2], h->W32[3], h->qs, h->qc};
   for (float* b : fbufs)
     if (b) cudaFree(b);
   if (h->pinned) cudaFreeHost(h->pinned);
@@ -2017,7 +2009,15 @@ mfwh_status mfwh_autotune(const mfwh_problem* prob, void* stream, int* time_bloc
   if (P.order == 4 || P.c2_field || (P.dim == 3 && P.precision == MFWH_PREC_FP64)) {
     cand = {{1, 0}};
   } else if (P.dim == 3) {
-    cand = {{1, 0}, {2, 0}, {4, 0}};
+    // grids of at most one tile per SM: launches are bound by latency, and 1 (Kahan sums of every
+    // step, in launches of 4) is as fast as 4
+    int sms = 0;
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int64_t tiles = ((P.n[0] + 56) / 56) * ((P.n[1] + 8) / 8) * ((P.n[2] + 12) / 12);
+    if (tiles <= sms)
+      cand = {{1, 0}};
+    else
+      cand = {{1, 0}, {2, 0}, {4, 0}};
   } else if (P.precision == MFWH_PREC_FP64) {
     cand = {{1, 0}, {2, 5}, {3, 5}, {4, 5}, {4, 4}, {4, 3}, {8, 3}};
   } else {

@@ -20,8 +20,8 @@ struct Geom {
   int layer_axis;            // axis whose index selects the c^2 layer
   int64_t layer_split;       // indices >= layer_split use the upper-layer coefficients
   int order;                 // order of L_{ph}: 2 or 4 (0 reads as 2)
-  int64_t syw, szw;          // strides of j and k in the FP32 arrays W, D and f (2D FP32 handles
-                             // pad rows to 32 floats for 16-byte accesses; else sy, sz)
+  int64_t syw, szw;          // strides of j and k in the FP32 arrays W, D and f (FP32 handles pad
+                             // rows to 32 floats for 16-byte accesses; else sy, sz)
   int64_t wpoints;           // entries of one of them (stride between the frequencies of f)
   const double* c2f;         // c^2 per point [points] (MFWH_C_FIELD), else null; with a field
                              // the layer coefficients are those of c = 1 (lower layer only)
@@ -100,10 +100,8 @@ struct Step32Host {
 };
 struct TB32Host {
   Coef32 reg_lo, reg_hi, first_lo, first_hi;
-  const float* wq;         // device [(N_t + 1) * nf]
-  const float* fc;         // device [N_t * nf]
-  const float* wq_host;    // host copies of the two (the 2D kernel's travel as parameters)
-  const float* fc_host;
+  const float* wq_host;    // [(N_t + 1) * nf] (a launch's weights travel as parameters)
+  const float* fc_host;    // [N_t * nf]
   const double* binv;      // host [MFWH_MAX_NF * MFWH_MAX_NF], row-major, leading dim 16 (C)
   const double* emat;      // host, same layout (E of the explicit filter)
   int has_e;

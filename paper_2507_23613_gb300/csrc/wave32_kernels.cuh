@@ -16,11 +16,12 @@
 // q_m = s_m - c_m.  The filter solve V = B^{-1} q (eq. waveHoltzMatrixIteration)
 // and everything after it are FP64.
 //
-// Two kernels advance the scheme:
+// Three kernels advance the scheme:
 //  * k_tb2d32: 2D, T steps per launch on overlapped tiles whose points, halo included, live
 //    in the registers of one CTA for all T steps;
-//  * k_step32 / k_last32: one step per launch, 2D or 3D, second- or fourth-order L_h.
-// Both perform the same FP32 operations per point in the same order, so their
+//  * k_tb3d32: the same in 3D with T = 2 or 4;
+//  * k_step32 / k_last32: one step per launch, the fourth-order L_h and 2D at time_block 1.
+// All perform the same FP32 operations per point in the same order, so their
 // results are bit-identical.
 #pragma once
 
@@ -268,15 +269,6 @@ constexpr size_t rt32_smem_bytes() {
                           (size_t)2 * kRtWarps * 2 * kRtEX);
 }
 
-// One parameter block for the kernel and the 3D kernel's table-driven coefficients.
-template <int NF>
-struct TB32Args {
-  Coef32 reg_lo, reg_hi, first_lo, first_hi;
-  const float* wq;   // [(N_t + 1) * NF]
-  const float* fc;   // [N_t * NF]
-  int n0, steps, forced, last, subtract;
-};
-
 // Fold a partial sum x into the Kahan pair (s, c).
 __device__ __forceinline__ void kahan_fold(float& s, float& c, float x) {
   const float y = x - c;
@@ -523,154 +515,234 @@ k_init32(const double* __restrict__ v, float* __restrict__ W0, float* __restrict
 }
 
 // ---- temporally blocked 3D kernel ------------------------------------------------
-// Overlapped tiling in all three axes: a CTA owns a (32 - 2T) x 8 x 8 tile and keeps the tile
-// plus a halo of T points per side of W^n, W^{n+1} and D in shared memory, 32 points wide in
-// x so that a warp covers a row.  At step s of a launch of S steps it updates every interior
-// point of the tile grown by S - 1 - s points per side (reading the values of the previous
-// step one point further out), so the owned points are exact after S steps.  The rows (y, z)
-// of the region are spread over the warps and a row's points over the lanes.  Thread (x, y)
-// with x < 32 - 2T owns the 8 points of tile column (x, y) and keeps their filter sums in
-// registers (ACC as in k_tb2d32).  Each point update performs the operations of
-// step_point<NF, 3, 2> in the same order, so with ACC = 0 every depth is bit-identical to
-// one step per launch.
-constexpr int kT3W = 32, kT3Y = 8, kT3Z = 8, kT3Threads = kT3W * kT3Y;
+// The 2D kernel's scheme in 3D: one CTA per SM (16 warps) holds an extended tile of 64 x 16 x 20
+// points in registers, warp w the row y = w, lane l its columns 2l, 2l + 1 of all 20 planes, and
+// steps all of it T times (T = 2 or 4; planes and rows that no later step reads rest), after
+// which the (64 - 2T) x (16 - 2T) x (20 - 2T) points in the middle are exact.  Neighbours along z
+// are in the thread, along x in the thread or one shuffle away; along y they come from a copy of
+// the whole tile in shared memory, rewritten every step (two barriers a step).  As in 2D the new
+// values of the owned points are kept in shared memory and all filter updates made after the last
+// step, with the weights as constant operands.  Per point the operations are those of
+// step_point<NF, 3, 2> in the same order, so with ACC = 0 every depth is bit-identical to one step
+// per launch.
+//
+// HBM bounds it: 16 + 16 N_f bytes per owned point and launch, and the halo of W and D.  257^3,
+// N_f = 4, two layers, depth 4 (one map of 885 steps): 235 ms for the form it replaces (a flat tile
+// in shared memory, 61 % issue, 13 % DRAM), 141 ms for this one.
+constexpr int kR3X = 64, kR3Y = 16, kR3Z = 20, kR3Threads = 32 * kR3Y;
+
+template <int NF, int T>
+struct R3Args {
+  Coef32 reg_lo, reg_hi, first_lo, first_hi;
+  int n0, steps, forced, last, subtract;
+  float wq[T * NF];   // w_{n+1,m} of step s: [s * NF + m]
+  float fc[T * NF];   // kappa_n cos(omega~_m t^n)
+};
+
+template <int T>
+constexpr size_t r3_smem_bytes() {
+  return sizeof(float) * ((size_t)kR3X * kR3Y * kR3Z +
+                          (size_t)T * (kR3X - 2 * T) * (kR3Y - 2 * T) * (kR3Z - 2 * T));
+}
 
 template <int NF, int T, int ACC>
-__global__ void __launch_bounds__(kT3Threads, ACC == 1 ? 2 : 1)
+__global__ void __launch_bounds__(kR3Threads, 1)
 k_tb3d32(const float* __restrict__ W_in, const float* __restrict__ D_in,
          float* __restrict__ W_out, float* __restrict__ D_out, const float* __restrict__ f,
          float* __restrict__ qs, float* __restrict__ qc, double* vout, const double* vsub,
-         const TB32Args<NF> a, const Last32Binv<NF> b, const Geom g) {
-  constexpr int BX = kT3W - 2 * T;
-  constexpr int EX = kT3W, EY = kT3Y + 2 * T, EZ = kT3Z + 2 * T;
-  constexpr int SXY = EX * EY, E = SXY * EZ;
+         const __grid_constant__ R3Args<NF, T> a, const __grid_constant__ Last32Binv<NF> b,
+         const Geom g) {
+  constexpr int VX = kR3X - 2 * T, VY = kR3Y - 2 * T, VZ = kR3Z - 2 * T;   // owned points
+  constexpr int VXY = VX * VY, V = VXY * VZ;
   extern __shared__ __align__(16) float sm3[];
-  float* Wc = sm3;
-  float* Wn = sm3 + E;
-  float* Dv = sm3 + 2 * E;
-  float* s_wq = sm3 + 3 * E;    // [T][NF]
-  float* s_fc = s_wq + T * NF;  // [T][NF]
-  const int tid = threadIdx.x;
-  const int tx = tid % kT3W, ty = tid / kT3W;   // lanes along x, warps along rows
-  const int64_t x0 = (int64_t)blockIdx.x * BX - T, y0 = (int64_t)blockIdx.y * kT3Y - T,
-                z0 = (int64_t)blockIdx.z * kT3Z - T;
+  float* tile = sm3;                          // [z][y][x] the level being read
+  float* hist = sm3 + kR3X * kR3Y * kR3Z;     // [T][VZ][VY][VX] owned values step by step
+  const int tid = threadIdx.x, lane = tid & 31, ly = tid >> 5, lx = 2 * lane;
+  const int64_t x0 = (int64_t)blockIdx.x * VX - T, y0 = (int64_t)blockIdx.y * VY - T,
+                z0 = (int64_t)blockIdx.z * VZ - T;
+  // local bounds (32-bit): interior columns, rows and planes, planes of the grid
+  auto local = [](int64_t v) { return v < -1 ? -1 : (v > 64 ? 64 : (int)v); };
+  const int ilx = local(1 - x0), ihx = local(g.nx - 1 - x0);
+  const int ily = local(1 - y0), ihy = local(g.ny - 1 - y0);
+  const int ilz = local(1 - z0), ihz = local(g.nz - 1 - z0);
+  const bool in_y = ly >= ily && ly <= ihy;
+  const bool in0 = in_y && lx >= ilx && lx <= ihx, in1 = in_y && lx + 1 >= ilx && lx + 1 <= ihx;
+  // c^2 layer: local index along the layer axis from which hi holds
+  const int thr = local(g.layer_split - (g.layer_axis == 0 ? x0 : (g.layer_axis == 1 ? y0 : z0)));
+  const bool owner_xy = lx >= T && lx < T + VX && ly >= T && ly < T + VY;
+  const int64_t gbase = z0 * g.szw + (y0 + ly) * g.syw + x0 + lx;
+
+  float w[kR3Z][2], d[kR3Z][2];
   {
-    const int64_t gx = x0 + tx;
-    for (int row = ty; row < EY * EZ; row += kT3Y) {
-      const int lz = row / EY, ly = row - lz * EY;
-      const int64_t gy = y0 + ly, gz = z0 + lz;
-      const bool in = gz >= 0 && gz <= g.nz && gy >= 0 && gy <= g.ny && gx >= 0 && gx <= g.nx;
-      const int64_t q = gz * g.szw + gy * g.syw + gx;
-      const int e = lz * SXY + ly * EX + tx;
-      const float w = in ? W_in[q] : 0.0f;
-      Wc[e] = w;
-      Wn[e] = w;
-      Dv[e] = (in && D_in != nullptr) ? D_in[q] : 0.0f;
+    // x0 + lx is even and rows are padded: both columns lie in a row of the arrays or none
+    const bool col = y0 + ly >= 0 && y0 + ly <= g.ny && x0 + lx >= 0 && x0 + lx < g.syw;
+#pragma unroll
+    for (int k = 0; k < kR3Z; ++k) {
+      float2 v = make_float2(0.0f, 0.0f), u = v;
+      if (col && k >= ilz && k <= ihz) {   // outside the interior W = 0
+        v = *reinterpret_cast<const float2*>(W_in + gbase + k * g.szw);
+        if (D_in != nullptr) u = *reinterpret_cast<const float2*>(D_in + gbase + k * g.szw);
+      }
+      w[k][0] = in0 ? v.x : 0.0f;
+      w[k][1] = in1 ? v.y : 0.0f;
+      d[k][0] = in0 ? u.x : 0.0f;
+      d[k][1] = in1 ? u.y : 0.0f;
     }
   }
-  for (int e = tid; e < a.steps * NF; e += kT3Threads) {
-    const int st = e / NF, m = e - st * NF;
-    const int n = a.n0 + st;
-    s_wq[e] = a.wq[(n + 1) * NF + m];
-    s_fc[e] = a.forced ? a.fc[n * NF + m] : 0.0f;
+  // Ask L2 for the sums that the end of the launch updates.
+  if (owner_xy && (lane & 7) == T / 2) {
+    const int64_t p = (z0 + T) * g.sz + (y0 + ly) * g.sy + x0 + lx;
+    for (int e = 0; e < 2 * NF; ++e) {
+      const float* base = (e & 1 ? qc : qs) + (int64_t)(e >> 1) * g.points;
+      for (int k = 0; k < VZ; ++k)
+        if (in0 && k + T >= ilz && k + T <= ihz)
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(base + p + k * g.sz));
+    }
   }
-  // the owned column (threads with tx < BX)
-  const bool owner = tx < BX;
-  const int64_t gx = x0 + T + tx, gy = y0 + T + ty;
-  const bool col_int = owner && gx > 0 && gx < g.nx && gy > 0 && gy < g.ny;
-  bool own_int[kT3Z];
-  float ks[kT3Z][NF], kc[kT3Z][NF], part[kT3Z][NF];
+  // PLAIN: all points of the CTA are interior with one c^2, no forcing; the values are the same.
+  auto run_steps = [&](auto plain_c) {
+    constexpr bool PLAIN = decltype(plain_c)::value;
+    float* mine = tile + ly * kR3X + lx;
+    for (int s = 0; s < a.steps; ++s) {
+      const int r = a.steps - 1 - s;   // later steps read the owned points grown by r
+      const bool first = a.n0 + s == 0;
+      const Coef32 lo = first ? a.first_lo : a.reg_lo, hi = first ? a.first_hi : a.reg_hi;
+      const Coef32 one = thr <= 0 ? hi : lo;
+      const bool upper_y = g.layer_axis == 1 && ly >= thr;
+      const bool upper0 = upper_y || (g.layer_axis == 0 && lx >= thr);
+      const bool upper1 = upper_y || (g.layer_axis == 0 && lx + 1 >= thr);
+      // rows read at this step: those updated and one beyond
+      if (ly >= T - r - 1 && ly <= T + VY + r) {
 #pragma unroll
-  for (int k = 0; k < kT3Z; ++k) {
-    const int64_t gz = z0 + T + k;
-    own_int[k] = col_int && gz > 0 && gz < g.nz;
-    const int64_t p = gz * g.sz + gy * g.sy + gx;
+        for (int k = 0; k < kR3Z; ++k)
+          *reinterpret_cast<float2*>(mine + k * (kR3X * kR3Y)) = make_float2(w[k][0], w[k][1]);
+      }
+      __syncthreads();
+      if (ly >= T - r && ly < T + VY + r) {
+        float dz0 = 0.0f, dz1 = 0.0f;   // W - W_below of the current plane
+#pragma unroll
+        for (int k = 0; k < kR3Z; ++k) {
+          const float w0 = w[k][0], w1 = w[k][1];
+          float dn0 = 0.0f, dn1 = 0.0f;
+          if (k + 1 < kR3Z) {
+            dn0 = w[k + 1 < kR3Z ? k + 1 : k][0] - w0;
+            dn1 = w[k + 1 < kR3Z ? k + 1 : k][1] - w1;
+          }
+          if (k >= T - r && k < T + VZ + r) {
+            const float left = __shfl_up_sync(0xffffffffu, w1, 1);
+            const float right = __shfl_down_sync(0xffffffffu, w0, 1);
+            const float2 ym = *reinterpret_cast<const float2*>(mine + k * (kR3X * kR3Y) - kR3X);
+            const float2 yp = *reinterpret_cast<const float2*>(mine + k * (kR3X * kR3Y) + kR3X);
+            const float dx0 = w0 - left, dx1 = w1 - w0, dx2 = right - w1;
+            const float dxx0 = dx1 - dx0, dxx1 = dx2 - dx1;
+            const float dyy0 = (ym.x - w0) + (yp.x - w0), dyy1 = (ym.y - w1) + (yp.y - w1);
+            const float dzz0 = dn0 - dz0, dzz1 = dn1 - dz1;
+            const bool uz = !PLAIN && g.layer_axis == 2 && k >= thr;
+            const Coef32 L0 = PLAIN ? one : ((upper0 || uz) ? hi : lo);
+            const Coef32 L1 = PLAIN ? one : ((upper1 || uz) ? hi : lo);
+            float i0 = L0.Ay * dyy0, i1 = L1.Ay * dyy1;
+            i0 = fmaf(L0.Az, dzz0, i0);
+            i1 = fmaf(L1.Az, dzz1, i1);
+            i0 = fmaf(L0.Ax, dxx0, i0);
+            i1 = fmaf(L1.Ax, dxx1, i1);
+            if (!PLAIN && a.forced && (in0 || in1) && k >= ilz && k <= ihz) {
+              const float* fp = f + gbase + k * g.szw;   // rows of f are padded like those of W
+#pragma unroll 4
+              for (int m = 0; m < NF; ++m) {
+                const float2 v = *reinterpret_cast<const float2*>(fp + m * g.wpoints);
+                i0 = fmaf(-a.fc[s * NF + m], v.x, i0);
+                i1 = fmaf(-a.fc[s * NF + m], v.y, i1);
+              }
+            }
+            float d0 = d[k][0] + i0, d1 = d[k][1] + i1;
+            float n0 = w0 + d0, n1 = w1 + d1;
+            if (!PLAIN) {   // boundary and outside points keep W = 0
+              const bool iz = k >= ilz && k <= ihz;
+              if (!(in0 && iz)) d0 = n0 = 0.0f;
+              if (!(in1 && iz)) d1 = n1 = 0.0f;
+            }
+            d[k][0] = d0;
+            d[k][1] = d1;
+            w[k][0] = n0;
+            w[k][1] = n1;
+          }
+          dz0 = dn0;
+          dz1 = dn1;
+        }
+        if (owner_xy) {
+          float* h = hist + (size_t)s * V + (ly - T) * VX + lx - T;
+#pragma unroll
+          for (int k = T; k < T + VZ; ++k)
+            *reinterpret_cast<float2*>(h + (k - T) * VXY) = make_float2(w[k][0], w[k][1]);
+        }
+      }
+      __syncthreads();
+    }
+  };
+  const bool simple = !a.forced && ilx <= 0 && ihx >= kR3X - 1 && ily <= 0 && ihy >= kR3Y - 1 &&
+                      ilz <= 0 && ihz >= kR3Z - 1 &&
+                      (thr <= 0 || thr >= (g.layer_axis == 0 ? kR3X : (g.layer_axis == 1 ? kR3Y : kR3Z)));
+  if (simple)
+    run_steps(std::true_type{});
+  else
+    run_steps(std::false_type{});
+  if (owner_xy && !a.last && y0 + ly <= g.ny && x0 + lx < g.syw) {
+#pragma unroll
+    for (int k = T; k < T + VZ; ++k) {
+      if (z0 + k > g.nz) continue;
+      *reinterpret_cast<float2*>(W_out + gbase + k * g.szw) = make_float2(w[k][0], w[k][1]);
+      *reinterpret_cast<float2*>(D_out + gbase + k * g.szw) = make_float2(d[k][0], d[k][1]);
+    }
+  }
+  // The filter sums of the owned points.
+#pragma unroll 2
+  for (int i = tid; i < V; i += kR3Threads) {
+    const int rz = i / VXY, rest = i - rz * VXY, ry = rest / VX, rx = rest - ry * VX;
+    const int64_t x = x0 + T + rx, y = y0 + T + ry, z = z0 + T + rz;
+    const bool in = x > 0 && x < g.nx && y > 0 && y < g.ny && z > 0 && z < g.nz;
+    if (!in && !(a.last && x <= g.nx && y <= g.ny && z <= g.nz)) continue;
+    const int64_t p = z * g.sz + y * g.sy + x;
+    float ks[NF], kc[NF];
 #pragma unroll
     for (int m = 0; m < NF; ++m) {
-      part[k][m] = 0.0f;
-      ks[k][m] = (ACC == 0 && own_int[k]) ? qs[m * g.points + p] : 0.0f;
-      kc[k][m] = (ACC == 0 && own_int[k]) ? qc[m * g.points + p] : 0.0f;
+      ks[m] = in ? qs[m * g.points + p] : 0.0f;
+      kc[m] = in ? qc[m * g.points + p] : 0.0f;
     }
-  }
-  __syncthreads();
-  for (int s = 0; s < a.steps; ++s) {
-    const int r = a.steps - 1 - s;
-    const bool first = a.n0 + s == 0;
-    const Coef32 lo = first ? a.first_lo : a.reg_lo;
-    const Coef32 hi = first ? a.first_hi : a.reg_hi;
-    const float* fc = s_fc + s * NF;
-    // the region [T - r, T + tile + r) per axis
-    const int l0 = T - r, RY = kT3Y + 2 * r, RZ = kT3Z + 2 * r;
-    const int lx = l0 + tx;
-    const int64_t px = x0 + lx;
-    const bool x_ok = lx < T + BX + r && px > 0 && px < g.nx;
-    for (int row = ty; row < RY * RZ; row += kT3Y) {
-      const int rz = row / RY, ry = row - rz * RY;
-      const int ly = l0 + ry, lz = l0 + rz;
-      const int64_t py = y0 + ly, pz = z0 + lz;
-      if (!x_ok || py <= 0 || py >= g.ny || pz <= 0 || pz >= g.nz) continue;
-      const int l = lz * SXY + ly * EX + lx;
-      const int64_t li = g.layer_axis == 0 ? px : (g.layer_axis == 1 ? py : pz);
-      const Coef32& L = li >= g.layer_split ? hi : lo;
-      const float w = Wc[l];
-      const float dxx = (Wc[l - 1] - w) + (Wc[l + 1] - w);
-      const float dyy = (Wc[l - EX] - w) + (Wc[l + EX] - w);
-      const float dzz = (Wc[l - SXY] - w) + (Wc[l + SXY] - w);
-      const int64_t q = pz * g.szw + py * g.syw + px;
-      const float inc = increment<NF, 3>(L, dxx, dyy, dzz, fc, f, q, g.wpoints, a.forced);
-      const float dn = Dv[l] + inc;
-      Dv[l] = dn;
-      Wn[l] = w + dn;
-    }
-    __syncthreads();
+    if (in) {
+      float part[ACC == 1 ? NF : 1];
+      if constexpr (ACC == 1) {
 #pragma unroll
-    for (int k = 0; k < kT3Z; ++k) {
-      if (!own_int[k]) continue;
-      const float wn = Wn[(T + k) * SXY + (T + ty) * EX + T + tx];
-#pragma unroll
-      for (int m = 0; m < NF; ++m) {
-        if (ACC == 0)
-          kahan_add(ks[k][m], kc[k][m], s_wq[s * NF + m], wn);
-        else
-          part[k][m] = fmaf(s_wq[s * NF + m], wn, part[k][m]);
+        for (int m = 0; m < NF; ++m) part[m] = 0.0f;
       }
-    }
-    float* t = Wc;
-    Wc = Wn;
-    Wn = t;
-  }
-  // Wc holds W^{n0+steps} and Dv the matching D on the owned points
-  if (!owner) return;
+      auto add = [&](int s, float v) {
 #pragma unroll
-  for (int k = 0; k < kT3Z; ++k) {
-    const int64_t gz = z0 + T + k;
-    if (gx > g.nx || gy > g.ny || gz > g.nz) continue;
-    const int64_t p = gz * g.sz + gy * g.sy + gx;
-    const int l = (T + k) * SXY + (T + ty) * EX + T + tx;
-    if (ACC == 1 && own_int[k]) {
+        for (int m = 0; m < NF; ++m) {
+          if constexpr (ACC == 1)
+            part[m] = fmaf(a.wq[s * NF + m], v, part[m]);
+          else
+            kahan_add(ks[m], kc[m], a.wq[s * NF + m], v);
+        }
+      };
+      if (a.steps == T) {
 #pragma unroll
-      for (int m = 0; m < NF; ++m) {
-        ks[k][m] = qs[m * g.points + p];
-        kc[k][m] = qc[m * g.points + p];
-        kahan_fold(ks[k][m], kc[k][m], part[k][m]);
+        for (int s = 0; s < T; ++s) add(s, hist[s * V + i]);
+      } else {
+#pragma unroll 1
+        for (int s = 0; s < a.steps; ++s) add(s, hist[s * V + i]);
+      }
+      if constexpr (ACC == 1) {
+#pragma unroll
+        for (int m = 0; m < NF; ++m) kahan_fold(ks[m], kc[m], part[m]);
       }
     }
     if (!a.last) {
-      if (!own_int[k]) continue;
-      const int64_t q = gz * g.szw + gy * g.syw + gx;
-      W_out[q] = Wc[l];
-      D_out[q] = Dv[l];
 #pragma unroll
       for (int m = 0; m < NF; ++m) {
-        qs[m * g.points + p] = ks[k][m];
-        qc[m * g.points + p] = kc[k][m];
+        qs[m * g.points + p] = ks[m];
+        qc[m * g.points + p] = kc[m];
       }
     } else {
-      if (!own_int[k]) {
-#pragma unroll
-        for (int m = 0; m < NF; ++m) ks[k][m] = kc[k][m] = 0.0f;
-      }
-      filter_solve_out<NF>(ks[k], kc[k], b, a.subtract, vsub, vout, p, g.points, own_int[k]);
+      filter_solve_out<NF>(ks, kc, b, a.subtract, vsub, vout, p, g.points, in);
     }
   }
 }
@@ -719,9 +791,7 @@ void step32_nf(const Geom& g, const float* W, const float* D_in, float* W_out, f
       k_step32<NF, 3, 4><<<grid, blk, 0, st>>>(W, D_in, W_out, D_out, f, qs, qc, a, g);
     else
       k_step32<NF, 2, 4><<<grid, blk, 0, st>>>(W, D_in, W_out, D_out, f, qs, qc, a, g);
-  } else if (g.dim == 3) {
-    k_step32<NF, 3, 2><<<grid, blk, 0, st>>>(W, D_in, W_out, D_out, f, qs, qc, a, g);
-  } else {
+  } else {   // (second-order 3D steps are those of k_tb3d32)
     k_step32<NF, 2, 2><<<grid, blk, 0, st>>>(W, D_in, W_out, D_out, f, qs, qc, a, g);
   }
 }
@@ -739,8 +809,6 @@ void last32_nf(const Geom& g, const float* W, const float* D, const float* f, co
       k_last32<NF, 3, 4><<<grid, blk, 0, st>>>(W, D, f, qs, qc, vout, vsub, a, b, sub, g);
     else
       k_last32<NF, 2, 4><<<grid, blk, 0, st>>>(W, D, f, qs, qc, vout, vsub, a, b, sub, g);
-  } else if (g.dim == 3) {
-    k_last32<NF, 3, 2><<<grid, blk, 0, st>>>(W, D, f, qs, qc, vout, vsub, a, b, sub, g);
   } else {
     k_last32<NF, 2, 2><<<grid, blk, 0, st>>>(W, D, f, qs, qc, vout, vsub, a, b, sub, g);
   }
@@ -818,9 +886,7 @@ template <int NF, int T, int ACC>
 void tb3d32_launch(const Geom& g, const float* W_in, const float* D_in, float* W_out,
                    float* D_out, const float* f, float* qs, float* qc, double* vout,
                    const double* vsub, const TB32Host& h, cudaStream_t st) {
-  constexpr int E = kT3W * (kT3Y + 2 * T) * (kT3Z + 2 * T);
-  constexpr int BX = kT3W - 2 * T;
-  constexpr size_t smem = sizeof(float) * (3 * E + 2 * T * NF);
+  constexpr size_t smem = r3_smem_bytes<T>();
   static bool configured[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
@@ -829,23 +895,27 @@ void tb3d32_launch(const Geom& g, const float* W_in, const float* D_in, float* W
                          (int)smem);
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
-  TB32Args<NF> a;
+  R3Args<NF, T> a;
   a.reg_lo = h.reg_lo;
   a.reg_hi = h.reg_hi;
   a.first_lo = h.first_lo;
   a.first_hi = h.first_hi;
-  a.wq = h.wq;
-  a.fc = h.fc;
   a.n0 = h.n0;
   a.steps = h.steps;
   a.forced = h.forced;
   a.last = h.last;
   a.subtract = vsub != nullptr;
+  for (int s = 0; s < T; ++s)
+    for (int m = 0; m < NF; ++m) {
+      a.wq[s * NF + m] = s < h.steps ? h.wq_host[(size_t)(h.n0 + s + 1) * NF + m] : 0.0f;
+      a.fc[s * NF + m] = s < h.steps && h.forced ? h.fc_host[(size_t)(h.n0 + s) * NF + m] : 0.0f;
+    }
   const Last32Binv<NF> b = binv_args<NF>(h.binv, h.emat, h.has_e, h.vprev);
-  const dim3 grid((unsigned)((g.nx + BX) / BX), (unsigned)((g.ny + kT3Y) / kT3Y),
-                  (unsigned)((g.nz + kT3Z) / kT3Z));
-  k_tb3d32<NF, T, ACC><<<grid, kT3Threads, smem, st>>>(W_in, D_in, W_out, D_out, f, qs, qc,
-                                                          vout, vsub, a, b, g);
+  constexpr int VX = kR3X - 2 * T, VY = kR3Y - 2 * T, VZ = kR3Z - 2 * T;
+  const dim3 grid((unsigned)((g.nx + VX) / VX), (unsigned)((g.ny + VY) / VY),
+                  (unsigned)((g.nz + VZ) / VZ));
+  k_tb3d32<NF, T, ACC><<<grid, kR3Threads, smem, st>>>(W_in, D_in, W_out, D_out, f, qs, qc, vout,
+                                                       vsub, a, b, g);
 }
 
 // Depth 2 or 4 (a launch of at most T steps; the halo is T points).
