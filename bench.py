@@ -200,8 +200,17 @@ def blocked_kernel_source_key():
     argument structs (kernels.h) and the float-pair arithmetic (fpair.cuh)."""
     h = hashlib.sha256()
     h.update(_region("wave_tb_kernels.cuh", "\0"))
-    h.update(_region("kernels.h", "// ---- FP32 path"))
+    h.update(_region("kernels.h", "// ---- FP64 wave solve of 2D grids in 64-bit fixed point"))
     h.update(_region("fpair.cuh", "\0"))
+    return h.hexdigest()[:16]
+
+
+def fixed_kernel_source_key():
+    """Hash of the FP64 fixed-point kernels' source (wave_fx_kernels.cuh, wave_fx.cu) and of their
+    arithmetic (fixed64.cuh)."""
+    h = hashlib.sha256()
+    for name in ("wave_fx_kernels.cuh", "wave_fx.cu", "fixed64.cuh"):
+        h.update(_region(name, "\0"))
     return h.hexdigest()[:16]
 
 
@@ -1156,7 +1165,8 @@ def workload_config(wl, n_t):
             "grid": [wl.n[0] + 1, wl.n[1] + 1], "nf": wl.nf, "n_p": wl.n_p, "n_t": n_t,
             "omega_band": [10.0, 60.0], "gaussian_b": 400.0, "cfl": wl.cfl,
             "restart": RESTART, "tol": TOL,
-            "precision": "fp64 wave levels, steps and filter solve; filter sums as float pairs",
+            "precision": "fp64 interface, forcing and filter solve; wave levels and filter sums as "
+                         "64-bit integers (steps rounded to 2^-58 of the largest level)",
             "l2": "working set (forcing, accumulators, Krylov basis: > 1 GB) is larger than L2"}
 
 
@@ -1324,19 +1334,17 @@ def main():
                     "unit": "TFLOP/s", "frac": round(achieved_tf / FP64_PEAK_TFLOPS, 4)}
         roof["alg_bytes_per_launch"] = round(alg_bytes / max(step_launches, 1))
     else:
-        # Blocked launches move (4 + 2 N_f (+ N_f forced)) words per point whatever their depth;
-        # the bound is the FP64 pipe (5 FP64 instructions per homogeneous point-step).
+        # Blocked launches move (4 + 2 N_f (+ N_f forced)) words per point whatever their depth.
+        # The fixed-point kernel (the default) is bound by instruction issue; its rate is given
+        # against the FP64 pipe that the FP64 form of the step would need (5 FP64 instructions per
+        # homogeneous point-step) and may exceed 1.
         blk_bytes = wl.interior_points * (
             forced_apps * -(-n_t // depth) * blocked_bytes_per_point_launch(wl.nf, True)
             + homog_apps * -(-n_t // depth) * blocked_bytes_per_point_launch(wl.nf, False))
         blk_gbs = blk_bytes / (step_ms_total * 1e-3) / 1e9
-        shape = args.tile_shape if args.time_block else 5
-        pipe = depth <= 4 and shape == 5 and wl.nf <= 8
-        traffic = (kernel_traffic("k_tb2d_pipe_square1025_nf8.txt", blocked_kernel_source_key())
-                   if pipe else None)
-        kernel = ("k_tb2d_pipe (%d leapfrog steps + N_f filters per pass, persistent CTAs "
-                  "copying the next tile while stepping one)" % depth if pipe else
-                  "k_tb2d (%d leapfrog steps + N_f filters per launch)" % depth)
+        traffic = kernel_traffic("k_fx2d_square1025_nf8.txt", fixed_kernel_source_key())
+        kernel = ("k_fx2d (%d leapfrog steps in 64-bit fixed point + N_f filters per launch, warp "
+                  "roles: stepping and summing)" % depth)
         roof = {"bound": "alu", "achieved": round(achieved_tf, 4), "peak": round(FP64_PEAK_TFLOPS, 4),
                 "unit": "TFLOP/s", "frac": round(achieved_tf / FP64_PEAK_TFLOPS, 4),
                 "alg_bytes_per_launch": round(blk_bytes / max(step_launches, 1)),

@@ -54,11 +54,15 @@ typedef enum {
 } mfwh_status;
 
 enum { MFWH_FILTER_OPTIMIZED = 0, MFWH_FILTER_TRADITIONAL = 1, MFWH_FILTER_USER = 2 };
-/* Arithmetic of the wave solve.  FP64: wave levels, steps and the filter solve in FP64; with
-   explicit time stepping the filter sums q_m are unevaluated float pairs (hi + lo, updated
-   with two-product/two-sum on the FP32 pipe, about 2^-47 relative per update), so their
-   magnitudes must stay below the float range (3.4e38) and keep full accuracy above about
-   1e-30.  FP32_KAHAN: wave levels and
+/* Arithmetic of the wave solve.  FP64: wave levels, steps and the filter solve at least as accurate
+   as in FP64.  Explicit steps in 2D with a constant or two-layer c advance 64-bit integers in
+   units of a quantum of 2^-58 to 2^-54 of the largest level, which follows that level, over the
+   whole range of double; beyond (infinities, NaN, magnitudes outside 1e-250 .. 1e250) they step
+   in FP64.  The other explicit FP64 problems (3D, a c^2 field, grids with dt^2 c^2 / h^2 below
+   2^-10, at least 1 or a multiple of 2^-24 along an axis, grids of very few rows or columns) keep
+   wave levels in FP64 and the filter sums q_m as unevaluated float pairs (hi + lo, updated with
+   two-product/two-sum on the FP32 pipe, about 2^-47 relative per update), so their magnitudes
+   must stay below the float range (3.4e38) and keep full accuracy above about 1e-30.  FP32_KAHAN: wave levels and
    steps in FP32 (increment form of the leapfrog scheme), filter sums with a Kahan update at
    every step; the filter solve B^{-1} q, GMRES and the residual stay FP64.  FP32_BLOCKSUM:
    as FP32_KAHAN, but a blocked launch of T steps sums its T filter terms in plain FP32 and
@@ -97,13 +101,15 @@ typedef struct {
   int n_delta;               /* N_delta of eq. LambdaRange (paper: 20) */
   double c_delta;            /* c_delta of eq. LambdaRange (paper: 2) */
   int precision;             /* MFWH_PREC_FP64, MFWH_PREC_FP32_KAHAN or MFWH_PREC_FP32_BLOCKSUM */
-  int time_block;            /* leapfrog steps per pass over HBM: 0 = library default (3 for
-                                FP64 2D problems of up to 8 frequencies with second order,
-                                explicit steps and constant or two-layer c, on tile shape 5;
-                                1 for the other FP64 problems and for 3D; 16 for FP32 in 2D),
-                                1 = one step per kernel launch; 2D: 2, 3, 4 or 8 for FP64, 4, 8
-                                or 16 for FP32 = temporal blocking with that depth; 3D: 2 or 4
-                                for the FP32 precisions.  Results are bit-identical for every
+  int time_block;            /* leapfrog steps per pass over HBM: 0 = library default (16 for
+                                FP32 in 2D; FP64 problems in 64-bit integers, see the precision:
+                                8 whatever this says, for the fourth order 4; other FP64 2D
+                                problems of up to 8 frequencies with second order, explicit steps
+                                and constant or two-layer c: 3 on tile shape 5; else 1),
+                                1 = one step per kernel launch (FP32 3D, second order: Kahan sums
+                                of one step each, in launches of 4); 2D: 2, 3, 4 or 8 for FP64,
+                                4, 8 or 16 for FP32 = temporal blocking with that depth; 3D: 2 or
+                                4 for the FP32 precisions.  Results are bit-identical for every
                                 depth (FP32_BLOCKSUM: for every depth with the same partial-sum
                                 length). */
   int order;                 /* order p of the spatial operator L_{ph}: 2 (0 means 2) or 4.
@@ -340,9 +346,10 @@ mfwh_status mfwh_solve_batch_graph(const mfwh_handle_t* handles, int count, int 
 
 /* Autotuner for the blocked wave kernels.  Times the first steps (at most 96) of a
  * homogeneous wave solve of prob on the current device for each candidate temporal depth and
- * tile shape (FP32, 2D: depths 4, 8, 16; FP64, 2D: depth 1, and depths
- * 4, 8 x tile shapes 1, 3; FP32, 3D: depths 1, 2, 4; FP64 3D, fourth order and c^2 fields:
- * depth 1), keeping the fastest:
+ * tile shape (FP32, 2D: depths 4, 8, 16; FP64, 2D: (8, 3), which has no effect, for problems in
+ * 64-bit integers, else depths 1 to 8 and their tile shapes; FP32, 3D: depths 1, 2, 4, only 1 for
+ * grids of at most one tile per SM; FP64 3D, fourth order and c^2 fields: depth 1), keeping the
+ * fastest:
  * *time_block and *tile_shape receive it, *ms_per_step
  * (may be NULL) its time per leapfrog step.  Results are cached per device, grid, number of
  * frequencies and precision for the life of the process.  Allocates (and frees) one handle's

@@ -18,6 +18,7 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include "fixed64.cuh"
 #include "internal.h"
 #include "kernels.h"
 
@@ -151,6 +152,19 @@ struct mfwh_handle_s {
   double* Wb = nullptr;
   double* Wc2 = nullptr;            // second pair of wave levels (temporal blocking:
   double* Wp2 = nullptr;            // a launch reads one pair and writes the other)
+  // FP64 wave solves in fixed point (Plan::fixed): the four arrays above hold 64-bit integers, W
+  // and D of the one pair and of the other, and q the tiled integer sums
+  int64_t* fx_force = nullptr;      // forcing of a launch's steps [8][PW]
+  unsigned long long* fx_max = nullptr;   // [0] max |W^0|, [1 + m] max |f_m|, as bits
+  FxForcing* fx_forcing = nullptr;
+  FxScale* fx_scale = nullptr;
+  FxState* fx_state = nullptr;      // [3]
+  FxCoef fx_cx[2][2], fx_cy[2][2];  // [first step][upper layer]: kappa c^2 / h_x^2 and / h_y^2
+  double fx_gw = 0.0, fx_gd = 0.0, fx_gf = 0.0;   // growth of the levels over 8 steps
+  std::vector<int64_t> fx_wint;     // [(N_t + 1) * nf] w_{n,m} 2^wexp[m]
+  int fx_wexp[MFWH_MAX_NF] = {};
+  int fx_else[2] = {1, 0};          // time_block and tile_shape of the FP64 kernels (fx_drop)
+  int fx_wsum = 0, fx_nw = 0;       // sum_n |fx_wint| < 2^fx_wsum; step warps
   double* d_wq = nullptr;           // [(N_t + 1) * nf] filter weights w_{n,m}
   double* d_cos = nullptr;          // [(N_t + 1) * nf] cos(omega~_m t^n)
   double* q = nullptr;              // filter accumulators [nf][P]
@@ -345,6 +359,9 @@ mfwh_status apply_pi32(mfwh_handle_t h, const double* vin, double* vout, int for
 mfwh_status apply_pi_tb(mfwh_handle_t h, const double* vin, double* vout, int forced,
                         const double* vsub);
 
+mfwh_status apply_pi_fx(mfwh_handle_t h, const double* vin, double* vout, int forced,
+                        const double* vsub, bool add = false);
+
 // Implicit trapezoidal wave solve: one init launch, then one launch per step (multigrid solve
 // of A Z = rhs and the update of W, q and the next rhs; the last one writes v_out).
 mfwh_status apply_pi_implicit(mfwh_handle_t h, const double* vin, double* vout, int forced,
@@ -403,6 +420,7 @@ mfwh_status apply_pi_direct(mfwh_handle_t h, const double* vin, double* vout, in
                             const double* vsub) {
   if (h->implicit) return apply_pi_implicit(h, vin, vout, forced, vsub);
   if (h->use32) return apply_pi32(h, vin, vout, forced, vsub);
+  if (h->plan.fixed) return apply_pi_fx(h, vin, vout, forced, vsub);
   // The FP64 blocked kernel (depth 2, 3, 4 or 8) serves the FP64 wave solves of FP64 handles
   // with time_block > 1 and those of 2D FP32 handles (the FP64 residuals and products of
   // mfwh_solve_refined and mfwh_solve_relaxed).
@@ -518,6 +536,168 @@ mfwh_status apply_pi_tb(mfwh_handle_t h, const double* vin, double* vout, int fo
   return MFWH_OK;
 }
 
+// kappa c^2 / h^2 as a 64-bit fraction (exact: see Plan::fixed).
+FxCoef fx_coef(double a) {
+  const uint64_t v = (uint64_t)std::ldexp(a, 64) & ~1ull;
+  return FxCoef{(uint32_t)v, (uint32_t)(v >> 32), v >> 1};
+}
+
+// Growth of the levels over at most 8 leapfrog steps in the maximum norm: |W^{n+k}| <= gw max |W^n|
+// + gd max |D^n| + gf dt^2 sum_m max |f_m|.  W^{n+k} = P_k W^n + Q_k D^n with the steps D' = D + L W,
+// W' = W + D' (L = dt^2 c^2 Delta_h; the first step of a wave solve has L / 2 and D = 0), and the
+// bounds are the largest absolute row sums of P_k and Q_k; a step's forcing acts like D of that
+// step, so gf is the sum over k of those of Q_k.  A row of P_k and Q_k is found by applying the
+// steps' transpose to a unit vector on a 19 x 19 patch, for every position of the layer
+// interface within reach.  The Dirichlet boundary (an odd reflection) only shortens rows.
+void fx_growth(const mfwh_handle_t h, double* gw, double* gd, double* gf) {
+  constexpr int R = 8, C = R + 1, E = 2 * C + 1;   // steps, centre and edge of the patch
+  const Plan& P = h->plan;
+  const double k = P.s.dt * P.s.dt;
+  const bool layers = P.c2_lo != P.c2_hi && P.layer_split > 0 && P.layer_split <= P.n[P.layer_axis];
+  *gw = 1.0;
+  *gd = *gf = 0.0;
+  double qmax[R + 1] = {}, u[E][E], v[E][E], t[E][E], c2[E];
+  // off: first index of the upper layer relative to the row's point (R + 1: all lower, R + 2: all
+  // upper)
+  for (int off = layers ? -R : R + 1; off <= R + 2; ++off) {
+    for (int i = 0; i < E; ++i) c2[i] = off == R + 2 || (off <= R && i - C >= off) ? P.c2_hi : P.c2_lo;
+    for (int j = 0; j < E; ++j)
+      for (int i = 0; i < E; ++i) u[j][i] = v[j][i] = t[j][i] = 0.0;
+    u[C][C] = 1.0;
+    const double kx = k * h->inv_h2[0], ky = k * h->inv_h2[1];
+    for (int s = 1; s <= R; ++s) {
+      // t = L^T (u + v), on the points reached
+      for (int j = C - s; j <= C + s; ++j)
+        for (int i = C - s; i <= C + s; ++i) {
+          auto at = [&](int ii, int jj) {
+            return c2[P.layer_axis == 0 ? ii : jj] * (u[jj][ii] + v[jj][ii]);
+          };
+          t[j][i] = kx * (at(i - 1, j) + at(i + 1, j)) + ky * (at(i, j - 1) + at(i, j + 1)) -
+                    2.0 * (kx + ky) * at(i, j);
+        }
+      double pu = 0.0, pf = 0.0, pv = 0.0;
+      for (int j = C - s; j <= C + s; ++j)
+        for (int i = C - s; i <= C + s; ++i) {
+          pf += std::fabs(u[j][i] + 0.5 * t[j][i]);
+          v[j][i] += u[j][i];
+          u[j][i] += t[j][i];
+          pu += std::fabs(u[j][i]);
+          pv += std::fabs(v[j][i]);
+        }
+      *gw = std::max(*gw, std::max(pu, pf));
+      qmax[s] = std::max(qmax[s], pv);
+    }
+  }
+  for (int s = 1; s <= R; ++s) {
+    *gd = std::max(*gd, qmax[s]);
+    *gf += qmax[s];
+  }
+  const double margin = 1.0 + 1e-6;   // roundings of the steps and of these sums
+  *gw *= margin;
+  *gd *= margin;
+  *gf *= margin;
+}
+
+// The weights as integers: |w_{n,m}| 2^wexp[m] below 2^60, their sum over n below 2^fx_wsum.
+void fx_weights(mfwh_handle_t h) {
+  const Plan& P = h->plan;
+  const int nf = h->nf;
+  h->fx_wint.resize(P.w.size());
+  h->fx_wsum = kFxWSumMin;
+  for (int m = 0; m < nf; ++m) {
+    double mx = 0.0, sum = 0.0;
+    for (int n = 0; n <= P.s.n_t; ++n) {
+      const double w = std::fabs(P.w[(size_t)n * nf + m]);
+      mx = std::max(mx, w);
+      sum += w;
+    }
+    int em = 0, es = 0;   // mx < 2^em, sum < 2^es
+    std::frexp(mx, &em);
+    std::frexp(sum, &es);
+    const int k = mx > 0.0 && std::isfinite(sum) ? std::min(60 - em, kFxWSumMax - 1 - es) : 0;
+    h->fx_wexp[m] = k;
+    if (mx > 0.0 && std::isfinite(sum)) h->fx_wsum = std::max(h->fx_wsum, es + k + 1);
+    for (int n = 0; n <= P.s.n_t; ++n) {
+      const double w = std::ldexp(P.w[(size_t)n * nf + m], k);
+      h->fx_wint[(size_t)n * nf + m] = std::isfinite(w) ? std::llrint(w) : 0;
+    }
+  }
+}
+
+// The forcing h->f as integers, after it has changed.
+cudaError_t fx_set_forcing(mfwh_handle_t h) {
+  if (!h->plan.fixed) return cudaSuccess;
+  launch_fx_forcing(h->nf, h->geom, h->f, h->fx_max + 1, h->fx_forcing, h->stream);
+  h->total_launches += 2;
+  return cudaGetLastError();
+}
+
+// Fixed-point wave solve (2D): three launches for the quantum, W^0 and the first filter terms, then
+// ceil(N_t / 8) launches alternating between the two pairs of level arrays; the last one writes
+// v_out (add: v_sub + V instead of v_sub - V).
+mfwh_status apply_pi_fx(mfwh_handle_t h, const double* vin, double* vout, int forced,
+                        const double* vsub, bool add) {
+  const Plan& P = h->plan;
+  const int nf = h->nf;
+  const int n_t = P.s.n_t;
+  const int n_run = h->tune_steps > 0 ? std::min(h->tune_steps, n_t) : n_t;
+  const double dt = P.s.dt;
+  cudaStream_t st = h->stream;
+  const FxArrays lev[2] = {
+      {reinterpret_cast<int64_t*>(h->Wa), reinterpret_cast<int64_t*>(h->Wb)},
+      {reinterpret_cast<int64_t*>(h->Wc2), reinterpret_cast<int64_t*>(h->Wp2)}};
+  int64_t* q = reinterpret_cast<int64_t*>(h->q);
+  launch_fx_init(nf, h->geom, vin, lev[0].W, q, &P.w[0], h->fx_wexp, h->fx_wsum, h->fx_nw,
+                 forced ? h->fx_gf * dt * dt : 0.0, h->fx_max, h->fx_forcing, h->fx_scale, h->fx_state, st);
+  h->total_launches += 3;
+  const bool timed = h->ev_used + 2 <= (int)h->ev.size();
+  if (timed) CK(cudaEventRecord(h->ev[h->ev_used], st));
+  FxHost a;
+  a.cx = h->fx_cx;
+  a.cy = h->fx_cy;
+  for (int first = 0; first < 2; ++first) {
+    const double kappa = first ? 0.5 * dt * dt : dt * dt, a_cur = first ? 1.0 : 2.0;
+    layer_coef(h, P.c2_lo, a_cur, kappa, &a.lay[first][0]);
+    layer_coef(h, P.c2_hi, a_cur, kappa, &a.lay[first][1]);
+  }
+  a.iso = a.lay[0][0].Ax == a.lay[0][0].Ay && a.lay[0][1].Ax == a.lay[0][1].Ay;
+  a.gw = h->fx_gw;
+  a.gd = h->fx_gd;
+  a.f = h->f;
+  a.force = h->fx_force;
+  a.wq_host = P.w.data();
+  a.wint = h->fx_wint.data();
+  a.wexp = h->fx_wexp;
+  a.wsum = h->fx_wsum;
+  a.warps = h->fx_nw;
+  a.cos_host = P.cosf.data();
+  a.dt2 = dt * dt;
+  a.forced = forced;
+  a.add = add;
+  a.binv = h->sh.binv;
+  a.emat = h->sh.emat;
+  a.has_e = h->sh.has_e;
+  a.vprev = vin;
+  a.scale = h->fx_scale;
+  a.state = h->fx_state;
+  int launches = 0;
+  for (int n0 = 0; n0 < n_run; ++launches) {
+    a.n0 = n0;
+    a.steps = std::min(8, n_run - n0);
+    n0 += a.steps;
+    a.last = n0 == n_t;
+    launch_fx2d(nf, h->geom, lev[launches & 1], lev[1 - (launches & 1)], q, vout, vsub, a, st);
+  }
+  h->step_launches += launches;
+  h->total_launches += forced ? 2 * launches : launches;
+  if (timed) {
+    CK(cudaEventRecord(h->ev[h->ev_used + 1], st));
+    h->ev_used += 2;
+  }
+  CK(cudaGetLastError());
+  return MFWH_OK;
+}
+
 // One wave solve: replayed from a captured graph in graph mode, launched directly otherwise.
 mfwh_status apply_pi(mfwh_handle_t h, const double* vin, double* vout, int forced,
                      const double* vsub) {
@@ -616,12 +796,39 @@ mfwh_status residual_dev(mfwh_handle_t h, const double* v_dev, double* r_out) {
   return MFWH_OK;
 }
 
+// Leaves fixed point for the FP64 kernels, which need less memory.
+void fx_drop(mfwh_handle_t h) {
+  cudaStreamSynchronize(h->stream);
+  if (h->gstream) cudaStreamSynchronize(h->gstream);
+  for (auto& x : h->gexec) {   // captured with the old buffers
+    if (x) cudaGraphExecDestroy(x);
+    x = nullptr;
+  }
+  if (h->fx_force) cudaFree(h->fx_force);
+  h->fx_force = nullptr;
+  h->plan.fixed = false;
+  if (h->plan.precision == MFWH_PREC_FP64) {
+    h->plan.time_block = h->depth64 = h->fx_else[0];
+    h->plan.tile_shape = h->shape64 = h->fx_else[1];
+  }
+}
+
+// Workspace of n values; where memory ends, a handle in fixed point gives up its own for it.
+template <typename T>
+cudaError_t alloc_workspace(mfwh_handle_t h, T** p, int64_t n) {
+  cudaError_t e = cudaMalloc(p, sizeof(T) * n);
+  if (e != cudaErrorMemoryAllocation || !h->fx_force) return e;
+  (void)cudaGetLastError();
+  fx_drop(h);
+  return cudaMalloc(p, sizeof(T) * n);
+}
+
 mfwh_status ensure_basis(mfwh_handle_t h, int vectors) {
   if (h->basis_vectors >= vectors) return MFWH_OK;
   if (h->basis) cudaFree(h->basis);
   h->basis = nullptr;
   h->basis_vectors = 0;
-  CK(cudaMalloc(&h->basis, sizeof(double) * h->N * vectors));
+  CK(alloc_workspace(h, &h->basis, h->N * vectors));
   h->basis_vectors = vectors;
   return MFWH_OK;
 }
@@ -904,8 +1111,8 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
   g.layer_axis = P.layer_axis;
   g.layer_split = P.layer_split;
   g.order = P.order;
-  // FP32 wave levels and forcing: rows padded to 32 floats (16-byte aligned)
-  const bool pad_w = P.precision != MFWH_PREC_FP64;
+  // wave levels in FP32 (and its forcing) and in fixed point: rows padded to 32 points
+  const bool pad_w = P.precision != MFWH_PREC_FP64 || P.fixed;
   g.syw = pad_w ? (g.nx + 1 + 31) / 32 * 32 : g.sy;
   g.szw = pad_w ? g.syw * (g.ny + 1) : g.sz;
   h->PW = pad_w ? g.szw * (g.dim == 3 ? g.nz + 1 : 1) : h->P;
@@ -917,18 +1124,25 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
   };
   cudaError_t e = cudaGetDevice(&h->device);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaGetDevice"));
+  if (P.fixed) {
+    int sms = 0;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+    if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaDeviceGetAttribute"));
+    h->fx_nw = fx_warps(g.nx, g.ny, sms);
+  }
   const int64_t tables = (int64_t)(P.s.n_t + 1) * h->nf;
   struct {
     double** p;
     int64_t n;
   } bufs[] = {{&h->f, h->N},
-              {&h->Wa, h->P},
-              {&h->Wb, h->P},
-              {&h->Wc2, h->P},
-              {&h->Wp2, h->P},
+              {&h->Wa, h->PW},     // PW >= P
+              {&h->Wb, h->PW},
+              {&h->Wc2, h->PW},
+              {&h->Wp2, h->PW},
               {&h->d_wq, tables},
               {&h->d_cos, tables},
-              {&h->q, h->N},
+              {&h->q, P.fixed ? std::max(h->N, fx_tiles(g.nx, g.ny, h->fx_nw) * kFxTile * h->nf)
+                              : h->N},
               {&h->res_partial, residual_partial_size(MFWH_MAX_NF)},
               {&h->res_out, 2 * MFWH_MAX_NF},
               {&h->dot_partial, dot_partial_size()},
@@ -938,6 +1152,36 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
   for (auto& b : bufs) {
     e = cudaMalloc(b.p, sizeof(double) * b.n);
     if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaMalloc (workspace)"));
+  }
+  if (P.fixed) {
+    const bool blocked = prob->time_block == 0 && h->nf <= 8;
+    h->fx_else[0] = prob->time_block != 0 ? prob->time_block : (blocked ? 3 : 1);
+    h->fx_else[1] = blocked && prob->tile_shape == 0 ? 5 : prob->tile_shape;
+    e = cudaMalloc(&h->fx_force, sizeof(int64_t) * h->PW * 8);
+    if (e == cudaErrorMemoryAllocation) {
+      (void)cudaGetLastError();
+      e = cudaSuccess;
+      fx_drop(h);
+    }
+  }
+  if (P.fixed) {
+    if (e == cudaSuccess)
+      e = cudaMalloc(&h->fx_max, sizeof(unsigned long long) * (1 + MFWH_MAX_NF));
+    if (e == cudaSuccess)
+      e = cudaMemsetAsync(h->fx_max, 0, sizeof(unsigned long long) * (1 + MFWH_MAX_NF), h->stream);
+    if (e == cudaSuccess) e = cudaMalloc(&h->fx_forcing, sizeof(FxForcing));
+    if (e == cudaSuccess) e = cudaMalloc(&h->fx_scale, sizeof(FxScale));
+    if (e == cudaSuccess) e = cudaMalloc(&h->fx_state, 3 * sizeof(FxState));
+    if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaMalloc (fixed-point workspace)"));
+    for (int first = 0; first < 2; ++first)
+      for (int up = 0; up < 2; ++up) {
+        LayerCoef L;
+        layer_coef(h, up ? P.c2_hi : P.c2_lo, 2.0, (first ? 0.5 : 1.0) * P.s.dt * P.s.dt, &L);
+        h->fx_cx[first][up] = fx_coef(L.Ax);
+        h->fx_cy[first][up] = fx_coef(L.Ay);
+      }
+    fx_growth(h, &h->fx_gw, &h->fx_gd, &h->fx_gf);
+    fx_weights(h);
   }
   if (P.precision != MFWH_PREC_FP64) {
     const int nf = h->nf;
@@ -957,7 +1201,7 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
     } fb[] = {{&h->f32, h->PW * h->nf}, {&h->W32[0], h->PW}, {&h->W32[1], h->PW}, {&h->W32[2], h->PW},
               {&h->W32[3], h->PW}, {&h->qs, h->N}, {&h->qc, h->N}};
     for (auto& b : fb) {
-      e = cudaMalloc(b.p, sizeof(float) * std::max<int64_t>(b.n, 1));
+      e = alloc_workspace(h, b.p, std::max<int64_t>(b.n, 1));
       if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaMalloc (FP32 workspace)"));
     }
     for (int i = 0; i < 4 && e == cudaSuccess; ++i)
@@ -1097,13 +1341,14 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
     launch_forcing32(h->nf, h->geom, h->f, h->f32, h->stream);
     e = cudaGetLastError();
   }
+  if (e == cudaSuccess) e = fx_set_forcing(h);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "initialising workspace"));
   h->use32 = P.precision != MFWH_PREC_FP64;
   if (P.precision == MFWH_PREC_FP64) {
     h->depth64 = P.time_block;
     h->shape64 = P.tile_shape;
-  } else if (P.dim == 2 && P.order == 2 && !P.c2_field && h->nf <= 8) {
+  } else if (P.dim == 2 && P.order == 2 && !P.c2_field && h->nf <= 8) {   // (unless fixed)
     // the FP64 wave solves of an FP32 handle take the FP64 default: 3 steps per pass on the
     // persistent pipelined kernel (bit-identical to one step per launch)
     h->depth64 = 3;
@@ -1133,6 +1378,7 @@ mfwh_status mfwh_set_forcing(mfwh_handle_t h, const double* forcing) {
     h->total_launches++;
     CK(cudaGetLastError());
   }
+  CK(fx_set_forcing(h));
   return MFWH_OK;
 }
 
@@ -1151,8 +1397,16 @@ mfwh_status mfwh_solve_fpi(mfwh_handle_t h, int iters, double* v) {
   bool on_dev = false;
   mfwh_status st = stage_in(h, v, &x, &on_dev);
   if (st != MFWH_OK) return st;
+  // The map is affine: Pi(x) = S x + b with b = Pi(0), and a homogeneous wave solve costs a
+  // fraction of a forced one (no forcing grids to read and sum at every step), so from three
+  // iterations on b is formed once.
+  const bool affine = h->plan.fixed && !h->use32 && iters >= 3;
+  if (affine) {
+    st = apply_pi(h, nullptr, h->vec_b, 1, nullptr);
+    if (st != MFWH_OK) return st;
+  }
   for (int k = 0; k < iters; ++k) {
-    st = apply_pi(h, x, x, 1, nullptr);
+    st = affine ? apply_pi_fx(h, x, x, 0, h->vec_b, true) : apply_pi(h, x, x, 1, nullptr);
     if (st != MFWH_OK) return st;
   }
   if (!on_dev) CK(cudaMemcpyAsync(v, x, sizeof(double) * h->N, cudaMemcpyDeviceToHost, h->stream));
@@ -1231,8 +1485,8 @@ mfwh_status refine_core(mfwh_handle_t h, int restart, double inner_tol, int max_
   reset_timing(h);
   mfwh_status st = ensure_basis(h, restart + 1);
   if (st != MFWH_OK) return st;
-  if (!h->vec_r) CK(cudaMalloc(&h->vec_r, sizeof(double) * h->N));
-  if (!h->vec_e) CK(cudaMalloc(&h->vec_e, sizeof(double) * h->N));
+  if (!h->vec_r) CK(alloc_workspace(h, &h->vec_r, h->N));
+  if (!h->vec_e) CK(alloc_workspace(h, &h->vec_e, h->N));
   mfwh_solve_info local{};
   mfwh_solve_info& I = info ? *info : local;
   I.iterations = I.pi_applications = I.restarts = I.refinements = 0;
@@ -1403,6 +1657,11 @@ void mfwh_destroy(mfwh_handle_t h) {
                     h->dot_partial, h->dot_out, h->vec_b,     h->vec_x,   h->basis};
   for (double* b : bufs)
     if (b) cudaFree(b);
+  if (h->fx_force) cudaFree(h->fx_force);
+  if (h->fx_max) cudaFree(h->fx_max);
+  if (h->fx_forcing) cudaFree(h->fx_forcing);
+  if (h->fx_state) cudaFree(h->fx_state);
+  if (h->fx_scale) cudaFree(h->fx_scale);
   if (h->d_err) cudaFree(h->d_err);
   if (h->c2f) cudaFree(h->c2f);
   if (h->fault) cudaFree(h->fault);
@@ -1453,8 +1712,8 @@ mfwh_status mfwh_set_graphs(mfwh_handle_t h, int enable) {
   if (h->gstream) CK(cudaStreamSynchronize(h->gstream));
   drop_graphs(h);
   if (enable && !h->g_in) {
-    CK(cudaMalloc(&h->g_in, sizeof(double) * h->N));
-    CK(cudaMalloc(&h->g_out, sizeof(double) * h->N));
+    CK(alloc_workspace(h, &h->g_in, h->N));
+    CK(alloc_workspace(h, &h->g_out, h->N));
     CK(cudaMemsetAsync(h->g_in, 0, sizeof(double) * h->N, h->stream));
     CK(cudaStreamCreateWithFlags(&h->gstream, cudaStreamNonBlocking));
     for (auto& e : h->gev) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -2019,7 +2278,9 @@ mfwh_status mfwh_autotune(const mfwh_problem* prob, void* stream, int* time_bloc
     else
       cand = {{1, 0}, {2, 0}, {4, 0}};
   } else if (P.precision == MFWH_PREC_FP64) {
-    cand = {{1, 0}, {2, 5}, {3, 5}, {4, 5}, {4, 4}, {4, 3}, {8, 3}};
+    cand = P.fixed ? std::vector<std::pair<int, int>>{{8, 3}}   // (no effect)
+                   : std::vector<std::pair<int, int>>{{1, 0}, {2, 5}, {3, 5}, {4, 5}, {4, 4}, {4, 3},
+                                                      {8, 3}};
   } else {
     cand = {{4, 0}, {8, 0}, {16, 0}};
   }
@@ -2094,8 +2355,8 @@ mfwh_status mfwh_warm_start(mfwh_handle_t h, mfwh_cnn_t net, double omega_scale,
   if (st != MFWH_OK) return st;
   // Amplitude of each predicted shape phi_m: alpha_m = <A phi_m, f_m> / <A phi_m, A phi_m>
   // with A = L_h + omega_m^2 minimises the L2 Helmholtz residual ||f_m - alpha A phi_m||.
-  if (!h->vec_r) CK(cudaMalloc(&h->vec_r, sizeof(double) * h->N));
-  if (!h->vec_e) CK(cudaMalloc(&h->vec_e, sizeof(double) * h->N));
+  if (!h->vec_r) CK(alloc_workspace(h, &h->vec_r, h->N));
+  if (!h->vec_e) CK(alloc_workspace(h, &h->vec_e, h->N));
   CK(cudaMemsetAsync(h->vec_e, 0, sizeof(double) * h->N, h->stream));
   // defect of phi against a zero forcing is -A phi at interior points, 0 on the boundary
   launch_residual_field(h->nf, h->geom, x, h->vec_e, h->omega2, h->plan.c2_lo, h->plan.c2_hi,

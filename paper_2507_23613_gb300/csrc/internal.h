@@ -22,8 +22,9 @@ struct Plan {
   bool c2_field = false;             // MFWH_C_FIELD: c^2 per point (c2_lo = c2_hi = 1 then)
   int layer_axis = 0;
   int dim = 2;
-  int time_block = 1;          // steps per wave-kernel launch (1, 4, 8 or 16)
+  int time_block = 1;          // steps per wave-kernel launch at most
   int tile_shape = 0;          // tile of the FP64 blocked kernels (wave_tb.cu)
+  bool fixed = false;          // FP64 wave solves in 64-bit fixed point (wave_fx.cu)
   int precision = MFWH_PREC_FP64;
   int order = 2;               // order of L_{ph}: 2 or 4
   int filter_update = MFWH_UPDATE_IMPLICIT;

@@ -21,7 +21,8 @@ struct Geom {
   int64_t layer_split;       // indices >= layer_split use the upper-layer coefficients
   int order;                 // order of L_{ph}: 2 or 4 (0 reads as 2)
   int64_t syw, szw;          // strides of j and k in the FP32 arrays W, D and f (FP32 handles pad
-                             // rows to 32 floats for 16-byte accesses; else sy, sz)
+                             // rows to 32 floats for 16-byte accesses) and in the fixed-point
+                             // levels (rows of 32 points); else sy, sz
   int64_t wpoints;           // entries of one of them (stride between the frequencies of f)
   const double* c2f;         // c^2 per point [points] (MFWH_C_FIELD), else null; with a field
                              // the layer coefficients are those of c = 1 (lower layer only)
@@ -85,6 +86,80 @@ struct TBHost {
 void launch_tb2d(int nf, const Geom& g, const double* Wc_in, const double* Wp_in, double* Wc_out,
                  double* Wp_out, const double* f, double* q, double* vout, const double* vsub,
                  const TBHost& h, cudaStream_t st);
+
+// ---- FP64 wave solve of 2D grids in 64-bit fixed point (wave_fx.cu) -----------------
+// W and D = W^n - W^{n-1} in units of the quantum, rows padded as syw, wpoints entries each.
+struct FxArrays {
+  int64_t* W;
+  int64_t* D;
+};
+// Device state of one wave solve.  mode 1: FP64 steps (the arrays then hold W^n and W^{n-1} as
+// doubles); fe: the unit 2^fe of the forcing's integers; fm 2^fx: bound of the forcing's part of a
+// launch's levels, gf dt^2 sum_m max |f_m| (fm 0 if unforced).
+struct FxScale {
+  float fm;
+  int fx, fe, mode;
+};
+struct FxForcing {
+  double fsum;
+  int fe;
+};
+// Quantum 2^e of a launch's input and its largest |W| and |D| in quanta (or bounds of them); the unit
+// 2^(eq - wexp[m]) of the sums.  Three states rotate: a launch reads one, writes the next and
+// resets the third's maxima.
+struct FxState {
+  unsigned long long wmax, dmax;
+  int e, eq;
+};
+constexpr int kFxWSumMin = 67, kFxWSumMax = 72;   // log2 of the bound of sum_n |w_{n,m}|, weight units
+constexpr int kFxTileX = 48, kFxTileY = 32;   // points that a tile owns at most (4 warps - 16 rows)
+constexpr int kFxTile = kFxTileX * kFxTileY;
+// Tiles of a grid with a number of step warps; the sums take fx_tiles * kFxTile entries per
+// frequency.
+inline int64_t fx_tiles(int64_t nx, int64_t ny, int warps) {
+  const int vy = 4 * warps - 16;
+  return ((nx + kFxTileX) / kFxTileX) * ((ny + vy) / vy);
+}
+int fx_warps(int64_t nx, int64_t ny, int sms);   // the number of step warps for a grid
+struct FxCoef;
+struct FxHost {
+  const FxCoef (*cx)[2];     // [first step][upper layer]: kappa c^2 / h_x^2
+  const FxCoef (*cy)[2];     //                            kappa c^2 / h_y^2
+  LayerCoef lay[2][2];       // the same steps in FP64
+  double gw, gd;             // |W^{n+k}| <= gw max |W^n| + gd max |D^n| (+ the forcing's part), k <= 8
+  const double* f;           // device forcing [nf][points]
+  int64_t* force;            // device [8][wpoints]: its sum at the launch's steps (rows as the levels')
+  const double* wq_host;     // [(N_t + 1) * nf] w_{n,m}
+  const int64_t* wint;       // the same times 2^wexp[m], rounded, below 2^60
+  const int* wexp;
+  int wsum;                  // sum_n |wint| < 2^wsum
+  int warps;                 // step warps of a CTA (fx_warps)
+  const double* cos_host;    // [(N_t + 1) * nf] cos(omega~_m t^n)
+  double dt2;
+  int n0, steps;             // first level (a multiple of 8), steps of this launch (at most 8)
+  int iso;                   // equal spacings: cx = cy
+  int forced, last;
+  int add;                   // v_out = v_sub + V instead of v_sub - V
+  const double* binv;        // epilogue as in StepHost
+  const double* emat;
+  int has_e;
+  const double* vprev;
+  const FxScale* scale;      // device
+  FxState* state;            // device [3]
+};
+// The unit of the forcing's integers and sum_m max |f_m|.  fmax: device scratch [nf].
+void launch_fx_forcing(int nf, const Geom& g, const double* f, unsigned long long* fmax,
+                       FxForcing* unit, cudaStream_t st);
+// The first quantum, W^0 = sum_m v_m (v == nullptr: 0) and q_m = w0_m W^0: three launches.  gf_dt2: 0 if
+// unforced.  wmax: device scratch, 0 on entry and on return.
+void launch_fx_init(int nf, const Geom& g, const double* v, int64_t* W, int64_t* q,
+                    const double* w0, const int* wexp, int wsum, int warps,
+                    double gf_dt2, unsigned long long* wmax, const FxForcing* forcing, FxScale* scale,
+                    FxState* state, cudaStream_t st);
+// Up to 8 steps (always 8 but for the last launch); the last one writes v_out.  q: sums
+// [tile][nf][owned point] in units of 2^(eq - wexp[m]).  Two launches when forced.
+void launch_fx2d(int nf, const Geom& g, const FxArrays& in, const FxArrays& out, int64_t* q,
+                 double* vout, const double* vsub, const FxHost& h, cudaStream_t st);
 
 // ---- FP32 path with compensated filter sums (wave32.cu) ----------------------------
 // Increment form: D' = D + kappa c^2 Delta_h W - sum_m fc_m f_m, W' = W + D', with
