@@ -542,16 +542,21 @@ FxCoef fx_coef(double a) {
   return FxCoef{(uint32_t)v, (uint32_t)(v >> 32), v >> 1};
 }
 
-// Growth of the levels over at most 8 leapfrog steps in the maximum norm: |W^{n+k}| <= gw max |W^n|
+// Growth of the levels over a launch's leapfrog steps (8, fourth order 4) in the maximum norm: |W^{n+k}| <= gw max |W^n|
 // + gd max |D^n| + gf dt^2 sum_m max |f_m|.  W^{n+k} = P_k W^n + Q_k D^n with the steps D' = D + L W,
 // W' = W + D' (L = dt^2 c^2 Delta_h; the first step of a wave solve has L / 2 and D = 0), and the
 // bounds are the largest absolute row sums of P_k and Q_k; a step's forcing acts like D of that
 // step, so gf is the sum over k of those of Q_k.  A row of P_k and Q_k is found by applying the
-// steps' transpose to a unit vector on a 19 x 19 patch, for every position of the layer
-// interface within reach.  The Dirichlet boundary (an odd reflection) only shortens rows.
+// steps' transpose to a unit vector on a patch of the 8 points reached each way and a margin, for
+// every position of the layer interface within reach.  The Dirichlet boundary (an odd reflection)
+// only shortens rows.
 void fx_growth(const mfwh_handle_t h, double* gw, double* gd, double* gf) {
-  constexpr int R = 8, C = R + 1, E = 2 * C + 1;   // steps, centre and edge of the patch
+  constexpr int R = 8, C = R + 2, E = 2 * C + 1;   // reach, centre and edge of the patch
   const Plan& P = h->plan;
+  const int steps = fx_launch_steps(P.order), reach = P.order / 2;
+  // weights of the centre, the first and the second neighbours along an axis
+  const double w0 = P.order == 4 ? -30.0 / 12.0 : -2.0, w1 = P.order == 4 ? 16.0 / 12.0 : 1.0,
+               w2 = P.order == 4 ? -1.0 / 12.0 : 0.0;
   const double k = P.s.dt * P.s.dt;
   const bool layers = P.c2_lo != P.c2_hi && P.layer_split > 0 && P.layer_split <= P.n[P.layer_axis];
   *gw = 1.0;
@@ -565,19 +570,21 @@ void fx_growth(const mfwh_handle_t h, double* gw, double* gd, double* gf) {
       for (int i = 0; i < E; ++i) u[j][i] = v[j][i] = t[j][i] = 0.0;
     u[C][C] = 1.0;
     const double kx = k * h->inv_h2[0], ky = k * h->inv_h2[1];
-    for (int s = 1; s <= R; ++s) {
+    for (int s = 1; s <= steps; ++s) {
       // t = L^T (u + v), on the points reached
-      for (int j = C - s; j <= C + s; ++j)
-        for (int i = C - s; i <= C + s; ++i) {
+      const int lo = C - s * reach, hi = C + s * reach;
+      for (int j = lo; j <= hi; ++j)
+        for (int i = lo; i <= hi; ++i) {
           auto at = [&](int ii, int jj) {
             return c2[P.layer_axis == 0 ? ii : jj] * (u[jj][ii] + v[jj][ii]);
           };
-          t[j][i] = kx * (at(i - 1, j) + at(i + 1, j)) + ky * (at(i, j - 1) + at(i, j + 1)) -
-                    2.0 * (kx + ky) * at(i, j);
+          t[j][i] = w1 * (kx * (at(i - 1, j) + at(i + 1, j)) + ky * (at(i, j - 1) + at(i, j + 1))) +
+                    w2 * (kx * (at(i - 2, j) + at(i + 2, j)) + ky * (at(i, j - 2) + at(i, j + 2))) +
+                    w0 * (kx + ky) * at(i, j);
         }
       double pu = 0.0, pf = 0.0, pv = 0.0;
-      for (int j = C - s; j <= C + s; ++j)
-        for (int i = C - s; i <= C + s; ++i) {
+      for (int j = lo; j <= hi; ++j)
+        for (int i = lo; i <= hi; ++i) {
           pf += std::fabs(u[j][i] + 0.5 * t[j][i]);
           v[j][i] += u[j][i];
           u[j][i] += t[j][i];
@@ -588,7 +595,7 @@ void fx_growth(const mfwh_handle_t h, double* gw, double* gd, double* gf) {
       qmax[s] = std::max(qmax[s], pv);
     }
   }
-  for (int s = 1; s <= R; ++s) {
+  for (int s = 1; s <= steps; ++s) {
     *gd = std::max(*gd, qmax[s]);
     *gf += qmax[s];
   }
@@ -603,7 +610,7 @@ void fx_weights(mfwh_handle_t h) {
   const Plan& P = h->plan;
   const int nf = h->nf;
   h->fx_wint.resize(P.w.size());
-  h->fx_wsum = kFxWSumMin;
+  h->fx_wsum = fx_wsum_min(P.order);
   for (int m = 0; m < nf; ++m) {
     double mx = 0.0, sum = 0.0;
     for (int n = 0; n <= P.s.n_t; ++n) {
@@ -633,7 +640,7 @@ cudaError_t fx_set_forcing(mfwh_handle_t h) {
 }
 
 // Fixed-point wave solve (2D): three launches for the quantum, W^0 and the first filter terms, then
-// ceil(N_t / 8) launches alternating between the two pairs of level arrays; the last one writes
+// ceil(N_t / 8 or 4) launches alternating between the two pairs of level arrays; the last one writes
 // v_out (add: v_sub + V instead of v_sub - V).
 mfwh_status apply_pi_fx(mfwh_handle_t h, const double* vin, double* vout, int forced,
                         const double* vsub, bool add) {
@@ -683,7 +690,7 @@ mfwh_status apply_pi_fx(mfwh_handle_t h, const double* vin, double* vout, int fo
   int launches = 0;
   for (int n0 = 0; n0 < n_run; ++launches) {
     a.n0 = n0;
-    a.steps = std::min(8, n_run - n0);
+    a.steps = std::min(fx_launch_steps(P.order), n_run - n0);
     n0 += a.steps;
     a.last = n0 == n_t;
     launch_fx2d(nf, h->geom, lev[launches & 1], lev[1 - (launches & 1)], q, vout, vsub, a, st);
@@ -1154,7 +1161,7 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
     if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaMalloc (workspace)"));
   }
   if (P.fixed) {
-    const bool blocked = prob->time_block == 0 && h->nf <= 8;
+    const bool blocked = prob->time_block == 0 && h->nf <= 8 && P.order == 2;
     h->fx_else[0] = prob->time_block != 0 ? prob->time_block : (blocked ? 3 : 1);
     h->fx_else[1] = blocked && prob->tile_shape == 0 ? 5 : prob->tile_shape;
     e = cudaMalloc(&h->fx_force, sizeof(int64_t) * h->PW * 8);
@@ -1177,8 +1184,8 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
       for (int up = 0; up < 2; ++up) {
         LayerCoef L;
         layer_coef(h, up ? P.c2_hi : P.c2_lo, 2.0, (first ? 0.5 : 1.0) * P.s.dt * P.s.dt, &L);
-        h->fx_cx[first][up] = fx_coef(L.Ax);
-        h->fx_cy[first][up] = fx_coef(L.Ay);
+        h->fx_cx[first][up] = fx_coef(P.order == 4 ? -L.Bx : L.Ax);
+        h->fx_cy[first][up] = fx_coef(P.order == 4 ? -L.By : L.Ay);
       }
     fx_growth(h, &h->fx_gw, &h->fx_gd, &h->fx_gf);
     fx_weights(h);

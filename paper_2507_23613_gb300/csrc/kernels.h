@@ -111,7 +111,12 @@ struct FxState {
   unsigned long long wmax, dmax;
   int e, eq;
 };
-constexpr int kFxWSumMin = 67, kFxWSumMax = 72;   // log2 of the bound of sum_n |w_{n,m}|, weight units
+// Steps of a launch (all but the last): 8 of the second-order operator, 4 of the fourth-order one;
+// bits of a level's bound; log2 of the bound of sum_n |w_{n,m}| in weight units.
+constexpr int fx_launch_steps(int order) { return order == 4 ? 4 : 8; }
+constexpr int fx_bits(int order) { return order == 4 ? 56 : 59; }
+constexpr int fx_wsum_min(int order) { return 126 - fx_bits(order); }
+constexpr int kFxWSumMax = 72;
 constexpr int kFxTileX = 48, kFxTileY = 32;   // points that a tile owns at most (4 warps - 16 rows)
 constexpr int kFxTile = kFxTileX * kFxTileY;
 // Tiles of a grid with a number of step warps; the sums take fx_tiles * kFxTile entries per
@@ -123,10 +128,11 @@ inline int64_t fx_tiles(int64_t nx, int64_t ny, int warps) {
 int fx_warps(int64_t nx, int64_t ny, int sms);   // the number of step warps for a grid
 struct FxCoef;
 struct FxHost {
-  const FxCoef (*cx)[2];     // [first step][upper layer]: kappa c^2 / h_x^2
+  const FxCoef (*cx)[2];     // [first step][upper layer]: kappa c^2 / h_x^2 (fourth order: / 12)
   const FxCoef (*cy)[2];     //                            kappa c^2 / h_y^2
   LayerCoef lay[2][2];       // the same steps in FP64
-  double gw, gd;             // |W^{n+k}| <= gw max |W^n| + gd max |D^n| (+ the forcing's part), k <= 8
+  double gw, gd;             // |W^{n+k}| <= gw max |W^n| + gd max |D^n| (+ the forcing's part)
+                             // over a launch's steps
   const double* f;           // device forcing [nf][points]
   int64_t* force;            // device [8][wpoints]: its sum at the launch's steps (rows as the levels')
   const double* wq_host;     // [(N_t + 1) * nf] w_{n,m}
@@ -136,7 +142,7 @@ struct FxHost {
   int warps;                 // step warps of a CTA (fx_warps)
   const double* cos_host;    // [(N_t + 1) * nf] cos(omega~_m t^n)
   double dt2;
-  int n0, steps;             // first level (a multiple of 8), steps of this launch (at most 8)
+  int n0, steps;             // first level, steps of this launch
   int iso;                   // equal spacings: cx = cy
   int forced, last;
   int add;                   // v_out = v_sub + V instead of v_sub - V
@@ -156,10 +162,36 @@ void launch_fx_init(int nf, const Geom& g, const double* v, int64_t* W, int64_t*
                     const double* w0, const int* wexp, int wsum, int warps,
                     double gf_dt2, unsigned long long* wmax, const FxForcing* forcing, FxScale* scale,
                     FxState* state, cudaStream_t st);
-// Up to 8 steps (always 8 but for the last launch); the last one writes v_out.  q: sums
+// One launch; the last one writes v_out.  q: sums
 // [tile][nf][owned point] in units of 2^(eq - wexp[m]).  Two launches when forced.
 void launch_fx2d(int nf, const Geom& g, const FxArrays& in, const FxArrays& out, int64_t* q,
                  double* vout, const double* vsub, const FxHost& h, cudaStream_t st);
+
+// ---- Programmatic dependent launch ---------------------------------------------------
+#ifdef __CUDACC__
+// A step kernel launched by launch_dependent starts where and when the launch before it leaves an
+// SM free; pdl_begin, before the first access to memory, waits for the end of that launch.  (The
+// arrays that the launch before writes must not be const __restrict__: such reads may move up.)
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... P, typename... A>
+inline void launch_dependent(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                             A&&... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
+}
+#endif
 
 // ---- FP32 path with compensated filter sums (wave32.cu) ----------------------------
 // Increment form: D' = D + kappa c^2 Delta_h W - sum_m fc_m f_m, W' = W + D', with

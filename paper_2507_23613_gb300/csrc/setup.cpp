@@ -447,18 +447,18 @@ mfwh_status plan_problem(const mfwh_problem* p, Plan* out, double c2_field_max) 
   }
   const double dt = s.dt;
 
-  // FP64 wave solves in 64-bit fixed point (wave_fx.cu): 2D, second order, constant or two-layer
-  // c, explicit steps, coefficients kappa c^2 / h^2 that a 64-bit fraction holds exactly (a double
+  // FP64 wave solves in 64-bit fixed point (wave_fx.cu): 2D, constant or two-layer c,
+  // explicit steps, coefficients kappa c^2 / h^2 (fourth order: / 12) that a 64-bit fraction holds exactly (a double
   // of at least 2^-10 has no bit below 2^-62, half of it none below 2^-63) and whose products do not
   // end in exact halves often (not a multiple of 2^-24: these round up, and a bias of the
   // increments grows with the square of the steps), and a grid that tiles of 48 x 32 points do not
   // pad to more than twice its size and a few tiles.
-  if (!implicit && !field && P.dim == 2 && P.order == 2) {
+  if (!implicit && !field && P.dim == 2) {
     const int64_t padded = ((P.n[0] + 48) / 48 * 48) * ((P.n[1] + 32) / 32 * 32);
     P.fixed = padded <= 2 * s.points + 65536;
     for (int a = 0; a < 2; ++a)
       for (double c2 : {P.c2_lo, P.c2_hi}) {
-        const double k = dt * dt * c2 / (s.h[a] * s.h[a]);
+        const double k = dt * dt * c2 / (s.h[a] * s.h[a]) / (P.order == 4 ? 12.0 : 1.0);
         const double k24 = std::ldexp(k, 24);
         P.fixed = P.fixed && k >= 0x1p-10 && k < 1.0 && k24 != std::floor(k24);
       }
@@ -472,7 +472,7 @@ mfwh_status plan_problem(const mfwh_problem* p, Plan* out, double c2_field_max) 
   P.time_block = p->time_block;
   if (p->time_block == 0)
     P.time_block = fp32 && p->dim == 2 && P.order != 4 ? 16
-                   : (!fp32 && P.fixed)                ? 8
+                   : (!fp32 && P.fixed)                ? (P.order == 4 ? 4 : 8)
                                                        : (fp64_blocked ? 3 : 1);
   P.tile_shape = (p->time_block == 0 && fp64_blocked && p->tile_shape == 0) ? 5 : p->tile_shape;
 

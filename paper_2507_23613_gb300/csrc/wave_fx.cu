@@ -84,6 +84,8 @@ struct FxForceArgs {
   int gh[8 * MFWH_MAX_NF];                              // high digits, [m * 8 + s]
   float ghf[8 * MFWH_MAX_NF], glf[8 * MFWH_MAX_NF];     // the digits / 2^32 in FP32
 };
+// STEPS: of a launch.
+template <int STEPS>
 __global__ void __launch_bounds__(128, 4)
 k_fx_force(const double* __restrict__ f, int64_t* __restrict__ force,
            const __grid_constant__ FxForceArgs a, const FxScale* __restrict__ scale,
@@ -91,7 +93,7 @@ k_fx_force(const double* __restrict__ f, int64_t* __restrict__ force,
   const FxScale sc = *scale;
   if (sc.mode) return;
   // the sum of high products is in units of 2^(fe + ce + 64)
-  const int sh = sc.fe + a.ce + 64 - fx_quantum(*state, sc, a.gw, a.gd, a.wsum).e;
+  const int sh = sc.fe + a.ce + 64 - fx_quantum(*state, sc, a.gw, a.gd, a.wsum, STEPS == 4 ? 4 : 2).e;
   const int64_t x = 1 + (int64_t)blockIdx.x * 32 + threadIdx.x;
   if (x >= g.nx) return;
   // two rows per thread
@@ -101,10 +103,10 @@ k_fx_force(const double* __restrict__ f, int64_t* __restrict__ force,
     const bool two = y + 4 < g.ny && MFWH_IDX(g.fault, p + 4 * g.sy, g.points) &&
                      MFWH_IDX(g.fault, o + 4 * g.syw, g.wpoints);
     const int64_t p2 = two ? p + 4 * g.sy : p;
-    int64_t S[2][8];
-    float r[2][8];
+    int64_t S[2][STEPS];
+    float r[2][STEPS];
 #pragma unroll
-    for (int s = 0; s < 8; ++s) {
+    for (int s = 0; s < STEPS; ++s) {
       S[0][s] = S[1][s] = 0;
       r[0][s] = r[1][s] = 0.0f;
     }
@@ -130,7 +132,7 @@ k_fx_force(const double* __restrict__ f, int64_t* __restrict__ force,
           lf[k] = (float)lo;
         }
 #pragma unroll
-        for (int s = 0; s < 8; ++s) {
+        for (int s = 0; s < STEPS; ++s) {
           const int i = (m0 + j) * 8 + s;
 #pragma unroll
           for (int k = 0; k < 2; ++k) {
@@ -144,7 +146,7 @@ k_fx_force(const double* __restrict__ f, int64_t* __restrict__ force,
 #pragma unroll
     for (int k = 0; k < 2; ++k)
 #pragma unroll
-      for (int s = 0; s < 8; ++s)
+      for (int s = 0; s < STEPS; ++s)
         if (s < a.steps && (k == 0 || two))
           force[s * g.wpoints + o + k * 4 * g.syw] =
               fx_rescale(S[k][s] + __float2int_rn(r[k][s]), sh);
@@ -287,8 +289,9 @@ void launch_fx2d(int nf, const Geom& g, const FxArrays& in, const FxArrays& out,
       }
     const unsigned bx = (unsigned)((g.nx + 30) / 32), by = (unsigned)((g.ny + 6) / 8);
     const unsigned cap = bx < 608 ? 608 / bx : 1;   // blocks: what 152 SMs hold
-    k_fx_force<<<dim3(bx, by < cap ? by : cap), dim3(32, 4), 0, st>>>(
-        h.f, h.force, a, h.scale, h.state + h.n0 / 8 % 3, g);
+    auto* fn = g.order == 4 ? k_fx_force<4> : k_fx_force<8>;
+    fn<<<dim3(bx, by < cap ? by : cap), dim3(32, 4), 0, st>>>(
+        h.f, h.force, a, h.scale, h.state + h.n0 / fx_launch_steps(g.order) % 3, g);
   }
   fx_fn(nf)(g, in, out, q, vout, vsub, h, st);
 }

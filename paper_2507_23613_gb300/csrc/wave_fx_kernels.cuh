@@ -1,5 +1,5 @@
 // Temporally blocked 2D wave step in 64-bit fixed point (fixed64.cuh): the FP64 wave solve of
-// 2D second-order problems with a constant or two-layer c^2.
+// 2D problems, second or fourth order, with a constant or two-layer c^2.
 //
 // The scheme is advanced in its increment form, D^{n+1/2} = D^{n-1/2} + kappa_n (c^2 Delta_h W^n -
 // F^n), W^{n+1} = W^n + D^{n+1/2} (kappa_0 = dt^2/2 with D^{-1/2} = 0, else dt^2; eq. WaveSchemeA,
@@ -25,7 +25,8 @@
 // HBM (32 + 16 N_f bytes per point and launch of 8 steps).  N_f = 8, homogeneous, per 8 steps: 76
 // us on 1025^2 (111 Gpts/s) against 162 us for the FP64 form (k_tb2d_pipe), 248 us on 2049^2, 26 us
 // on 513^2.  Small grids are bound by the latency of a launch: 10.4 us on 65^2, of which 5 with
-// nothing stepped and no sums made.
+// nothing stepped and no sums made.  Fourth order, 513^2, N_f = 3: 22.5 us per 4 steps against 4 x
+// 12.2 us for the FP64 one-step kernel.
 //
 // Roles.  A persistent CTA per SM has kFxStep warps that step tiles and kFxTail warps that make
 // the filter sums of the tile stepped before, so that the one's loads, stores and barriers
@@ -39,7 +40,10 @@
 // through shared memory (double buffered: one barrier per step).  An owned point's new value
 // is stored per step as two digits in shared memory (64 bytes per owned point, double buffered
 // between the roles); a thread of the tail warps takes owned points one by one and forms their N_f
-// contributions in registers, with the weights as constant operands.  The sums are laid out tile
+// contributions in registers, with the weights as constant operands.  (All of this for the
+// second-order operator; the fourth-order one reaches two points, so a launch makes 4 steps within
+// the same halo, the warps exchange all their rows, and its 68-fold neighbour sums leave the
+// levels 56 bits.)  The sums are laid out tile
 // by tile, [tile][m][owned point], so that their addresses are a pointer plus constants and the
 // loop has no index arithmetic or masks (points outside the interior have zero levels).
 #pragma once
@@ -55,7 +59,7 @@
 namespace mfwh {
 namespace {
 
-constexpr int kFxT = 8;                          // steps per launch at most
+constexpr int kFxT = 8;                          // halo points: 8 steps of reach 1 or 4 of reach 2
 constexpr int kFxStep = 12, kFxTail = 8;         // warps of the two roles (step warps: at most)
 constexpr int kFxThreads = 32 * (kFxStep + kFxTail);
 constexpr int kFxEX = 64, kFxEY = 4 * kFxStep;   // extended tile
@@ -86,8 +90,13 @@ struct FxArgs {
   double fc[kFxT * NF];      // kappa_n cos(omega~_m t^n)
 };
 
-constexpr size_t kFxHist = (size_t)kFxT * kFxTile * sizeof(int2);   // one buffer
-constexpr size_t kFxSmem = 2 * kFxHist + (size_t)2 * kFxStep * 2 * kFxEX * 8;
+// Shared memory: the two buffers of new values, the two of edge rows (2 or 4 per warp).
+constexpr size_t fx_hist_bytes(int order) {
+  return (size_t)fx_launch_steps(order) * kFxTile * sizeof(int2);
+}
+constexpr size_t fx_smem_bytes(int order) {
+  return 2 * fx_hist_bytes(order) + (size_t)2 * kFxStep * order * kFxEX * 8;
+}
 
 // Barriers among part of the CTA's warps (0 is __syncthreads).
 __device__ __forceinline__ void fx_bar_sync(int id, int threads) {
@@ -102,14 +111,14 @@ __device__ __forceinline__ void fx_prefetch(const void* p) {
 
 // The quantum 2^e of a launch from its input's state, the factor 2^shift of the input and the
 // unit of the sums.  b: bound of the launch's levels in the input's quanta, which the quantum puts
-// just below 2^59.  In FP32, rounding up: every warp makes it before its first load is used, and
+// just below 2^fx_bits.  In FP32, rounding up: every warp makes it before its first load is used, and
 // the few FP64 instructions it would take cost a launch a microsecond (64 cycles a warp each).
 struct FxQuantum {
   float b;
   int shift, e, eq;
 };
 __device__ __forceinline__ FxQuantum fx_quantum(const FxState& st, const FxScale& sc, float gw,
-                                                float gd, int wsum) {
+                                                float gd, int wsum, int order) {
   FxQuantum r;
   r.b = __fmaf_ru(gw, __ull2float_ru(st.wmax), __fmul_ru(gd, __ull2float_ru(st.dmax)));
   // (a quantum keeps the forcing's part below 2^59: no overflow; far below the levels it may
@@ -119,7 +128,7 @@ __device__ __forceinline__ FxQuantum fx_quantum(const FxState& st, const FxScale
   r.eq = st.eq;
   if (r.b > 0.0f) {
     const int ex = (__float_as_int(r.b) >> 23) - 126;   // b < 2^ex (b is normal)
-    r.shift = 59 - ex;
+    r.shift = fx_bits(order) - ex;
     r.eq = max(r.eq, ex + st.e + wsum - 62);
   }
   r.e = st.e - r.shift;
@@ -135,7 +144,7 @@ __device__ __forceinline__ int fx_clamp(int64_t v, int lo, int hi) {
 // magnitudes near the ends of the double range): A and B hold W^n and W^{n-1} on the extended
 // tile in shared memory, the sums (qi: the tile's) are updated in place in global memory.  The
 // arrays hold doubles.
-template <int NF>
+template <int NF, int ORDER>
 __device__ __noinline__ void fx_double_steps(double* A, double* B, const FxArrays& in,
                                              const FxArrays& out, const double* f, int64_t* qi,
                                              const FxArgs<NF>& a, const Geom& g, int64_t x0,
@@ -156,7 +165,8 @@ __device__ __noinline__ void fx_double_steps(double* A, double* B, const FxArray
     for (int e = tid; e < kFxEX * EY; e += blockDim.x) {
       const int lx = e % kFxEX, ly = e / kFxEX;
       const int64_t x = x0 + lx, y = y0 + ly;
-      if (lx < 1 || lx > kFxEX - 2 || ly < 1 || ly > EY - 2 || x <= 0 || x >= g.nx || y <= 0 ||
+      constexpr int H = ORDER / 2;   // reach
+      if (lx < H || lx >= kFxEX - H || ly < H || ly >= EY - H || x <= 0 || x >= g.nx || y <= 0 ||
           y >= g.ny)
         continue;
       const LayerCoef& L = a.lay[first][(g.layer_axis == 0 ? x : y) >= g.layer_split];
@@ -164,6 +174,13 @@ __device__ __noinline__ void fx_double_steps(double* A, double* B, const FxArray
       double acc = fma(L.A0, A[e], -B[e]);
       acc = fma(L.Ax, sx, acc);
       acc = fma(L.Ay, sy, acc);
+      if constexpr (ORDER == 4) {   // the ghost value beyond the boundary is minus the centre's
+        const double tx = (x == 1 ? -A[e] : A[e - 2]) + (x == g.nx - 1 ? -A[e] : A[e + 2]);
+        const double ty =
+            (y == 1 ? -A[e] : A[e - 2 * kFxEX]) + (y == g.ny - 1 ? -A[e] : A[e + 2 * kFxEX]);
+        acc = fma(L.Bx, tx, acc);
+        acc = fma(L.By, ty, acc);
+      }
       const int64_t p = y * g.sy + x;
       if (a.forced)
         for (int m = 0; m < NF; ++m) acc = fma(-a.fc[s * NF + m], f[m * g.points + p], acc);
@@ -218,33 +235,33 @@ __device__ __noinline__ void fx_finish(const int64_t* q, const double* unit, boo
 
 // Reads W, D (level n0; D is not read when n0 = 0) and writes those of level n0 + steps, with the
 // sums updated in place; the last launch writes v_out instead.  state[0]: the input's quantum and
-// maxima; state[1]: the output's, its maxima 0 on entry; state[2]: reset to 0.  ISO: equal
-// spacings (one product per step instead of two).
-template <int NF, bool ISO, bool FORCED>
+// maxima; state[1]: the output's, its maxima 0 on entry; state[2]: reset to 0.  ISO (second
+// order): equal spacings (one product per step instead of two).
+template <int NF, bool ISO, bool FORCED, int ORDER>
 __global__ void __launch_bounds__(kFxThreads, 1)
 k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
-       const int64_t* __restrict__ force, int64_t* __restrict__ q, double* vout, const double* vsub,
-       const __grid_constant__ FxArgs<NF> a, const FxScale* __restrict__ scale,
+       const int64_t* force, int64_t* __restrict__ q, double* vout, const double* vsub,
+       const __grid_constant__ FxArgs<NF> a, const FxScale* scale,
        const FxState* s_in, FxState* s_out, FxState* s_reset, const Geom g, int tiles_x,
        int tiles) {
-  constexpr int T = kFxT, VX = kFxVX;
+  constexpr int T = kFxT, VX = kFxVX, REACH = ORDER / 2, STEPS = fx_launch_steps(ORDER);
+  constexpr size_t kHist = fx_hist_bytes(ORDER);
   const int NW = a.warps, EY = 4 * NW, VY = EY - 2 * T;   // step warps, rows of the tile, owned rows
   const int threads = 32 * (NW + kFxTail);
   constexpr int kBarStep = 1, kBarFull = 2, kBarEmpty = 4;   // (and + 1: second buffer)
   extern __shared__ __align__(16) unsigned char fx_smem[];
   __shared__ double s_unit[NF];   // last launch: unit of the sums
   __shared__ int64_t s_off[NF];   // start of the contributions, with half a unit of the sums
-  int64_t* edge = reinterpret_cast<int64_t*>(fx_smem + 2 * kFxHist);   // [2][warp][2][64]
+  int64_t* edge = reinterpret_cast<int64_t*>(fx_smem + 2 * kHist);   // [2][warp][ORDER][64]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");   // the launch before is complete
+  pdl_begin();
   const FxScale sc = *scale;
   if (sc.mode) {   // FP64 steps by the whole CTA
     double* A = reinterpret_cast<double*>(fx_smem);
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
       const int64_t x0 = (int64_t)(tile % tiles_x) * VX - T, y0 = (int64_t)(tile / tiles_x) * VY - T;
       int64_t* qt = q + (int64_t)tile * NF * kFxTile;
-      fx_double_steps<NF>(A, A + kFxEX * EY, in, out, f, qt, a, g, x0, y0);
+      fx_double_steps<NF, ORDER>(A, A + kFxEX * EY, in, out, f, qt, a, g, x0, y0);
       __syncthreads();
       if (!a.last) continue;
       for (int i = tid; i < VX * VY; i += threads) {
@@ -257,11 +274,11 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
     return;
   }
   const FxState st = *s_in;
-  const FxQuantum Q = fx_quantum(st, sc, a.gw, a.gd, a.wsum);
+  const FxQuantum Q = fx_quantum(st, sc, a.gw, a.gd, a.wsum, ORDER);
   const int shift = Q.shift;
   const bool zero = Q.b == 0.0f;   // all levels are 0
   // shifts of the stored sums and of the launch's contributions (units of 2^(e + 64)): eq - e - 64
-  // >= wsum - 67 >= 0 as the bound's exponent is e + 59
+  // >= wsum + fx_bits - 126 >= 0 as the bound's exponent is e + fx_bits
   const int q_old = Q.eq - st.eq, q_new = Q.eq - Q.e - 64;
   const bool wide = q_new >= 32;   // the contributions' high words only
   if (blockIdx.x == 0 && tid == 0) {
@@ -281,7 +298,7 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
     int mw = 0, md = 0;                        // largest high words of |W| and |D|
     int it = 0;
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++it) {
-      int2* hist = reinterpret_cast<int2*>(fx_smem + (it & 1) * kFxHist);   // [T][kFxTile]
+      int2* hist = reinterpret_cast<int2*>(fx_smem + (it & 1) * kHist);   // [T][kFxTile]
       const int64_t x0 = (int64_t)(tile % tiles_x) * VX - T, y0 = (int64_t)(tile / tiles_x) * VY - T;
       // local bounds of grid rows and of interior points; first local index of the upper layer
       const int ghy = fx_clamp(g.ny - y0, -1, EY - 1);
@@ -326,8 +343,16 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
           d[k][c] = is ? fx_rescale(d[k][c], shift) : 0;
         }
       }
-      auto edge_row = [&](int buf, int wp, int which) {
-        return reinterpret_cast<longlong2*>(edge + ((buf * kFxStep + wp) * 2 + which) * kFxEX) + lane;
+      // the rows a warp shows its neighbours: second order 0 and 3, fourth order all
+      auto edge_row = [&](int buf, int wp, int row) {
+        return reinterpret_cast<longlong2*>(
+                   edge + ((buf * kFxStep + wp) * ORDER + (ORDER == 4 ? row : row / 3)) * kFxEX) +
+               lane;
+      };
+      auto put_edges = [&](int buf) {
+#pragma unroll
+        for (int k = 0; k < 4; k += ORDER == 4 ? 1 : 3)
+          *edge_row(buf, warp, k) = make_longlong2(w[k][0], w[k][1]);
       };
       // forced: the step's forcing, loaded while the step before ends
       int64_t fs[FORCED ? 4 : 1][2];
@@ -351,20 +376,52 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
         const FxAxes one = a.coef[first][hi_mask & 1u];
         const FxAxes clo = PLAIN ? one : a.coef[first][0], chi = PLAIN ? one : a.coef[first][1];
         // the outermost rows have no neighbour warp: their values are never read
-        const longlong2 up = *edge_row(buf, warp > 0 ? warp - 1 : 0, 1);
-        const longlong2 bl = *edge_row(buf, warp < NW - 1 ? warp + 1 : warp, 0);
+        const int wu = warp > 0 ? warp - 1 : 0, wb = warp < NW - 1 ? warp + 1 : warp;
+        const longlong2 up = *edge_row(buf, wu, 3);
+        const longlong2 bl = *edge_row(buf, wb, 0);
         const int64_t below[2] = {bl.x, bl.y};
         int64_t dv[2] = {w[0][0] - up.x, w[0][1] - up.y};   // W - W_above of the current row
+        // fourth order: the same of the row above, and the second row below
+        int64_t dv2[2] = {0, 0}, below2[2] = {0, 0};
+        if constexpr (ORDER == 4) {
+          const longlong2 up2 = *edge_row(buf, wu, 2), bl2 = *edge_row(buf, wb, 1);
+          dv2[0] = up.x - up2.x;
+          dv2[1] = up.y - up2.y;
+          below2[0] = bl2.x;
+          below2[1] = bl2.y;
+        }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const int64_t left = __shfl_up_sync(0xffffffffu, w[k][1], 1);
           const int64_t right = __shfl_down_sync(0xffffffffu, w[k][0], 1);
-          // W - W_left of columns 0 .. 2
+          // W - W_left of columns 0 .. 2, fourth order also -1 and 3
           const int64_t dx[3] = {w[k][0] - left, w[k][1] - w[k][0], right - w[k][1]};
+          int64_t dxl = 0, dxr = 0;
+          if constexpr (ORDER == 4) {
+            dxl = left - __shfl_up_sync(0xffffffffu, w[k][0], 1);
+            dxr = __shfl_down_sync(0xffffffffu, w[k][1], 1) - right;
+          }
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
             const int64_t dn = (k < 3 ? w[k < 3 ? k + 1 : 3][c] : below[c]) - w[k][c];
-            const int64_t dxx = dx[c + 1] - dx[c], dyy = dn - dv[c];
+            int64_t dxx = dx[c + 1] - dx[c], dyy = dn - dv[c];
+            if constexpr (ORDER == 4) {
+              // 16 times the first neighbours' sum of differences less the second neighbours', which
+              // is dxx + (difference two to the right) - (two to the left)
+              int64_t ra = c == 0 ? dx[2] : dxr, la = c == 0 ? dxl : dx[0];
+              const int64_t w1 = k < 3 ? w[k < 3 ? k + 1 : 3][c] : below[c];
+              const int64_t w2 = k < 2 ? w[k < 2 ? k + 2 : 3][c] : (k == 2 ? below[c] : below2[c]);
+              int64_t ba = w2 - w1, ab = dv2[c];
+              if (!PLAIN) {   // a ghost value beyond the boundary is minus the centre's
+                if (lx + c == ihx) ra = -w[k][c];
+                if (lx + c == ilx) la = w[k][c];
+                if (ly + k == ihy) ba = -w[k][c];
+                if (ly + k == ily) ab = w[k][c];
+              }
+              dxx = 15 * dxx - (ra - la);
+              dyy = 15 * dyy - (ba - ab);
+              dv2[c] = dv[c];
+            }
             dv[c] = dn;
             const bool upper = !PLAIN && (hi_mask >> (2 * k + c) & 1u);
             const FxAxes& L = upper ? chi : clo;
@@ -383,16 +440,17 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
           }
         }
       };
+      // (fourth order: not the rows next to the boundary, which have a ghost neighbour)
       const bool plain = __all_sync(0xffffffffu, in_mask == 0xFFu) &&
+                         (ORDER == 2 || (y0 + ly > 1 && y0 + ly + 3 < g.ny - 1)) &&
                          (__all_sync(0xffffffffu, hi_mask == 0u) ||
                           __all_sync(0xffffffffu, hi_mask == 0xFFu));
       load_force(0);
-      *edge_row(0, warp, 0) = make_longlong2(w[0][0], w[0][1]);
-      *edge_row(0, warp, 1) = make_longlong2(w[3][0], w[3][1]);
+      put_edges(0);
       fx_bar_sync(kBarStep, 32 * NW);
       if (it >= 2) fx_bar_sync(kBarEmpty + (it & 1), threads);   // the buffer's sums are made
       for (int s = 0; s < a.steps; ++s) {
-        const int r = a.steps - 1 - s;   // later steps read the owned points grown by r
+        const int r = REACH * (a.steps - 1 - s);   // later steps read the owned points grown by r
         if (ly + 3 >= T - r && ly < T + VY + r) {
           if (plain)
             step_points(s, s & 1, std::true_type{});
@@ -400,8 +458,7 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
             step_points(s, s & 1, std::false_type{});
           if (r > 0) {
             load_force(s + 1);
-            *edge_row((s + 1) & 1, warp, 0) = make_longlong2(w[0][0], w[0][1]);
-            *edge_row((s + 1) & 1, warp, 1) = make_longlong2(w[3][0], w[3][1]);
+            put_edges((s + 1) & 1);
           }
           if (owner) {
             int2* h = hist + s * kFxTile + (ly - T) * VX + lx - T;
@@ -459,7 +516,7 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
     int it = 0;
     if ((int)blockIdx.x < tiles) prefetch(blockIdx.x);
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++it) {
-      const int2* hist = reinterpret_cast<const int2*>(fx_smem + (it & 1) * kFxHist);
+      const int2* hist = reinterpret_cast<const int2*>(fx_smem + (it & 1) * kHist);
       int64_t* qt = q + (int64_t)tile * NF * kFxTile;
       // the sums are loaded one group of MG frequencies ahead
       int64_t qm[MG], qn[MG];
@@ -501,9 +558,9 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
                   r[j] = fmaf(a.wl[e], vf, r[j]);
                 }
             };
-            if (a.steps == T) {
+            if (a.steps == STEPS) {
 #pragma unroll
-              for (int s = 0; s < T; ++s) add(s);
+              for (int s = 0; s < STEPS; ++s) add(s);
             } else {
 #pragma unroll 1
               for (int s = 0; s < a.steps; ++s) add(s);
@@ -552,16 +609,17 @@ inline double fx_forcing_coef(const FxHost& h, int n, int nf, int m) {
 
 // ---- host launchers ------------------------------------------------------------------------
 
-template <int NF, bool ISO, bool FORCED>
+template <int NF, bool ISO, bool FORCED, int ORDER>
 void fx_launch(const Geom& g, const FxArrays& in, const FxArrays& out, int64_t* q, double* vout,
                const double* vsub, const FxHost& h, cudaStream_t st) {
+  constexpr size_t smem = fx_smem_bytes(ORDER);
   static int sms[64] = {};   // SMs of the device; the attribute is set on first use
   int dev = 0;
   cudaGetDevice(&dev);
   int n = (dev >= 0 && dev < 64) ? sms[dev] : 0;
   if (n == 0) {
-    cudaFuncSetAttribute(k_fx2d<NF, ISO, FORCED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)kFxSmem);
+    cudaFuncSetAttribute(k_fx2d<NF, ISO, FORCED, ORDER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem);
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
       n = 1;
     if (dev >= 0 && dev < 64) sms[dev] = n;
@@ -608,35 +666,30 @@ void fx_launch(const Geom& g, const FxArrays& in, const FxArrays& out, int64_t* 
       a.fc[i] = is && h.forced ? fx_forcing_coef(h, k, NF, m) : 0.0;
     }
   const int64_t tx = (g.nx + kFxVX) / kFxVX, tiles = fx_tiles(g.nx, g.ny, h.warps);
-  const int L = h.n0 / kFxT;
-  // Programmatic dependent launch: a launch's CTAs start where and when the one before leaves an SM
-  // free, and wait in the kernel for its end.
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(tiles < n ? tiles : n));
-  cfg.blockDim = dim3(32 * (h.warps + kFxTail));
-  cfg.dynamicSmemBytes = kFxSmem;
-  cfg.stream = st;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, k_fx2d<NF, ISO, FORCED>, in, out, h.f, (const int64_t*)h.force, q, vout,
-                     vsub, a, h.scale, (const FxState*)(h.state + L % 3), h.state + (L + 1) % 3,
-                     h.state + (L + 2) % 3, g, (int)tx, (int)tiles);
+  const int L = h.n0 / fx_launch_steps(ORDER);
+  launch_dependent(k_fx2d<NF, ISO, FORCED, ORDER>, dim3((unsigned)(tiles < n ? tiles : n)),
+                   dim3(32 * (h.warps + kFxTail)), smem, st, in, out, h.f, h.force, q, vout, vsub, a,
+                   h.scale, h.state + L % 3, h.state + (L + 1) % 3, h.state + (L + 2) % 3, g, (int)tx,
+                   (int)tiles);
 }
 
 template <int NF>
 void fx_launch_nf(const Geom& g, const FxArrays& in, const FxArrays& out, int64_t* q, double* vout,
                   const double* vsub, const FxHost& h, cudaStream_t st) {
-  if (h.iso && h.forced)
-    fx_launch<NF, true, true>(g, in, out, q, vout, vsub, h, st);
+  auto go = [&](auto iso, auto order) {
+    constexpr bool I = decltype(iso)::value;
+    constexpr int O = decltype(order)::value;
+    if (h.forced)
+      fx_launch<NF, I, true, O>(g, in, out, q, vout, vsub, h, st);
+    else
+      fx_launch<NF, I, false, O>(g, in, out, q, vout, vsub, h, st);
+  };
+  if (g.order == 4)
+    go(std::false_type{}, std::integral_constant<int, 4>{});
   else if (h.iso)
-    fx_launch<NF, true, false>(g, in, out, q, vout, vsub, h, st);
-  else if (h.forced)
-    fx_launch<NF, false, true>(g, in, out, q, vout, vsub, h, st);
+    go(std::true_type{}, std::integral_constant<int, 2>{});
   else
-    fx_launch<NF, false, false>(g, in, out, q, vout, vsub, h, st);
+    go(std::false_type{}, std::integral_constant<int, 2>{});
 }
 
 }  // namespace

@@ -68,8 +68,10 @@ def check(n, length, om, f, v, layer, forced, n_p=1, order=2):
     level = 8.0 * np.abs(v).sum(0).max()
     if forced:
         level += n_t ** 2 * dt ** 2 * np.abs(f).sum(0).max()
+    kw = {} if layer is None else dict(c_lo=1.0, c_hi=layer[2], interface=layer[1],
+                                       layer_axis=layer[0])
     p, keep = M.make_problem(n, length, om, None, n_p=n_p, filter_mode=_lib.FILTER_TRADITIONAL,
-                             order=order)
+                             order=order, **kw)
     w = np.abs(M.plan_weights(p, n_t, nf)).sum(0)
     bound = n_t ** 2 * 2.0 ** -52 * level * (np.abs(s["B_inv"]) @ w)
     err = np.abs(got - want).max((1, 2))
@@ -118,3 +120,70 @@ def test_zero_input_and_values_without_a_quantum():
             want, _ = maps(n, length, om, g, w, general=True, forced=True)
             assert np.array_equal(np.isfinite(got), np.isfinite(want))
             assert not np.isfinite(got).all()
+
+
+def fourth_order_reference(n, length, s, w, f, v, layer, forced):
+    """Extended-precision map with the fourth-order operator (odd reflection at the boundary)."""
+    L = np.longdouble
+    c2 = np.ones((n[1] + 1, n[0] + 1), L)
+    if layer is not None:
+        axis, at, c = layer
+        x = np.arange(n[axis] + 1) * (length[axis] / n[axis])
+        c2 = c2 * (np.where(x < at, 1.0, c * c) if axis == 0 else
+                   np.where(x < at, 1.0, c * c)[:, None])
+    dt, n_t = L(s["dt"]), s["n_t"]
+    u = v.astype(L).sum(0)
+    f = f.astype(L)
+    cos = np.cos(np.arange(n_t)[:, None] * s["dt"] * np.asarray(s["omega_tilde"])[None]).astype(L)
+    w = w.astype(L)
+    q = w[0][:, None, None] * u[None]
+    d = np.zeros_like(u)
+    h = [length[a] / n[a] for a in (0, 1)]
+
+    def second(u, axis):
+        e = np.moveaxis(u, axis, 0)
+        e = np.concatenate([-e[1:2], e, -e[-2:-1]])
+        t = -e[:-4] + 16 * e[1:-3] - 30 * e[2:-2] + 16 * e[3:-1] - e[4:]
+        out = np.zeros_like(u)
+        np.moveaxis(out, axis, 0)[1:-1] = t / 12
+        return out
+    for k in range(n_t):
+        inc = dt * dt * c2 * (second(u, 1) / L(h[0]) ** 2 + second(u, 0) / L(h[1]) ** 2)
+        if forced:
+            inc = inc - dt * dt * np.tensordot(cos[k], f, 1)
+        inc[[0, -1]] = 0
+        inc[:, [0, -1]] = 0
+        d = d + (inc / 2 if k == 0 else inc)
+        u = u + d
+        q = q + w[k + 1][:, None, None] * u[None]
+    out = np.tensordot(np.asarray(s["B_inv"]).astype(L), q, 1)
+    out[:, [0, -1]] = 0
+    out[:, :, [0, -1]] = 0
+    return out
+
+
+@pytest.mark.parametrize("n,nf,layer", [
+    ((2, 3), 1, None), ((3, 2), 2, None), ((47, 15), 3, (0, 0.4, 1.5)), ((49, 17), 5, None),
+    ((65, 64), 2, (1, 0.93, 0.8)), ((96, 33), 9, None), ((95, 31), 1, (1, 0.3, 1.2)),
+    ((71, 47), 1, None), ((150, 60), 4, None), ((90, 62), 2, None), ((144, 65), 3, None),
+    ((145, 97), 16, None)])
+@pytest.mark.parametrize("forced", [False, True])
+def test_fourth_order_map(n, nf, layer, forced):
+    om = np.linspace(6.0, 6.0 + 2.5 * (nf - 1), nf) + 0.37
+    f, v = data(n, nf, 5)
+    length = (1.0, 1.1 * n[1] / n[0])
+    lay = None if layer is None else (layer[0], layer[1] * length[layer[0]], layer[2])
+    n_p = 2 if nf > 4 else 1
+    got, s = maps(n, length, om, f, v, lay, False, forced, n_p, 4)
+    kw = {} if lay is None else dict(c_lo=1.0, c_hi=lay[2], interface=lay[1], layer_axis=lay[0])
+    p, keep = M.make_problem(n, length, om, None, n_p=n_p, filter_mode=_lib.FILTER_TRADITIONAL,
+                             order=4, **kw)
+    w = M.plan_weights(p, s["n_t"], nf)
+    want = fourth_order_reference(n, length, s, w, f, v, lay, forced)
+    level = 8.0 * np.abs(v).sum(0).max()
+    if forced:
+        level += s["n_t"] ** 2 * s["dt"] ** 2 * np.abs(f).sum(0).max()
+    # as in check(); the products' coefficients are rounded to 53 bits in the map only
+    bound = s["n_t"] ** 2 * 2.0 ** -52 * level * (np.abs(s["B_inv"]) @ np.abs(w).sum(0))
+    err = np.abs(got - want).max((1, 2))
+    assert np.isfinite(got).all() and np.all(err <= bound), (err, bound)
