@@ -106,10 +106,11 @@ typedef struct {
                                 8 whatever this says, for the fourth order 4; other FP64 2D
                                 problems of up to 8 frequencies with second order, explicit steps
                                 and constant or two-layer c: 3 on tile shape 5; else 1),
-                                1 = one step per kernel launch (FP32 3D, second order: Kahan sums
-                                of one step each, in launches of 4); 2D: 2, 3, 4 or 8 for FP64,
+                                1 = one step per kernel launch (FP32 3D, second order, beyond L2: the
+                                same sums in launches of 4); 2D: 2, 3, 4 or 8 for FP64,
                                 4, 8 or 16 for FP32 = temporal blocking with that depth; 3D: 2 or
-                                4 for the FP32 precisions.  Results are bit-identical for every
+                                4 for the FP32 precisions (grids that L2 holds: one step per
+                                launch with the sums of that depth).  Results are bit-identical for every
                                 depth (FP32_BLOCKSUM: for every depth with the same partial-sum
                                 length). */
   int order;                 /* order p of the spatial operator L_{ph}: 2 (0 means 2) or 4.
@@ -348,7 +349,7 @@ mfwh_status mfwh_solve_batch_graph(const mfwh_handle_t* handles, int count, int 
  * homogeneous wave solve of prob on the current device for each candidate temporal depth and
  * tile shape (FP32, 2D: depths 4, 8, 16; FP64, 2D: (8, 3), which has no effect, for problems in
  * 64-bit integers, else depths 1 to 8 and their tile shapes; FP32, 3D: depths 1, 2, 4, only 1 for
- * grids of at most one tile per SM; FP64 3D, fourth order and c^2 fields: depth 1), keeping the
+ * grids that L2 holds; FP64 3D, fourth order and c^2 fields: depth 1), keeping the
  * fastest:
  * *time_block and *tile_shape receive it, *ms_per_step
  * (may be NULL) its time per leapfrog step.  Results are cached per device, grid, number of

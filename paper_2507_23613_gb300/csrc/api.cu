@@ -188,6 +188,8 @@ struct mfwh_handle_s {
   float* W32[4] = {};               // (W, D) pairs: W32[0], W32[1] and W32[2], W32[3]
   float* qs = nullptr;              // Kahan sums [nf][P]
   float* qc = nullptr;              // Kahan compensations [nf][P]
+  float* part32 = nullptr;          // FP32_BLOCKSUM in 3D on grids that L2 holds: partial sums [N]
+  int l2_bytes = 0;                 // of the device
   std::vector<float> wq32_h, fc32_h;   // [(N_t + 1) * nf] w_{n,m}, [N_t * nf] kappa_n cos(omega~_m t^n)
   // implicit time stepping (MFWH_TIME_IMPLICIT)
   bool implicit = false;
@@ -288,8 +290,16 @@ mfwh_status apply_pi32(mfwh_handle_t h, const double* vin, double* vout, int for
   int launches = 0;
   // One step per launch (time_block 1, the 3D default) makes a Kahan update at every step, and
   // the blocked kernels with such updates give the same bits: 3D runs 4 steps per launch then.
+  // While L2 holds what a step reads and writes (W, D, the sums, f), one step per launch is faster
+  // than either depth and runs instead, with partial sums over as many steps as the depth: 65^3, N_f
+  // = 8, 7.5 us per step against 9.6 (depth 4) and 15.3 (2); 17^3, N_f = 2, 2.5 against 3.9 and 6.3.
+  // At 129^3, N_f = 4 (94 MB) 29.1 against 28.1 and 44.1, at 161^3 (184 MB) 76 against 42 and 70.
+  const bool steps3 = P.dim == 3 && P.order == 2 &&
+                      h->P * (12 + 8 * nf + (h->part32 ? 4 * nf : 0) + (forced ? 4 * nf : 0)) <=
+                          h->l2_bytes &&
+                      (h->part32 || P.precision != MFWH_PREC_FP32_BLOCKSUM || P.time_block <= 1);
   const bool kahan3 = P.dim == 3 && P.order == 2 && P.time_block <= 1;
-  const int depth = kahan3 ? 4 : P.time_block;
+  const int depth = steps3 ? 1 : (kahan3 ? 4 : P.time_block);
   if (depth > 1) {
     TB32Host a;
     a.reg_lo = reg_lo;
@@ -324,6 +334,9 @@ mfwh_status apply_pi32(mfwh_handle_t h, const double* vin, double* vout, int for
   } else {
     Step32Host a;
     a.forced = forced;
+    a.group = 0;
+    a.part = h->part32;
+    const int T = h->part32 ? P.time_block : 1;   // steps of a partial sum
     float* Wc = h->W32[0];
     float* Wn = h->W32[2];
     float* D = h->W32[1];
@@ -334,6 +347,8 @@ mfwh_status apply_pi32(mfwh_handle_t h, const double* vin, double* vout, int for
         a.fc[m] = h->fc32_h[(size_t)n * nf + m];
         a.wq[m] = h->wq32_h[(size_t)(n + 1) * nf + m];
       }
+      if (T > 1) a.group = (n % T == 0 ? 1 : 0) | (n % T == T - 1 || n + 1 == n_t ? 2 : 0);
+      if (T > 1 && a.group == 0) a.group = 4;   // neither: the partial sum goes on
       const float* D_in = n == 0 ? nullptr : D;
       if (n + 1 < n_t) {
         launch_step32(nf, h->geom, Wc, D_in, Wn, D, h->f32, h->qs, h->qc, a, st);
@@ -1131,6 +1146,8 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
   };
   cudaError_t e = cudaGetDevice(&h->device);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaGetDevice"));
+  e = cudaDeviceGetAttribute(&h->l2_bytes, cudaDevAttrL2CacheSize, h->device);
+  if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaDeviceGetAttribute"));
   if (P.fixed) {
     int sms = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
@@ -1210,6 +1227,13 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
     for (auto& b : fb) {
       e = alloc_workspace(h, b.p, std::max<int64_t>(b.n, 1));
       if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaMalloc (FP32 workspace)"));
+    }
+    // (at most 1/3 of L2's size; without it the blocked kernels run)
+    if (P.dim == 3 && P.order == 2 && P.precision == MFWH_PREC_FP32_BLOCKSUM && P.time_block > 1 &&
+        h->P * (12 + 12 * nf) <= h->l2_bytes &&
+        cudaMalloc(&h->part32, sizeof(float) * h->N) != cudaSuccess) {
+      (void)cudaGetLastError();
+      h->part32 = nullptr;
     }
     for (int i = 0; i < 4 && e == cudaSuccess; ++i)
       e = cudaMemsetAsync(h->W32[i], 0, sizeof(float) * h->PW, h->stream);
@@ -1677,7 +1701,7 @@ void mfwh_destroy(mfwh_handle_t h) {
   if (h->d_bar) cudaFree(h->d_bar);
   if (h->d_mgc) cudaFree(h->d_mgc);
   delete h->imp;
-  float* fbufs[] = {h->f32, h->W32[0], h->W32[1], h->W32[2], h->W32[3], h->qs, h->qc};
+  float* fbufs[] = {h->f32, h->W32[0], h->W32[1], h->W32[2], h->W32[3], h->qs, h->qc, h->part32};
   for (float* b : fbufs)
     if (b) cudaFree(b);
   if (h->pinned) cudaFreeHost(h->pinned);
@@ -2275,12 +2299,10 @@ mfwh_status mfwh_autotune(const mfwh_problem* prob, void* stream, int* time_bloc
   if (P.order == 4 || P.c2_field || (P.dim == 3 && P.precision == MFWH_PREC_FP64)) {
     cand = {{1, 0}};
   } else if (P.dim == 3) {
-    // grids of at most one tile per SM: launches are bound by latency, and 1 (Kahan sums of every
-    // step, in launches of 4) is as fast as 4
-    int sms = 0;
-    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int64_t tiles = ((P.n[0] + 56) / 56) * ((P.n[1] + 8) / 8) * ((P.n[2] + 12) / 12);
-    if (tiles <= sms)
+    // in L2 every depth runs one step per launch; the sums of 1 are the most accurate
+    int l2 = 0;
+    CK(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
+    if (P.s.points * (12 + 12 * P.s.nf) <= l2)
       cand = {{1, 0}};
     else
       cand = {{1, 0}, {2, 0}, {4, 0}};

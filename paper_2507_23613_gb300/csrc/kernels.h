@@ -204,6 +204,8 @@ struct Step32Host {
   float fc[MFWH_MAX_NF];   // kappa_n cos(omega~_m t^n), rounded to FP32
   float wq[MFWH_MAX_NF];   // w_{n+1,m}, rounded to FP32
   int forced;
+  int group;               // filter terms: 0 Kahan, else a partial sum: 1 its first, 2 its last step
+  float* part;             // device [nf][points] partial sums (group)
 };
 struct TB32Host {
   Coef32 reg_lo, reg_hi, first_lo, first_hi;

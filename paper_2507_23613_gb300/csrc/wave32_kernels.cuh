@@ -20,7 +20,7 @@
 //  * k_tb2d32: 2D, T steps per launch on overlapped tiles whose points, halo included, live
 //    in the registers of one CTA for all T steps;
 //  * k_tb3d32: the same in 3D with T = 2 or 4;
-//  * k_step32 / k_last32: one step per launch, the fourth-order L_h and 2D at time_block 1.
+//  * k_step32 / k_last32: one step per launch, 2D or 3D, second- or fourth-order L_h.
 // All are dependent launches (launch_dependent): one step on 33^3, N_f = 2, took 4.3 us, now 2.6.
 // All perform the same FP32 operations per point in the same order, so their
 // results are bit-identical.
@@ -69,6 +69,8 @@ struct Step32Args {
   float fc[NF];     // kappa_n cos(omega~_m t^n)
   float wq[NF];     // w_{n+1,m}
   int forced;
+  int group;        // sums: 0 Kahan, else partial over several steps, 1 the first, 2 the last, 3 both
+  float* part;      // [NF][points] partial sums
 };
 
 __device__ __forceinline__ bool interior2(int64_t gx, int64_t gy, const Geom& g) {
@@ -77,6 +79,14 @@ __device__ __forceinline__ bool interior2(int64_t gx, int64_t gy, const Geom& g)
 
 __device__ __forceinline__ void kahan_add(float& s, float& c, float w, float x) {
   const float y = fmaf(w, x, -c);
+  const float t = s + y;
+  c = (t - s) - y;
+  s = t;
+}
+
+// Fold a partial sum x into the Kahan pair (s, c).
+__device__ __forceinline__ void kahan_fold(float& s, float& c, float x) {
+  const float y = x - c;
   const float t = s + y;
   c = (t - s) - y;
   s = t;
@@ -153,8 +163,24 @@ __device__ __forceinline__ void step_point(const float* W, const float* D,
   wn = w + dn;
 }
 
-// W_out = W + D', D' = D + increment (D_out may alias D_in; W_out must not alias W_in);
-// Kahan sums updated in place.
+// The term of one step added to the pair (s, c), or (a.group) to the partial sum of the steps of one
+// launch of the blocked kernels, which the last of them folds into the pair: the same operations as
+// theirs.  Returns whether the pair has changed; a partial sum that goes on is in t.
+template <int NF>
+__device__ __forceinline__ bool add_term(float& s, float& c, float& t, const Step32Args<NF>& a,
+                                         int m, int64_t o, float wn) {
+  if (a.group == 0) {
+    kahan_add(s, c, a.wq[m], wn);
+    return true;
+  }
+  t = fmaf(a.wq[m], wn, (a.group & 1) ? 0.0f : a.part[o]);
+  if (!(a.group & 2)) return false;
+  kahan_fold(s, c, t);
+  return true;
+}
+
+// W_out = W + D', D' = D + increment (D_out may alias D_in; W_out must not alias W_in); sums
+// updated in place.
 template <int NF, int DIM, int ORDER>
 __global__ void __launch_bounds__(kBX * kBY)
 k_step32(const float* W, const float* D_in, float* __restrict__ W_out, float* D_out,
@@ -171,10 +197,18 @@ k_step32(const float* W, const float* D_in, float* __restrict__ W_out, float* D_
   D_out[wpos(g, i, j, k)] = dn;
 #pragma unroll
   for (int m = 0; m < NF; ++m) {
-    float s = qs[m * g.points + p], c = qc[m * g.points + p];
-    kahan_add(s, c, a.wq[m], wn);
-    qs[m * g.points + p] = s;
-    qc[m * g.points + p] = c;
+    const int64_t o = m * g.points + p;
+    float s = 0.0f, c = 0.0f, t = 0.0f;
+    if (a.group == 0 || (a.group & 2)) {
+      s = qs[o];
+      c = qc[o];
+    }
+    if (add_term(s, c, t, a, m, o, wn)) {
+      qs[o] = s;
+      qc[o] = c;
+    } else {
+      a.part[o] = t;
+    }
   }
 }
 
@@ -224,7 +258,8 @@ k_last32(const float* W, const float* D, const float* __restrict__ f,
     for (int m = 0; m < NF; ++m) {
       s[m] = qs[m * g.points + p];
       c[m] = qc[m * g.points + p];
-      kahan_add(s[m], c[m], a.wq[m], wn);
+      float t;
+      add_term(s[m], c[m], t, a, m, m * g.points + p, wn);   // (a last step ends its group)
     }
   }
   filter_solve_out<NF>(s, c, b, subtract, vsub, vout, p, g.points, interior);
@@ -271,15 +306,6 @@ constexpr size_t rt32_smem_bytes() {
   return sizeof(float) * ((size_t)T * (kRtEX - 2 * T) * (kRtEY - 2 * T) +
                           (size_t)2 * kRtWarps * 2 * kRtEX);
 }
-
-// Fold a partial sum x into the Kahan pair (s, c).
-__device__ __forceinline__ void kahan_fold(float& s, float& c, float x) {
-  const float y = x - c;
-  const float t = s + y;
-  c = (t - s) - y;
-  s = t;
-}
-
 
 template <int NF, int T, int ACC>
 __global__ void __launch_bounds__(kRtThreads, 1)
@@ -764,6 +790,8 @@ Step32Args<NF> step_args(const Step32Host& h) {
     a.wq[m] = h.wq[m];
   }
   a.forced = h.forced;
+  a.group = h.group;
+  a.part = h.part;
   return a;
 }
 
@@ -796,7 +824,9 @@ void step32_nf(const Geom& g, const float* W, const float* D_in, float* W_out, f
       launch_dependent(k_step32<NF, 3, 4>, grid, blk, 0, st, W, D_in, W_out, D_out, f, qs, qc, a, g);
     else
       launch_dependent(k_step32<NF, 2, 4>, grid, blk, 0, st, W, D_in, W_out, D_out, f, qs, qc, a, g);
-  } else {   // (second-order 3D steps are those of k_tb3d32)
+  } else if (g.dim == 3) {
+    launch_dependent(k_step32<NF, 3, 2>, grid, blk, 0, st, W, D_in, W_out, D_out, f, qs, qc, a, g);
+  } else {
     launch_dependent(k_step32<NF, 2, 2>, grid, blk, 0, st, W, D_in, W_out, D_out, f, qs, qc, a, g);
   }
 }
@@ -814,6 +844,8 @@ void last32_nf(const Geom& g, const float* W, const float* D, const float* f, co
       launch_dependent(k_last32<NF, 3, 4>, grid, blk, 0, st, W, D, f, qs, qc, vout, vsub, a, b, sub, g);
     else
       launch_dependent(k_last32<NF, 2, 4>, grid, blk, 0, st, W, D, f, qs, qc, vout, vsub, a, b, sub, g);
+  } else if (g.dim == 3) {
+    launch_dependent(k_last32<NF, 3, 2>, grid, blk, 0, st, W, D, f, qs, qc, vout, vsub, a, b, sub, g);
   } else {
     launch_dependent(k_last32<NF, 2, 2>, grid, blk, 0, st, W, D, f, qs, qc, vout, vsub, a, b, sub, g);
   }

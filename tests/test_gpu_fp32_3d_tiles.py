@@ -56,3 +56,30 @@ def test_blocked_depths_agree_at_tile_edges(n, nf, layer):
             assert np.array_equal(a, b), (key, np.max(np.abs(a - b)))
     for a, b in zip(outs[4], outs["fp64"]):
         assert np.max(np.abs(a - b)) <= 2e-5 * np.max(np.abs(b))
+
+
+@pytest.mark.parametrize("n,prec,tb,layer", [
+    ((112, 128, 144), _lib.PREC_FP32_BLOCKSUM, 4, 0), ((111, 127, 143), _lib.PREC_FP32_BLOCKSUM, 4, None),
+    ((119, 131, 127), _lib.PREC_FP32_BLOCKSUM, 2, 2), ((120, 132, 124), _lib.PREC_FP32_BLOCKSUM, 2, None),
+    ((112, 136, 159), _lib.PREC_FP32_KAHAN, 1, 1), ((113, 135, 156), _lib.PREC_FP32_KAHAN, 2, None),
+    ((167, 119, 131), _lib.PREC_FP32_KAHAN, 4, 0)])
+def test_one_step_launches_give_the_bits_of_the_blocked_ones(n, prec, tb, layer):
+    """Grids that fill L2 without the forcing (one step per launch, partial sums over as many steps
+    as the depth) but not with it (blocked launches): with a forcing of zeros the forced map is the
+    homogeneous one, bit for bit."""
+    om = np.linspace(30.0, 60.0, 4)
+    length = tuple(k / n[0] for k in n)
+    rng = np.random.default_rng(4)
+    v = np.zeros((4, n[2] + 1, n[1] + 1, n[0] + 1))
+    v[:, 1:-1, 1:-1, 1:-1] = rng.normal(size=(4, n[2] - 1, n[1] - 1, n[0] - 1))
+    v = torch.from_numpy(v).cuda()
+    kw = {} if layer is None else dict(c_lo=1.0, c_hi=1.4, interface=0.37, layer_axis=layer)
+    s = M.Solver(n, length, om, torch.zeros_like(v), n_p=1, time_block=tb, precision=prec,
+                 filter_mode=_lib.FILTER_TRADITIONAL, **kw)
+    out = []
+    for forced in (True, False):
+        o = torch.full_like(v, float("nan"))
+        s.apply_Pi(v, o, forced=forced)
+        out.append(o.cpu().numpy())
+    s.close()
+    assert np.array_equal(out[0], out[1])
