@@ -1166,7 +1166,7 @@ def workload_config(wl, n_t):
             "omega_band": [10.0, 60.0], "gaussian_b": 400.0, "cfl": wl.cfl,
             "restart": RESTART, "tol": TOL,
             "precision": "fp64 interface, forcing and filter solve; wave levels and filter sums as "
-                         "64-bit integers (steps rounded to 2^-58 of the largest level)",
+                         "64-bit integers (steps rounded to about 2^-55 of the largest level)",
             "l2": "working set (forcing, accumulators, Krylov basis: > 1 GB) is larger than L2"}
 
 

@@ -56,7 +56,7 @@ typedef enum {
 enum { MFWH_FILTER_OPTIMIZED = 0, MFWH_FILTER_TRADITIONAL = 1, MFWH_FILTER_USER = 2 };
 /* Arithmetic of the wave solve.  FP64: wave levels, steps and the filter solve at least as accurate
    as in FP64.  Explicit steps in 2D with a constant or two-layer c advance 64-bit integers in
-   units of a quantum of 2^-58 to 2^-54 of the largest level, which follows that level, over the
+   units of a quantum of 2^-58 to 2^-51 of the largest level, which follows that level, over the
    whole range of double; beyond (infinities, NaN, magnitudes outside 1e-250 .. 1e250) they step
    in FP64.  The other explicit FP64 problems (3D, a c^2 field, grids with dt^2 c^2 / h^2 below
    2^-10, at least 1 or a multiple of 2^-24 along an axis, grids of very few rows or columns) keep

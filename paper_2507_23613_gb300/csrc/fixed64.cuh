@@ -2,10 +2,11 @@
 //
 // On sm_103a the FP64 pipe runs two lanes per SM and cycle, 1/64 of the FP32 rate, while integer
 // additions with carry run at about 64 lanes and 32 x 32 -> 64-bit multiply-adds at 50.  The
-// levels of a wave solve are kept as integers in units of a quantum 2^e that follows their largest
-// magnitude from launch to launch (57 or 58 bits are in use), so additions are exact and the only
-// rounding of a step is that of the product with dt^2 c^2 / h^2, to the nearest quantum: 2^-58 of
-// the largest level, against the several 2^-53 relative roundings of an FP64 step.  The functions
+// levels of a wave solve are kept as integers in units of a quantum 2^e that puts a bound of a
+// launch's levels just below 2^59 (fourth order 2^56) and follows it from launch to launch, so
+// additions are exact and the only rounding of a step is that of the product with dt^2 c^2 / h^2, to
+// the nearest quantum: about 2^-55 of the largest level, against the several 2^-53 relative roundings
+// of an FP64 step and the 2^-47 of its float-pair sums.  The functions
 // also compile for the host, where tests compare them with exact arithmetic.
 #pragma once
 
@@ -30,17 +31,16 @@ __device__ __forceinline__ int64_t fx_mac(int64_t d, int64_t x, const FxCoef& A)
   return (int64_t)((uint64_t)d + p - A.half);
 }
 
-// Exact sums of products of two 64-bit factors.  A factor is two signed digits, hi 2^32 + lo; a sum
-// is kept as s1 = sum of hi hi' and s2 = sum of hi lo' + lo hi' (three 32 x 32 + 64-bit
-// multiply-adds a term; lo lo', at most 2^62 and of either sign, is dropped) and stands for
-// s1 2^64 + s2 2^32.
+// Sums of products of two 64-bit factors of two signed digits each, hi 2^32 + lo: s1 = sum of hi hi'
+// and s2 = sum of hi lo' exactly (two 32 x 32 + 64-bit multiply-adds a term), which stand for
+// s1 2^64 + s2 2^32.  The kernel adds lo hi' in FP32, to 2^-24 of terms below 2^-28 of the largest;
+// lo lo', at most 2^62 and of either sign, is dropped.
 struct FxSum {
   int64_t s1, s2;
 };
-__device__ __forceinline__ void fx_madd(FxSum& s, int ahi, int alo, int bhi, int blo) {
-  s.s1 += (int64_t)ahi * bhi;
-  s.s2 += (int64_t)ahi * blo;
-  s.s2 += (int64_t)alo * bhi;
+__device__ __forceinline__ void fx_madd(FxSum& s, int ahi, const int2& b) {
+  s.s1 += (int64_t)ahi * b.x;
+  s.s2 += (int64_t)ahi * b.y;
 }
 // v as two signed digits, for |v| < 2^62.
 __host__ __device__ __forceinline__ void fx_digits(int64_t v, int& hi, int& lo) {

@@ -553,8 +553,7 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
               for (int j = 0; j < MG; ++j)
                 if (m0 + j < NF) {
                   const int e = s * NF + m0 + j;
-                  S[j].s1 += (int64_t)a.wh[e] * v.x;
-                  S[j].s2 += (int64_t)a.wh[e] * v.y;
+                  fx_madd(S[j], a.wh[e], v);
                   r[j] = fmaf(a.wl[e], vf, r[j]);
                 }
             };

@@ -32,7 +32,8 @@ void products(const int64_t* w, const int64_t* x, int n, int64_t* s) {
     int hi, lo;
     fx_digits(w[i], hi, lo);
     const int2 v = fx_level_digits(x[i]);
-    fx_madd(S, hi, lo, v.x, v.y);
+    fx_madd(S, hi, v);
+    S.s2 += (int64_t)lo * v.x;   // (in FP32 in the kernel)
   }
   s[0] = S.s1; s[1] = S.s2;
 }
