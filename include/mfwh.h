@@ -492,6 +492,12 @@ mfwh_status mfwh_set_wait_limit(mfwh_handle_t h, double seconds);
 mfwh_status mfwh_debug_bounds(mfwh_handle_t h, int64_t* count, int64_t* index, int64_t* extent,
                               int* line);
 
+/* Out-of-memory test (a debugging aid; the paper has none): of the workspace allocations that the
+ * calling thread's next calls make (handle buffers, Krylov basis, graph buffers), `after` succeed
+ * and the `count` that follow report that device memory has ended, without asking the device.
+ * (0, 0) ends it. */
+mfwh_status mfwh_debug_fail_allocations(int after, int count);
+
 /* Release the handle and its device workspace (waits for its stream). */
 void mfwh_destroy(mfwh_handle_t h);
 

@@ -151,6 +151,7 @@ _SIGNATURES = {
     "mfwh_mg_stats": (C.c_int, [C.c_void_p, C.POINTER(C.c_int64), C.POINTER(C.c_int64),
                                 C.POINTER(C.c_int64), C.POINTER(C.c_int), C.c_int]),
     "mfwh_set_wait_limit": (C.c_int, [C.c_void_p, C.c_double]),
+    "mfwh_debug_fail_allocations": (C.c_int, [C.c_int, C.c_int]),
     "mfwh_debug_bounds": (C.c_int, [C.c_void_p, C.POINTER(C.c_int64), C.POINTER(C.c_int64),
                                     C.POINTER(C.c_int64), C.POINTER(C.c_int)]),
     "mfwh_destroy": (None, [C.c_void_p]),

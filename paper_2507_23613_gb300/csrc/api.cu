@@ -818,31 +818,57 @@ mfwh_status residual_dev(mfwh_handle_t h, const double* v_dev, double* r_out) {
   return MFWH_OK;
 }
 
-// Leaves fixed point for the FP64 kernels, which need less memory.
-void fx_drop(mfwh_handle_t h) {
-  cudaStreamSynchronize(h->stream);
-  if (h->gstream) cudaStreamSynchronize(h->gstream);
+// mfwh_debug_fail_allocations: of this thread's coming workspace allocations, t_fail_after succeed
+// and t_fail_count then report that memory has ended.
+thread_local int t_fail_after = 0, t_fail_count = 0;
+
+cudaError_t device_alloc(void** p, size_t bytes) {
+  if (t_fail_count > 0 && t_fail_after-- <= 0) {
+    t_fail_after = 0;
+    --t_fail_count;
+    return cudaErrorMemoryAllocation;
+  }
+  return cudaMalloc(p, bytes);
+}
+
+// Leaves fixed point for the FP64 kernels, which need less memory.  They read the level arrays on
+// the boundary and write the interior alone, so what fixed point left there (integers, in longer
+// rows) is cleared.
+cudaError_t fx_drop(mfwh_handle_t h) {
+  cudaError_t e = cudaStreamSynchronize(h->stream);
+  if (e == cudaSuccess && h->gstream) e = cudaStreamSynchronize(h->gstream);
   for (auto& x : h->gexec) {   // captured with the old buffers
     if (x) cudaGraphExecDestroy(x);
     x = nullptr;
   }
+  for (double* w : {h->Wa, h->Wb, h->Wc2, h->Wp2})
+    if (e == cudaSuccess) e = cudaMemsetAsync(w, 0, sizeof(double) * h->PW, h->stream);
   if (h->fx_force) cudaFree(h->fx_force);
   h->fx_force = nullptr;
   h->plan.fixed = false;
   if (h->plan.precision == MFWH_PREC_FP64) {
     h->plan.time_block = h->depth64 = h->fx_else[0];
     h->plan.tile_shape = h->shape64 = h->fx_else[1];
+    Geom& g = h->geom;   // (an FP32 handle's FP32 arrays keep their rows)
+    g.syw = g.sy;
+    g.szw = g.sz;
+    g.wpoints = g.points;
   }
+  return e;
 }
 
 // Workspace of n values; where memory ends, a handle in fixed point gives up its own for it.
 template <typename T>
 cudaError_t alloc_workspace(mfwh_handle_t h, T** p, int64_t n) {
-  cudaError_t e = cudaMalloc(p, sizeof(T) * n);
-  if (e != cudaErrorMemoryAllocation || !h->fx_force) return e;
-  (void)cudaGetLastError();
-  fx_drop(h);
-  return cudaMalloc(p, sizeof(T) * n);
+  void* v = nullptr;
+  cudaError_t e = device_alloc(&v, sizeof(T) * n);
+  if (e == cudaErrorMemoryAllocation && h->fx_force) {
+    (void)cudaGetLastError();
+    e = fx_drop(h);
+    if (e == cudaSuccess) e = device_alloc(&v, sizeof(T) * n);
+  }
+  if (e == cudaSuccess) *p = static_cast<T*>(v);
+  return e;
 }
 
 mfwh_status ensure_basis(mfwh_handle_t h, int vectors) {
@@ -1174,19 +1200,23 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
               {&h->vec_b, h->N},
               {&h->vec_x, h->N}};
   for (auto& b : bufs) {
-    e = cudaMalloc(b.p, sizeof(double) * b.n);
+    void* v = nullptr;
+    e = device_alloc(&v, sizeof(double) * b.n);
     if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaMalloc (workspace)"));
+    *b.p = static_cast<double*>(v);
   }
   if (P.fixed) {
     const bool blocked = prob->time_block == 0 && h->nf <= 8 && P.order == 2;
     h->fx_else[0] = prob->time_block != 0 ? prob->time_block : (blocked ? 3 : 1);
     h->fx_else[1] = blocked && prob->tile_shape == 0 ? 5 : prob->tile_shape;
-    e = cudaMalloc(&h->fx_force, sizeof(int64_t) * h->PW * 8);
+    void* force = nullptr;
+    e = device_alloc(&force, sizeof(int64_t) * h->PW * 8);
+    h->fx_force = static_cast<int64_t*>(force);
     if (e == cudaErrorMemoryAllocation) {
       (void)cudaGetLastError();
-      e = cudaSuccess;
-      fx_drop(h);
+      e = fx_drop(h);
     }
+    if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaMalloc (fixed-point workspace)"));
   }
   if (P.fixed) {
     if (e == cudaSuccess)
@@ -1666,6 +1696,13 @@ mfwh_status mfwh_debug_bounds(mfwh_handle_t h, int64_t* count, int64_t* index, i
   if (index) *index = r.index;
   if (extent) *extent = r.extent;
   if (line) *line = r.line;
+  return MFWH_OK;
+}
+
+mfwh_status mfwh_debug_fail_allocations(int after, int count) {
+  if (after < 0 || count < 0) return fail(MFWH_ERR_INVALID_ARG, "negative count");
+  t_fail_after = after;
+  t_fail_count = count;
   return MFWH_OK;
 }
 

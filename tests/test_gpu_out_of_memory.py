@@ -1,0 +1,110 @@
+"""Where device memory ends (mfwh_debug_fail_allocations stands in for it), an FP64 2D handle in
+fixed point gives up its own workspace and goes on with the FP64 kernels.  What it computes then is
+what a handle computes that left fixed point before its first map, bit for bit."""
+
+import numpy as np
+import pytest
+
+import paper_2507_23613_gb300 as M
+from paper_2507_23613_gb300 import _lib, build
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    build.build()
+    yield _lib.load()
+    _lib.load().mfwh_debug_fail_allocations(0, 0)
+
+
+def solver(n, nf, **kw):
+    rng = np.random.default_rng(3)
+    om = np.linspace(6.0, 6.0 + 2.5 * (nf - 1), nf) + 0.37
+    f = torch.from_numpy(rng.normal(size=(nf, n[1] + 1, n[0] + 1))).cuda()
+    return M.Solver(n, (1.0, n[1] / n[0]), om, f, n_p=2 if nf > 4 else 1,
+                    filter_mode=_lib.FILTER_TRADITIONAL, **kw)
+
+
+def drop(s):
+    """The next workspace allocation fails once: the handle leaves fixed point."""
+    _lib.check(_lib.load().mfwh_debug_fail_allocations(0, 1))
+    s.set_graphs(True)
+    s.set_graphs(False)
+
+
+def results(s, v):
+    out = []
+    for forced in (True, False):
+        o = torch.full(v.shape, float("nan"), dtype=torch.float64, device="cuda")
+        s.apply_Pi(v, o, forced=forced)
+        out.append(o.cpu().numpy())
+    launches = s.last_timing()[1]
+    x = torch.zeros_like(v)
+    s.solve_gmres(x, restart=4, tol=0.0, max_iters=6, raise_on_error=False)
+    return out + [x.cpu().numpy()], launches
+
+
+# rows of 71 points (not a multiple of 32): the pipelined, the one-step and the fourth-order kernel
+@pytest.mark.parametrize("nf,order,depth", [(3, 2, 3), (12, 2, 1), (3, 4, 1)])
+@pytest.mark.parametrize("forced", [True, False])
+def test_maps_after_leaving_fixed_point(nf, order, depth, forced):
+    n = (70, 45)
+    v = torch.from_numpy(np.random.default_rng(4).normal(size=(nf, n[1] + 1, n[0] + 1))).cuda()
+    ref = solver(n, nf, order=order)
+    drop(ref)
+    want, launches = results(ref, v)
+    assert launches == -(-ref.setup["n_t"] // depth)   # (of the last map)
+    s = solver(n, nf, order=order)
+    o = torch.empty_like(v)
+    s.apply_Pi(v, o, forced=forced)
+    assert s.last_timing()[1] == -(-s.setup["n_t"] // (4 if order == 4 else 8))
+    fixed = o.cpu().numpy()
+    drop(s)
+    got, launches = results(s, v)
+    assert launches == -(-s.setup["n_t"] // depth)
+    for a, b in zip(got, want):
+        assert np.array_equal(a, b)
+    # and the two arithmetics agree
+    scale = np.abs(fixed).max()
+    assert np.abs(want[0 if forced else 1] - fixed).max() <= 1e-10 * scale
+
+
+def test_krylov_basis_that_does_not_fit():
+    """GMRES whose basis meets the end of memory after maps in fixed point."""
+    n, nf = (70, 45), 3
+    v = torch.from_numpy(np.random.default_rng(5).normal(size=(nf, n[1] + 1, n[0] + 1))).cuda()
+    xs = []
+    for first in (False, True):
+        s = solver(n, nf)
+        if first:
+            s.solve_fpi(v.clone(), 3)
+            _lib.check(_lib.load().mfwh_debug_fail_allocations(0, 1))
+        else:
+            drop(s)
+        x = torch.zeros_like(v)
+        s.solve_gmres(x, restart=4, tol=0.0, max_iters=6, raise_on_error=False)
+        xs.append(x.cpu().numpy())
+    assert np.array_equal(xs[0], xs[1])
+
+
+def test_refined_solve_that_does_not_fit():
+    """The FP64 residuals of an FP32 handle leave fixed point between two solves."""
+    n, nf = (70, 45), 3
+    xs = []
+    for first in (False, True):
+        s = solver(n, nf, precision=_lib.PREC_FP32_KAHAN)
+        if first:
+            x = torch.zeros((nf, n[1] + 1, n[0] + 1), dtype=torch.float64, device="cuda")
+            s.solve_relaxed(x, restart=4, inner_tol=1e-3, max_iters=4, target=1e-3, max_refinements=1,
+                            raise_on_error=False)
+        drop(s)
+        x = torch.zeros((nf, n[1] + 1, n[0] + 1), dtype=torch.float64, device="cuda")
+        s.solve_relaxed(x, restart=6, inner_tol=1e-6, max_iters=12, target=1e-9, max_refinements=2,
+                        raise_on_error=False)
+        xs.append(x.cpu().numpy())
+    assert np.isfinite(xs[0]).all() and np.array_equal(xs[0], xs[1])
