@@ -169,12 +169,19 @@ void launch_fx2d(int nf, const Geom& g, const FxArrays& in, const FxArrays& out,
 
 // ---- Programmatic dependent launch ---------------------------------------------------
 #ifdef __CUDACC__
-// A step kernel launched by launch_dependent starts where and when the launch before it leaves an
-// SM free; pdl_begin, before the first access to memory, waits for the end of that launch.  (The
-// arrays that the launch before writes must not be const __restrict__: such reads may move up.)
-__device__ __forceinline__ void pdl_begin() {
+// A step kernel launched by launch_dependent starts once every block of the launch before has called
+// pdl_release or ended; pdl_wait, before the first access to memory, waits for the end of that
+// launch.  (The arrays that the launch before writes must not be const __restrict__: such reads may
+// move up.)  Kernels of many small blocks release at their end: blocks that come while most of
+// the launch before still runs fill the places that happen to be free and then sit unevenly on the
+// SMs (k_step).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_begin() {
+  pdl_release();
+  pdl_wait();
 }
 template <typename... P, typename... A>
 inline void launch_dependent(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,

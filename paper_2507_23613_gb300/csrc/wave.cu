@@ -14,8 +14,11 @@
 // accumulators are float pairs updated on the FP32 pipe (fpair.cuh); k_last adds the
 // final term in FP64 and solves for V in FP64.
 //
-// k_step and k_last are dependent launches (launch_dependent): the gap between two steps was 2 us,
-// 5 % of a step on 129^3 (17.6 ms for a map of N_f = 4, now 16.4) and half of one on 33^3.
+// k_step and k_last are dependent launches (launch_dependent), released at the end of a step: us per
+// step as plain launches, released at the start and at the end, second order, N_f = 4: 33^3 6.4,
+// 4.9, 4.0; 49^3 7.5, 7.0, 5.4; 129^3 39.5, 37.2, 36.6; forced 41^3 8.4, 8.6, 5.8; fourth order 41^3
+// 10.4, 12.2, 7.9 (released at the start, the next step's blocks crowd the SMs that have room while
+// the others still work: grids of 3 to 6 blocks per SM lost up to 30 %).
 #include <cuda_runtime.h>
 
 #include "fpair.cuh"
@@ -158,7 +161,7 @@ template <int NF, int DIM, int ORDER, bool FIELD, bool FORCED>
 __global__ void __launch_bounds__(kBX * kBY)
 k_step(const double* Wc, double* __restrict__ Wp, const double* __restrict__ f,
        float2* __restrict__ q, const StepParams<NF> a, const Geom g) {
-  pdl_begin();
+  pdl_wait();
   const PointIndex x = point_index<DIM>(g);
   if (!x.interior) return;           // boundary values stay 0 (Dirichlet, g = 0)
   // index-checked build: the nearest neighbours along the outermost axis lie in the arrays
@@ -174,6 +177,7 @@ k_step(const double* Wc, double* __restrict__ Wp, const double* __restrict__ f,
     float2* qm = q + m * g.points + x.p;
     *qm = fpair_fma(a.wq_hi[m], a.wq_lo[m], xw.x, xw.y, *qm);
   }
+  pdl_release();
 }
 
 template <int NF, int DIM, int ORDER, bool FIELD>
