@@ -347,13 +347,12 @@ mfwh_status mfwh_solve_batch_graph(const mfwh_handle_t* handles, int count, int 
 
 /* Autotuner for the blocked wave kernels.  Times the first steps (at most 96) of a
  * homogeneous wave solve of prob on the current device for each candidate temporal depth and
- * tile shape (FP32, 2D: depths 4, 8, 16; FP64, 2D: (8, 3), which has no effect, for problems in
- * 64-bit integers, else depths 1 to 8 and their tile shapes; FP32, 3D: depths 1, 2, 4, only 1 for
- * grids that L2 holds; FP64 3D, fourth order and c^2 fields: depth 1), keeping the
- * fastest:
- * *time_block and *tile_shape receive it, *ms_per_step
- * (may be NULL) its time per leapfrog step.  Results are cached per device, grid, number of
- * frequencies and precision for the life of the process.  Allocates (and frees) one handle's
+ * tile shape (FP32, 2D: depths 4, 8, 16; FP64, 2D: depths 1 to 8 and their tile shapes, but for
+ * problems in 64-bit integers, which neither concerns, only the FP64 kernels' default; FP32, 3D:
+ * depths 1, 2, 4, only 1 for grids that L2 holds; FP64 3D, fourth order and c^2 fields: depth 1),
+ * keeping the fastest: *time_block and *tile_shape receive it, *ms_per_step (may be NULL) its time
+ * per leapfrog step.  Results are cached for the life of the process per device, grid, number of
+ * frequencies, precision, order, kind of c^2 and arithmetic (64-bit integers or not).  Allocates (and frees) one handle's
  * workspace per candidate on the given stream; synchronous.  Implicit time stepping has no
  * candidates: depth 1, tile shape 0 and *ms_per_step = 0 without timing. */
 mfwh_status mfwh_autotune(const mfwh_problem* prob, void* stream, int* time_block,

@@ -2317,11 +2317,11 @@ mfwh_status mfwh_autotune(const mfwh_problem* prob, void* stream, int* time_bloc
   }
   int dev = 0;
   CK(cudaGetDevice(&dev));
-  using Key = std::tuple<int, int, int64_t, int64_t, int64_t, int, int, int>;
+  using Key = std::tuple<int, int, int64_t, int64_t, int64_t, int, int, int, int, bool>;
   static std::mutex mu;
   static std::map<Key, std::tuple<int, int, double>> cache;
   const Key key{dev, P.dim, P.n[0], P.n[1], P.dim == 3 ? P.n[2] : 0, P.s.nf, P.precision,
-                P.c2_field ? 1 : 0};
+                P.c2_field ? 1 : 0, P.order, P.fixed};   // what selects kernels and candidates
   {
     std::lock_guard<std::mutex> lk(mu);
     auto it = cache.find(key);
@@ -2344,9 +2344,11 @@ mfwh_status mfwh_autotune(const mfwh_problem* prob, void* stream, int* time_bloc
     else
       cand = {{1, 0}, {2, 0}, {4, 0}};
   } else if (P.precision == MFWH_PREC_FP64) {
-    cand = P.fixed ? std::vector<std::pair<int, int>>{{8, 3}}   // (no effect)
-                   : std::vector<std::pair<int, int>>{{1, 0}, {2, 5}, {3, 5}, {4, 5}, {4, 4}, {4, 3},
-                                                      {8, 3}};
+    // (fixed point runs whatever these say: the FP64 kernels' default, for a handle that leaves it)
+    if (P.fixed)
+      cand = {P.s.nf <= 8 ? std::pair<int, int>{3, 5} : std::pair<int, int>{1, 0}};
+    else
+      cand = {{1, 0}, {2, 5}, {3, 5}, {4, 5}, {4, 4}, {4, 3}, {8, 3}};
   } else {
     cand = {{4, 0}, {8, 0}, {16, 0}};
   }
