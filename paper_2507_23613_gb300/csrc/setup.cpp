@@ -447,15 +447,16 @@ mfwh_status plan_problem(const mfwh_problem* p, Plan* out, double c2_field_max) 
   }
   const double dt = s.dt;
 
-  // FP64 wave solves in 64-bit fixed point (wave_fx.cu): 2D, constant or two-layer c,
-  // explicit steps, coefficients kappa c^2 / h^2 (fourth order: / 12) that a 64-bit fraction holds exactly (a double
-  // of at least 2^-10 has no bit below 2^-62, half of it none below 2^-63) and whose products do not
-  // end in exact halves often (not a multiple of 2^-24: these round up, and a bias of the
-  // increments grows with the square of the steps), and a grid that tiles of 48 x 32 points do not
-  // pad to more than twice its size and a few tiles.
+  // FP64 wave solves in 64-bit fixed point (wave_fx.cu): 2D, constant or two-layer c, explicit
+  // steps, coefficients kappa c^2 / h^2 (fourth order: / 12) that a 64-bit fraction holds exactly (a
+  // double of at least 2^-10 has no bit below 2^-62, half of it none below 2^-63) and whose products
+  // do not end in exact halves often (not a multiple of 2^-24: these round up, and a bias of the
+  // increments grows with the square of the steps), a grid that tiles of 48 x 32 points do not pad
+  // to more than twice its size and a few tiles, and more than two launches of steps (a map's three
+  // launches before them cost a 3^2 grid of 10 steps 35 us against 28).
   if (!implicit && !field && P.dim == 2) {
     const int64_t padded = ((P.n[0] + 48) / 48 * 48) * ((P.n[1] + 32) / 32 * 32);
-    P.fixed = padded <= 2 * s.points + 65536;
+    P.fixed = padded <= 2 * s.points + 65536 && n_t >= 24;
     for (int a = 0; a < 2; ++a)
       for (double c2 : {P.c2_lo, P.c2_hi}) {
         const double k = dt * dt * c2 / (s.h[a] * s.h[a]) / (P.order == 4 ? 12.0 : 1.0);
