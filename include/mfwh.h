@@ -249,7 +249,10 @@ mfwh_status mfwh_set_forcing(mfwh_handle_t h, const double* forcing);
  * v_in, v_out: device [nf][points]; they may alias.  Asynchronous on the stream. */
 mfwh_status mfwh_apply_Pi(mfwh_handle_t h, const double* v_in, double* v_out, int forced);
 
-/* Fixed-point iteration of Algorithm 1: v <- Pi(v), `iters` times.
+/* Fixed-point iteration of Algorithm 1: v <- Pi(v), `iters` times.  From 3 iterations on, problems
+ * whose wave solves run in 64-bit integers (see the precision) form b = Pi(0) once and iterate
+ * v <- S v + b, the same map (one wave solve more, each of a fraction of the time); the last bits
+ * then differ from those of as many single maps.  Graph mode replays either form.
  * v: host or device [nf][points], in: V^0, out: V^iters.  Synchronous. */
 mfwh_status mfwh_solve_fpi(mfwh_handle_t h, int iters, double* v);
 
