@@ -188,6 +188,8 @@ struct mfwh_handle_s {
   float* W32[4] = {};               // (W, D) pairs: W32[0], W32[1] and W32[2], W32[3]
   float* qs = nullptr;              // Kahan sums [nf][P]
   float* qc = nullptr;              // Kahan compensations [nf][P]
+  float* wq32 = nullptr;            // device copies of wq32_h and fc32_h
+  float* fc32 = nullptr;
   float* part32 = nullptr;          // FP32_BLOCKSUM in 3D on grids that L2 holds: partial sums [N]
   int l2_bytes = 0;                 // of the device
   std::vector<float> wq32_h, fc32_h;   // [(N_t + 1) * nf] w_{n,m}, [N_t * nf] kappa_n cos(omega~_m t^n)
@@ -308,6 +310,8 @@ mfwh_status apply_pi32(mfwh_handle_t h, const double* vin, double* vout, int for
     a.first_hi = first_hi;
     a.wq_host = h->wq32_h.data();
     a.fc_host = h->fc32_h.data();
+    a.wq = h->wq32;
+    a.fc = h->fc32;
     a.binv = h->sh.binv;
     a.emat = h->sh.emat;
     a.has_e = h->sh.has_e;
@@ -1257,7 +1261,8 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
       float** p;
       int64_t n;
     } fb[] = {{&h->f32, h->PW * h->nf}, {&h->W32[0], h->PW}, {&h->W32[1], h->PW}, {&h->W32[2], h->PW},
-              {&h->W32[3], h->PW}, {&h->qs, h->N}, {&h->qc, h->N}};
+              {&h->W32[3], h->PW}, {&h->qs, h->N}, {&h->qc, h->N},
+              {&h->wq32, (int64_t)h->wq32_h.size()}, {&h->fc32, (int64_t)h->fc32_h.size()}};
     for (auto& b : fb) {
       e = alloc_workspace(h, b.p, std::max<int64_t>(b.n, 1));
       if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaMalloc (FP32 workspace)"));
@@ -1271,6 +1276,12 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
     }
     for (int i = 0; i < 4 && e == cudaSuccess; ++i)
       e = cudaMemsetAsync(h->W32[i], 0, sizeof(float) * h->PW, h->stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(h->wq32, h->wq32_h.data(), sizeof(float) * h->wq32_h.size(),
+                          cudaMemcpyHostToDevice, h->stream);
+    if (e == cudaSuccess && !h->fc32_h.empty())
+      e = cudaMemcpyAsync(h->fc32, h->fc32_h.data(), sizeof(float) * h->fc32_h.size(),
+                          cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cleanup(cuda_fail(e, "initialising FP32 workspace"));
   }
@@ -1743,7 +1754,8 @@ void mfwh_destroy(mfwh_handle_t h) {
   if (h->d_bar) cudaFree(h->d_bar);
   if (h->d_mgc) cudaFree(h->d_mgc);
   delete h->imp;
-  float* fbufs[] = {h->f32, h->W32[0], h->W32[1], h->W32[2], h->W32[3], h->qs, h->qc, h->part32};
+  float* fbufs[] = {h->f32, h->W32[0], h->W32[1], h->W32[2], h->W32[3], h->qs, h->qc, h->part32,
+                    h->wq32, h->fc32};
   for (float* b : fbufs)
     if (b) cudaFree(b);
   if (h->pinned) cudaFreeHost(h->pinned);

@@ -218,6 +218,8 @@ struct TB32Host {
   Coef32 reg_lo, reg_hi, first_lo, first_hi;
   const float* wq_host;    // [(N_t + 1) * nf] (a launch's weights travel as parameters)
   const float* fc_host;    // [N_t * nf]
+  const float* wq;         // the same on the device (small 2D grids)
+  const float* fc;
   const double* binv;      // host [MFWH_MAX_NF * MFWH_MAX_NF], row-major, leading dim 16 (C)
   const double* emat;      // host, same layout (E of the explicit filter)
   int has_e;

@@ -16,9 +16,10 @@
 // q_m = s_m - c_m.  The filter solve V = B^{-1} q (eq. waveHoltzMatrixIteration)
 // and everything after it are FP64.
 //
-// Three kernels advance the scheme:
+// Four kernels advance the scheme:
 //  * k_tb2d32: 2D, T steps per launch on overlapped tiles whose points, halo included, live
 //    in the registers of one CTA for all T steps;
+//  * k_ring2d32: the same on smaller tiles in shared memory, for grids of few tiles;
 //  * k_tb3d32: the same in 3D with T = 2 or 4;
 //  * k_step32 / k_last32: one step per launch, 2D or 3D, second- or fourth-order L_h.
 // All are dependent launches (launch_dependent): one step on 33^3, N_f = 2, took 4.3 us, now 2.6.
@@ -28,6 +29,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
@@ -267,8 +269,8 @@ k_last32(const float* W, const float* D, const float* __restrict__ f,
 
 // ---- temporally blocked 2D kernel ----------------------------------------------
 //
-// One CTA per SM (16 warps) holds an extended tile of 128 x 64 points in registers, W and D of
-// 4 x 4 points per thread: lane l has columns 4l .. 4l + 3, warp w rows 4w .. 4w + 3.  Every step
+// One CTA per SM (16 warps) holds an extended tile of 128 x 64 points (fewer rows where the grid
+// would leave SMs idle: rt_warps) in registers, W and D of 4 x 4 points per thread: lane l has columns 4l .. 4l + 3, warp w rows 4w .. 4w + 3.  Every step
 // updates all of them (the outermost ring of valid values shrinks by one point a step, so after
 // T steps the (128 - 2T) x (64 - 2T) points in the middle are exact), except that a warp rests
 // once no later step reads its rows.  Left and right neighbours come from the thread itself or by
@@ -297,6 +299,7 @@ template <int NF, int T>
 struct RT32Args {
   Coef32 reg_lo, reg_hi, first_lo, first_hi;
   int n0, steps, forced, last, subtract;
+  int warps;          // that step: the tile has 4 warps rows (k_tb2d32)
   float wq[T * NF];   // w_{n+1,m} of step s: [s * NF + m]
   float fc[T * NF];   // kappa_n cos(omega~_m t^n)
 };
@@ -315,11 +318,12 @@ k_tb2d32(const float* W_in, const float* D_in,
          const __grid_constant__ RT32Args<NF, T> a, const __grid_constant__ Last32Binv<NF> b,
          const Geom g) {
   pdl_begin();
-  constexpr int VX = kRtEX - 2 * T, VY = kRtEY - 2 * T;   // owned points
-  static_assert(T % 4 == 0 && VX > 0 && VY > 0, "owned points are whole 4 x 4 blocks");
+  constexpr int VX = kRtEX - 2 * T, VYM = kRtEY - 2 * T;   // owned columns, rows at most
+  static_assert(T % 4 == 0 && VX > 0 && VYM > 0, "owned points are whole 4 x 4 blocks");
+  const int VY = 4 * a.warps - 2 * T;                      // owned rows
   extern __shared__ __align__(16) float sm32[];
-  float* hist = sm32;                       // [T][VY][VX] owned values step by step
-  float* edge = sm32 + T * VX * VY;         // [2][warp][top, bottom][128] edge rows
+  float* hist = sm32;                       // [T][VYM][VX] owned values step by step
+  float* edge = sm32 + T * VX * VYM;        // [2][warp][top, bottom][128] edge rows
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t x0 = (int64_t)blockIdx.x * VX - T, y0 = (int64_t)blockIdx.y * VY - T;
   const int lx = 4 * lane, ly = 4 * warp;
@@ -332,7 +336,7 @@ k_tb2d32(const float* W_in, const float* D_in,
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int64_t y = gy + k;
-    const bool row = y >= 0 && y <= g.ny;
+    const bool row = warp < a.warps && y >= 0 && y <= g.ny;
     const int64_t base = y * g.syw + gx;
     if (row && gx >= 0 && gx + 3 <= g.nx) {
       const float4 v = *reinterpret_cast<const float4*>(W_in + base);
@@ -451,7 +455,7 @@ k_tb2d32(const float* W_in, const float* D_in,
         step_points(s, s & 1, std::false_type{}, std::false_type{});
       put_edges((s + 1) & 1);
       if (owner) {
-        float* h = hist + (size_t)s * VX * VY + (ly - T) * VX + lx - T;
+        float* h = hist + (size_t)s * VX * VYM + (ly - T) * VX + lx - T;
 #pragma unroll
         for (int k = 0; k < 4; ++k)
           *reinterpret_cast<float4*>(h + k * VX) =
@@ -499,10 +503,10 @@ k_tb2d32(const float* W_in, const float* D_in,
       };
       if (a.steps == T) {
 #pragma unroll
-        for (int s = 0; s < T; ++s) add(s, hist[s * VX * VY + i]);
+        for (int s = 0; s < T; ++s) add(s, hist[s * VX * VYM + i]);
       } else {
 #pragma unroll 1
-        for (int s = 0; s < a.steps; ++s) add(s, hist[s * VX * VY + i]);
+        for (int s = 0; s < a.steps; ++s) add(s, hist[s * VX * VYM + i]);
       }
       if constexpr (ACC == 1) {
 #pragma unroll
@@ -517,6 +521,233 @@ k_tb2d32(const float* W_in, const float* D_in,
       }
     } else {
       filter_solve_out<NF>(ks, kc, b, a.subtract, vsub, vout, p, g.points, in);
+    }
+  }
+}
+
+// ---- temporally blocked 2D kernel for grids of few tiles ------------------------------
+//
+// Where a grid has fewer tiles than the device has SMs, k_tb2d32 leaves a launch to a few CTAs, and
+// what it does for a tile's many points after and (forced) during the steps is a long chain of L2
+// latencies.  This kernel has tiles of 32 x 16 points (32 x 32 up to 4 frequencies), 512 threads: the
+// tile plus a halo of T points in shared memory, a thread's one or two points and their sums in
+// registers, the ring of the halo that later steps still read spread evenly over all threads.  It
+// stages nothing for the sums and has all of a point's f in flight at once, but issues about three
+// times the instructions per point-step, so larger grids are slower (ring_faster).  Per point the
+// operations are those of k_tb2d32 in the same order.  us per launch of 16 steps with Kahan sums, in
+// k_tb2d32 with 64 rows a tile, with the rows that rt_warps picks, and here: 129^2, N_f = 8,
+// homogeneous 42, 20, 18, forced 67, 46, 25; 257^2, N_f = 16, homogeneous 65, 32, 26, forced 121, 85,
+// 48.  (513^2, N_f = 6, homogeneous 25 there and 39 here.)
+constexpr int kRingX = 32, kRingRows = 16, kRingThreads = kRingX * kRingRows;
+constexpr int kRingNF = 4;   // frequencies from which it is used (tb32_launch)
+__host__ __device__ constexpr int ring_k(int nf) { return nf <= 4 ? 2 : 1; }   // rows of a thread
+
+struct RingArgs {
+  Coef32 reg_lo, reg_hi, first_lo, first_hi;
+  int n0, steps, forced, last, subtract;
+};
+
+template <int NF, int T>
+constexpr size_t ring_smem_bytes() {
+  return sizeof(float) *
+         (3 * (kRingX + 2 * T) * (kRingRows * ring_k(NF) + 2 * T) + 2 * T * NF + 2 * T);
+}
+
+template <int NF, int T, int ACC>
+__global__ void __launch_bounds__(kRingThreads, ACC == 0 || NF > 8 ? 1 : 2)
+k_ring2d32(const float* W_in, const float* D_in,
+           float* __restrict__ W_out, float* __restrict__ D_out, const float* __restrict__ f,
+           float* __restrict__ qs, float* __restrict__ qc, double* vout, const double* vsub,
+           const float* __restrict__ wq_table, const float* __restrict__ fc_table,
+           const __grid_constant__ RingArgs a, const __grid_constant__ Last32Binv<NF> b,
+           const Geom g) {
+  pdl_wait();
+  constexpr int K = ring_k(NF), BX = kRingX, BY = kRingRows * K;
+  constexpr int EX = BX + 2 * T, EY = BY + 2 * T, E = EX * EY;
+  extern __shared__ __align__(16) float sm32[];
+  float* Wc = sm32;          // W^n on the extended tile
+  float* Wn = sm32 + E;      // W^{n+1}
+  float* Dv = sm32 + 2 * E;  // D on the halo (the tile's own is in registers)
+  float* s_wq = sm32 + 3 * E;   // [T][NF] w_{n+1,m} and kappa_n cos(omega~_m t^n) of step s
+  float* s_fc = s_wq + T * NF;
+  unsigned* s_div = reinterpret_cast<unsigned*>(s_fc + T * NF);   // [T][2] divisors of radius r
+  const int tid = threadIdx.x, tx = tid % BX, ty = tid / BX;
+  const int64_t x0 = (int64_t)blockIdx.x * BX - T, y0 = (int64_t)blockIdx.y * BY - T;
+  auto local = [](int64_t v) { return v < -1 ? -1 : (v > 128 ? 128 : (int)v); };
+  // local bounds of the interior and of the grid; first local index of the upper layer
+  const int ilx = local(1 - x0), ihx = local(g.nx - 1 - x0);
+  const int ily = local(1 - y0), ihy = local(g.ny - 1 - y0);
+  const bool lay_x = g.layer_axis == 0;
+  const int thr = local(g.layer_split - (lay_x ? x0 : y0));
+  // points outside the grid are 0, and so is the padding of its rows
+  for (int e = tid; e < E / 4; e += kRingThreads) {
+    const int ly = e / (EX / 4), lx = 4 * (e % (EX / 4));
+    const int64_t x = x0 + lx, y = y0 + ly;
+    float4 w = make_float4(0.0f, 0.0f, 0.0f, 0.0f), d = w;
+    if (x >= 0 && x < g.syw && y >= 0 && y <= g.ny) {
+      w = *reinterpret_cast<const float4*>(W_in + y * g.syw + x);
+      if (D_in != nullptr) d = *reinterpret_cast<const float4*>(D_in + y * g.syw + x);
+    }
+    reinterpret_cast<float4*>(Wc)[e] = w;
+    reinterpret_cast<float4*>(Wn)[e] = w;   // (boundary values of the next level)
+    reinterpret_cast<float4*>(Dv)[e] = d;
+  }
+  for (int e = tid; e < a.steps * NF; e += kRingThreads) {
+    s_wq[e] = wq_table[(int64_t)(a.n0 + 1) * NF + e];
+    if (a.forced) s_fc[e] = fc_table[(int64_t)a.n0 * NF + e];
+  }
+  // e / d = umulhi(e, 2^32 / d rounded up), exact for e < 2^16 and 2 <= d < 2^7
+  if (tid < T) {
+    s_div[2 * tid] = 0xFFFFFFFFu / (unsigned)(BX + 2 * tid) + 1u;
+    s_div[2 * tid + 1] = tid > 0 ? 0xFFFFFFFFu / (unsigned)(2 * tid) + 1u : 0u;
+  }
+  // every point that is updated is interior, with one c^2
+  const bool simple = ilx <= 1 && ihx >= EX - 2 && ily <= 1 && ihy >= EY - 2 &&
+                      (thr <= 0 || thr >= (lay_x ? EX : EY));
+  const int lxo = T + tx, lyo = T + ty * K;   // this thread's first point
+  const int64_t p0 = (y0 + lyo) * g.sy + x0 + lxo, f0 = (y0 + lyo) * g.syw + x0 + lxo;
+  bool own[K], up[K];
+  float wr[K], dr[K], ks[K][NF], kc[K][NF], part[K][NF];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    own[k] = lxo >= ilx && lxo <= ihx && lyo + k >= ily && lyo + k <= ihy;
+    up[k] = (lay_x ? lxo : lyo + k) >= thr;
+#pragma unroll
+    for (int m = 0; m < NF; ++m) {
+      part[k][m] = 0.0f;
+      const int64_t o = m * g.points + p0 + k * g.sy;
+      if (ACC == 0) {
+        ks[k][m] = own[k] ? qs[o] : 0.0f;
+        kc[k][m] = own[k] ? qc[o] : 0.0f;
+      } else if (own[k] && (tid & 7) == 0) {   // read at the end of the launch
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(qs + o));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(qc + o));
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    wr[k] = Wc[(lyo + k) * EX + lxo];
+    dr[k] = Dv[(lyo + k) * EX + lxo];
+  }
+  // PLAIN: homogeneous launches of such CTAs; the values are the same.
+  auto run_steps = [&](auto plain_c) {
+    constexpr bool PLAIN = decltype(plain_c)::value;
+    const int forced = PLAIN ? 0 : a.forced;
+    for (int s = 0; s < a.steps; ++s) {
+      const int r = a.steps - 1 - s;   // later steps read the tile grown by r
+      const bool first = a.n0 + s == 0;
+      const Coef32 lo = first ? a.first_lo : a.reg_lo, hi = first ? a.first_hi : a.reg_hi;
+      const Coef32 one = thr <= 0 ? hi : lo;
+      const float* fc = s_fc + s * NF;
+      constexpr int R = ACC == 0 && NF > 12 ? NF : 1;   // (in registers where that spares loads)
+      float wr_q[R];
+#pragma unroll
+      for (int m = 0; m < R; ++m) wr_q[m] = s_wq[s * NF + m];
+      auto wq = [&](int m) { return R > 1 ? wr_q[R > 1 ? m : 0] : s_wq[s * NF + m]; };
+      {
+        const float above = Wc[(lyo - 1) * EX + lxo], below = Wc[(lyo + K) * EX + lxo];
+        float wnew[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          const float w = wr[k];
+          wnew[k] = w;
+          if (!PLAIN && !own[k]) continue;   // boundary and outside points keep W = 0
+          const int l = (lyo + k) * EX + lxo;
+          const float wu = k == 0 ? above : wr[k > 0 ? k - 1 : 0];
+          const float wd = k == K - 1 ? below : wr[k < K - 1 ? k + 1 : k];
+          const Coef32 L = PLAIN ? one : (up[k] ? hi : lo);
+          const float inc =
+              increment<NF, 2>(L, (Wc[l - 1] - w) + (Wc[l + 1] - w), (wu - w) + (wd - w), 0.0f, fc,
+                               f, f0 + k * g.syw, g.wpoints, forced);
+          dr[k] = dr[k] + inc;
+          wnew[k] = w + dr[k];
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          wr[k] = wnew[k];
+          Wn[(lyo + k) * EX + lxo] = wnew[k];
+          if (!PLAIN && !own[k]) continue;
+#pragma unroll
+          for (int m = 0; m < NF; ++m) {
+            if (ACC == 0)
+              kahan_add(ks[k][m], kc[k][m], wq(m), wnew[k]);
+            else
+              part[k][m] = fmaf(wq(m), wnew[k], part[k][m]);
+          }
+        }
+      }
+      // The ring of radius r around the tile: first the 2 r rows of BX + 2 r points above and
+      // below it, then the BY rows of 2 r points at its sides.
+      const int RW = BX + 2 * r, top = 2 * r * RW, ring = top + 2 * r * BY;
+      const unsigned m_rw = s_div[2 * r], m_2r = s_div[2 * r + 1];
+      auto ring_pass = [&](auto simple_c) {
+        constexpr bool SIMPLE = decltype(simple_c)::value;
+        for (int e = tid; e < ring; e += kRingThreads) {
+          int lx, ly;
+          if (e < top) {
+            const int row = (int)__umulhi((unsigned)e, m_rw);
+            lx = T - r + (e - row * RW);
+            ly = row < r ? T - r + row : T + BY + row - r;
+          } else {
+            const int row = (int)__umulhi((unsigned)(e - top), m_2r), col = e - top - row * 2 * r;
+            ly = T + row;
+            lx = col < r ? T - r + col : T + BX + col - r;
+          }
+          if (!SIMPLE && (lx < ilx || lx > ihx || ly < ily || ly > ihy)) continue;
+          const int l = ly * EX + lx;
+          const float w = Wc[l];
+          const Coef32 L = SIMPLE ? one : ((lay_x ? lx : ly) >= thr ? hi : lo);
+          const float inc = increment<NF, 2>(L, (Wc[l - 1] - w) + (Wc[l + 1] - w),
+                                             (Wc[l - EX] - w) + (Wc[l + EX] - w), 0.0f, fc, f,
+                                             (y0 + ly) * g.syw + x0 + lx, g.wpoints, forced);
+          const float dn = Dv[l] + inc;
+          Dv[l] = dn;
+          Wn[l] = w + dn;
+        }
+      };
+      if (PLAIN || simple)
+        ring_pass(std::true_type{});
+      else
+        ring_pass(std::false_type{});
+      __syncthreads();
+      float* t = Wc;
+      Wc = Wn;
+      Wn = t;
+    }
+  };
+  if (simple && !a.forced)
+    run_steps(std::true_type{});
+  else
+    run_steps(std::false_type{});
+  pdl_release();
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int64_t p = p0 + k * g.sy;
+    if (ACC == 1 && own[k]) {
+#pragma unroll
+      for (int m = 0; m < NF; ++m) {
+        ks[k][m] = qs[m * g.points + p];
+        kc[k][m] = qc[m * g.points + p];
+        kahan_fold(ks[k][m], kc[k][m], part[k][m]);
+      }
+    }
+    if (!a.last) {
+      if (!own[k]) continue;
+      W_out[f0 + k * g.syw] = wr[k];
+      D_out[f0 + k * g.syw] = dr[k];
+#pragma unroll
+      for (int m = 0; m < NF; ++m) {
+        qs[m * g.points + p] = ks[k][m];
+        qc[m * g.points + p] = kc[k][m];
+      }
+    } else if (x0 + lxo <= g.nx && y0 + lyo + k <= g.ny) {
+      if (!own[k]) {
+#pragma unroll
+        for (int m = 0; m < NF; ++m) ks[k][m] = kc[k][m] = 0.0f;
+      }
+      filter_solve_out<NF>(ks[k], kc[k], b, a.subtract, vsub, vout, p, g.points, own[k]);
     }
   }
 }
@@ -862,18 +1093,68 @@ void init32_nf(const Geom& g, const double* v, float* W0, float* qs, float* qc, 
     k_init32<NF, 2><<<grid_of(g), dim3(kBX, kBY), 0, st>>>(v, W0, qs, qc, a, g);
 }
 
+// Step warps of k_tb2d32: a launch takes about as many rounds as the grid has tiles per SM, of a time
+// that grows with the tile's rows (step warps and, more with more frequencies, sums of the rows
+// owned).
+inline int rt_warps(const Geom& g, int nf, int T, int sms) {
+  const int64_t tx = (g.nx + kRtEX - 2 * T) / (kRtEX - 2 * T);
+  int best = kRtWarps;
+  double cost = 0.0;
+  for (int w = kRtWarps; w > T / 2; --w) {
+    const int vy = 4 * w - 2 * T;
+    const int64_t t = tx * ((g.ny + vy) / vy);
+    const double r = 0.5 * ((double)((t + sms - 1) / sms) + std::max(1.0, (double)t / sms));
+    const double c = r * (2.0 + w + 0.15 * nf * (w - T / 2));
+    if (w == kRtWarps || c < 0.95 * cost) {
+      best = w;
+      cost = c;
+    }
+  }
+  return best;
+}
+
+// Whether k_ring2d32 is the faster one: up to a number of 32 x 32 tiles per SM (of 152: 257^2 0.53,
+// 385^2 1.1, 449^2 1.5) that grows with the frequencies, more so forced and for shallow launches.
+// Measured on 16 grids of 65^2 to 1501^2, N_f 1 to 16, depths 4, 8, 16.
+inline bool ring_faster(const Geom& g, int nf, int T, bool kahan, int forced, int sms) {
+  const double r = (double)((g.nx + 32) / 32 * ((g.ny + 32) / 32)) / sms;
+  const double up_to = nf >= 14 ? 1.5 : 1.25;
+  if (T == 16) return forced ? r <= 1.0 && (nf >= 5 || kahan) : r <= 0.55 && nf >= (kahan ? 5 : 12);
+  if (T == 8)
+    return forced ? r <= (nf >= 5 || kahan ? up_to : 0.55) : nf >= 5 && r <= (nf >= 14 ? 1.5 : 0.55);
+  return nf >= 5 || kahan ? r <= up_to : forced && r <= 0.55;
+}
+
 template <int NF, int T, int ACC>
 void tb32_launch(const Geom& g, const float* W_in, const float* D_in, float* W_out, float* D_out,
                  const float* f, float* qs, float* qc, double* vout, const double* vsub,
                  const TB32Host& h, cudaStream_t st) {
   constexpr size_t smem = rt32_smem_bytes<T>();
-  static bool configured[64] = {};
+  static int sms[64] = {};   // SMs of the device; the attributes are set on first use
   int dev = 0;
   cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64 || !configured[dev]) {
+  int n = (dev >= 0 && dev < 64) ? sms[dev] : 0;
+  if (n == 0) {
     cudaFuncSetAttribute(k_tb2d32<NF, T, ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);
-    if (dev >= 0 && dev < 64) configured[dev] = true;
+    if constexpr (NF >= kRingNF)
+      cudaFuncSetAttribute(k_ring2d32<NF, T, ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)ring_smem_bytes<NF, T>());
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
+      n = 1;
+    if (dev >= 0 && dev < 64) sms[dev] = n;
+  }
+  const Last32Binv<NF> b = binv_args<NF>(h.binv, h.emat, h.has_e, h.vprev);
+  if constexpr (NF >= kRingNF) {
+    constexpr int BY = kRingRows * ring_k(NF);
+    const dim3 grid((unsigned)((g.nx + kRingX) / kRingX), (unsigned)((g.ny + BY) / BY));
+    if (ring_faster(g, NF, T, ACC == 0, h.forced, n)) {
+      const RingArgs r{h.reg_lo, h.reg_hi, h.first_lo, h.first_hi, h.n0, h.steps, h.forced, h.last,
+                       vsub != nullptr};
+      launch_dependent(k_ring2d32<NF, T, ACC>, grid, dim3(kRingThreads), ring_smem_bytes<NF, T>(), st,
+                       W_in, D_in, W_out, D_out, f, qs, qc, vout, vsub, h.wq, h.fc, r, b, g);
+      return;
+    }
   }
   RT32Args<NF, T> a;
   a.reg_lo = h.reg_lo;
@@ -885,13 +1166,14 @@ void tb32_launch(const Geom& g, const float* W_in, const float* D_in, float* W_o
   a.forced = h.forced;
   a.last = h.last;
   a.subtract = vsub != nullptr;
+  a.warps = rt_warps(g, NF, T, n);
   for (int s = 0; s < T; ++s)
     for (int m = 0; m < NF; ++m) {
       a.wq[s * NF + m] = s < h.steps ? h.wq_host[(size_t)(h.n0 + s + 1) * NF + m] : 0.0f;
       a.fc[s * NF + m] = s < h.steps && h.forced ? h.fc_host[(size_t)(h.n0 + s) * NF + m] : 0.0f;
     }
-  const Last32Binv<NF> b = binv_args<NF>(h.binv, h.emat, h.has_e, h.vprev);
-  constexpr int VX = kRtEX - 2 * T, VY = kRtEY - 2 * T;
+  constexpr int VX = kRtEX - 2 * T;
+  const int VY = 4 * a.warps - 2 * T;
   const dim3 grid((unsigned)((g.nx + VX) / VX), (unsigned)((g.ny + VY) / VY));
   launch_dependent(k_tb2d32<NF, T, ACC>, grid, dim3(kRtThreads), smem, st, W_in, D_in, W_out, D_out, f, qs, qc, vout,
                                                        vsub, a, b, g);
@@ -911,9 +1193,9 @@ template <int NF>
 void tb32_nf(const Geom& g, const float* W_in, const float* D_in, float* W_out, float* D_out,
              const float* f, float* qs, float* qc, double* vout, const double* vsub,
              const TB32Host& h, cudaStream_t st) {
-  // Depth 4 runs on the depth-8 instantiation: a launch of at most 4 steps only needs the
-  // inner 4 points of its 8-point halo, and the arithmetic per point is the same.
-  if (h.depth <= 8)
+  if (h.depth <= 4)
+    tb32_acc<NF, 4>(g, W_in, D_in, W_out, D_out, f, qs, qc, vout, vsub, h, st);
+  else if (h.depth <= 8)
     tb32_acc<NF, 8>(g, W_in, D_in, W_out, D_out, f, qs, qc, vout, vsub, h, st);
   else
     tb32_acc<NF, 16>(g, W_in, D_in, W_out, D_out, f, qs, qc, vout, vsub, h, st);
