@@ -1138,16 +1138,30 @@ mfwh_status mfwh_opt_parameters(int nf, const double* omega, int n_p, int n_t, i
   return optimise_parameters(nf, omega, n_p, n_t, n_delta, c_delta, params_out, lam_max, n_lambda);
 }
 
-mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* out) {
-  Range range("mfwh: create");
-  if (!out) return fail(MFWH_ERR_INVALID_ARG, "null output");
-  *out = nullptr;
+// The FP64 kernels' time_block and tile_shape for a 2D problem that fixed point would take.
+static void fp64_choice(const mfwh_problem* prob, const Plan& P, int out[2]) {
+  const bool blocked = prob->time_block == 0 && P.s.nf <= 8 && P.order == 2;
+  out[0] = prob->time_block != 0 ? prob->time_block : (blocked ? 3 : 1);
+  out[1] = blocked && prob->tile_shape == 0 ? 5 : prob->tile_shape;
+}
+
+// compact: without the workspace that is there for speed alone (fixed point, whole 128-byte rows).
+static mfwh_status create_handle(const mfwh_problem* prob, void* stream, bool compact,
+                                 mfwh_handle_t* out) {
   auto* h = new (std::nothrow) mfwh_handle_s();
   if (!h) return fail(MFWH_ERR_NOMEM, "host allocation failed");
   mfwh_status st = plan_with_field(prob, &h->plan);
   if (st != MFWH_OK) {
     delete h;
     return st;
+  }
+  if (h->plan.fixed) fp64_choice(prob, h->plan, h->fx_else);
+  if (compact && h->plan.fixed) {
+    h->plan.fixed = false;
+    if (h->plan.precision == MFWH_PREC_FP64) {
+      h->plan.time_block = h->fx_else[0];
+      h->plan.tile_shape = h->fx_else[1];
+    }
   }
   const Plan& P = h->plan;
   h->stream = static_cast<cudaStream_t>(stream);
@@ -1167,9 +1181,12 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
   g.layer_axis = P.layer_axis;
   g.layer_split = P.layer_split;
   g.order = P.order;
-  // wave levels in FP32 (and its forcing) and in fixed point: rows padded to 32 points
+  // Rows of the wave levels in FP32 (and its forcing) and in fixed point: whole 128-byte lines in 2D,
+  // where memory is short whole accesses of 16 bytes; in 3D accesses of 8 bytes (padding to 32
+  // points nearly doubled 33^3 and gave nothing: 257^3, N_f = 4, 162.5 and 162.7 us per step).
   const bool pad_w = P.precision != MFWH_PREC_FP64 || P.fixed;
-  g.syw = pad_w ? (g.nx + 1 + 31) / 32 * 32 : g.sy;
+  const int64_t pad = P.dim == 3 ? 2 : (compact ? 4 : 32);
+  g.syw = pad_w ? (g.nx + pad) / pad * pad : g.sy;
   g.szw = pad_w ? g.syw * (g.ny + 1) : g.sz;
   h->PW = pad_w ? g.szw * (g.dim == 3 ? g.nz + 1 : 1) : h->P;
   g.wpoints = h->PW;
@@ -1214,17 +1231,10 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
     *b.p = static_cast<double*>(v);
   }
   if (P.fixed) {
-    const bool blocked = prob->time_block == 0 && h->nf <= 8 && P.order == 2;
-    h->fx_else[0] = prob->time_block != 0 ? prob->time_block : (blocked ? 3 : 1);
-    h->fx_else[1] = blocked && prob->tile_shape == 0 ? 5 : prob->tile_shape;
     void* force = nullptr;
     e = device_alloc(&force, sizeof(int64_t) * h->PW * 8);
-    h->fx_force = static_cast<int64_t*>(force);
-    if (e == cudaErrorMemoryAllocation) {
-      (void)cudaGetLastError();
-      e = fx_drop(h);
-    }
     if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaMalloc (fixed-point workspace)"));
+    h->fx_force = static_cast<int64_t*>(force);
   }
   if (P.fixed) {
     if (e == cudaSuccess)
@@ -1264,8 +1274,10 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
               {&h->W32[3], h->PW}, {&h->qs, h->N}, {&h->qc, h->N},
               {&h->wq32, (int64_t)h->wq32_h.size()}, {&h->fc32, (int64_t)h->fc32_h.size()}};
     for (auto& b : fb) {
-      e = alloc_workspace(h, b.p, std::max<int64_t>(b.n, 1));
+      void* v = nullptr;
+      e = device_alloc(&v, sizeof(float) * std::max<int64_t>(b.n, 1));
       if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaMalloc (FP32 workspace)"));
+      *b.p = static_cast<float*>(v);
     }
     // (at most 1/3 of L2's size; without it the blocked kernels run)
     if (P.dim == 3 && P.order == 2 && P.precision == MFWH_PREC_FP32_BLOCKSUM && P.time_block > 1 &&
@@ -1444,6 +1456,18 @@ mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* o
   h->sh.vprev = nullptr;
   *out = h;
   return MFWH_OK;
+}
+
+mfwh_status mfwh_create(const mfwh_problem* prob, void* stream, mfwh_handle_t* out) {
+  Range range("mfwh: create");
+  if (!out) return fail(MFWH_ERR_INVALID_ARG, "null output");
+  *out = nullptr;
+  mfwh_status st = create_handle(prob, stream, false, out);
+  if (st == MFWH_ERR_NOMEM) {   // (a failed attempt has released what it had)
+    (void)cudaGetLastError();
+    st = create_handle(prob, stream, true, out);
+  }
+  return st;
 }
 
 mfwh_status mfwh_set_forcing(mfwh_handle_t h, const double* forcing) {

@@ -108,3 +108,70 @@ def test_refined_solve_that_does_not_fit():
                         raise_on_error=False)
         xs.append(x.cpu().numpy())
     assert np.isfinite(xs[0]).all() and np.array_equal(xs[0], xs[1])
+
+
+@pytest.mark.parametrize("after", [0, 3, 14])
+def test_creation_without_the_workspace_for_speed(after):
+    """Memory that ends during mfwh_create: the handle is made without fixed point (its 15th
+    allocation, the forcing of a launch, is the first that the FP64 kernels do without)."""
+    n, nf = (70, 45), 3
+    v = torch.from_numpy(np.random.default_rng(6).normal(size=(nf, n[1] + 1, n[0] + 1))).cuda()
+    ref = solver(n, nf)
+    drop(ref)
+    want, _ = results(ref, v)
+    _lib.check(_lib.load().mfwh_debug_fail_allocations(after, 1))
+    s = solver(n, nf)
+    _lib.check(_lib.load().mfwh_debug_fail_allocations(0, 0))
+    got, launches = results(s, v)
+    assert launches == -(-s.setup["n_t"] // 3)
+    for a, b in zip(got, want):
+        assert np.array_equal(a, b)
+    _lib.check(_lib.load().mfwh_debug_fail_allocations(after, 1000))   # and where nothing helps
+    with pytest.raises(_lib.MfwhError) as e:
+        solver(n, nf)
+    _lib.check(_lib.load().mfwh_debug_fail_allocations(0, 0))
+    assert e.value.status == _lib.ERR_NOMEM
+
+
+@pytest.mark.parametrize("n", [(70, 45), (3, 90), (191, 130)])
+@pytest.mark.parametrize("tb", [1, 4, 16])
+def test_fp32_rows_where_memory_is_short(n, tb):
+    """FP32 handles made at the second attempt have rows of whole 16-byte accesses: same bits."""
+    nf = 3
+    v = torch.from_numpy(np.random.default_rng(7).normal(size=(nf, n[1] + 1, n[0] + 1))).cuda()
+    out = []
+    for short in (False, True):
+        if short:
+            _lib.check(_lib.load().mfwh_debug_fail_allocations(2, 1))
+        s = solver(n, nf, precision=_lib.PREC_FP32_KAHAN, time_block=tb)
+        res = []
+        for forced in (True, False):
+            o = torch.full_like(v, float("nan"))
+            s.apply_Pi(v, o, forced=forced)
+            res.append(o.cpu().numpy())
+        out.append(res)
+        s.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+
+
+def cube(n, nf, tb, **kw):
+    rng = np.random.default_rng(9)
+    om = np.linspace(6.0, 6.0 + 2.5 * (nf - 1), nf)
+    f = torch.from_numpy(rng.normal(size=(nf,) + tuple(k + 1 for k in reversed(n)))).cuda()
+    return M.Solver(n, tuple(k / n[0] for k in n), om, f, n_p=2 if nf > 2 else 1, time_block=tb,
+                    filter_mode=_lib.FILTER_TRADITIONAL, precision=_lib.PREC_FP32_BLOCKSUM, **kw)
+
+
+def test_fp32_rows_of_3d_grids_are_hardly_padded():
+    """A 3D FP32 handle of 33 points a row takes about 33 / 32 of one of 32."""
+    used = []
+    for nx in (31, 32):
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        s = cube((nx, 200, 200), 4, 4)
+        torch.cuda.empty_cache()
+        before = torch.cuda.mem_get_info()[0]
+        s.close()
+        used.append(torch.cuda.mem_get_info()[0] - before)
+    assert used[0] > 0 and used[1] < 1.15 * used[0], used
