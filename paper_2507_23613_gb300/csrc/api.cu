@@ -191,7 +191,7 @@ struct mfwh_handle_s {
   float* wq32 = nullptr;            // device copies of wq32_h and fc32_h
   float* fc32 = nullptr;
   float* part32 = nullptr;          // FP32_BLOCKSUM in 3D on grids that L2 holds: partial sums [N]
-  int l2_bytes = 0;                 // of the device
+  int l2_bytes = 0, sms = 0;        // of the device
   std::vector<float> wq32_h, fc32_h;   // [(N_t + 1) * nf] w_{n,m}, [N_t * nf] kappa_n cos(omega~_m t^n)
   // implicit time stepping (MFWH_TIME_IMPLICIT)
   bool implicit = false;
@@ -269,6 +269,40 @@ void layer_coef32(const mfwh_handle_t h, double c2, double kappa, Coef32* L) {
   L->Az = (float)(k * h->inv_h2[2]);
 }
 
+// 3D FP32, second order: whether a launch per step is faster than launches of T = 2 or 4 steps with
+// partial sums, or (T = 1) than launches of 4 with a Kahan update at every step.  Both in us per step.
+//  * A launch per step is bound by L2, or by HBM once what it touches is beyond L2: W and D (16 bytes
+//    a point), per frequency 16 bytes of Kahan sums, or 12 (T = 2) or 10 (T = 4) with partial sums,
+//    and f.
+//  * A blocked launch by the time of a tile (of 56 x 8 x 12 or 60 x 12 x 16 points), which the
+//    loads and the latency of a tile's phases set, times the tiles an SM takes.
+// Forced tiles read all of f for every point stepped, 2 to 4 for each owned: with partial sums a
+// launch per step was faster on all of 57^3 .. 257^3, N_f 1 .. 16 (161^3, N_f = 6: 93 us against 122
+// at T = 2, 92 against 103 at T = 4).  The others, one step and blocked, in us: homogeneous Kahan
+// 89^3, N_f = 4, 10.4 and 14.9; 105^3, 8, 28.6 and 21.9; 129^3, 4, 29.4 and 28.8; 257^3, 4, 287 and
+// 163; 257^3, 1, 117 and 125; forced 129^3, 4, 42 and 47; 161^3, 6, 116 and 105; T = 4 105^3, 8, 26.3
+// and 21.4; 129^3, 4, 24.7 and 28.4; T = 2 145^3, 6, 63 and 69; 257^3, 6, 315 and 277.  The constants
+// are fits to 15 sizes and 8 frequency counts; where they pick the slower one it is by 7 % at most,
+// but for a few grids of one round of tiles.
+bool step3_faster(int64_t points, const int64_t* n, int nf, int T, int forced, int64_t l2, int sms) {
+  if (T > 1 && forced) return true;
+  const double touched = (double)points * (12 + nf * (T > 1 ? 12 : 8) + (forced ? 4 * nf : 0));
+  const double bytes =
+      (double)points * (16 + nf * (T == 1 ? 16 : (T == 2 ? 12 : 10)) + (forced ? 4 * nf : 0));
+  double one;
+  if (T == 1)
+    one = 2.5 + bytes / (touched <= 0.95 * l2 ? 6.6e6 : (forced ? 5.1e6 : 4.8e6));
+  else
+    one = 1.5 + bytes / (touched <= 1.1 * l2 ? (T == 2 ? 5.3e6 : 5.0e6) : (T == 2 ? 4.7e6 : 4.3e6));
+  const int64_t v[3] = {T == 2 ? 60 : 56, T == 2 ? 12 : 8, T == 2 ? 16 : 12};
+  double rounds = 1.0 / sms;
+  for (int a = 0; a < 3; ++a) rounds *= (double)((n[a] + v[a]) / v[a]);
+  const double tile = T == 2     ? 12.5 + (1.7 + 0.13 * nf) * nf
+                      : forced   ? 7.0 + (1.4 + 0.04 * nf) * nf
+                                 : 5.4 + (0.65 + 0.022 * nf) * nf;
+  return one < tile * (rounds <= 1.06 ? 1.05 : std::max(1.85, 0.9 * rounds));
+}
+
 // FP32 wave solve (increment form, Kahan filter sums), FP64 filter solve.
 mfwh_status apply_pi32(mfwh_handle_t h, const double* vin, double* vout, int forced,
                        const double* vsub) {
@@ -291,16 +325,14 @@ mfwh_status apply_pi32(mfwh_handle_t h, const double* vin, double* vout, int for
   layer_coef32(h, P.c2_hi, 0.5 * dt * dt, &first_hi);
   int launches = 0;
   // One step per launch (time_block 1, the 3D default) makes a Kahan update at every step, and
-  // the blocked kernels with such updates give the same bits: 3D runs 4 steps per launch then.
-  // While L2 holds what a step reads and writes (W, D, the sums, f), one step per launch is faster
-  // than either depth and runs instead, with partial sums over as many steps as the depth: 65^3, N_f
-  // = 8, 7.5 us per step against 9.6 (depth 4) and 15.3 (2); 17^3, N_f = 2, 2.5 against 3.9 and 6.3.
-  // At 129^3, N_f = 4 (94 MB) 29.1 against 28.1 and 44.1, at 161^3 (184 MB) 76 against 42 and 70.
-  const bool steps3 = P.dim == 3 && P.order == 2 &&
-                      h->P * (12 + 8 * nf + (h->part32 ? 4 * nf : 0) + (forced ? 4 * nf : 0)) <=
-                          h->l2_bytes &&
-                      (h->part32 || P.precision != MFWH_PREC_FP32_BLOCKSUM || P.time_block <= 1);
-  const bool kahan3 = P.dim == 3 && P.order == 2 && P.time_block <= 1;
+  // the blocked kernels with such updates give the same bits: in 3D any depth with Kahan updates runs
+  // 4 steps per launch or one, whichever is faster.  The partial sums of a depth are made by the
+  // blocked kernel of that depth or, with part32, by as many launches of a step.
+  const bool partial = P.precision == MFWH_PREC_FP32_BLOCKSUM && P.time_block > 1;
+  const bool kahan3 = P.dim == 3 && P.order == 2 && !partial;
+  const bool steps3 = P.dim == 3 && P.order == 2 && (!partial || h->part32) &&
+                      step3_faster(h->P, P.n, nf, partial ? P.time_block : 1, forced, h->l2_bytes,
+                                   h->sms);
   const int depth = steps3 ? 1 : (kahan3 ? 4 : P.time_block);
   if (depth > 1) {
     TB32Host a;
@@ -340,7 +372,7 @@ mfwh_status apply_pi32(mfwh_handle_t h, const double* vin, double* vout, int for
     a.forced = forced;
     a.group = 0;
     a.part = h->part32;
-    const int T = h->part32 ? P.time_block : 1;   // steps of a partial sum
+    const int T = partial && steps3 ? P.time_block : 1;   // steps of a partial sum
     float* Wc = h->W32[0];
     float* Wn = h->W32[2];
     float* D = h->W32[1];
@@ -845,10 +877,7 @@ cudaError_t device_alloc(void** p, size_t bytes) {
 cudaError_t fx_drop(mfwh_handle_t h) {
   cudaError_t e = cudaStreamSynchronize(h->stream);
   if (e == cudaSuccess && h->gstream) e = cudaStreamSynchronize(h->gstream);
-  for (auto& x : h->gexec) {   // captured with the old buffers
-    if (x) cudaGraphExecDestroy(x);
-    x = nullptr;
-  }
+  drop_graphs(h);   // captured with the old buffers
   for (double* w : {h->Wa, h->Wb, h->Wc2, h->Wp2})
     if (e == cudaSuccess) e = cudaMemsetAsync(w, 0, sizeof(double) * h->PW, h->stream);
   if (h->fx_force) cudaFree(h->fx_force);
@@ -865,14 +894,24 @@ cudaError_t fx_drop(mfwh_handle_t h) {
   return e;
 }
 
-// Workspace of n values; where memory ends, a handle in fixed point gives up its own for it.
+// Gives up the partial sums of steps: the blocked kernels run then.
+cudaError_t part_drop(mfwh_handle_t h) {
+  cudaError_t e = cudaStreamSynchronize(h->stream);
+  if (e == cudaSuccess && h->gstream) e = cudaStreamSynchronize(h->gstream);
+  drop_graphs(h);   // captured with the old buffer
+  cudaFree(h->part32);
+  h->part32 = nullptr;
+  return e;
+}
+
+// Workspace of n values; where memory ends, a handle gives up for it what it has for speed alone.
 template <typename T>
 cudaError_t alloc_workspace(mfwh_handle_t h, T** p, int64_t n) {
   void* v = nullptr;
   cudaError_t e = device_alloc(&v, sizeof(T) * n);
-  if (e == cudaErrorMemoryAllocation && h->fx_force) {
+  if (e == cudaErrorMemoryAllocation && (h->fx_force || h->part32)) {
     (void)cudaGetLastError();
-    e = fx_drop(h);
+    e = h->fx_force ? fx_drop(h) : part_drop(h);
     if (e == cudaSuccess) e = device_alloc(&v, sizeof(T) * n);
   }
   if (e == cudaSuccess) *p = static_cast<T*>(v);
@@ -1198,13 +1237,10 @@ static mfwh_status create_handle(const mfwh_problem* prob, void* stream, bool co
   cudaError_t e = cudaGetDevice(&h->device);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaGetDevice"));
   e = cudaDeviceGetAttribute(&h->l2_bytes, cudaDevAttrL2CacheSize, h->device);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaDeviceGetAttribute"));
-  if (P.fixed) {
-    int sms = 0;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-    if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaDeviceGetAttribute"));
-    h->fx_nw = fx_warps(g.nx, g.ny, sms);
-  }
+  if (P.fixed) h->fx_nw = fx_warps(g.nx, g.ny, h->sms);
   const int64_t tables = (int64_t)(P.s.n_t + 1) * h->nf;
   struct {
     double** p;
@@ -1279,12 +1315,14 @@ static mfwh_status create_handle(const mfwh_problem* prob, void* stream, bool co
       if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaMalloc (FP32 workspace)"));
       *b.p = static_cast<float*>(v);
     }
-    // (at most 1/3 of L2's size; without it the blocked kernels run)
-    if (P.dim == 3 && P.order == 2 && P.precision == MFWH_PREC_FP32_BLOCKSUM && P.time_block > 1 &&
-        h->P * (12 + 12 * nf) <= h->l2_bytes &&
-        cudaMalloc(&h->part32, sizeof(float) * h->N) != cudaSuccess) {
-      (void)cudaGetLastError();
-      h->part32 = nullptr;
+    // (without it the blocked kernels run)
+    if (P.dim == 3 && P.order == 2 && P.precision == MFWH_PREC_FP32_BLOCKSUM && P.time_block > 1) {
+      void* v = nullptr;
+      if (device_alloc(&v, sizeof(float) * h->N) != cudaSuccess) {
+        (void)cudaGetLastError();
+        v = nullptr;
+      }
+      h->part32 = static_cast<float*>(v);
     }
     for (int i = 0; i < 4 && e == cudaSuccess; ++i)
       e = cudaMemsetAsync(h->W32[i], 0, sizeof(float) * h->PW, h->stream);

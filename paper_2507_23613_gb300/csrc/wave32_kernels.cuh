@@ -23,6 +23,7 @@
 //  * k_tb3d32: the same in 3D with T = 2 or 4;
 //  * k_step32 / k_last32: one step per launch, 2D or 3D, second- or fourth-order L_h.
 // All are dependent launches (launch_dependent): one step on 33^3, N_f = 2, took 4.3 us, now 2.6.
+// (k_step32 releases the next one at its end, for the reason that k_step does.)
 // All perform the same FP32 operations per point in the same order, so their
 // results are bit-identical.
 #pragma once
@@ -183,12 +184,13 @@ __device__ __forceinline__ bool add_term(float& s, float& c, float& t, const Ste
 
 // W_out = W + D', D' = D + increment (D_out may alias D_in; W_out must not alias W_in); sums
 // updated in place.
-template <int NF, int DIM, int ORDER>
+// GROUP: partial sums (a.group not 0).
+template <int NF, int DIM, int ORDER, bool GROUP>
 __global__ void __launch_bounds__(kBX * kBY)
 k_step32(const float* W, const float* D_in, float* __restrict__ W_out, float* D_out,
          const float* __restrict__ f, float* __restrict__ qs, float* __restrict__ qc,
          const Step32Args<NF> a, const Geom g) {
-  pdl_begin();
+  pdl_wait();
   int64_t i, j, k, p;
   bool interior;
   index_of<DIM>(g, i, j, k, p, interior);
@@ -200,18 +202,26 @@ k_step32(const float* W, const float* D_in, float* __restrict__ W_out, float* D_
 #pragma unroll
   for (int m = 0; m < NF; ++m) {
     const int64_t o = m * g.points + p;
-    float s = 0.0f, c = 0.0f, t = 0.0f;
-    if (a.group == 0 || (a.group & 2)) {
-      s = qs[o];
-      c = qc[o];
-    }
-    if (add_term(s, c, t, a, m, o, wn)) {
+    if constexpr (GROUP) {
+      float s = 0.0f, c = 0.0f, t = 0.0f;
+      if (a.group & 2) {
+        s = qs[o];
+        c = qc[o];
+      }
+      if (add_term(s, c, t, a, m, o, wn)) {
+        qs[o] = s;
+        qc[o] = c;
+      } else {
+        a.part[o] = t;
+      }
+    } else {
+      float s = qs[o], c = qc[o];
+      kahan_add(s, c, a.wq[m], wn);
       qs[o] = s;
       qc[o] = c;
-    } else {
-      a.part[o] = t;
     }
   }
+  pdl_release();
 }
 
 template <int NF>
@@ -1052,13 +1062,16 @@ void step32_nf(const Geom& g, const float* W, const float* D_in, float* W_out, f
   const dim3 grid = grid_of(g), blk(kBX, kBY);
   if (g.order == 4) {
     if (g.dim == 3)
-      launch_dependent(k_step32<NF, 3, 4>, grid, blk, 0, st, W, D_in, W_out, D_out, f, qs, qc, a, g);
+      launch_dependent(k_step32<NF, 3, 4, false>, grid, blk, 0, st, W, D_in, W_out, D_out, f, qs, qc, a, g);
     else
-      launch_dependent(k_step32<NF, 2, 4>, grid, blk, 0, st, W, D_in, W_out, D_out, f, qs, qc, a, g);
+      launch_dependent(k_step32<NF, 2, 4, false>, grid, blk, 0, st, W, D_in, W_out, D_out, f, qs, qc, a, g);
   } else if (g.dim == 3) {
-    launch_dependent(k_step32<NF, 3, 2>, grid, blk, 0, st, W, D_in, W_out, D_out, f, qs, qc, a, g);
+    if (h.group)
+      launch_dependent(k_step32<NF, 3, 2, true>, grid, blk, 0, st, W, D_in, W_out, D_out, f, qs, qc, a, g);
+    else
+      launch_dependent(k_step32<NF, 3, 2, false>, grid, blk, 0, st, W, D_in, W_out, D_out, f, qs, qc, a, g);
   } else {
-    launch_dependent(k_step32<NF, 2, 2>, grid, blk, 0, st, W, D_in, W_out, D_out, f, qs, qc, a, g);
+    launch_dependent(k_step32<NF, 2, 2, false>, grid, blk, 0, st, W, D_in, W_out, D_out, f, qs, qc, a, g);
   }
 }
 

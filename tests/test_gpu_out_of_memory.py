@@ -163,6 +163,42 @@ def cube(n, nf, tb, **kw):
                     filter_mode=_lib.FILTER_TRADITIONAL, precision=_lib.PREC_FP32_BLOCKSUM, **kw)
 
 
+@pytest.mark.parametrize("n,nf,layer", [
+    ((2, 2, 2), 1, None), ((3, 30, 5), 2, 1), ((54, 7, 11), 2, None), ((55, 8, 12), 1, 0),
+    ((56, 9, 13), 3, 2), ((57, 11, 15), 2, None), ((60, 12, 16), 9, 1), ((61, 13, 17), 2, 2),
+    ((120, 33, 40), 4, 0)])
+@pytest.mark.parametrize("tb", [2, 4])
+def test_partial_sums_of_steps_and_of_blocked_launches(n, nf, layer, tb):
+    """The 3D FP32 sums over 2 or 4 steps: one step per launch with an array of partial sums, and,
+    where that array does not fit, the blocked kernel, at its tile edges: same bits."""
+    shape = (nf,) + tuple(k + 1 for k in reversed(n))
+    v = np.random.default_rng(10).normal(size=shape)
+    for a in (1, 2, 3):
+        v[tuple([slice(None)] * a + [[0, -1]])] = 0.0
+    v = torch.from_numpy(v).cuda()
+    kw = {} if layer is None else dict(c_lo=1.0, c_hi=1.4, interface=0.37 * n[layer] / n[0],
+                                       layer_axis=layer)
+
+    def maps(s):
+        out = []
+        for forced in (True, False):
+            o = torch.full_like(v, float("nan"))
+            s.apply_Pi(v, o, forced=forced)
+            out.append(o.cpu().numpy())
+        launches = s.last_timing()[1]   # (of the homogeneous map)
+        return out, launches
+    s = cube(n, nf, tb, **kw)
+    want, launches = maps(s)
+    n_t = s.setup["n_t"]
+    assert launches == n_t
+    # give the array up for a workspace that does not fit
+    drop(s)
+    got, launches = maps(s)
+    assert launches == -(-n_t // tb)
+    for a, b in zip(got, want):
+        assert np.array_equal(a, b)
+
+
 def test_fp32_rows_of_3d_grids_are_hardly_padded():
     """A 3D FP32 handle of 33 points a row takes about 33 / 32 of one of 32."""
     used = []
