@@ -14,6 +14,18 @@
 
 namespace mfwh {
 
+// Sums of levels.  Points beyond the valid ring of a tile are stepped too, on values that no bound
+// covers; they are never read, and wrap around.
+__host__ __device__ __forceinline__ int64_t fx_add(int64_t a, int64_t b) {
+  return (int64_t)((uint64_t)a + (uint64_t)b);
+}
+__host__ __device__ __forceinline__ int64_t fx_sub(int64_t a, int64_t b) {
+  return (int64_t)((uint64_t)a - (uint64_t)b);
+}
+__host__ __device__ __forceinline__ int64_t fx_mul15(int64_t a) {
+  return (int64_t)(15ull * (uint64_t)a);
+}
+
 // A coefficient A in [0, 1) as an even integer A 2^64 = hi 2^32 + lo, and half = A 2^63.
 struct FxCoef {
   uint32_t lo, hi;
@@ -45,7 +57,7 @@ __device__ __forceinline__ void fx_madd(FxSum& s, int ahi, const int2& b) {
 // v as two signed digits, for |v| < 2^62.
 __host__ __device__ __forceinline__ void fx_digits(int64_t v, int& hi, int& lo) {
   lo = (int)(uint32_t)(uint64_t)v;
-  hi = (int)((v - lo) >> 32);
+  hi = (int)(fx_sub(v, lo) >> 32);
 }
 // The digits of a level as a factor, of W less the constant 2^31 (which makes the low word's
 // excess over 2^31 a signed digit); the sums take the constant back once per launch.
@@ -72,7 +84,7 @@ __device__ __forceinline__ int64_t fx_from_bits(uint64_t bits, int e) {
 // x 2^k below 2^62.
 __device__ __forceinline__ int64_t fx_rescale(int64_t x, int k) {
   if (k >= 0) return (int64_t)((uint64_t)x << k);
-  return -k > 62 ? 0 : (x + (((int64_t)1 << (-k - 1)) - 1) + (x >> -k & 1)) >> -k;
+  return -k > 62 ? 0 : fx_add(x, (((int64_t)1 << (-k - 1)) - 1) + (x >> -k & 1)) >> -k;
 }
 
 }  // namespace mfwh

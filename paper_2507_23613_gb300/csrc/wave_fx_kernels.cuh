@@ -380,13 +380,13 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
         const longlong2 up = *edge_row(buf, wu, 3);
         const longlong2 bl = *edge_row(buf, wb, 0);
         const int64_t below[2] = {bl.x, bl.y};
-        int64_t dv[2] = {w[0][0] - up.x, w[0][1] - up.y};   // W - W_above of the current row
+        int64_t dv[2] = {fx_sub(w[0][0], up.x), fx_sub(w[0][1], up.y)};   // W - W_above of the row
         // fourth order: the same of the row above, and the second row below
         int64_t dv2[2] = {0, 0}, below2[2] = {0, 0};
         if constexpr (ORDER == 4) {
           const longlong2 up2 = *edge_row(buf, wu, 2), bl2 = *edge_row(buf, wb, 1);
-          dv2[0] = up.x - up2.x;
-          dv2[1] = up.y - up2.y;
+          dv2[0] = fx_sub(up.x, up2.x);
+          dv2[1] = fx_sub(up.y, up2.y);
           below2[0] = bl2.x;
           below2[1] = bl2.y;
         }
@@ -395,31 +395,32 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
           const int64_t left = __shfl_up_sync(0xffffffffu, w[k][1], 1);
           const int64_t right = __shfl_down_sync(0xffffffffu, w[k][0], 1);
           // W - W_left of columns 0 .. 2, fourth order also -1 and 3
-          const int64_t dx[3] = {w[k][0] - left, w[k][1] - w[k][0], right - w[k][1]};
+          const int64_t dx[3] = {fx_sub(w[k][0], left), fx_sub(w[k][1], w[k][0]),
+                                 fx_sub(right, w[k][1])};
           int64_t dxl = 0, dxr = 0;
           if constexpr (ORDER == 4) {
-            dxl = left - __shfl_up_sync(0xffffffffu, w[k][0], 1);
-            dxr = __shfl_down_sync(0xffffffffu, w[k][1], 1) - right;
+            dxl = fx_sub(left, __shfl_up_sync(0xffffffffu, w[k][0], 1));
+            dxr = fx_sub(__shfl_down_sync(0xffffffffu, w[k][1], 1), right);
           }
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
-            const int64_t dn = (k < 3 ? w[k < 3 ? k + 1 : 3][c] : below[c]) - w[k][c];
-            int64_t dxx = dx[c + 1] - dx[c], dyy = dn - dv[c];
+            const int64_t dn = fx_sub(k < 3 ? w[k < 3 ? k + 1 : 3][c] : below[c], w[k][c]);
+            int64_t dxx = fx_sub(dx[c + 1], dx[c]), dyy = fx_sub(dn, dv[c]);
             if constexpr (ORDER == 4) {
               // 16 times the first neighbours' sum of differences less the second neighbours', which
               // is dxx + (difference two to the right) - (two to the left)
               int64_t ra = c == 0 ? dx[2] : dxr, la = c == 0 ? dxl : dx[0];
               const int64_t w1 = k < 3 ? w[k < 3 ? k + 1 : 3][c] : below[c];
               const int64_t w2 = k < 2 ? w[k < 2 ? k + 2 : 3][c] : (k == 2 ? below[c] : below2[c]);
-              int64_t ba = w2 - w1, ab = dv2[c];
+              int64_t ba = fx_sub(w2, w1), ab = dv2[c];
               if (!PLAIN) {   // a ghost value beyond the boundary is minus the centre's
-                if (lx + c == ihx) ra = -w[k][c];
+                if (lx + c == ihx) ra = fx_sub(0, w[k][c]);
                 if (lx + c == ilx) la = w[k][c];
-                if (ly + k == ihy) ba = -w[k][c];
+                if (ly + k == ihy) ba = fx_sub(0, w[k][c]);
                 if (ly + k == ily) ab = w[k][c];
               }
-              dxx = 15 * dxx - (ra - la);
-              dyy = 15 * dyy - (ba - ab);
+              dxx = fx_sub(fx_mul15(dxx), fx_sub(ra, la));
+              dyy = fx_sub(fx_mul15(dyy), fx_sub(ba, ab));
               dv2[c] = dv[c];
             }
             dv[c] = dn;
@@ -427,13 +428,13 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
             const FxAxes& L = upper ? chi : clo;
             int64_t dnew = d[k][c];
             if constexpr (ISO) {
-              dnew = fx_mac(dnew, dxx + dyy, L.x);
+              dnew = fx_mac(dnew, fx_add(dxx, dyy), L.x);
             } else {
               dnew = fx_mac(dnew, dxx, L.x);
               dnew = fx_mac(dnew, dyy, L.y);
             }
-            if constexpr (FORCED) dnew -= fs[k][c];
-            int64_t wnew = w[k][c] + dnew;
+            if constexpr (FORCED) dnew = fx_sub(dnew, fs[k][c]);
+            int64_t wnew = fx_add(w[k][c], dnew);
             if (!PLAIN && !(in_mask >> (2 * k + c) & 1u)) dnew = wnew = 0;
             d[k][c] = dnew;
             w[k][c] = wnew;
@@ -574,7 +575,7 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
                   c = (int64_t)((uint64_t)(uint32_t)(c >> 32 >> q_new) << 32 |
                                 __funnelshift_r((uint32_t)c, (uint32_t)(c >> 32), q_new));
                 if (q_old != 0) v = fx_rescale(v, -q_old);
-                qi[(m0 + j) * kFxTile] = v + c;
+                qi[(m0 + j) * kFxTile] = fx_add(v, c);
               }
 #pragma unroll
             for (int j = 0; j < MG; ++j) qm[j] = qn[j];
