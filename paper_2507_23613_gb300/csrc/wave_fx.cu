@@ -205,8 +205,10 @@ k_fx_init(int64_t* W, int64_t* q, int nf, const FxInit a, const FxScale* scale,
   const double w = __longlong_as_double(W[i]);
   if (!scale->mode) W[i] = fx_from_bits((uint64_t)__double_as_longlong(w), state->e);
   if (x >= tiles_x * kFxTileX) return;
-  int64_t* qp = q + (y / vy * tiles_x + x / kFxTileX) * nf * kFxTile + y % vy * kFxTileX +
-                x % kFxTileX;
+  const int64_t o = (y / vy * tiles_x + x / kFxTileX) * nf * kFxTile + y % vy * kFxTileX +
+                    x % kFxTileX;
+  if (!MFWH_IDX(g.fault, o + (nf - 1) * kFxTile, (g.ny + vy) / vy * tiles_x * nf * kFxTile)) return;
+  int64_t* qp = q + o;
   for (int m = 0; m < nf; ++m) {
     const double t = a.w0[m] * w;
     qp[m * kFxTile] = scale->mode ? __double_as_longlong(t)

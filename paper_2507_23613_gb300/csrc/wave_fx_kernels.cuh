@@ -153,9 +153,12 @@ __device__ __noinline__ void fx_double_steps(double* A, double* B, const FxArray
   const int EY = 4 * a.warps;
   double* q = reinterpret_cast<double*>(qi);
   const int tid = threadIdx.x;
+  constexpr int kTileValues = kFxEX * kFxEY;   // of A and of B
   for (int e = tid; e < kFxEX * EY; e += blockDim.x) {
     const int64_t x = x0 + e % kFxEX, y = y0 + e / kFxEX;
-    const bool is = x >= 0 && x <= g.nx && y >= 0 && y <= g.ny;
+    const bool is = x >= 0 && x <= g.nx && y >= 0 && y <= g.ny &&
+                    MFWH_IDX(g.fault, y * g.syw + x, g.wpoints);
+    if (!MFWH_IDX(g.fault, e, kTileValues)) continue;
     A[e] = is ? __longlong_as_double(in.W[y * g.syw + x]) : 0.0;
     B[e] = (is && a.n0 > 0) ? __longlong_as_double(in.D[y * g.syw + x]) : 0.0;
   }
@@ -182,11 +185,13 @@ __device__ __noinline__ void fx_double_steps(double* A, double* B, const FxArray
         acc = fma(L.By, ty, acc);
       }
       const int64_t p = y * g.sy + x;
+      if (!MFWH_IDX(g.fault, p, g.points)) continue;
       if (a.forced)
         for (int m = 0; m < NF; ++m) acc = fma(-a.fc[s * NF + m], f[m * g.points + p], acc);
       B[e] = acc;
       if (lx >= T && lx < kFxEX - T && ly >= T && ly < EY - T) {
         double* qp = q + (ly - T) * kFxVX + lx - T;
+        if (!MFWH_IDX(g.fault, (ly - T) * kFxVX + lx - T, kFxTile)) continue;
         for (int m = 0; m < NF; ++m)
           qp[m * kFxTile] = fma(a.wd[s * NF + m], acc, qp[m * kFxTile]);
       }
@@ -201,6 +206,7 @@ __device__ __noinline__ void fx_double_steps(double* A, double* B, const FxArray
     const int lx = e % kFxEX, ly = e / kFxEX;
     const int64_t x = x0 + lx, y = y0 + ly;
     if (lx < T || lx >= kFxEX - T || ly < T || ly >= EY - T || x > g.nx || y > g.ny) continue;
+    if (!MFWH_IDX(g.fault, y * g.syw + x, g.wpoints)) continue;
     out.W[y * g.syw + x] = __double_as_longlong(A[e]);
     out.D[y * g.syw + x] = __double_as_longlong(B[e]);
   }
@@ -266,7 +272,7 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
       if (!a.last) continue;
       for (int i = tid; i < VX * VY; i += threads) {
         const int64_t x = x0 + T + i % VX, y = y0 + T + i / VX;
-        if (x > g.nx || y > g.ny) continue;
+        if (x > g.nx || y > g.ny || !MFWH_IDX(g.fault, y * g.sy + x, g.points)) continue;
         const bool is = x > 0 && x < g.nx && y > 0 && y < g.ny;
         fx_finish<NF>(qt + i, nullptr, is, vout, vsub, a, g.points, y * g.sy + x);
       }
@@ -345,9 +351,9 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
       }
       // the rows a warp shows its neighbours: second order 0 and 3, fourth order all
       auto edge_row = [&](int buf, int wp, int row) {
-        return reinterpret_cast<longlong2*>(
-                   edge + ((buf * kFxStep + wp) * ORDER + (ORDER == 4 ? row : row / 3)) * kFxEX) +
-               lane;
+        const int i = ((buf * kFxStep + wp) * ORDER + (ORDER == 4 ? row : row / 3)) * kFxEX;
+        const bool ok = MFWH_IDX(g.fault, i + 2 * lane + 1, 2 * kFxStep * ORDER * kFxEX);
+        return reinterpret_cast<longlong2*>(edge + (ok ? i : 0)) + lane;
       };
       auto put_edges = [&](int buf) {
 #pragma unroll
@@ -361,7 +367,8 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             longlong2 v = make_longlong2(0, 0);
-            if (in_mask >> (2 * k) & 3u)
+            if ((in_mask >> (2 * k) & 3u) &&
+                MFWH_IDX(g.fault, s * g.wpoints + base + k * g.syw + 1, 8 * g.wpoints))
               v = *reinterpret_cast<const longlong2*>(force + s * g.wpoints + base + k * g.syw);
             fs[k][0] = v.x;
             fs[k][1] = v.y;
@@ -462,9 +469,11 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
             put_edges((s + 1) & 1);
           }
           if (owner) {
-            int2* h = hist + s * kFxTile + (ly - T) * VX + lx - T;
+            const int i = s * kFxTile + (ly - T) * VX + lx - T;
+            int2* h = hist + i;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
+              if (!MFWH_IDX(g.fault, i + k * VX + 1, STEPS * kFxTile)) continue;
               const int2 p = fx_level_digits(w[k][0]), r2 = fx_level_digits(w[k][1]);
               *reinterpret_cast<int4*>(h + k * VX) = make_int4(p.x, p.y, r2.x, r2.y);
             }
@@ -521,10 +530,13 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
       int64_t* qt = q + (int64_t)tile * NF * kFxTile;
       // the sums are loaded one group of MG frequencies ahead
       int64_t qm[MG], qn[MG];
+      auto in_sums = [&](const int64_t* p) {
+        return MFWH_IDX(g.fault, p - q, (int64_t)tiles * NF * kFxTile);
+      };
       auto load = [&](const int64_t* p, int m0, int64_t* v) {
 #pragma unroll
         for (int j = 0; j < MG; ++j)
-          if (m0 + j < NF) v[j] = p[(m0 + j) * kFxTile];
+          if (m0 + j < NF && in_sums(p + (m0 + j) * kFxTile)) v[j] = p[(m0 + j) * kFxTile];
       };
       load(qt + t0, 0, qm);
       if (tile + (int)gridDim.x < tiles) prefetch(tile + (int)gridDim.x);
@@ -548,6 +560,7 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
                 r[j] = 0.0f;
               }
             auto add = [&](int s) {
+              if (!MFWH_IDX(g.fault, s * kFxTile + i, STEPS * kFxTile)) return;
               const int2 v = hist[s * kFxTile + i];
               const float vf = (float)v.x;
 #pragma unroll
@@ -575,7 +588,7 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
                   c = (int64_t)((uint64_t)(uint32_t)(c >> 32 >> q_new) << 32 |
                                 __funnelshift_r((uint32_t)c, (uint32_t)(c >> 32), q_new));
                 if (q_old != 0) v = fx_rescale(v, -q_old);
-                qi[(m0 + j) * kFxTile] = fx_add(v, c);
+                if (in_sums(qi + (m0 + j) * kFxTile)) qi[(m0 + j) * kFxTile] = fx_add(v, c);
               }
 #pragma unroll
             for (int j = 0; j < MG; ++j) qm[j] = qn[j];
@@ -586,7 +599,9 @@ k_fx2d(const FxArrays in, const FxArrays out, const double* __restrict__ f,
         const int64_t x1 = (int64_t)(tile % tiles_x) * VX, y1 = (int64_t)(tile / tiles_x) * VY;
         for (int i = t0; i < VX * VY; i += 32 * kFxTail) {
           const int64_t x = x1 + i % VX, y = y1 + i / VX;
-          if (x > g.nx || y > g.ny || !MFWH_IDX(g.fault, y * g.sy + x, g.points)) continue;
+          if (x > g.nx || y > g.ny || !MFWH_IDX(g.fault, y * g.sy + x, g.points) ||
+              !in_sums(qt + (NF - 1) * kFxTile + i))
+            continue;
           const bool is = x > 0 && x < g.nx && y > 0 && y < g.ny;
           fx_finish<NF>(qt + i, s_unit, is, vout, vsub, a, g.points, y * g.sy + x);
         }
