@@ -729,6 +729,7 @@ mfwh_status apply_pi_fx(mfwh_handle_t h, const double* vin, double* vout, int fo
   a.wexp = h->fx_wexp;
   a.wsum = h->fx_wsum;
   a.warps = h->fx_nw;
+  a.sms = h->sms;
   a.cos_host = P.cosf.data();
   a.dt2 = dt * dt;
   a.forced = forced;

@@ -140,6 +140,7 @@ struct FxHost {
   const int* wexp;
   int wsum;                  // sum_n |wint| < 2^wsum
   int warps;                 // step warps of a CTA (fx_warps)
+  int sms;                   // of the device
   const double* cos_host;    // [(N_t + 1) * nf] cos(omega~_m t^n)
   double dt2;
   int n0, steps;             // first level, steps of this launch

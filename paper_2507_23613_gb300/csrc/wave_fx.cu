@@ -293,13 +293,14 @@ void launch_fx2d(int nf, const Geom& g, const FxArrays& in, const FxArrays& out,
         a.glf[m * 8 + s] = std::ldexp((float)lo, -32);
       }
     const unsigned bx = (unsigned)((g.nx + 30) / 32), by = (unsigned)((g.ny + 6) / 8);
-    const unsigned cap = bx < 608 ? 608 / bx : 1;   // blocks: what 152 SMs hold
+    const unsigned held = 4u * (unsigned)h.sms;   // blocks that the SMs hold
+    const unsigned cap = bx < held ? held / bx : 1;
     auto* fn = g.order == 4 ? k_fx_force<4> : k_fx_force<8>;
     const dim3 grid(bx, by < cap ? by : cap);
     const FxState* state = h.state + h.n0 / fx_launch_steps(g.order) % 3;
     // A dependent launch saves 2 us; of more blocks than a few SMs hold, those that come early fill
     // the SMs that k_fx2d leaves idle and take longer there (401^2, N_f = 16: 9.4 ms against 8.1 a map).
-    if (grid.x * grid.y <= 128)
+    if (grid.x * grid.y < (unsigned)h.sms)
       launch_dependent(fn, grid, dim3(32, 4), 0, st, h.f, h.force, a, h.scale, state, g);
     else
       fn<<<grid, dim3(32, 4), 0, st>>>(h.f, h.force, a, h.scale, state, g);
