@@ -319,7 +319,8 @@ k_conv_tc(const __nv_bfloat16* __restrict__ in, const __nv_bfloat16* __restrict_
 // tensor-core product would round it; 2 * 9 * Cin * Cout flops per pixel).
 //
 // A persistent CTA of 8 warps walks over strips of the images (up to kWgX columns by kWgRows
-// rows of one image).  The rows it needs are in shared memory: four rows of `in` (the three of
+// rows of one image, fewer where the images make fewer strips than CTAs: one row after the other,
+// each behind a barrier, a strip of 16 rows takes 16 us however few columns it has).  The rows it needs are in shared memory: four rows of `in` (the three of
 // the window and the one being copied) and two of g, copied a row ahead by cp.async.  A warp
 // takes CO output channels and one part of the strip's columns, a lane one input channel (Cp < 32:
 // 32 / Cp lanes share a channel and split the columns again).  The lane keeps its CO x 9 sums and
@@ -337,7 +338,7 @@ __host__ __device__ constexpr int wgrad_parts(int cout) {
 template <int CO>
 __global__ void __launch_bounds__(32 * kWgWarps, 2)
 k_wgrad(const __nv_bfloat16* __restrict__ in, const float* __restrict__ g, int Cp, int Cin,
-        int Cout, int Gp, int B, int H, int W, int xc, int chunks, int segs,
+        int Cout, int Gp, int B, int H, int W, int xc, int chunks, int rows, int segs,
         float* __restrict__ part) {
   extern __shared__ __align__(16) unsigned char wg_smem[];
   const int inrow = (xc + 2) * Cp;                                   // BF16 values of a row
@@ -358,7 +359,7 @@ k_wgrad(const __nv_bfloat16* __restrict__ in, const float* __restrict__ g, int C
   for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
     const int seg = (int)(it % segs), ch = (int)(it / segs % chunks), b = (int)(it / segs / chunks);
     const int x0 = ch * xc, xn = W - x0 < xc ? W - x0 : xc;
-    const int y0 = seg * kWgRows, yn = H - y0 < kWgRows ? H - y0 : kWgRows;
+    const int y0 = seg * rows, yn = H - y0 < rows ? H - y0 : rows;
     // copy row y of `in` (columns x0 - 1 .. x0 + xn, zeros outside the image) into slot y & 3
     auto copy_in = [&](int y) {
       const int per = Cp / 8, n = (xn + 2) * per;
@@ -711,17 +712,19 @@ void wgrad(mfwh_cnn_t c, int l, const float* g, int B, int H, int W) {
   const int cin = c->cin[l], cout = c->cout[l], cp = chan_pad(cin);
   const int gp = cout == 1 ? 1 : chan_pad(cout);
   const int chunks = (W + kWgX - 1) / kWgX, xc = (W + chunks - 1) / chunks;   // even strips
-  const int segs = (H + kWgRows - 1) / kWgRows;
+  const int64_t want = ((int64_t)B * chunks * H + 2 * c->sms - 1) / (2 * c->sms);
+  const int rows = (int)std::min<int64_t>(kWgRows, std::max<int64_t>(2, want));
+  const int segs = (H + rows - 1) / rows;
   const int blocks =
       (int)std::min<int64_t>((int64_t)B * chunks * segs, (int64_t)2 * c->sms);
   const size_t smem = (size_t)4 * (xc + 2) * cp * 2 + (size_t)2 * xc * gp * 4;
   const int E = cout * cin * 9 + cout;
   if (cout == 1)
     k_wgrad<1><<<blocks, 32 * kWgWarps, smem, c->stream>>>(c->act[l], g, cp, cin, cout, gp, B, H,
-                                                           W, xc, chunks, segs, c->wpart);
+                                                           W, xc, chunks, rows, segs, c->wpart);
   else
     k_wgrad<8><<<blocks, 32 * kWgWarps, smem, c->stream>>>(c->act[l], g, cp, cin, cout, gp, B, H,
-                                                           W, xc, chunks, segs, c->wpart);
+                                                           W, xc, chunks, rows, segs, c->wpart);
   k_wgrad_sum<<<(E + 31) / 32, 256, 0, c->stream>>>(c->wpart, blocks * wgrad_parts(cout), E,
                                                     c->grad + c->woff[l]);
 }
