@@ -859,11 +859,13 @@ mfwh_status residual_dev(mfwh_handle_t h, const double* v_dev, double* r_out) {
   return MFWH_OK;
 }
 
+}  // namespace
+
 // mfwh_debug_fail_allocations: of this thread's coming workspace allocations, t_fail_after succeed
 // and t_fail_count then report that memory has ended.
-thread_local int t_fail_after = 0, t_fail_count = 0;
+static thread_local int t_fail_after = 0, t_fail_count = 0;
 
-cudaError_t device_alloc(void** p, size_t bytes) {
+cudaError_t mfwh::device_alloc(void** p, size_t bytes) {
   if (t_fail_count > 0 && t_fail_after-- <= 0) {
     t_fail_after = 0;
     --t_fail_count;
@@ -871,6 +873,8 @@ cudaError_t device_alloc(void** p, size_t bytes) {
   }
   return cudaMalloc(p, bytes);
 }
+
+namespace {
 
 // Leaves fixed point for the FP64 kernels, which need less memory.  They read the level arrays on
 // the boundary and write the interior alone, so what fixed point left there (integers, in longer

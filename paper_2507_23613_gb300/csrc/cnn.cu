@@ -18,9 +18,11 @@
 #include <cstring>
 #include <random>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "internal.h"
+#include "kernels.h"
 #include "mfwh.h"
 
 namespace mfwh {
@@ -450,9 +452,10 @@ k_wgrad(const __nv_bfloat16* __restrict__ in, const float* __restrict__ g, int C
   if (lane < CO && co0 + lane < Cout) slot[Cout * Cin * 9 + co0 + lane] = accb;
 }
 
-// out[e] = the sum over the slots of part[slot][e]: 8 interleaved partial sums per output.
+// out[e] = (add: out[e] +) the sum over the slots of part[slot][e]: 8 interleaved partial sums per
+// output.
 __global__ void __launch_bounds__(256)
-k_wgrad_sum(const float* __restrict__ part, int slots, int E, float* __restrict__ out) {
+k_wgrad_sum(const float* __restrict__ part, int slots, int E, int add, float* __restrict__ out) {
   const int e = blockIdx.x * 32 + (threadIdx.x & 31), s0 = threadIdx.x >> 5;
   float v = 0.0f;
   if (e < E)
@@ -463,7 +466,7 @@ k_wgrad_sum(const float* __restrict__ part, int slots, int E, float* __restrict_
   if (s0 == 0 && e < E) {
 #pragma unroll
     for (int i = 1; i < 8; ++i) v += red[i][threadIdx.x];
-    out[e] = v;
+    out[e] = add ? out[e] + v : v;
   }
 }
 
@@ -505,11 +508,11 @@ k_mask_sum(const float* __restrict__ mask, int64_t n, int B, float* __restrict__
 }
 
 // Masked mean squared error: g = 2 (y - t) m / count (FP32, and BF16 images of 8 channels, 7 of
-// them 0), partial sums of (y - t)^2 m per block.
+// them 0), partial sums of (y - t)^2 m per block (add: on those of the images before).
 __global__ void __launch_bounds__(256)
 k_mse(const float* __restrict__ y, const float* __restrict__ t, const float* __restrict__ mask,
       int64_t plane, int64_t n, const float* __restrict__ inv_count, float* __restrict__ g,
-      __nv_bfloat16* __restrict__ gbf, float* __restrict__ part) {
+      __nv_bfloat16* __restrict__ gbf, int add, float* __restrict__ part) {
   const float inv = *inv_count;
   float s = 0.0f;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -528,7 +531,7 @@ k_mse(const float* __restrict__ y, const float* __restrict__ t, const float* __r
   if (threadIdx.x == 0) {
     float v = 0.0f;
     for (int w = 0; w < 8; ++w) v += red[w];
-    part[blockIdx.x] = v;
+    part[blockIdx.x] = add ? part[blockIdx.x] + v : v;
   }
 }
 
@@ -637,6 +640,7 @@ struct mfwh_cnn_s {
   std::vector<int> Kp, Kpt, Np, Npt;
   // activation workspace, sized for cap elements per channel plane times the batch
   int64_t cap = 0;                     // B * H * W the workspace holds
+  int64_t refused = 0;                 // the smallest one that did not fit (0: none so far)
   std::vector<__nv_bfloat16*> act;     // inputs of each layer (BF16), [B][H][W][chan_pad(C)]
   float* y = nullptr;                  // network output [B][1][H][W]
   float* g0 = nullptr;                 // gradients of a layer's output, [B][H][W][chan_pad(C)]
@@ -661,28 +665,57 @@ constexpr int kLossBlocks = 256;
       return cnn_fail(MFWH_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
   } while (0)
 
-mfwh_status ensure_ws(mfwh_cnn_t c, int64_t bhw) {
-  if (bhw <= c->cap) return MFWH_OK;
+void free_ws(mfwh_cnn_t c) {
   for (auto& a : c->act)
     if (a) cudaFree(a);
-  if (c->y) cudaFree(c->y);
-  if (c->g0) cudaFree(c->g0);
-  if (c->g1) cudaFree(c->g1);
+  for (float* b : {c->y, c->g0, c->g1})
+    if (b) cudaFree(b);
   if (c->gbf0) cudaFree(c->gbf0);
   if (c->gbf1) cudaFree(c->gbf1);
   c->y = c->g0 = c->g1 = nullptr;
   c->gbf0 = c->gbf1 = nullptr;
   c->act.assign(c->layers, nullptr);
   c->cap = 0;
+}
+
+cudaError_t alloc_ws(mfwh_cnn_t c, int64_t bhw) {
+  cudaError_t e = cudaSuccess;
+  auto take = [&](auto** p, int64_t n) {
+    void* v = nullptr;
+    if (e == cudaSuccess) e = device_alloc(&v, sizeof(**p) * n);
+    if (e == cudaSuccess) *p = static_cast<std::remove_reference_t<decltype(*p)>>(v);
+  };
   const int gc = chan_pad(c->channels);
-  for (int l = 0; l < c->layers; ++l)
-    CKC(cudaMalloc(&c->act[l], sizeof(__nv_bfloat16) * bhw * chan_pad(c->cin[l])));
-  CKC(cudaMalloc(&c->y, sizeof(float) * bhw));
-  CKC(cudaMalloc(&c->g0, sizeof(float) * bhw * gc));
-  CKC(cudaMalloc(&c->g1, sizeof(float) * bhw * gc));
-  CKC(cudaMalloc(&c->gbf0, sizeof(__nv_bfloat16) * bhw * gc));
-  CKC(cudaMalloc(&c->gbf1, sizeof(__nv_bfloat16) * bhw * gc));
-  c->cap = bhw;
+  for (int l = 0; l < c->layers; ++l) take(&c->act[l], bhw * chan_pad(c->cin[l]));
+  take(&c->y, bhw);
+  take(&c->g0, bhw * gc);
+  take(&c->g1, bhw * gc);
+  take(&c->gbf0, bhw * gc);
+  take(&c->gbf1, bhw * gc);
+  return e;
+}
+
+// Workspace for a batch of B images of hw pixels, or, where memory ends, for as many of them at a
+// time as fit (the padded channels take up to 8 times the memory of the images' own): *images.
+mfwh_status ensure_ws(mfwh_cnn_t c, int B, int64_t hw, int* images) {
+  int n = B;
+  if (c->refused > 0 && n * hw >= c->refused && c->cap >= hw) n = (int)(c->cap / hw);
+  while (n * hw > c->cap) {
+    free_ws(c);
+    const cudaError_t e = alloc_ws(c, n * hw);
+    if (e == cudaSuccess) {
+      c->cap = n * hw;
+      break;
+    }
+    free_ws(c);
+    if (e != cudaErrorMemoryAllocation || n == 1)
+      return cnn_fail(e == cudaErrorMemoryAllocation ? MFWH_ERR_NOMEM : MFWH_ERR_CUDA,
+                      std::string("cnn workspace: ") + cudaGetErrorString(e));
+    (void)cudaGetLastError();
+    c->refused = c->refused > 0 ? std::min(c->refused, n * hw) : n * hw;
+    n = (n + 1) / 2;
+  }
+  *images = std::min(n, B);
   return MFWH_OK;
 }
 
@@ -707,8 +740,8 @@ void conv(mfwh_cnn_t c, const __nv_bfloat16* in, const __nv_bfloat16* Wk, const 
 }
 
 // Weight and bias gradients of layer l from the gradient g of its output, into c->grad (w and b
-// of a layer are adjacent in the flat parameter vector).
-void wgrad(mfwh_cnn_t c, int l, const float* g, int B, int H, int W) {
+// of a layer are adjacent in the flat parameter vector); add: added to those of the images before.
+void wgrad(mfwh_cnn_t c, int l, const float* g, int B, int H, int W, int add) {
   const int cin = c->cin[l], cout = c->cout[l], cp = chan_pad(cin);
   const int gp = cout == 1 ? 1 : chan_pad(cout);
   const int chunks = (W + kWgX - 1) / kWgX, xc = (W + chunks - 1) / chunks;   // even strips
@@ -726,7 +759,7 @@ void wgrad(mfwh_cnn_t c, int l, const float* g, int B, int H, int W) {
     k_wgrad<8><<<blocks, 32 * kWgWarps, smem, c->stream>>>(c->act[l], g, cp, cin, cout, gp, B, H,
                                                            W, xc, chunks, rows, segs, c->wpart);
   k_wgrad_sum<<<(E + 31) / 32, 256, 0, c->stream>>>(c->wpart, blocks * wgrad_parts(cout), E,
-                                                    c->grad + c->woff[l]);
+                                                    add, c->grad + c->woff[l]);
 }
 
 // The convolution kernels' shared-memory limit, once per device.
@@ -766,11 +799,10 @@ mfwh_status pack_all(mfwh_cnn_t c) {
   return MFWH_OK;
 }
 
-// The network on planar images x; its output (one channel) to y.
+// The network on planar images x (as many as the workspace holds at most); its output (one
+// channel) to y.
 mfwh_status forward_impl(mfwh_cnn_t c, const float* x, int B, int H, int W, float* y) {
   const int64_t bhw = (int64_t)B * H * W;
-  mfwh_status st = ensure_ws(c, bhw);
-  if (st != MFWH_OK) return st;
   k_to_images<<<8 * c->sms, 256, 0, c->stream>>>(x, c->act[0], c->in_channels,
                                                  chan_pad(c->in_channels), (int64_t)H * W, bhw);
   for (int l = 0; l < c->layers; ++l) {
@@ -898,31 +930,42 @@ mfwh_status mfwh_cnn_get_params(mfwh_cnn_t c, float* host, float* grads_host, in
 mfwh_status mfwh_cnn_forward(mfwh_cnn_t c, const float* x, int B, int H, int W, float* y) {
   if (!c || !x || !y || B < 1 || H < 1 || W < 1)
     return cnn_fail(MFWH_ERR_INVALID_ARG, "cnn: bad forward arguments");
-  return forward_impl(c, x, B, H, W, y);
+  const int64_t hw = (int64_t)H * W;
+  int images = 0;
+  mfwh_status st = ensure_ws(c, B, hw, &images);
+  for (int b = 0; b < B && st == MFWH_OK; b += images)
+    st = forward_impl(c, x + b * hw * c->in_channels, std::min(images, B - b), H, W, y + b * hw);
+  return st;
 }
 
 mfwh_status mfwh_cnn_train_step(mfwh_cnn_t c, const float* x, const float* target,
                                 const float* mask, int B, int H, int W, float lr, float* loss) {
   if (!c || !x || !target || !mask || B < 1 || H < 1 || W < 1 || !(lr > 0.0f))
     return cnn_fail(MFWH_ERR_INVALID_ARG, "cnn: bad training arguments");
-  mfwh_status st = ensure_ws(c, (int64_t)B * H * W);
-  if (st == MFWH_OK) st = forward_impl(c, x, B, H, W, c->y);
+  const int64_t hw = (int64_t)H * W;
+  int images = 0;
+  mfwh_status st = ensure_ws(c, B, hw, &images);
   if (st != MFWH_OK) return st;
-  const int64_t hw = (int64_t)H * W, n = (int64_t)B * hw;
-  float* g = c->g0;
-  float* gnext = c->g1;
-  __nv_bfloat16* gb = c->gbf0;
-  __nv_bfloat16* gbnext = c->gbf1;
   float* inv = c->part + kLossBlocks;
   k_mask_sum<<<1, 1024, 0, c->stream>>>(mask, hw, B, inv);
-  k_mse<<<kLossBlocks, 256, 0, c->stream>>>(c->y, target, mask, hw, n, inv, g, gb, c->part);
-  for (int l = c->layers - 1; l >= 0; --l) {
-    wgrad(c, l, g, B, H, W);
-    if (l > 0) {   // the input gradient, through the ReLU of the layer below
-      conv(c, gb, c->Wt[l], nullptr, c->cout[l], c->cin[l], c->Kpt[l], c->Npt[l], B, H, W, 0,
-           c->act[l], gbnext, gnext);
-      std::swap(g, gnext);
-      std::swap(gb, gbnext);
+  for (int b = 0; b < B; b += images) {
+    const int n = std::min(images, B - b);
+    st = forward_impl(c, x + b * hw * c->in_channels, n, H, W, c->y);
+    if (st != MFWH_OK) return st;
+    float* g = c->g0;
+    float* gnext = c->g1;
+    __nv_bfloat16* gb = c->gbf0;
+    __nv_bfloat16* gbnext = c->gbf1;
+    k_mse<<<kLossBlocks, 256, 0, c->stream>>>(c->y, target + b * hw, mask, hw, n * hw, inv, g, gb,
+                                              b > 0, c->part);
+    for (int l = c->layers - 1; l >= 0; --l) {
+      wgrad(c, l, g, n, H, W, b > 0);
+      if (l > 0) {   // the input gradient, through the ReLU of the layer below
+        conv(c, gb, c->Wt[l], nullptr, c->cout[l], c->cin[l], c->Kpt[l], c->Npt[l], n, H, W, 0,
+             c->act[l], gbnext, gnext);
+        std::swap(g, gnext);
+        std::swap(gb, gbnext);
+      }
     }
   }
   c->step++;
@@ -944,10 +987,9 @@ mfwh_status mfwh_cnn_train_step(mfwh_cnn_t c, const float* x, const float* targe
 void mfwh_cnn_destroy(mfwh_cnn_t c) {
   if (!c) return;
   cudaStreamSynchronize(c->stream);
-  for (float* b : {c->p, c->grad, c->m, c->v, c->y, c->g0, c->g1, c->part, c->wpart})
+  free_ws(c);
+  for (float* b : {c->p, c->grad, c->m, c->v, c->part, c->wpart})
     if (b) cudaFree(b);
-  if (c->gbf0) cudaFree(c->gbf0);
-  if (c->gbf1) cudaFree(c->gbf1);
   for (auto* w : c->Wk)
     if (w) cudaFree(w);
   for (auto* w : c->Wt)

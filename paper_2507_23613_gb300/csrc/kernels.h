@@ -168,6 +168,9 @@ void launch_fx_init(int nf, const Geom& g, const double* v, int64_t* W, int64_t*
 void launch_fx2d(int nf, const Geom& g, const FxArrays& in, const FxArrays& out, int64_t* q,
                  double* vout, const double* vsub, const FxHost& h, cudaStream_t st);
 
+// cudaMalloc of a workspace; fails as mfwh_debug_fail_allocations says (api.cu).
+cudaError_t device_alloc(void** p, size_t bytes);
+
 // ---- Programmatic dependent launch ---------------------------------------------------
 #ifdef __CUDACC__
 // A step kernel launched by launch_dependent starts once every block of the launch before has called
