@@ -54,20 +54,28 @@ typedef enum {
 } mfwh_status;
 
 enum { MFWH_FILTER_OPTIMIZED = 0, MFWH_FILTER_TRADITIONAL = 1, MFWH_FILTER_USER = 2 };
-/* Arithmetic of the wave solve.  FP64: wave levels, steps and the filter solve at least as accurate
-   as in FP64.  Explicit steps in 2D with a constant or two-layer c advance 64-bit integers in
-   units of a quantum of 2^-58 to 2^-51 of the largest level, which follows that level, over the
-   whole range of double; beyond (infinities, NaN, magnitudes outside 1e-250 .. 1e250) they step
-   in FP64.  The other explicit FP64 problems (3D, a c^2 field, grids with dt^2 c^2 / h^2 below
-   2^-10, at least 1 or a multiple of 2^-24 along an axis, grids of very few rows or columns) keep
-   wave levels in FP64 and the filter sums q_m as unevaluated float pairs (hi + lo, updated with
-   two-product/two-sum on the FP32 pipe, about 2^-47 relative per update), so their magnitudes
-   must stay below the float range (3.4e38) and keep full accuracy above about 1e-30.  FP32_KAHAN: wave levels and
-   steps in FP32 (increment form of the leapfrog scheme), filter sums with a Kahan update at
-   every step; the filter solve B^{-1} q, GMRES and the residual stay FP64.  FP32_BLOCKSUM:
-   as FP32_KAHAN, but a blocked launch of T steps sums its T filter terms in plain FP32 and
-   folds that partial sum into the Kahan pair once (compensated across launches); with one
-   step per launch it is FP32_KAHAN. */
+/* Arithmetic of the wave solve.  FP64: the filter solve, GMRES and the residual in FP64, and the wave
+   levels, steps and filter sums in one of two ways.
+   Explicit steps in 2D with a constant or two-layer c advance 64-bit integers in units of a quantum
+   of 2^-58 to 2^-51 of the largest level, which follows that level over the whole range of double;
+   beyond (infinities, NaN, magnitudes outside 1e-250 .. 1e250) they step in FP64.  The error of V
+   is then relative to the largest values on the grid.  In the maximum norm it was 1e-15 to 1.3e-10 of
+   max |V| in maps of 100 to 3000 steps and short solves, where the FP64 kernels had 2e-14 to
+   2.3e-10, and for iterates that fill the grid it was no larger at values down to 1e-8 of the
+   largest either.  Where a field decays steeply (ahead of a wave front, around a source 2^-20 of
+   another's), values below about 1e-5 of the largest keep fewer correct digits than FP64 steps give
+   them; a c^2 given at every point (MFWH_C_FIELD, 1 for a constant c) selects FP64 steps.
+   The other explicit FP64 problems (3D, a c^2 field, grids with dt^2 c^2 / h^2 below 2^-10, at least 1
+   or a multiple of 2^-24 along an axis (fourth order: / 12), grids of very few rows or columns, fewer
+   than 24 steps, and handles whose workspace does not fit) keep wave levels in FP64, accurate
+   relative to the local values, and the filter sums q_m as unevaluated float pairs (hi + lo, updated
+   with two-product/two-sum on the FP32 pipe, about 2^-47 relative per update), so their magnitudes
+   must stay below the float range (3.4e38) and keep full accuracy above about 1e-30.
+   FP32_KAHAN: wave levels and steps in FP32 (increment form of the leapfrog scheme), filter sums with
+   a Kahan update at every step; the filter solve B^{-1} q, GMRES and the residual stay FP64.
+   FP32_BLOCKSUM: as FP32_KAHAN, but the terms of T steps (time_block) are summed in plain FP32 and
+   that partial sum is folded into the Kahan pair once (compensated across them); with a time_block
+   of 1 it is FP32_KAHAN. */
 enum { MFWH_PREC_FP64 = 0, MFWH_PREC_FP32_KAHAN = 1, MFWH_PREC_FP32_BLOCKSUM = 2 };
 /* How the filter sums become the next iterate (Section "The MFWH algorithm"). */
 enum { MFWH_UPDATE_IMPLICIT = 0, MFWH_UPDATE_EXPLICIT = 1 };
@@ -106,25 +114,25 @@ typedef struct {
                                 8 whatever this says, for the fourth order 4; other FP64 2D
                                 problems of up to 8 frequencies with second order, explicit steps
                                 and constant or two-layer c: 3 on tile shape 5; else 1),
-                                1 = one step per kernel launch (FP32 3D, second order, beyond L2: the
-                                same sums in launches of 4); 2D: 2, 3, 4 or 8 for FP64,
-                                4, 8 or 16 for FP32 = temporal blocking with that depth; 3D: 2 or
-                                4 for the FP32 precisions (grids that L2 holds: one step per
-                                launch with the sums of that depth).  Results are bit-identical for every
+                                1 = one step per kernel launch; 2D: 2, 3, 4 or 8 for FP64, 4, 8
+                                or 16 for FP32 = temporal blocking with that depth; 3D: 2 or 4
+                                for the FP32 precisions.  FP32 3D problems of second order make
+                                the sums of their depth in launches of that depth (Kahan sums: 4)
+                                or of one step, whichever is faster.  Results are bit-identical for every
                                 depth (FP32_BLOCKSUM: for every depth with the same partial-sum
                                 length). */
   int order;                 /* order p of the spatial operator L_{ph}: 2 (0 means 2) or 4.
                                 Order 4: (-W_{j-2} + 16 W_{j-1} - 30 W_j + 16 W_{j+1} - W_{j+2})
                                 / (12 h^2) per axis, ghost values W_{-1} = -W_1 and
                                 W_{N+1} = -W_{N-1} (odd reflection of homogeneous Dirichlet data),
-                                time step limit sqrt(3)/2 of the second-order one, one step
-                                per kernel launch (time_block 0 or 1) */
+                                time step limit sqrt(3)/2 of the second-order one, time_block 0
+                                or 1 */
   int filter_update;         /* MFWH_UPDATE_IMPLICIT (0, default): B V^{k+1} = q, the implicit
                                 filter of eq. vkUpdate; MFWH_UPDATE_EXPLICIT: B_mm V_m^{k+1} =
                                 q_m - sum_{j != m} B_mj V_j^k, the explicit filter of the
                                 footnote to eq. filterII (same fixed point) */
   int tile_shape;            /* FP32: 0, 1 or 2, no effect (the 2D blocked kernel has one tile:
-                                128x64 points with the halo).  FP64 blocked kernel tile (points x by
+                                128x64 points with the halo, or fewer, by the grid).  FP64 blocked kernel tile (points x by
                                 y): 0 = 32x64, 512 threads; 1 = 32x32, 512 threads; 2 = 32x48,
                                 512 threads; 3 = 32x32, 256 threads, two CTAs per SM; 4 =
                                 32x16, 512 threads, two CTAs per SM; 5 = 32x16 tiles stepped by
