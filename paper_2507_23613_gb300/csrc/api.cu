@@ -143,8 +143,9 @@ struct mfwh_handle_s {
   cudaEvent_t gev[2] = {};          // orders gstream after / before the caller's stream
   double* g_in = nullptr;
   double* g_out = nullptr;
-  cudaGraphExec_t gexec[32] = {};
-  int64_t g_steps[32] = {}, g_total[32] = {};
+  cudaGraphExec_t gexec[64] = {};
+  int64_t g_steps[64] = {}, g_total[64] = {};
+  int share = 1;                    // wave solves that have the device at the same time (batches)
   int tune_steps = 0;               // autotuner only: stop the wave solve after this many steps
   double* vec_r = nullptr;          // outer residual of the refined solve [nf][P] (lazy)
   double* vec_e = nullptr;          // correction of the refined solve [nf][P] (lazy)
@@ -342,6 +343,7 @@ mfwh_status apply_pi32(mfwh_handle_t h, const double* vin, double* vout, int for
     a.first_hi = first_hi;
     a.wq_host = h->wq32_h.data();
     a.fc_host = h->fc32_h.data();
+    a.sms = h->share > 1 ? 1 : h->sms;   // (1: tiles of least work in all)
     a.wq = h->wq32;
     a.fc = h->fc32;
     a.binv = h->sh.binv;
@@ -768,7 +770,7 @@ mfwh_status apply_pi(mfwh_handle_t h, const double* vin, double* vout, int force
       h->implicit)
     return apply_pi_direct(h, vin, vout, forced, vsub, add);
   const int key = (vin ? 1 : 0) | (forced ? 2 : 0) | (vsub ? 4 : 0) | (h->use32 ? 8 : 0) |
-                  (add ? 16 : 0);
+                  (add ? 16 : 0) | (h->share > 1 ? 32 : 0);
   cudaStream_t st = h->gstream;
   CK(cudaEventRecord(h->gev[0], h->stream));
   CK(cudaStreamWaitEvent(st, h->gev[0], 0));
@@ -1915,6 +1917,7 @@ mfwh_status mfwh_solve_batch(const mfwh_handle_t* handles, int count, int restar
       if (status[i] != MFWH_OK) msg[i] = g_error;
     }
   };
+  for (int i = 0; i < count; ++i) handles[i]->share = (int)groups.size();
   std::vector<std::thread> pool;
   pool.reserve(groups.size());
   for (auto& grp : groups) pool.emplace_back(work, &grp);
@@ -1922,6 +1925,7 @@ mfwh_status mfwh_solve_batch(const mfwh_handle_t* handles, int count, int restar
   t0 = std::chrono::steady_clock::now();
   go.store(true);
   for (auto& t : pool) t.join();
+  for (int i = 0; i < count; ++i) handles[i]->share = 1;
   if (seconds)
     for (int i = 0; i < count; ++i) seconds[i] = secs[i];
   for (int i = 0; i < count; ++i)
@@ -2105,8 +2109,10 @@ mfwh_status mfwh_solve_batch_graph(const mfwh_handle_t* handles, int count, int 
     if (cap) cudaStreamDestroy(cap);
   };
   for (auto& P : Ps) {
+    P.h->share = count;
     for (int k = 0; k < 2 && st == MFWH_OK; ++k)
       st = capture_child(P.h, cap, k, &P.child[k], &P.child_steps[k], &P.child_total[k]);
+    P.h->share = 1;
     if (st != MFWH_OK) {
       restore();
       return st;

@@ -222,6 +222,7 @@ struct TB32Host {
   Coef32 reg_lo, reg_hi, first_lo, first_hi;
   const float* wq_host;    // [(N_t + 1) * nf] (a launch's weights travel as parameters)
   const float* fc_host;    // [N_t * nf]
+  int sms;                 // that the wave solve has (a batch shares the device's)
   const float* wq;         // the same on the device (small 2D grids)
   const float* fc;
   const double* binv;      // host [MFWH_MAX_NF * MFWH_MAX_NF], row-major, leading dim 16 (C)

@@ -1108,7 +1108,9 @@ void init32_nf(const Geom& g, const double* v, float* W0, float* qs, float* qc, 
 
 // Step warps of k_tb2d32: a launch takes about as many rounds as the grid has tiles per SM, of a time
 // that grows with the tile's rows (step warps and, more with more frequencies, sums of the rows
-// owned).
+// owned).  Problems of a batch share the SMs: with each one's tiles for the whole device, whose halos
+// are more work in all, six of 257^2 to 1025^2 took 65.0 ms for a map and four products, and take
+// 61.8 with tiles as for one SM.
 inline int rt_warps(const Geom& g, int nf, int T, int sms) {
   const int64_t tx = (g.nx + kRtEX - 2 * T) / (kRtEX - 2 * T);
   int best = kRtWarps;
@@ -1143,25 +1145,22 @@ void tb32_launch(const Geom& g, const float* W_in, const float* D_in, float* W_o
                  const float* f, float* qs, float* qc, double* vout, const double* vsub,
                  const TB32Host& h, cudaStream_t st) {
   constexpr size_t smem = rt32_smem_bytes<T>();
-  static int sms[64] = {};   // SMs of the device; the attributes are set on first use
+  static bool configured[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
-  int n = (dev >= 0 && dev < 64) ? sms[dev] : 0;
-  if (n == 0) {
+  if (dev < 0 || dev >= 64 || !configured[dev]) {
     cudaFuncSetAttribute(k_tb2d32<NF, T, ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);
     if constexpr (NF >= kRingNF)
       cudaFuncSetAttribute(k_ring2d32<NF, T, ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)ring_smem_bytes<NF, T>());
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
-      n = 1;
-    if (dev >= 0 && dev < 64) sms[dev] = n;
+    if (dev >= 0 && dev < 64) configured[dev] = true;
   }
   const Last32Binv<NF> b = binv_args<NF>(h.binv, h.emat, h.has_e, h.vprev);
   if constexpr (NF >= kRingNF) {
     constexpr int BY = kRingRows * ring_k(NF);
     const dim3 grid((unsigned)((g.nx + kRingX) / kRingX), (unsigned)((g.ny + BY) / BY));
-    if (ring_faster(g, NF, T, ACC == 0, h.forced, n)) {
+    if (ring_faster(g, NF, T, ACC == 0, h.forced, h.sms)) {
       const RingArgs r{h.reg_lo, h.reg_hi, h.first_lo, h.first_hi, h.n0, h.steps, h.forced, h.last,
                        vsub != nullptr};
       launch_dependent(k_ring2d32<NF, T, ACC>, grid, dim3(kRingThreads), ring_smem_bytes<NF, T>(), st,
@@ -1179,7 +1178,7 @@ void tb32_launch(const Geom& g, const float* W_in, const float* D_in, float* W_o
   a.forced = h.forced;
   a.last = h.last;
   a.subtract = vsub != nullptr;
-  a.warps = rt_warps(g, NF, T, n);
+  a.warps = rt_warps(g, NF, T, h.sms);
   for (int s = 0; s < T; ++s)
     for (int m = 0; m < NF; ++m) {
       a.wq[s * NF + m] = s < h.steps ? h.wq_host[(size_t)(h.n0 + s + 1) * NF + m] : 0.0f;
@@ -1189,7 +1188,7 @@ void tb32_launch(const Geom& g, const float* W_in, const float* D_in, float* W_o
   const int VY = 4 * a.warps - 2 * T;
   const dim3 grid((unsigned)((g.nx + VX) / VX), (unsigned)((g.ny + VY) / VY));
   launch_dependent(k_tb2d32<NF, T, ACC>, grid, dim3(kRtThreads), smem, st, W_in, D_in, W_out, D_out, f, qs, qc, vout,
-                                                       vsub, a, b, g);
+                   vsub, a, b, g);
 }
 
 template <int NF, int T>
