@@ -320,7 +320,9 @@ constexpr size_t rt32_smem_bytes() {
                           (size_t)2 * kRtWarps * 2 * kRtEX);
 }
 
-template <int NF, int T, int ACC>
+// FULL: all kRtWarps warps step (with their number at run time the loop over the sums is 4 to 20 %
+// slower above 6 frequencies: 769^2, N_f = 16, depth 16, partial sums, 82 us a launch and 91).
+template <int NF, int T, int ACC, bool FULL>
 __global__ void __launch_bounds__(kRtThreads, 1)
 k_tb2d32(const float* W_in, const float* D_in,
          float* __restrict__ W_out, float* __restrict__ D_out, const float* __restrict__ f,
@@ -330,7 +332,8 @@ k_tb2d32(const float* W_in, const float* D_in,
   pdl_begin();
   constexpr int VX = kRtEX - 2 * T, VYM = kRtEY - 2 * T;   // owned columns, rows at most
   static_assert(T % 4 == 0 && VX > 0 && VYM > 0, "owned points are whole 4 x 4 blocks");
-  const int VY = 4 * a.warps - 2 * T;                      // owned rows
+  const int warps = FULL ? kRtWarps : a.warps;             // that step
+  const int VY = 4 * warps - 2 * T;                        // owned rows
   extern __shared__ __align__(16) float sm32[];
   float* hist = sm32;                       // [T][VYM][VX] owned values step by step
   float* edge = sm32 + T * VX * VYM;        // [2][warp][top, bottom][128] edge rows
@@ -346,7 +349,7 @@ k_tb2d32(const float* W_in, const float* D_in,
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int64_t y = gy + k;
-    const bool row = warp < a.warps && y >= 0 && y <= g.ny;
+    const bool row = warp < warps && y >= 0 && y <= g.ny;
     const int64_t base = y * g.syw + gx;
     if (row && gx >= 0 && gx + 3 <= g.nx) {
       const float4 v = *reinterpret_cast<const float4*>(W_in + base);
@@ -1108,19 +1111,23 @@ void init32_nf(const Geom& g, const double* v, float* W0, float* qs, float* qc, 
 
 // Step warps of k_tb2d32: a launch takes about as many rounds as the grid has tiles per SM, of a time
 // that grows with the tile's rows (step warps and, more with more frequencies, sums of the rows
-// owned).  Problems of a batch share the SMs: with each one's tiles for the whole device, whose halos
-// are more work in all, six of 257^2 to 1025^2 took 65.0 ms for a map and four products, and take
-// 61.8 with tiles as for one SM.
+// owned).  Lower tiles have to promise 5 % (7 % above 12 frequencies, 10 % at depth 16, where the
+// promise of a grid of just over a round of tiles is not kept: 1501 x 301, N_f = 4, forced, 60.8 us a
+// launch with 160 tiles of 64 rows, 67.9 with 208 of 56).  Problems of a batch share the SMs: with
+// each one's tiles for the whole device, whose halos are more work in all, six of 257^2 to 1025^2
+// took 65.0 ms for a map and four products, and take 61.8 with tiles as for one SM.
 inline int rt_warps(const Geom& g, int nf, int T, int sms) {
   const int64_t tx = (g.nx + kRtEX - 2 * T) / (kRtEX - 2 * T);
+  const double part = T == 16 ? 0.90 : nf > 12 ? 0.93 : 0.95;
   int best = kRtWarps;
   double cost = 0.0;
   for (int w = kRtWarps; w > T / 2; --w) {
     const int vy = 4 * w - 2 * T;
     const int64_t t = tx * ((g.ny + vy) / vy);
     const double r = 0.5 * ((double)((t + sms - 1) / sms) + std::max(1.0, (double)t / sms));
-    const double c = r * (2.0 + w + 0.15 * nf * (w - T / 2));
-    if (w == kRtWarps || c < 0.95 * cost) {
+    const double c = r * (2.0 + w + 0.15 * nf * (w - T / 2)) *
+                     (w < kRtWarps && nf > 6 ? 1.0 + 0.01 * (nf - 6) : 1.0);   // (FULL)
+    if (w == kRtWarps || c < part * cost) {
       best = w;
       cost = c;
     }
@@ -1149,8 +1156,11 @@ void tb32_launch(const Geom& g, const float* W_in, const float* D_in, float* W_o
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64 || !configured[dev]) {
-    cudaFuncSetAttribute(k_tb2d32<NF, T, ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(k_tb2d32<NF, T, ACC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);
+    if constexpr (T >= 8)
+      cudaFuncSetAttribute(k_tb2d32<NF, T, ACC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)smem);
     if constexpr (NF >= kRingNF)
       cudaFuncSetAttribute(k_ring2d32<NF, T, ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)ring_smem_bytes<NF, T>());
@@ -1187,7 +1197,10 @@ void tb32_launch(const Geom& g, const float* W_in, const float* D_in, float* W_o
   constexpr int VX = kRtEX - 2 * T;
   const int VY = 4 * a.warps - 2 * T;
   const dim3 grid((unsigned)((g.nx + VX) / VX), (unsigned)((g.ny + VY) / VY));
-  launch_dependent(k_tb2d32<NF, T, ACC>, grid, dim3(kRtThreads), smem, st, W_in, D_in, W_out, D_out, f, qs, qc, vout,
+  auto* fn = k_tb2d32<NF, T, ACC, false>;
+  if constexpr (T >= 8)
+    if (a.warps == kRtWarps) fn = k_tb2d32<NF, T, ACC, true>;
+  launch_dependent(fn, grid, dim3(kRtThreads), smem, st, W_in, D_in, W_out, D_out, f, qs, qc, vout,
                    vsub, a, b, g);
 }
 
