@@ -322,7 +322,8 @@ k_conv_tc(const __nv_bfloat16* __restrict__ in, const __nv_bfloat16* __restrict_
 //
 // A persistent CTA of 8 warps walks over strips of the images (up to kWgX columns by kWgRows
 // rows of one image, fewer where the images make fewer strips than CTAs: one row after the other,
-// each behind a barrier, a strip of 16 rows takes 16 us however few columns it has).  The rows it needs are in shared memory: four rows of `in` (the three of
+// each behind a barrier, a strip of 16 rows takes 16 us however few columns it has; FULL: kWgRows,
+// known at compile time).  The rows it needs are in shared memory: four rows of `in` (the three of
 // the window and the one being copied) and two of g, copied a row ahead by cp.async.  A warp
 // takes CO output channels and one part of the strip's columns, a lane one input channel (Cp < 32:
 // 32 / Cp lanes share a channel and split the columns again).  The lane keeps its CO x 9 sums and
@@ -337,11 +338,12 @@ __host__ __device__ constexpr int wgrad_parts(int cout) {
   return cout <= 8 ? kWgWarps : (cout <= 16 ? kWgWarps / 2 : kWgWarps / 4);
 }
 
-template <int CO>
+template <int CO, bool FULL>
 __global__ void __launch_bounds__(32 * kWgWarps, 2)
 k_wgrad(const __nv_bfloat16* __restrict__ in, const float* __restrict__ g, int Cp, int Cin,
-        int Cout, int Gp, int B, int H, int W, int xc, int chunks, int rows, int segs,
+        int Cout, int Gp, int B, int H, int W, int xc, int chunks, int rows_arg, int segs,
         float* __restrict__ part) {
+  const int rows = FULL ? kWgRows : rows_arg;
   extern __shared__ __align__(16) unsigned char wg_smem[];
   const int inrow = (xc + 2) * Cp;                                   // BF16 values of a row
   __nv_bfloat16* s_in = reinterpret_cast<__nv_bfloat16*>(wg_smem);   // [4][xc + 2][Cp]
@@ -752,12 +754,11 @@ void wgrad(mfwh_cnn_t c, int l, const float* g, int B, int H, int W, int add) {
       (int)std::min<int64_t>((int64_t)B * chunks * segs, (int64_t)2 * c->sms);
   const size_t smem = (size_t)4 * (xc + 2) * cp * 2 + (size_t)2 * xc * gp * 4;
   const int E = cout * cin * 9 + cout;
-  if (cout == 1)
-    k_wgrad<1><<<blocks, 32 * kWgWarps, smem, c->stream>>>(c->act[l], g, cp, cin, cout, gp, B, H,
-                                                           W, xc, chunks, rows, segs, c->wpart);
-  else
-    k_wgrad<8><<<blocks, 32 * kWgWarps, smem, c->stream>>>(c->act[l], g, cp, cin, cout, gp, B, H,
-                                                           W, xc, chunks, rows, segs, c->wpart);
+  const bool full = rows == kWgRows;
+  auto* fn = cout == 1 ? (full ? k_wgrad<1, true> : k_wgrad<1, false>)
+                       : (full ? k_wgrad<8, true> : k_wgrad<8, false>);
+  fn<<<blocks, 32 * kWgWarps, smem, c->stream>>>(c->act[l], g, cp, cin, cout, gp, B, H, W, xc, chunks,
+                                                 rows, segs, c->wpart);
   k_wgrad_sum<<<(E + 31) / 32, 256, 0, c->stream>>>(c->wpart, blocks * wgrad_parts(cout), E,
                                                     add, c->grad + c->woff[l]);
 }
