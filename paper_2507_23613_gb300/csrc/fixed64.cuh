@@ -5,9 +5,9 @@
 // levels of a wave solve are kept as integers in units of a quantum 2^e that puts a bound of a
 // launch's levels just below 2^59 (fourth order 2^56) and follows it from launch to launch, so
 // additions are exact and the only rounding of a step is that of the product with dt^2 c^2 / h^2, to
-// the nearest quantum: about 2^-55 of the largest level, against the several 2^-53 relative roundings
-// of an FP64 step and the 2^-47 of its float-pair sums.  The functions
-// also compile for the host, where tests compare them with exact arithmetic.
+// the nearest quantum: about 2^-55 of the largest level on the grid, whatever the local one (an FP64
+// step rounds several times to 2^-53 of the local values, its float-pair sums to 2^-47).  The
+// functions also compile for the host, where tests compare them with exact arithmetic.
 #pragma once
 
 #include <cstdint>

@@ -5,10 +5,13 @@
 // F^n), W^{n+1} = W^n + D^{n+1/2} (kappa_0 = dt^2/2 with D^{-1/2} = 0, else dt^2; eq. WaveSchemeA,
 // eq. implicitFirstStep with alpha = 0), W and D as integers in units of the launch's quantum.  A
 // step rounds once per point (the product with kappa c^2 / h^2; a second time for the forcing).
-// The filter sums q_m = sum_n w_{n,m} W^n (eq. pDefQ) are 64-bit integers too; the contribution of
-// a launch's 8 steps is summed exactly, from the weights as two 32-bit digits (58 bits), and
-// rounded once to the unit of the sums.  The filter solve is FP64.  The forcing of a launch's
-// steps is summed over the frequencies by a kernel before it (k_fx_force), once per point.
+// The filter sums q_m = sum_n w_{n,m} W^n (eq. pDefQ) are 64-bit integers too.  The contribution of
+// a launch's 8 steps is formed from the weights' and the levels' two 32-bit digits (60 bits of the
+// weights): high x high and high x low digits are summed exactly, the weights' low digits times the
+// levels' high ones in FP32 (2^-24 of terms below 2^-28 of the largest), low x low is dropped
+// (2^-60), and the sum is rounded once to the unit of the sums.  The filter solve is FP64.  The
+// forcing of a launch's steps is summed over the frequencies by a kernel before it (k_fx_force),
+// once per point, in the same way.
 //
 // The quantum.  A launch knows the largest |W| and |D| of its input (FxState, left by the launch
 // before), and with them bounds every level of its steps: |W^{n+k}| <= gw max |W| + gd max |D| + gf
@@ -42,10 +45,10 @@
 // between the roles); a thread of the tail warps takes owned points one by one and forms their N_f
 // contributions in registers, with the weights as constant operands.  (All of this for the
 // second-order operator; the fourth-order one reaches two points, so a launch makes 4 steps within
-// the same halo, the warps exchange all their rows, and its 68-fold neighbour sums leave the
-// levels 56 bits.)  The sums are laid out tile
-// by tile, [tile][m][owned point], so that their addresses are a pointer plus constants and the
-// loop has no index arithmetic or masks (points outside the interior have zero levels).
+// the same halo, the warps exchange all their rows, and its sums of 64 times a level along an axis
+// leave the levels 56 bits.)  The sums are laid out tile by tile, [tile][m][owned point], so that
+// their addresses are a pointer plus constants and the loop has no index arithmetic or masks (points
+// outside the interior have zero levels).
 #pragma once
 
 #include <cuda_runtime.h>
