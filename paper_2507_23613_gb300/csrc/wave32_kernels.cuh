@@ -280,9 +280,10 @@ k_last32(const float* W, const float* D, const float* __restrict__ f,
 // ---- temporally blocked 2D kernel ----------------------------------------------
 //
 // One CTA per SM (16 warps) holds an extended tile of 128 x 64 points (fewer rows where the grid
-// would leave SMs idle: rt_warps) in registers, W and D of 4 x 4 points per thread: lane l has columns 4l .. 4l + 3, warp w rows 4w .. 4w + 3.  Every step
-// updates all of them (the outermost ring of valid values shrinks by one point a step, so after
-// T steps the (128 - 2T) x (64 - 2T) points in the middle are exact), except that a warp rests
+// would leave SMs idle: rt_warps) in registers, W and D of 4 x 4 points per thread: lane l has
+// columns 4l .. 4l + 3, warp w rows 4w .. 4w + 3.  Every step updates all of them (the outermost
+// ring of valid values shrinks by one point a step, so after T steps the (128 - 2T) x (64 - 2T)
+// points in the middle are exact), except that a warp rests
 // once no later step reads its rows.  Left and right neighbours come from the thread itself or by
 // one shuffle per row and side, vertical neighbours from the thread itself or, above and below
 // its four rows, from the edge rows that the warps exchange through shared memory (double
@@ -1111,14 +1112,14 @@ void init32_nf(const Geom& g, const double* v, float* W0, float* qs, float* qc, 
 
 // Step warps of k_tb2d32: a launch takes about as many rounds as the grid has tiles per SM, of a time
 // that grows with the tile's rows (step warps and, more with more frequencies, sums of the rows
-// owned).  Lower tiles have to promise 5 % (7 % above 12 frequencies, 10 % at depth 16, where the
-// promise of a grid of just over a round of tiles is not kept: 1501 x 301, N_f = 4, forced, 60.8 us a
-// launch with 160 tiles of 64 rows, 67.9 with 208 of 56).  Problems of a batch share the SMs: with
-// each one's tiles for the whole device, whose halos are more work in all, six of 257^2 to 1025^2
-// took 65.0 ms for a map and four products, and take 61.8 with tiles as for one SM.
+// owned).  Lower tiles have to promise 5 % (7 % at depth 8 above 12 frequencies, 10 % at depth 16,
+// where the promise of a grid of just over a round of tiles is not kept: 1501 x 301, N_f = 4, forced,
+// 60.8 us a launch with 160 tiles of 64 rows, 67.9 with 208 of 56).  Problems of a batch share the
+// SMs: with each one's tiles for the whole device, whose halos are more work in all, six of 257^2 to
+// 1025^2 took 65.0 ms for a map and four products, and take 61.8 with tiles as for one SM.
 inline int rt_warps(const Geom& g, int nf, int T, int sms) {
   const int64_t tx = (g.nx + kRtEX - 2 * T) / (kRtEX - 2 * T);
-  const double part = T == 16 ? 0.90 : nf > 12 ? 0.93 : 0.95;
+  const double part = T == 16 ? 0.90 : (T == 8 && nf > 12 ? 0.93 : 0.95);
   int best = kRtWarps;
   double cost = 0.0;
   for (int w = kRtWarps; w > T / 2; --w) {
@@ -1126,7 +1127,7 @@ inline int rt_warps(const Geom& g, int nf, int T, int sms) {
     const int64_t t = tx * ((g.ny + vy) / vy);
     const double r = 0.5 * ((double)((t + sms - 1) / sms) + std::max(1.0, (double)t / sms));
     const double c = r * (2.0 + w + 0.15 * nf * (w - T / 2)) *
-                     (w < kRtWarps && nf > 6 ? 1.0 + 0.01 * (nf - 6) : 1.0);   // (FULL)
+                     (T >= 8 && w < kRtWarps && nf > 6 ? 1.0 + 0.01 * (nf - 6) : 1.0);   // (FULL)
     if (w == kRtWarps || c < part * cost) {
       best = w;
       cost = c;
